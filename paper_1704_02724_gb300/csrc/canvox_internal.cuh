@@ -49,9 +49,14 @@ __host__ __device__ __forceinline__ int64_t leaf_index(const Tree& t, int64_t re
 struct View {
     double eye[3];
     double f[3], u[3], r[3];  // orthonormal frame (Gram-Schmidt from forward)
-    double sx, sy;            // tan * aspect, tan
+    double sy;                // tan
     double aspect;            // width / height
-    double two_over_w, two_over_h;
+    double inv_w, inv_h;      // 1 / width, 1 / height (rounded to nearest)
+    // the eye from the canvas's low corner, in units of 2^-31 canvas sides: eye_unit[a] + eye_rest[a], the rest at
+    // most half a unit (a far eye: 0 and the whole distance)
+    double eye_rest[3];
+    int32_t eye_unit[3];
+    int32_t pad;
     float bg[4];
     int64_t out_offset;
     int64_t ray_begin;  // first ray index of this view in the launch (multiple of 32)
@@ -70,7 +75,6 @@ struct EyePath {
     int32_t len;                 // leaf level (0: not valid, trace from the root)
     uint2 val;                   // leaf value (0, 0 = empty)
     int32_t stored;              // 1 if the leaf has a stored value (slot < 0)
-    int32_t pad[2];
 };
 
 // Counters, in the order of canvox_stats.
@@ -112,6 +116,10 @@ struct MixedParams {
     int32_t smem_records;
     int32_t use_ropes;   // 1: neighbour links (Tree::ropes), 0: stack of ancestors
     int32_t count_reads; // 1: count slot reads, leaf loads and record loads (canvox_stats)
+    // set by launch_mixed
+    double inv_extent, unit;  // 1 / extent, extent 2^-31
+    float side;               // extent
+    float bound_t, bound_i;   // the colour bound of a boundary per local time and per ih (see ray_step)
 };
 
 struct PlainParams {
@@ -153,7 +161,7 @@ cudaError_t footprint_finish(const int32_t* nodes, const int64_t* level_begin, i
                              unsigned long long* d_count, int64_t* n_records, int64_t* n_leaves);
 
 // Host helpers of runtime.cu shared with other entry points.
-int build_views(const canvox_camera* cams, int n, int tile_w, View* out, int64_t* total_rays);
+int build_views(const canvox_camera* cams, int n, int tile_w, double extent, View* out, int64_t* total_rays);
 void builtin_render_opts(canvox_render_opts* o);
 int set_error(int code, const char* msg);
 void clear_error();
@@ -179,15 +187,37 @@ namespace canvox {
 //   d = (f + u r) + v up,  d /= sqrt((d0 d0 + d1 d1) + d2 d2).
 // A ray that lies exactly in a cell plane (d_a == 0) must come out exactly so,
 // since the side of the plane it runs on is decided by this value.
+//
+// The quotients take the reciprocal of their divisor, known for the width and height and formed once for the
+// norm: q = a r, then one correction by the exact remainder (Markstein 1990), 3 FP64 operations each instead of a
+// division's nine or so; the FP64 pipe (1/64 of the FP32 rate) bounds views of few leaves per ray. For the pixel
+// coordinates the result is the rounded quotient always: 2i + 1 < 2^32 and W < 2^31, so a quotient lies at least
+// 2^-32 of an ulp from a rounding boundary, far more than the correction's error of 2^-51.
+__device__ __forceinline__ double rcp64(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));  // about 20 bits; two Newton steps to 53
+    r = fma(fma(-x, r, 1.0), r, r);
+    return fma(fma(-x, r, 1.0), r, r);
+}
+__device__ __forceinline__ double div64(double a, double b, double rcp_b) {
+    const double q = __dmul_rn(a, rcp_b);
+    return fma(fma(-b, q, a), rcp_b, q);
+}
 __device__ __forceinline__ void pixel_ray(const View& V, int i, int j, double d[3]) {
-    const double x = __dadd_rn(__ddiv_rn(2.0 * i + 1.0, (double)V.width), -1.0);
-    const double y = __dsub_rn(1.0, __ddiv_rn(2.0 * j + 1.0, (double)V.height));
+    const double x = __dadd_rn(div64(2.0 * i + 1.0, (double)V.width, V.inv_w), -1.0);
+    const double y = __dsub_rn(1.0, div64(2.0 * j + 1.0, (double)V.height, V.inv_h));
     const double u = __dmul_rn(__dmul_rn(x, V.sy), V.aspect);
     const double v = __dmul_rn(y, V.sy);
 #pragma unroll
     for (int a = 0; a < 3; ++a) d[a] = __dadd_rn(__dadd_rn(V.f[a], __dmul_rn(u, V.r[a])), __dmul_rn(v, V.u[a]));
     const double n = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2])));
+    if (n < 1.0e100) {
+        const double r = rcp64(n);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) d[a] = __ddiv_rn(d[a], n);
+        for (int a = 0; a < 3; ++a) d[a] = div64(d[a], n, r);
+    } else {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) d[a] = __ddiv_rn(d[a], n);
+    }
 }
 }  // namespace canvox

@@ -99,7 +99,7 @@ extern "C" int canvox_render_noalloc(const int32_t* node_pool_dev, int64_t n_rec
     int64_t total_rays = 0;
     canvox_render_opts o;
     builtin_render_opts(&o);
-    int rc = build_views(cams, n_views, o.tile_w, vt.v, &total_rays);
+    int rc = build_views(cams, n_views, o.tile_w, extent, vt.v, &total_rays);
     if (rc) return rc;
     unsigned char* base = nullptr;
     rc = scratch_address(&base);

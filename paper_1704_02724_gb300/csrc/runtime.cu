@@ -187,7 +187,7 @@ bool finite3(const double* v) { return std::isfinite(v[0]) && std::isfinite(v[1]
 double dot3(const double* a, const double* b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; }
 
 // Per-view set-up in FP64: Gram-Schmidt frame from forward, pixel scale factors, tiling.
-int setup_views(const canvox_camera* cams, int n, int tile_w, View* out, int64_t* total_rays) {
+int setup_views(const canvox_camera* cams, int n, int tile_w, double extent, View* out, int64_t* total_rays) {
     const int wl = tile_w == 4 ? 2 : tile_w == 8 ? 3 : tile_w == 16 ? 4 : 5;
     const int tw = 1 << wl, th = 32 >> wl;
     int64_t ray = 0;
@@ -218,9 +218,21 @@ int setup_views(const canvox_camera* cams, int n, int tile_w, View* out, int64_t
         for (int a = 0; a < 3; ++a) V.eye[a] = c.eye[a];
         V.sy = c.tan_half_fov_y;
         V.aspect = (double)c.width / (double)c.height;
-        V.sx = c.tan_half_fov_y * V.aspect;
-        V.two_over_w = 2.0 / (double)c.width;
-        V.two_over_h = 2.0 / (double)c.height;
+        V.inv_w = 1.0 / (double)c.width;
+        V.inv_h = 1.0 / (double)c.height;
+        for (int a = 0; a < 3; ++a) {
+            // eye + half exactly as s + e (Knuth's two-sum); the rest of s over a unit count is exact (one fma)
+            const double half = 0.5 * extent, unit = std::ldexp(extent, -31);
+            const double s = c.eye[a] + half, b = s - c.eye[a], e = (c.eye[a] - (s - b)) + (half - b);
+            const double k = std::nearbyint(s / unit);
+            if (k >= 1.0 && k <= 2147483647.0) {
+                V.eye_unit[a] = (int32_t)k;
+                V.eye_rest[a] = (std::fma(-k, unit, s) + e) / unit;
+            } else {
+                V.eye_unit[a] = 0;
+                V.eye_rest[a] = s / unit;
+            }
+        }
         for (int a = 0; a < 4; ++a) V.bg[a] = c.background[a];
         V.out_offset = c.out_offset_px;
         V.width = c.width;
@@ -481,8 +493,8 @@ int paint_table(int32_t depth, double extent, int64_t* n_records, int64_t* n_lea
 }  // namespace
 
 namespace canvox {
-int build_views(const canvox_camera* cams, int n, int tile_w, View* out, int64_t* total_rays) {
-    return setup_views(cams, n, tile_w, out, total_rays);
+int build_views(const canvox_camera* cams, int n, int tile_w, double extent, View* out, int64_t* total_rays) {
+    return setup_views(cams, n, tile_w, extent, out, total_rays);
 }
 void builtin_render_opts(canvox_render_opts* o) { builtin_defaults(o); }
 int set_error(int code, const char* msg) { return fail(code, "%s", msg); }
@@ -714,7 +726,7 @@ int canvox_render_ex(const canvox_camera* cams, int32_t n_views, float* out_rgba
     if (n_views == 0) return CANVOX_OK;
     std::vector<View> views((size_t)n_views);
     int64_t total_rays = 0;
-    rc = setup_views(cams, n_views, o.tile_w, views.data(), &total_rays);
+    rc = setup_views(cams, n_views, o.tile_w, g.extent, views.data(), &total_rays);
     if (rc) return rc;
     if ((rc = ensure_views(n_views)) || (rc = ensure_scratch(o.per_view ? n_views : 1))) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -920,7 +932,7 @@ int canvox_footprint(const canvox_camera* cams, int32_t n_views, void* stream, i
     if ((rc = resolve_opts(&o, &o))) return rc;
     std::vector<View> views((size_t)(n_views > 0 ? n_views : 1));
     int64_t total_rays = 0;
-    if (n_views > 0 && (rc = setup_views(cams, n_views, o.tile_w, views.data(), &total_rays))) return rc;
+    if (n_views > 0 && (rc = setup_views(cams, n_views, o.tile_w, g.extent, views.data(), &total_rays))) return rc;
     if ((rc = ensure_views(n_views > 0 ? n_views : 1)) || (rc = ensure_scratch(1))) return rc;
     if (g.any_render) CK(cudaEventSynchronize(g.done), "cudaEventSynchronize");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);

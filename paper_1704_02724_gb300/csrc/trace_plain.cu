@@ -210,7 +210,7 @@ __global__ void eye_path_kernel(Tree t, const View* views, int n_views, EyePath*
     E.stored = 0;
     E.val = make_uint2(0u, 0u);
     for (int a = 0; a < 3; ++a)
-        if (!(V.eye[a] >= -t.half && V.eye[a] < t.half)) return;
+        if (!(V.eye[a] > -t.half && V.eye[a] < t.half)) return;  // (on the low face the direction decides)
     unsigned c[3] = {0u, 0u, 0u};
     int32_t rec = 0;
     for (int lev = 0; lev < kMaxDepth; ++lev) {
