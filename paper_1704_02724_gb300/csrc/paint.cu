@@ -22,14 +22,25 @@
 //     first cell s does not descend through lies inside s, or is partially
 //     covered and has its centre inside s.
 // Each level keeps, per refined cell, the ordered list of stamps that still
-// descend (undecided) or already paint its whole subtree (painted); one warp
-// per refined cell classifies that list against its eight children, 32
-// entries at a time (a cell around a room holds tens of thousands of stamps),
-// with each stamp's distances to the cell's three planes per axis shared by
-// the children. Levels of few cells take a warp per child instead, and cells
-// whose lists run long (near the root every stamp is on them; around a room,
-// its stamps) a warp per chunk of a child's list. Geometry is FP64 with the
-// same operations and order as the host painter, so the pools are identical.
+// descend (undecided) or already paint its whole subtree (painted). Eight lanes
+// take a cell, one per child, and walk its list in order: at stamp s a child
+// knows whether an earlier stamp (or s itself) refines it, so one pass gives its
+// firstref, its blend and which stamps its own list keeps; that decision is left
+// as two bits per stamp and child, from which the next level's lists are written.
+// Lists of more than kLongList entries (near the root every stamp is on them;
+// around a room, its stamps) are cut into items of kItem entries that octets
+// take in parallel: first the least refining stamp per child, then the decisions.
+// Geometry is FP32 with a proven margin, retaken in FP64 with the same operations
+// and order as the host painter inside the margin, so the pools are identical.
+//
+// What bounds it: near the root the latency of few octets walking lists, on the
+// levels of millions of cells instruction issue and the gathers of the stamps'
+// records. A lane per child suits the short lists most cells have: with a warp
+// per cell and a lane per stamp (32 stamps at a time, two passes), a list of five
+// left 27 lanes idle and its children were taken one after the other: the depth-24
+// table of 210,000 stamps took 251 ms then and 63 ms now (expand_count 32 ms of it,
+// its issue slots 52 % used at 26 of 48 possible warps), the 1,000 stamps of the
+// depth-8 cube with the read-back 7.5 and 2.4 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -44,12 +55,25 @@ namespace {
 
 constexpr uint64_t kInternal = 1ull << 63;  // child slot: internal cell, low bits = index at the next level
 constexpr uint64_t kNotCollapsed = 1ull << 63;
+constexpr unsigned kFullMask = 0xFFFFFFFFu;
+constexpr int kCells = 16;              // cells per block of the octet kernels (128 threads)
+constexpr int64_t kLongList = 512;      // longer lists are cut into items ...
+constexpr int64_t kItem = 128;          // ... of so many entries, one octet each
+constexpr int32_t kNoStamp = 0x7FFFFFFF;
+
+// What a child box test reads of a stamp: the centre as two FP32 words per axis, the squared radius, the target depth.
+struct StampRec {
+    float ch[3], cl0;
+    float cl1, cl2, r2;
+    int32_t kt;
+};
+static_assert(sizeof(StampRec) == 32, "two 16-byte loads, one L2 sector");
 
 struct StampDev {
-    const double* c;     // [n][3]
-    const double* r2;    // [n]
-    const int32_t* kt;   // [n] target depth
-    const float4* rgba;  // [n]
+    const double* c;       // [n][3]
+    const double* r2;      // [n]
+    const StampRec* rec;   // [n]
+    const float4* rgba;    // [n]
 };
 
 __device__ __forceinline__ double sq(double x) { return __dmul_rn(x, x); }
@@ -94,340 +118,148 @@ struct LevelIn {
     const uint32_t* coord;  // [n][3]
     const int64_t* off;     // [n + 1]
     const int32_t* ent;     // s: descends, ~s: paints the whole cell
+    double h;               // side of the children
+    float hf;
 };
+
+// How a stamp covers a box.
+enum { kOut = 0, kIn = 1, kPartCentreIn = 2, kPartCentreOut = 3 };
+
+// The box of one child. Its low corner is j h with the integer j = child coordinate - 2^level, formed for the screen
+// as two FP32 words without FP64 (whose pipe, converting and adding, bounded the levels of millions of cells at 74 %
+// busy): j as two words too (the second 0 up to 2^24), the product's error from one fma. Within 2^-46 of the
+// corner's own size of the exact one.
+struct Child {
+    uint32_t cc[3];   // child coordinates
+    float lh[3], ll[3];
+    float hf, hh;     // side, half side
+    float g;          // the screen's margin: 2 sides per axis plus 2^-22 of the corner
+};
+
+__device__ __forceinline__ Child child_box(const LevelIn& L, int64_t i, int k) {
+    Child B;
+    B.hf = L.hf;
+    B.hh = 0.5f * L.hf;
+    B.g = 6.0f * L.hf;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        B.cc[a] = 2u * L.coord[3 * i + a] + ((k >> a) & 1u);
+        const int32_t j = (int32_t)B.cc[a] - (1 << L.level);
+        const float jh = __int2float_rn(j), jl = __int2float_rn(j - __float2int_rn(jh));
+        const float p = __fmul_rn(jh, L.hf), t = __fmaf_rn(jl, L.hf, __fmaf_rn(jh, L.hf, -p));
+        B.lh[a] = __fadd_rn(p, t);
+        B.ll[a] = __fsub_rn(t, __fsub_rn(B.lh[a], p));
+        B.g += 2.384185791015625e-07f * fabsf(B.lh[a]);
+    }
+    return B;
+}
+
+// The cover of stamp v in FP64, in the host painter's operations and order (its skipped terms are +0, which is
+// exact). Taken on about one test in ten thousand, so it is kept out of line.
+__device__ __noinline__ int cover64(const double* c, double r2, uint32_t c0, uint32_t c1, uint32_t c2, double h,
+                                    double half) {
+    double dmin[3], dmax[3], cen[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double lo = fma((double)(a == 0 ? c0 : (a == 1 ? c1 : c2)), h, -half), up = __dadd_rn(lo, h);
+        const double A = sq(__dsub_rn(c[a], lo)), B = sq(__dsub_rn(c[a], up));
+        dmin[a] = c[a] < lo ? A : (c[a] > up ? B : 0.0);
+        dmax[a] = fmax(A, B);
+        cen[a] = sq(__dsub_rn(__dadd_rn(lo, 0.5 * h), c[a]));
+    }
+    if (__dadd_rn(__dadd_rn(dmin[0], dmin[1]), dmin[2]) >= r2) return kOut;
+    if (__dadd_rn(__dadd_rn(dmax[0], dmax[1]), dmax[2]) <= r2) return kIn;
+    return __dadd_rn(__dadd_rn(cen[0], cen[1]), cen[2]) < r2 ? kPartCentreIn : kPartCentreOut;
+}
+
+// The cover of a stamp, screened in FP32 (-1: open). With m >= M_a = |c_a - lo_a| + 2 h + 2^-22 |lo_a| on every axis,
+// the difference c_a - lo_a formed from two words each is within 2^-23 M_a of the exact one (the corner's words are
+// within 2^-46 of it, the centre's within 2^-48, and |c_a| <= |lo_a| + M_a), those to the far plane and the centre within 2^-22.4 M_a. The
+// squared distances to the far corner and the centre are then within 2^-20.9 m^2 (margin 2^-18 m^2), that to the box,
+// with n the sum of its terms' roots, within 2^-21.4 m n + 3 2^-44.8 m^2 + 2^-22 of itself (margin twice that and
+// more): a stamp far smaller than the box it lies in has n = 0 and is decided, where a margin in m^2 would leave
+// every room's stamps on every coarse level to FP64. Every comparison is false for a NaN or an infinite margin,
+// which leaves it open.
+__device__ __forceinline__ int cover32(const Child& B, const StampRec& R, bool centre) {
+    const float cl[3] = {R.cl0, R.cl1, R.cl2};
+    float dmin2 = 0.0f, dmax2 = 0.0f, cen2 = 0.0f, m = B.g, n = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float dl = __fadd_rn(__fsub_rn(R.ch[a], B.lh[a]), __fsub_rn(cl[a], B.ll[a]));
+        const float du = __fsub_rn(dl, B.hf), dc = __fsub_rn(dl, B.hh);
+        const float near = fmaxf(fmaxf(-dl, du), 0.0f), far = fmaxf(fabsf(dl), fabsf(du));
+        dmin2 = fmaf(near, near, dmin2);
+        dmax2 = fmaf(far, far, dmax2);
+        cen2 = fmaf(dc, dc, cen2);
+        m += fabsf(dl);
+        n += near;
+    }
+    // 2^-20 m n + 2^-41 m^2 + 2^-21 (dmin2 + r2)
+    const float e = fmaf(m, fmaf(4.547473508864641e-13f, m, 9.5367431640625e-07f * n), 4.76837158203125e-07f * (dmin2 + R.r2));
+    if (dmin2 > R.r2 + e) return kOut;
+    if (!(dmin2 < R.r2 - e)) return -1;
+    const float margin = fmaf(3.814697265625e-06f * m, m, 2.384185791015625e-07f * R.r2);  // 2^-18 m^2 + 2^-22 r2
+    const float lo = R.r2 - margin, hi = R.r2 + margin;
+    if (dmax2 < lo) return kIn;
+    if (!(dmax2 > hi)) return -1;
+    if (!centre || cen2 < lo) return kPartCentreIn;
+    return cen2 > hi ? kPartCentreOut : -1;
+}
+
+// Eight list entries of an octet: lane k loads entry q0 + k and its stamp's record, so the octet's eight loads are in
+// flight at once (one entry after the other, each step of the walk waits for an entry and then for its record, 2.7 us
+// a step on a level of few cells). The records are staged in shared memory, padded so that the four octets of a warp
+// read different banks; on the long lists the next eight are loaded while these are used.
+struct Entries {
+    int64_t q0, e;  // [q0, q0 + m) of the list that ends at e
+    int32_t v;      // lane k's entry
+    int m;
+    float4 x, y;    // its record
+};
+constexpr int kStageRow = 17;  // float4 per octet: eight records and a pad
+__device__ __forceinline__ void load_entries(Entries& E, const LevelIn& L, const StampDev& S, int k) {
+    E.m = (int)max((int64_t)0, min((int64_t)8, E.e - E.q0));
+    E.v = k < E.m ? L.ent[E.q0 + k] : -1;
+    if (E.v >= 0) {
+        const float4* r = reinterpret_cast<const float4*>(S.rec + E.v);
+        E.x = __ldg(r);
+        E.y = __ldg(r + 1);
+    }
+}
+__device__ __forceinline__ void stage_entries(const Entries& E, float4* row, int k) {
+    row[2 * k] = E.x;
+    row[2 * k + 1] = E.y;
+}
+__device__ __forceinline__ StampRec staged(const float4* row, int j) {
+    StampRec R;
+    const float4 x = row[2 * j], y = row[2 * j + 1];
+    R.ch[0] = x.x;
+    R.ch[1] = x.y;
+    R.ch[2] = x.z;
+    R.cl0 = x.w;
+    R.cl1 = y.x;
+    R.cl2 = y.y;
+    R.r2 = y.z;
+    R.kt = __float_as_int(y.w);
+    return R;
+}
+
+__device__ __forceinline__ int cover(const StampDev& S, int32_t v, const StampRec& R, const Child& B, double h,
+                                     double half, bool centre) {
+    const int c = cover32(B, R, centre);
+    return c >= 0 ? c : cover64(S.c + 3 * (int64_t)v, S.r2[v], B.cc[0], B.cc[1], B.cc[2], h, half);
+}
 
 enum { kDrop = 0, kPaint = 1, kKeep = 2 };
 
-// Lanes take a cell's stamp list 32 entries at a time, in order.
-constexpr unsigned kFullMask = 0xFFFFFFFFu;
-constexpr int kWarpsPerBlock = 4;
-constexpr int64_t kSplitCells = 8192;  // levels with fewer refined cells take one warp per child
-
-// One warp per refined cell, all eight children at once. Per axis a stamp's squared distances to the
-// cell's three planes (low, mid, high) serve both halves, so a child's box distances are sums of
-// per-axis terms already formed: (t0 + t1) + t2, the host painter's sums with its zero terms dropped,
-// which leaves them bit-identical (adding +0 is exact).
-struct ParentTerms {
-    double dmin[2][3], dmax[2][3];  // [bit][axis]
-    double cen[2][3];               // squared distance to the child centre's coordinate
-};
-
-__device__ __forceinline__ void parent_terms(const double* c, const double pl[3], const double pm[3], const double pu[3],
-                                             const double cl[3], const double cm[3], ParentTerms& T) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double A = sq(__dsub_rn(c[a], pl[a])), B = sq(__dsub_rn(c[a], pm[a])), C = sq(__dsub_rn(c[a], pu[a]));
-        T.dmin[0][a] = c[a] < pl[a] ? A : (c[a] > pm[a] ? B : 0.0);
-        T.dmin[1][a] = c[a] < pm[a] ? B : (c[a] > pu[a] ? C : 0.0);
-        T.dmax[0][a] = fmax(A, B);
-        T.dmax[1][a] = fmax(B, C);
-        T.cen[0][a] = sq(__dsub_rn(cl[a], c[a]));
-        T.cen[1][a] = sq(__dsub_rn(cm[a], c[a]));
-    }
-}
-
-// Term of child k on axis a (the half it lies in), picked without indexing by a runtime value.
-template <typename V>
-__device__ __forceinline__ V half_term(const V (&x)[2][3], int k, int a) {
-    return ((k >> a) & 1) ? x[1][a] : x[0][a];
-}
-
-// Child k: kDrop / kPaint / kKeep for an undecided stamp with squared radius r2.
-__device__ __forceinline__ int classify_child(const ParentTerms& T, int k, double r2, bool refined) {
-    const double dmin2 = __dadd_rn(__dadd_rn(half_term(T.dmin, k, 0), half_term(T.dmin, k, 1)), half_term(T.dmin, k, 2));
-    if (dmin2 >= r2) return kDrop;
-    const double dmax2 = __dadd_rn(__dadd_rn(half_term(T.dmax, k, 0), half_term(T.dmax, k, 1)), half_term(T.dmax, k, 2));
-    if (dmax2 <= r2) return kPaint;
-    if (refined) return kKeep;
-    const double d2 = __dadd_rn(__dadd_rn(half_term(T.cen, k, 0), half_term(T.cen, k, 1)), half_term(T.cen, k, 2));
-    return d2 < r2 ? kPaint : kDrop;
-}
-
-// FP32 screen of the same box distances. Each coordinate difference to the low plane is formed in FP64 and
-// rounded once; the rest is FP32. Every FP32 distance is within `margin` of its FP64 counterpart (a generous
-// bound: differences within 2^-23 M_a, squares within 2^-21 M_a^2, two additions), so a comparison with r2
-// farther than `margin` decides as the FP64 one does; closer ones are retaken in FP64.
-struct FastTerms {
-    float dmin[2][3], dmax[2][3], cen[2][3];
-    float r2, margin;
-};
-
-__device__ __forceinline__ void fast_terms(const double* c, const double pl[3], float h, float hh, double r2,
-                                           FastTerms& F) {
-    float mm = 0.0f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float dl = __double2float_rn(__dsub_rn(c[a], pl[a]));
-        const float dm = __fsub_rn(dl, h), du = __fsub_rn(dm, h);
-        const float A = __fmul_rn(dl, dl), B = __fmul_rn(dm, dm), C = __fmul_rn(du, du);
-        F.dmin[0][a] = dl < 0.0f ? A : (dm > 0.0f ? B : 0.0f);
-        F.dmin[1][a] = dm < 0.0f ? B : (du > 0.0f ? C : 0.0f);
-        F.dmax[0][a] = fmaxf(A, B);
-        F.dmax[1][a] = fmaxf(B, C);
-        const float el = __fsub_rn(dl, hh), em = __fsub_rn(dm, hh);
-        F.cen[0][a] = __fmul_rn(el, el);
-        F.cen[1][a] = __fmul_rn(em, em);
-        const float M = fabsf(dl) + 2.0f * h;
-        mm = __fmaf_rn(M, M, mm);
-    }
-    F.r2 = __double2float_rn(r2);
-    F.margin = 3.814697265625e-06f * mm + 2.384185791015625e-07f * F.r2;  // 2^-18 sum M^2 + 2^-22 r2
-}
-
-// kDrop / kPaint / kKeep when the screen decides, -1 when FP64 must.
-__device__ __forceinline__ int classify_fast(const FastTerms& F, int k, bool refined) {
-    const float lo = F.r2 - F.margin, hi = F.r2 + F.margin;
-    const float dmin2 = (half_term(F.dmin, k, 0) + half_term(F.dmin, k, 1)) + half_term(F.dmin, k, 2);
-    if (dmin2 >= hi) return kDrop;
-    if (dmin2 >= lo) return -1;
-    const float dmax2 = (half_term(F.dmax, k, 0) + half_term(F.dmax, k, 1)) + half_term(F.dmax, k, 2);
-    if (dmax2 <= lo) return kPaint;
-    if (dmax2 <= hi) return -1;
-    if (refined) return kKeep;
-    const float d2 = (half_term(F.cen, k, 0) + half_term(F.cen, k, 1)) + half_term(F.cen, k, 2);
-    if (d2 < lo) return kPaint;
-    if (d2 >= hi) return kDrop;
-    return -1;
-}
-
-// Partial cover (the refining test): 1 / 0 when the screen decides, -1 when FP64 must.
-__device__ __forceinline__ int partial_fast(const FastTerms& F, int k) {
-    const float lo = F.r2 - F.margin, hi = F.r2 + F.margin;
-    const float dmin2 = (half_term(F.dmin, k, 0) + half_term(F.dmin, k, 1)) + half_term(F.dmin, k, 2);
-    if (dmin2 >= hi) return 0;
-    if (dmin2 >= lo) return -1;
-    const float dmax2 = (half_term(F.dmax, k, 0) + half_term(F.dmax, k, 1)) + half_term(F.dmax, k, 2);
-    if (dmax2 <= lo) return 0;
-    if (dmax2 <= hi) return -1;
-    return 1;
-}
-
-__device__ __forceinline__ void parent_planes(const LevelIn& L, int64_t i, double extent, double half, double pl[3],
-                                              double pm[3], double pu[3], double cl[3], double cm[3]) {
-    const double H = extent * __longlong_as_double((long long)(1023 - L.level) << 52);
-    const double h = 0.5 * H, hh = 0.5 * h;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        pl[a] = fma((double)L.coord[3 * i + a], H, -half);  // exact: multiples of the cell size
-        pm[a] = __dadd_rn(pl[a], h);
-        pu[a] = __dadd_rn(pm[a], h);
-        cl[a] = __dadd_rn(pl[a], hh);
-        cm[a] = __dadd_rn(pm[a], hh);
-    }
-}
-
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) expand_parent_count(LevelIn L, StampDev S, int32_t depth,
-                                                                           double extent, double half, int32_t* firstref,
-                                                                           uint64_t* slot, int64_t* count, int64_t* is_int,
-                                                                           const uint8_t* skip) {
-    __shared__ int32_t s_idx[kWarpsPerBlock][32];
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    if (i >= L.n || (skip && skip[i])) return;  // warp-uniform (skipped cells take the chunked passes)
-    double pl[3], pm[3], pu[3], cl[3], cm[3];
-    parent_planes(L, i, extent, half, pl, pm, pu, cl, cm);
-    const float hf = (float)(pm[0] - pl[0]), hhf = 0.5f * hf;  // child side and half side (exact)
-    const int lc = L.level + 1;
-    const int64_t b = L.off[i], e = L.off[i + 1];
-    // the first refining stamp of each child
-    int32_t fr[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) fr[k] = 0x7FFFFFFF;
-    unsigned found = 0;
-    if (lc < depth) {
-        for (int64_t base = b; base < e && found != 0xFFu; base += 32) {
-            const int64_t q = base + lane;
-            int32_t v = -1;
-            bool cand = false;
-            FastTerms F;
-            double r2 = 0.0;
-            if (q < e) {
-                v = L.ent[q];
-                if (v >= 0 && S.kt[v] > lc) {
-                    cand = true;
-                    r2 = S.r2[v];
-                    fast_terms(S.c + 3 * (int64_t)v, pl, hf, hhf, r2, F);
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                bool qual = false;
-                if (cand) {
-                    const int f = partial_fast(F, k);
-                    if (f >= 0) {
-                        qual = f == 1;
-                    } else {
-                        ParentTerms T;
-                        parent_terms(S.c + 3 * (int64_t)v, pl, pm, pu, cl, cm, T);
-                        const double dmin2 = __dadd_rn(__dadd_rn(half_term(T.dmin, k, 0), half_term(T.dmin, k, 1)),
-                                                       half_term(T.dmin, k, 2));
-                        const double dmax2 = __dadd_rn(__dadd_rn(half_term(T.dmax, k, 0), half_term(T.dmax, k, 1)),
-                                                       half_term(T.dmax, k, 2));
-                        qual = dmin2 < r2 && dmax2 > r2;
-                    }
-                }
-                const unsigned m = __ballot_sync(kFullMask, qual);
-                const int32_t first = __shfl_sync(kFullMask, v, m ? __ffs(m) - 1 : 0);
-                if (m && !((found >> k) & 1u)) {
-                    fr[k] = first;
-                    found |= 1u << k;
-                }
-            }
-        }
-    }
-    // counts of the refined children, blends of the leaf children (lane k folds child k)
-    int64_t n[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) n[k] = 0;
-    float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t base = b; base < e; base += 32) {
-        const int64_t q = base + lane;
-        int32_t v = 0;
-        bool valid = false;
-        FastTerms F;
-        double r2 = 0.0;
-        if (q < e) {
-            valid = true;
-            v = L.ent[q];
-            if (v >= 0) {
-                r2 = S.r2[v];
-                fast_terms(S.c + 3 * (int64_t)v, pl, hf, hhf, r2, F);
-            }
-        }
-        s_idx[wib][lane] = v < 0 ? ~v : v;
-        unsigned pmask = 0;  // lane k: the entries that paint leaf child k
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const bool internal = fr[k] != 0x7FFFFFFF;
-            int c = kDrop;
-            if (valid) {
-                if (v < 0) {
-                    c = kPaint;
-                } else {
-                    const bool refined = internal && fr[k] <= v;
-                    c = classify_fast(F, k, refined);
-                    if (c < 0) {
-                        ParentTerms T;
-                        parent_terms(S.c + 3 * (int64_t)v, pl, pm, pu, cl, cm, T);
-                        c = classify_child(T, k, r2, refined);
-                    }
-                }
-            }
-            if (internal) {
-                n[k] += __popc(__ballot_sync(kFullMask, c != kDrop));
-            } else {
-                const unsigned m = __ballot_sync(kFullMask, c == kPaint);
-                if (lane == k) pmask = m;
-            }
-        }
-        __syncwarp();
-        if (lane < 8) {
-            while (pmask) {
-                const int j = __ffs(pmask) - 1;
-                pmask &= pmask - 1;
-                blend(val, S.rgba[s_idx[wib][j]]);
-            }
-        }
-        __syncwarp();
-    }
-    if (lane < 8) {
-        int64_t nk = 0;
-        int32_t fk = 0x7FFFFFFF;
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (lane == k) {
-                nk = n[k];
-                fk = fr[k];
-            }
-        const int64_t t = 8 * i + lane;
-        firstref[t] = fk;
-        if (fk != 0x7FFFFFFF) {
-            count[t] = nk;
-            is_int[t] = 1;
-            slot[t] = kInternal;
-        } else {
-            count[t] = 0;
-            is_int[t] = 0;
-            slot[t] = leaf_key(val);
-        }
-    }
-}
-
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) expand_parent_write(LevelIn L, StampDev S, double extent,
-                                                                           double half, const int32_t* firstref,
-                                                                           uint64_t* slot, const int64_t* ent_off,
-                                                                           const int64_t* next_idx, uint32_t* ncoord,
-                                                                           int64_t* noff, int32_t* nent, const uint8_t* skip) {
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (i >= L.n || (skip && skip[i])) return;
-    int32_t fr[8];
-    int64_t w[8];
-    unsigned internal = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        fr[k] = firstref[8 * i + k];
-        w[k] = ent_off[8 * i + k];
-        if (slot[8 * i + k] == kInternal) internal |= 1u << k;
-    }
-    if (!internal) return;  // warp-uniform
-    __syncwarp();
-    if (lane < 8 && ((internal >> lane) & 1u)) {
-        const int64_t t = 8 * i + lane, j = next_idx[t];
-        slot[t] = kInternal | (uint64_t)j;
-        ncoord[3 * j] = 2u * L.coord[3 * i] + (lane & 1u);
-        ncoord[3 * j + 1] = 2u * L.coord[3 * i + 1] + ((lane >> 1) & 1u);
-        ncoord[3 * j + 2] = 2u * L.coord[3 * i + 2] + ((lane >> 2) & 1u);
-        noff[j] = ent_off[t];
-    }
-    double pl[3], pm[3], pu[3], cl[3], cm[3];
-    parent_planes(L, i, extent, half, pl, pm, pu, cl, cm);
-    const float hf = (float)(pm[0] - pl[0]), hhf = 0.5f * hf;
-    const int64_t b = L.off[i], e = L.off[i + 1];
-    for (int64_t base = b; base < e; base += 32) {
-        const int64_t q = base + lane;
-        int32_t v = 0;
-        bool valid = false;
-        FastTerms F;
-        double r2 = 0.0;
-        if (q < e) {
-            valid = true;
-            v = L.ent[q];
-            if (v >= 0) {
-                r2 = S.r2[v];
-                fast_terms(S.c + 3 * (int64_t)v, pl, hf, hhf, r2, F);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if (!((internal >> k) & 1u)) continue;  // warp-uniform
-            int c = kDrop;
-            if (valid) {
-                if (v < 0) {
-                    c = kPaint;
-                } else {
-                    c = classify_fast(F, k, fr[k] <= v);
-                    if (c < 0) {
-                        ParentTerms T;
-                        parent_terms(S.c + 3 * (int64_t)v, pl, pm, pu, cl, cm, T);
-                        c = classify_child(T, k, r2, fr[k] <= v);
-                    }
-                }
-            }
-            const bool keep = c != kDrop;
-            const unsigned m = __ballot_sync(kFullMask, keep);
-            if (keep) nent[w[k] + __popc(m & ((1u << lane) - 1u))] = (v < 0 || c == kKeep) ? v : ~v;
-            w[k] += __popc(m);
-        }
-    }
-}
-
-// Squared radius and target depth of each stamp: the smallest k with extent 2^-k <= r/10, at most depth.
-__global__ void stamp_prep(const double* r, int64_t n, int32_t depth, double extent, double* r2, int32_t* kt) {
+// Squared radius, target depth (the smallest k with extent 2^-k <= r/10, at most depth) and record of each stamp.
+__global__ void stamp_prep(const double* c, const double* r, int64_t n, int32_t depth, double extent, double* r2,
+                           StampRec* rec) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const double rs = r[s];
-    r2[s] = __dmul_rn(rs, rs);
+    const double rr = __dmul_rn(rs, rs);
+    r2[s] = rr;
     const double tgt = __ddiv_rn(rs, 10.0);
     int32_t k = 0;
     double w = extent;
@@ -435,392 +267,457 @@ __global__ void stamp_prep(const double* r, int64_t n, int32_t depth, double ext
         w = __dmul_rn(w, 0.5);
         ++k;
     }
-    kt[s] = k;
-}
-
-// The same two passes with one warp per child, for levels of few refined cells: near the root and around the
-// rooms a cell's list holds tens of thousands of stamps, and eight warps per cell instead of one keep the GPU
-// busy. The per-child decisions are the ones above (the same screen and FP64 fallback), so the output is too.
-__device__ __forceinline__ int child_class(const StampDev& S, const FastTerms& F, int32_t v, double r2, int k,
-                                           bool refined, const double pl[3], const double pm[3], const double pu[3],
-                                           const double cl[3], const double cm[3]) {
-    int c = classify_fast(F, k, refined);
-    if (c < 0) {
-        ParentTerms T;
-        parent_terms(S.c + 3 * (int64_t)v, pl, pm, pu, cl, cm, T);
-        c = classify_child(T, k, r2, refined);
+    float h[3], l[3];
+    for (int a = 0; a < 3; ++a) {
+        h[a] = (float)c[3 * s + a];
+        l[a] = (float)(c[3 * s + a] - (double)h[a]);
     }
-    return c;
+    StampRec R;
+    R.ch[0] = h[0];
+    R.ch[1] = h[1];
+    R.ch[2] = h[2];
+    R.cl0 = l[0];
+    R.cl1 = l[1];
+    R.cl2 = l[2];
+    R.r2 = (float)rr;
+    R.kt = k;
+    rec[s] = R;
 }
 
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) expand_child_count(LevelIn L, StampDev S, int32_t depth,
-                                                                          double extent, double half, int32_t* firstref,
-                                                                          uint64_t* slot, int64_t* count, int64_t* is_int,
-                                                                          const uint8_t* skip) {
-    __shared__ int32_t s_idx[kWarpsPerBlock][32];
-    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    if (t >= 8 * L.n || (skip && skip[t >> 3])) return;  // warp-uniform
-    const int64_t i = t >> 3;
-    const int k = (int)(t & 7);
-    double pl[3], pm[3], pu[3], cl[3], cm[3];
-    parent_planes(L, i, extent, half, pl, pm, pu, cl, cm);
-    const float hf = (float)(pm[0] - pl[0]), hhf = 0.5f * hf;
-    const int lc = L.level + 1;
+// ---------------------------------------------------------------------------
+// Long lists: items of kItem entries, one octet (eight lanes, one per child) each.
+// ---------------------------------------------------------------------------
+
+struct LongCell {
+    int64_t cell, b, e;  // its list [b, e)
+    int64_t item;        // its first item
+};
+struct Item {
+    int64_t cell, b, e;
+    int64_t p;  // long cell
+};
+
+// Cells with lists longer than kLongList; ctr[0] counts them, ctr[1] their items.
+__global__ void find_long(LevelIn L, LongCell* out, unsigned long long* ctr) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.n) return;
     const int64_t b = L.off[i], e = L.off[i + 1];
-    int32_t fr = 0x7FFFFFFF;
-    if (lc < depth) {
-        for (int64_t base = b; base < e; base += 32) {
-            const int64_t q = base + lane;
-            int32_t v = -1;
-            bool qual = false;
-            if (q < e) {
-                v = L.ent[q];
-                if (v >= 0 && S.kt[v] > lc) {
-                    const double r2 = S.r2[v];
-                    FastTerms F;
-                    fast_terms(S.c + 3 * (int64_t)v, pl, hf, hhf, r2, F);
-                    const int f = partial_fast(F, k);
-                    if (f >= 0) {
-                        qual = f == 1;
-                    } else {
-                        ParentTerms T;
-                        parent_terms(S.c + 3 * (int64_t)v, pl, pm, pu, cl, cm, T);
-                        const double dmin2 = __dadd_rn(__dadd_rn(half_term(T.dmin, k, 0), half_term(T.dmin, k, 1)),
-                                                       half_term(T.dmin, k, 2));
-                        const double dmax2 = __dadd_rn(__dadd_rn(half_term(T.dmax, k, 0), half_term(T.dmax, k, 1)),
-                                                       half_term(T.dmax, k, 2));
-                        qual = dmin2 < r2 && dmax2 > r2;
-                    }
+    if (e - b <= kLongList) return;
+    const unsigned long long p = atomicAdd(&ctr[0], 1ull);
+    const unsigned long long w = atomicAdd(&ctr[1], (unsigned long long)((e - b + kItem - 1) / kItem));
+    out[p] = LongCell{i, b, e, (int64_t)w};
+}
+
+// One block per long cell: its items, and no refining stamp yet.
+__global__ void long_items(const LongCell* cells, Item* items, int32_t* fr) {
+    const LongCell C = cells[blockIdx.x];
+    for (int64_t j = threadIdx.x; C.b + j * kItem < C.e; j += blockDim.x)
+        items[C.item + j] = Item{C.cell, C.b + j * kItem, min(C.e, C.b + (j + 1) * kItem), (int64_t)blockIdx.x};
+    if (threadIdx.x < 8) fr[8 * (int64_t)blockIdx.x + threadIdx.x] = kNoStamp;
+}
+
+// The least stamp of each item that refines each child (entries are in stamp order, so the first that does).
+__global__ void __launch_bounds__(128) long_first(LevelIn L, StampDev S, double half, const Item* items,
+                                                  int64_t n_items, int32_t* fr) {
+    __shared__ float4 s_rec[16 * kStageRow];
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const int lane = threadIdx.x & 31, k = threadIdx.x & 7, lc = L.level + 1;
+    float4* row = s_rec + (threadIdx.x >> 3) * kStageRow;
+    const bool mine = w < n_items;
+    const Item I = mine ? items[w] : Item{0, 0, 0, 0};
+    const Child B = child_box(L, I.cell, k);
+    int32_t first = kNoStamp;
+    Entries E{I.b, I.e, -1, 0, {}, {}};
+    load_entries(E, L, S, k);
+    while (__any_sync(kFullMask, E.m > 0 && first == kNoStamp)) {
+        const Entries C = E;
+        stage_entries(C, row, k);
+        __syncwarp();
+        E.q0 += 8;
+        load_entries(E, L, S, k);
+        for (int j = 0; j < 8; ++j) {
+            const int32_t v = __shfl_sync(kFullMask, C.v, (lane & 24) + j);
+            if (v < 0 || first != kNoStamp) continue;
+            const StampRec R = staged(row, j);
+            if (R.kt > lc && cover(S, v, R, B, L.h, half, false) >= kPartCentreIn) first = v;
+        }
+        __syncwarp();
+    }
+    if (mine && first != kNoStamp) atomicMin(&fr[8 * I.p + k], first);
+}
+
+// Decision bits of one entry for the octet's eight children: low byte kept, high byte painted.
+__device__ __forceinline__ unsigned decision_bits(int c) {
+    const unsigned keep = __ballot_sync(kFullMask, c != kDrop), paint = __ballot_sync(kFullMask, c == kPaint);
+    const int o = threadIdx.x & 24;
+    return ((keep >> o) & 0xFFu) | (((paint >> o) & 0xFFu) << 8);
+}
+
+// Per item: the entries' decisions, and per child how many a refined child keeps or paint one that stays a leaf.
+__global__ void __launch_bounds__(128) long_count(LevelIn L, StampDev S, double half, const Item* items,
+                                                  int64_t n_items, const int32_t* fr, uint16_t* cls, int32_t* icnt) {
+    __shared__ float4 s_rec[16 * kStageRow];
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const int lane = threadIdx.x & 31, k = threadIdx.x & 7;
+    float4* row = s_rec + (threadIdx.x >> 3) * kStageRow;
+    const bool mine = w < n_items;
+    const Item I = mine ? items[w] : Item{0, 0, 0, 0};
+    const Child B = child_box(L, I.cell, k);
+    const int32_t f = mine ? fr[8 * I.p + k] : kNoStamp;
+    int32_t n = 0;
+    Entries E{I.b, I.e, -1, 0, {}, {}};
+    load_entries(E, L, S, k);
+    while (__any_sync(kFullMask, E.m > 0)) {
+        const Entries C = E;
+        stage_entries(C, row, k);
+        __syncwarp();
+        E.q0 += 8;
+        load_entries(E, L, S, k);
+        const int mm = __reduce_max_sync(kFullMask, C.m);
+        unsigned own = 0;
+        for (int j = 0; j < mm; ++j) {
+            const int32_t v = __shfl_sync(kFullMask, C.v, (lane & 24) + j);
+            int c = kDrop;
+            if (j < C.m) {
+                if (v < 0) {
+                    c = kPaint;
+                } else {
+                    const bool refined = f <= v;
+                    const int x = cover(S, v, staged(row, j), B, L.h, half, !refined);
+                    c = x == kIn ? kPaint : (x == kOut ? kDrop : (refined ? kKeep : (x == kPartCentreIn ? kPaint : kDrop)));
                 }
             }
-            const unsigned m = __ballot_sync(kFullMask, qual);
-            if (m) {
-                fr = __shfl_sync(kFullMask, v, __ffs(m) - 1);  // entries are in stamp order
-                break;
-            }
+            const unsigned bits = decision_bits(c);
+            if (k == j) own = bits;
+            n += f != kNoStamp ? c != kDrop : c == kPaint;
         }
+        if (k < C.m) cls[C.q0 + k] = (uint16_t)own;
+        __syncwarp();
     }
-    int64_t n = 0;
-    float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t base = b; base < e; base += 32) {
-        const int64_t q = base + lane;
-        int32_t v = 0;
-        int c = kDrop;
-        if (q < e) {
-            v = L.ent[q];
-            if (v < 0) {
-                c = kPaint;
-            } else {
-                const double r2 = S.r2[v];
-                FastTerms F;
-                fast_terms(S.c + 3 * (int64_t)v, pl, hf, hhf, r2, F);
-                c = child_class(S, F, v, r2, k, fr != 0x7FFFFFFF && fr <= v, pl, pm, pu, cl, cm);
-            }
+    if (mine) icnt[8 * w + k] = n;
+}
+
+// One block per long cell: the items' counts become exclusive sums per child; the child's total and slot.
+constexpr int kSumRows = 32;  // items at a time (a lane per item and child)
+__global__ void __launch_bounds__(8 * kSumRows) long_sums(const LongCell* cells, const int32_t* fr, int32_t* icnt,
+                                                          uint64_t* slot, int32_t* cnt, int32_t* npaint) {
+    __shared__ int32_t s_x[8][kSumRows + 1];
+    const int64_t p = blockIdx.x;
+    const int k = threadIdx.x & 7, row = threadIdx.x >> 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const LongCell C = cells[p];
+    const int64_t ni = (C.e - C.b + kItem - 1) / kItem;
+    int32_t sum = 0;  // warp w sums child w's items
+    for (int64_t j = 0; j < ni; j += kSumRows) {
+        int32_t* x = icnt + 8 * (C.item + j + row) + k;
+        s_x[k][row] = j + row < ni ? *x : 0;
+        __syncthreads();
+        const int32_t own = s_x[warp][lane];
+        int32_t pre = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t u = __shfl_up_sync(kFullMask, pre, o);
+            if (lane >= o) pre += u;
         }
-        if (fr != 0x7FFFFFFF) {
-            n += __popc(__ballot_sync(kFullMask, c != kDrop));
-        } else {
-            s_idx[wib][lane] = v < 0 ? ~v : v;
-            unsigned m = __ballot_sync(kFullMask, c == kPaint);
-            __syncwarp();
-            while (m) {  // every lane folds the same sequence
-                const int j = __ffs(m) - 1;
-                m &= m - 1;
-                blend(val, S.rgba[s_idx[wib][j]]);
-            }
-            __syncwarp();
-        }
+        s_x[warp][lane] = sum + pre - own;
+        sum += __shfl_sync(kFullMask, pre, 31);
+        __syncthreads();
+        if (j + row < ni) *x = s_x[k][row];
+        __syncthreads();
     }
     if (lane == 0) {
-        firstref[t] = fr;
-        if (fr != 0x7FFFFFFF) {
-            count[t] = n;
-            is_int[t] = 1;
-            slot[t] = kInternal;
-        } else {
-            count[t] = 0;
-            is_int[t] = 0;
-            slot[t] = leaf_key(val);
+        const int64_t t = 8 * C.cell + warp;
+        const bool internal = fr[8 * p + warp] != kNoStamp;
+        slot[t] = internal ? kInternal : 0ull;
+        cnt[t] = internal ? sum : 0;
+        npaint[8 * p + warp] = internal ? 0 : sum;
+    }
+}
+
+// One warp per child of a long cell that stays a leaf and is painted: the blend, in order, of the stamps that do.
+__global__ void __launch_bounds__(128) long_blend(LevelIn L, StampDev S, const LongCell* cells, int64_t n_long,
+                                                  const int32_t* npaint, const uint16_t* cls, uint64_t* slot) {
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (w >= 8 * n_long || npaint[w] == 0) return;  // warp-uniform
+    const LongCell C = cells[w >> 3];
+    const int k = (int)(w & 7);
+    float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t base = C.b; base < C.e; base += 32) {
+        const int64_t q = base + lane;
+        const bool p = q < C.e && ((cls[q] >> (8 + k)) & 1u);
+        const int32_t v = p ? L.ent[q] : 0;
+        unsigned m = __ballot_sync(kFullMask, p);
+        while (m) {  // every lane folds the same sequence
+            const int32_t x = __shfl_sync(kFullMask, v, __ffs(m) - 1);
+            m &= m - 1;
+            blend(val, S.rgba[x < 0 ? ~x : x]);
+        }
+    }
+    if (lane == 0) slot[8 * C.cell + k] = leaf_key(val);
+}
+
+// One octet per item: its kept entries at the child's list start plus the counts of the cell's earlier items.
+__global__ void __launch_bounds__(128) long_write(LevelIn L, const Item* items, int64_t n_items, const uint64_t* slot,
+                                                  const uint16_t* cls, const int32_t* icnt, const int64_t* noff,
+                                                  int32_t* nent) {
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const int k = threadIdx.x & 7;
+    if (w >= n_items) return;
+    const Item I = items[w];
+    const uint64_t s = slot[8 * I.cell + k];
+    if (!(s & kInternal)) return;
+    int64_t pos = noff[s & ~kInternal] + icnt[8 * w + k];
+    for (int64_t q = I.b; q < I.e; ++q) {
+        const unsigned bits = cls[q];
+        if ((bits >> k) & 1u) {
+            const int32_t v = L.ent[q];
+            nent[pos++] = (v >= 0 && ((bits >> (8 + k)) & 1u)) ? ~v : v;
         }
     }
 }
 
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) expand_child_write(LevelIn L, StampDev S, double extent,
-                                                                          double half, const int32_t* firstref,
-                                                                          uint64_t* slot, const int64_t* ent_off,
-                                                                          const int64_t* next_idx, uint32_t* ncoord,
-                                                                          int64_t* noff, int32_t* nent, const uint8_t* skip) {
-    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (t >= 8 * L.n || (skip && skip[t >> 3])) return;
-    if (slot[t] != kInternal) return;  // warp-uniform
-    const int64_t i = t >> 3;
-    const int k = (int)(t & 7);
-    const int32_t fr = firstref[t];
-    const int64_t j = next_idx[t];
-    int64_t w = ent_off[t];
-    __syncwarp();
+// ---------------------------------------------------------------------------
+// Every cell: one octet each (16 cells a block).
+// ---------------------------------------------------------------------------
+
+// Sums of a block of the octet kernels (entries and cells of the next level), then their exclusive sums over the
+// blocks (scan_sums).
+struct BlockSum {
+    int64_t ent, cells;
+};
+
+// Sum of x over the warp.
+__device__ __forceinline__ int64_t warp_total(int64_t x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFullMask, x, o);
+    return x;
+}
+
+// The children of every cell: slot (internal, or the leaf's key), list length, the entries' decisions; the block's
+// sums; tot[2] = the longest list. Cells with long lists only add their sums here.
+__global__ void __launch_bounds__(8 * kCells) expand_count(LevelIn L, StampDev S, double half, uint64_t* slot,
+                                                           int32_t* cnt, uint16_t* cls, BlockSum* bs, long long* tot) {
+    __shared__ float4 s_rec[kCells * kStageRow];
+    __shared__ int64_t s_ent[kCells / 4], s_int[kCells / 4];
+    const int64_t i = (int64_t)blockIdx.x * kCells + (threadIdx.x >> 3);
+    const int lane = threadIdx.x & 31, k = threadIdx.x & 7, lc = L.level + 1;
+    int64_t b = 0, e = 0;
+    if (i < L.n) {
+        b = L.off[i];
+        e = L.off[i + 1];
+    }
+    const bool is_long = e - b > kLongList;
+    if (is_long) e = b;
+    int32_t n = 0;
+    bool found = false;
+    float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (__any_sync(kFullMask, b < e)) {
+        const Child B = child_box(L, i < L.n ? i : 0, k);
+        float4* row = s_rec + (threadIdx.x >> 3) * kStageRow;
+        Entries C{b, e, -1, 0, {}, {}};
+        for (; __any_sync(kFullMask, C.q0 < C.e); C.q0 += 8) {
+            load_entries(C, L, S, k);  // (most lists are short: no loads ahead, which cost registers)
+            stage_entries(C, row, k);
+            __syncwarp();
+            const int mm = __reduce_max_sync(kFullMask, C.m);
+            unsigned own = 0;
+            for (int j = 0; j < mm; ++j) {
+                const int32_t v = __shfl_sync(kFullMask, C.v, (lane & 24) + j);
+                int c = kDrop;
+                if (j < C.m) {
+                    if (v < 0) {
+                        c = kPaint;
+                    } else {
+                        const StampRec R = staged(row, j);
+                        const bool refines = found || R.kt > lc;
+                        const int x = cover(S, v, R, B, L.h, half, !refines);
+                        if (x == kIn) {
+                            c = kPaint;
+                        } else if (x != kOut) {
+                            found = refines;  // (the first stamp that partially covers it with a deeper target)
+                            c = refines ? kKeep : (x == kPartCentreIn ? kPaint : kDrop);
+                        }
+                    }
+                }
+                const unsigned bits = decision_bits(c);
+                if (k == j) own = bits;
+                n += c != kDrop;
+                if (c == kPaint && !found) blend(val, S.rgba[v < 0 ? ~v : v]);
+            }
+            if (k < C.m) cls[C.q0 + k] = (uint16_t)own;
+            __syncwarp();
+        }
+    }
+    const int64_t t = 8 * i + k;
+    if (i < L.n) {
+        if (is_long) {
+            found = slot[t] == kInternal;
+            n = cnt[t];
+        } else {
+            if (!found) n = 0;
+            slot[t] = found ? kInternal : leaf_key(val);
+            cnt[t] = n;
+        }
+    }
+    const int32_t longest = __reduce_max_sync(kFullMask, n);
+    const int64_t ents = warp_total(n);
+    const int ints = __popc(__ballot_sync(kFullMask, found));
     if (lane == 0) {
+        s_ent[threadIdx.x >> 5] = ents;
+        s_int[threadIdx.x >> 5] = ints;
+        if (longest > kLongList) atomicMax(&tot[2], (long long)longest);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        BlockSum x{0, 0};
+        for (int w = 0; w < kCells / 4; ++w) {
+            x.ent += s_ent[w];
+            x.cells += s_int[w];
+        }
+        bs[blockIdx.x] = x;
+    }
+}
+
+// Exclusive sums over the blocks, two levels: within kScanItems of them in place, and over those groups (sup).
+constexpr int kScanThreads = 1024, kScanPer = 4, kScanItems = kScanThreads * kScanPer;
+
+// Exclusive sums of x over the block's threads; *total = the block's sum.
+__device__ __forceinline__ BlockSum block_scan(BlockSum x, BlockSum* total) {
+    __shared__ BlockSum s_w[kScanThreads / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    BlockSum v = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t a = __shfl_up_sync(kFullMask, v.ent, o), c = __shfl_up_sync(kFullMask, v.cells, o);
+        if (lane >= o) {
+            v.ent += a;
+            v.cells += c;
+        }
+    }
+    __syncthreads();
+    if (lane == 31) s_w[w] = v;
+    __syncthreads();
+    if (w == 0) {
+        BlockSum y = lane < (int)(blockDim.x >> 5) ? s_w[lane] : BlockSum{0, 0};
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t a = __shfl_up_sync(kFullMask, y.ent, o), c = __shfl_up_sync(kFullMask, y.cells, o);
+            if (lane >= o) {
+                y.ent += a;
+                y.cells += c;
+            }
+        }
+        s_w[lane] = y;
+    }
+    __syncthreads();
+    if (w > 0) {
+        v.ent += s_w[w - 1].ent;
+        v.cells += s_w[w - 1].cells;
+    }
+    *total = s_w[(blockDim.x >> 5) - 1];
+    return BlockSum{v.ent - x.ent, v.cells - x.cells};
+}
+
+// (with a single group, tot gets the whole sums here and scan_sup is not needed)
+__global__ void __launch_bounds__(kScanThreads) scan_groups(BlockSum* bs, int64_t n, BlockSum* sup, long long* tot) {
+    const int64_t g = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kScanPer;
+    BlockSum x[kScanPer], sum{0, 0};
+#pragma unroll
+    for (int j = 0; j < kScanPer; ++j) {
+        x[j] = g + j < n ? bs[g + j] : BlockSum{0, 0};
+        sum.ent += x[j].ent;
+        sum.cells += x[j].cells;
+    }
+    BlockSum total;
+    BlockSum pre = block_scan(sum, &total);
+#pragma unroll
+    for (int j = 0; j < kScanPer; ++j) {
+        if (g + j < n) bs[g + j] = pre;
+        pre.ent += x[j].ent;
+        pre.cells += x[j].cells;
+    }
+    if (threadIdx.x == 0) {
+        sup[blockIdx.x] = gridDim.x == 1 ? BlockSum{0, 0} : total;
+        if (gridDim.x == 1) {
+            tot[0] = total.ent;
+            tot[1] = total.cells;
+        }
+    }
+}
+
+// Exclusive sums over the groups (one block); tot[0], tot[1] = the whole sums.
+__global__ void __launch_bounds__(kScanThreads) scan_sup(BlockSum* sup, int64_t n, long long* tot) {
+    BlockSum carry{0, 0};
+    for (int64_t base = 0; base < n; base += kScanThreads) {
+        const int64_t g = base + threadIdx.x;
+        const BlockSum x = g < n ? sup[g] : BlockSum{0, 0};
+        BlockSum total;
+        const BlockSum pre = block_scan(x, &total);
+        if (g < n) sup[g] = BlockSum{carry.ent + pre.ent, carry.cells + pre.cells};
+        carry.ent += total.ent;
+        carry.cells += total.cells;
+    }
+    if (threadIdx.x == 0) {
+        tot[0] = carry.ent;
+        tot[1] = carry.cells;
+    }
+}
+
+// The next level: each refined child's index (into its slot), coordinates, list start and list, and with pid the
+// partition it belongs to. The lists of long cells are left to long_write.
+__global__ void __launch_bounds__(8 * kCells) expand_write(LevelIn L, uint64_t* slot, const int32_t* cnt, const uint16_t* cls,
+                                                           const BlockSum* bs, const BlockSum* sup, const int32_t* pid,
+                                                           uint32_t* ncoord, int64_t* noff, int32_t* nent, int32_t* npid) {
+    __shared__ int64_t s_ent[kCells / 4];
+    __shared__ int s_int[kCells / 4];
+    const int64_t i = (int64_t)blockIdx.x * kCells + (threadIdx.x >> 3);
+    const int lane = threadIdx.x & 31, k = threadIdx.x & 7, warp = threadIdx.x >> 5;
+    const int64_t t = 8 * i + k;
+    const bool internal = i < L.n && slot[t] == kInternal;
+    const int64_t n = internal ? cnt[t] : 0;
+    // offsets: the block's, the earlier warps', the earlier lanes'
+    int64_t pre = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t u = __shfl_up_sync(kFullMask, pre, o);
+        if (lane >= o) pre += u;
+    }
+    const unsigned im = __ballot_sync(kFullMask, internal);
+    if (lane == 31) {
+        s_ent[warp] = pre;
+        s_int[warp] = __popc(im);
+    }
+    __syncthreads();
+    const BlockSum base = bs[blockIdx.x], group = sup[blockIdx.x / kScanItems];
+    int64_t w = base.ent + group.ent + pre - n, j = base.cells + group.cells + __popc(im & ((1u << lane) - 1u));
+    for (int q = 0; q < warp; ++q) {
+        w += s_ent[q];
+        j += s_int[q];
+    }
+    if (internal) {
         slot[t] = kInternal | (uint64_t)j;
         ncoord[3 * j] = 2u * L.coord[3 * i] + (k & 1u);
         ncoord[3 * j + 1] = 2u * L.coord[3 * i + 1] + ((k >> 1) & 1u);
         ncoord[3 * j + 2] = 2u * L.coord[3 * i + 2] + ((k >> 2) & 1u);
         noff[j] = w;
+        if (pid) npid[j] = pid[i];
     }
-    double pl[3], pm[3], pu[3], cl[3], cm[3];
-    parent_planes(L, i, extent, half, pl, pm, pu, cl, cm);
-    const float hf = (float)(pm[0] - pl[0]), hhf = 0.5f * hf;
-    const int64_t b = L.off[i], e = L.off[i + 1];
-    for (int64_t base = b; base < e; base += 32) {
-        const int64_t q = base + lane;
-        int32_t out = 0;
-        bool keep = false;
-        if (q < e) {
-            const int32_t v = L.ent[q];
-            if (v < 0) {
-                out = v;
-                keep = true;
-            } else {
-                const double r2 = S.r2[v];
-                FastTerms F;
-                fast_terms(S.c + 3 * (int64_t)v, pl, hf, hhf, r2, F);
-                const int c = child_class(S, F, v, r2, k, fr <= v, pl, pm, pu, cl, cm);
-                keep = c != kDrop;
-                out = c == kPaint ? ~v : v;
-            }
+    int64_t b = 0, e = 0;
+    if (i < L.n) {
+        b = L.off[i];
+        e = L.off[i + 1];
+        if (e - b > kLongList) e = b;
+    }
+    for (int64_t q0 = b; __any_sync(kFullMask, q0 < e); q0 += 8) {
+        const int m = (int)max((int64_t)0, min((int64_t)8, e - q0));
+        const int32_t vv = k < m ? L.ent[q0 + k] : 0;
+        const int own = k < m ? (int)cls[q0 + k] : 0;
+        const int mm = __reduce_max_sync(kFullMask, m);
+        for (int x = 0; x < mm; ++x) {
+            const int32_t v = __shfl_sync(kFullMask, vv, (lane & 24) + x);
+            const int bits = __shfl_sync(kFullMask, own, (lane & 24) + x);
+            if (internal && ((bits >> k) & 1)) nent[w++] = (v >= 0 && ((bits >> (8 + k)) & 1)) ? ~v : v;
         }
-        const unsigned m = __ballot_sync(kFullMask, keep);
-        if (keep) nent[w + __popc(m & ((1u << lane) - 1u))] = out;
-        w += __popc(m);
-    }
-}
-
-// The per-child passes once more, for the cells whose lists are long (near the root every stamp is on them, and
-// around a room its tens of thousands of stamps are, level after level): a child's list is cut into chunks of
-// kChunk entries, one warp each, so that such a cell runs on hundreds of warps instead of one (or eight). The
-// first refining stamp is the least one any chunk finds (entries are in stamp order), the kept entries are counted
-// per chunk and written at the child's list start plus the counts of its earlier chunks (which keeps every
-// next-level list in stamp order), and a child that stays a leaf blends its painting stamps in order in one warp
-// (such children of long lists rarely have any, and skip it). Every per-entry decision is the one of the passes
-// above, so the pools are the same. The level's other cells take those passes, which skip the long ones.
-constexpr int64_t kChunk = 2048;         // entries per warp
-constexpr int64_t kChunkMinList = 8192;  // cells whose list is longer take the chunked passes
-constexpr int32_t kNoStamp = 0x7FFFFFFF;
-
-struct ChunkWork {
-    int64_t t;      // child 8 i + k of refined cell i
-    int64_t b, e;   // its entries [b, e) of cell i's list
-    int64_t fw;     // index of the child's first chunk
-    int32_t first;  // 1 for the child's first chunk
-};
-
-// Whether list entry v (a stamp that still descends) partially covers child k and has its target below level lc.
-__device__ __forceinline__ bool refines_child(const StampDev& S, int32_t v, int k, int lc, const double pl[3],
-                                              const double pm[3], const double pu[3], const double cl[3],
-                                              const double cm[3], float hf, float hhf) {
-    if (v < 0 || S.kt[v] <= lc) return false;
-    const double r2 = S.r2[v];
-    FastTerms F;
-    fast_terms(S.c + 3 * (int64_t)v, pl, hf, hhf, r2, F);
-    const int f = partial_fast(F, k);
-    if (f >= 0) return f == 1;
-    ParentTerms T;
-    parent_terms(S.c + 3 * (int64_t)v, pl, pm, pu, cl, cm, T);
-    const double dmin2 = __dadd_rn(__dadd_rn(half_term(T.dmin, k, 0), half_term(T.dmin, k, 1)), half_term(T.dmin, k, 2));
-    const double dmax2 = __dadd_rn(__dadd_rn(half_term(T.dmax, k, 0), half_term(T.dmax, k, 1)), half_term(T.dmax, k, 2));
-    return dmin2 < r2 && dmax2 > r2;
-}
-
-// kDrop / kPaint / kKeep of list entry x for child k whose first refining stamp is fr (kNoStamp: none).
-__device__ __forceinline__ int entry_class(const StampDev& S, int32_t x, int k, int32_t fr, const double pl[3],
-                                           const double pm[3], const double pu[3], const double cl[3],
-                                           const double cm[3], float hf, float hhf) {
-    if (x < 0) return kPaint;
-    const double r2 = S.r2[x];
-    FastTerms F;
-    fast_terms(S.c + 3 * (int64_t)x, pl, hf, hhf, r2, F);
-    return child_class(S, F, x, r2, k, fr != kNoStamp && fr <= x, pl, pm, pu, cl, cm);
-}
-
-// Cells with lists longer than kChunkMinList: skip[i] = flag[i] = 1.
-__global__ void flag_long(LevelIn L, uint8_t* skip, int64_t* flag) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L.n) return;
-    const bool lg = L.off[i + 1] - L.off[i] > kChunkMinList;
-    skip[i] = lg ? 1 : 0;
-    flag[i] = lg ? 1 : 0;
-}
-
-// The long cells in order, as (cell, list start, list end); pos = exclusive scan of their flags.
-__global__ void gather_long(LevelIn L, const uint8_t* skip, const int64_t* pos, int64_t* out) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L.n || !skip[i]) return;
-    const int64_t j = pos[i];
-    out[3 * j] = i;
-    out[3 * j + 1] = L.off[i];
-    out[3 * j + 2] = L.off[i + 1];
-}
-
-// Children of the long cells: cells[j >> 3] is the cell of the j-th.
-__global__ void chunk_init(const int64_t* cells, int64_t nj, int32_t* fr, int64_t* cnt, int64_t* npaint) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= nj) return;
-    const int64_t t = 8 * cells[j >> 3] + (j & 7);
-    fr[t] = kNoStamp;
-    cnt[t] = 0;
-    npaint[t] = 0;
-}
-
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) chunk_firstref(LevelIn L, StampDev S, int32_t depth, double extent,
-                                                                      double half, const ChunkWork* W, int64_t nw,
-                                                                      int32_t* fr) {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int lc = L.level + 1;
-    if (w >= nw || lc >= depth) return;  // warp-uniform
-    const ChunkWork cw = W[w];
-    const int k = (int)(cw.t & 7);
-    double pl[3], pm[3], pu[3], cl[3], cm[3];
-    parent_planes(L, cw.t >> 3, extent, half, pl, pm, pu, cl, cm);
-    const float hf = (float)(pm[0] - pl[0]), hhf = 0.5f * hf;
-    for (int64_t base = cw.b; base < cw.e; base += 32) {
-        const int64_t q = base + lane;
-        const int32_t v = q < cw.e ? L.ent[q] : -1;
-        const unsigned m = __ballot_sync(kFullMask, refines_child(S, v, k, lc, pl, pm, pu, cl, cm, hf, hhf));
-        if (m) {
-            const int32_t first = __shfl_sync(kFullMask, v, __ffs(m) - 1);
-            if (lane == 0) atomicMin(&fr[cw.t], first);
-            break;
-        }
-    }
-}
-
-// Per chunk: the entries a refined child keeps (chunk_cnt, summed into cnt), or the ones that paint a child that
-// stays a leaf (summed into npaint).
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) chunk_count(LevelIn L, StampDev S, double extent, double half,
-                                                                   const ChunkWork* W, int64_t nw, const int32_t* fr,
-                                                                   int64_t* chunk_cnt, int64_t* cnt, int64_t* npaint) {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= nw) return;
-    const ChunkWork cw = W[w];
-    const int k = (int)(cw.t & 7);
-    const int32_t f = fr[cw.t];
-    double pl[3], pm[3], pu[3], cl[3], cm[3];
-    parent_planes(L, cw.t >> 3, extent, half, pl, pm, pu, cl, cm);
-    const float hf = (float)(pm[0] - pl[0]), hhf = 0.5f * hf;
-    int64_t n = 0;
-    for (int64_t base = cw.b; base < cw.e; base += 32) {
-        const int64_t q = base + lane;
-        const int c = q < cw.e ? entry_class(S, L.ent[q], k, f, pl, pm, pu, cl, cm, hf, hhf) : kDrop;
-        n += __popc(__ballot_sync(kFullMask, f != kNoStamp ? c != kDrop : c == kPaint));
-    }
-    if (lane == 0) {
-        chunk_cnt[w] = f != kNoStamp ? n : 0;
-        if (n)
-            atomicAdd(reinterpret_cast<unsigned long long*>(f != kNoStamp ? &cnt[cw.t] : &npaint[cw.t]),
-                      (unsigned long long)n);
-    }
-}
-
-// Per child: an internal slot, or the leaf key of the blend, in stamp order, of the stamps that paint it.
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) chunk_child_finish(LevelIn L, StampDev S, double extent, double half,
-                                                                          const int64_t* cells, int64_t nj,
-                                                                          const int32_t* fr, const int64_t* npaint,
-                                                                          uint64_t* slot, int64_t* cnt, int64_t* is_int) {
-    __shared__ int32_t s_idx[kWarpsPerBlock][32];
-    const int64_t jj = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    if (jj >= nj) return;  // warp-uniform
-    const int64_t t = 8 * cells[jj >> 3] + (jj & 7);
-    if (fr[t] != kNoStamp) {
-        if (lane == 0) {
-            is_int[t] = 1;
-            slot[t] = kInternal;
-        }
-        return;
-    }
-    float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (npaint[t] > 0) {
-        const int64_t i = t >> 3;
-        const int k = (int)(t & 7);
-        double pl[3], pm[3], pu[3], cl[3], cm[3];
-        parent_planes(L, i, extent, half, pl, pm, pu, cl, cm);
-        const float hf = (float)(pm[0] - pl[0]), hhf = 0.5f * hf;
-        const int64_t b = L.off[i], e = L.off[i + 1];
-        for (int64_t base = b; base < e; base += 32) {
-            const int64_t q = base + lane;
-            int32_t x = 0;
-            int c = kDrop;
-            if (q < e) {
-                x = L.ent[q];
-                c = entry_class(S, x, k, kNoStamp, pl, pm, pu, cl, cm, hf, hhf);
-            }
-            s_idx[wib][lane] = x < 0 ? ~x : x;
-            unsigned m = __ballot_sync(kFullMask, c == kPaint);
-            __syncwarp();
-            while (m) {  // every lane folds the same sequence
-                const int j = __ffs(m) - 1;
-                m &= m - 1;
-                blend(val, S.rgba[s_idx[wib][j]]);
-            }
-            __syncwarp();
-        }
-    }
-    if (lane == 0) {
-        cnt[t] = 0;
-        is_int[t] = 0;
-        slot[t] = leaf_key(val);
-    }
-}
-
-// Per chunk of a refined child: its kept entries at the child's list start plus the kept entries of its earlier
-// chunks (chunk_scan, the exclusive scan of chunk_cnt over all chunks); the child's first chunk also writes its
-// cell and list start.
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) chunk_write(LevelIn L, StampDev S, double extent, double half,
-                                                                   const ChunkWork* W, int64_t nw, const int32_t* fr,
-                                                                   uint64_t* slot, const int64_t* ent_off,
-                                                                   const int64_t* next_idx, const int64_t* chunk_scan,
-                                                                   uint32_t* ncoord, int64_t* noff, int32_t* nent) {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= nw) return;
-    const ChunkWork cw = W[w];
-    const int32_t f = fr[cw.t];
-    if (f == kNoStamp) return;  // a leaf child
-    const int64_t i = cw.t >> 3;
-    const int k = (int)(cw.t & 7);
-    if (cw.first && lane == 0) {
-        const int64_t j = next_idx[cw.t];
-        slot[cw.t] = kInternal | (uint64_t)j;
-        ncoord[3 * j] = 2u * L.coord[3 * i] + (k & 1u);
-        ncoord[3 * j + 1] = 2u * L.coord[3 * i + 1] + ((k >> 1) & 1u);
-        ncoord[3 * j + 2] = 2u * L.coord[3 * i + 2] + ((k >> 2) & 1u);
-        noff[j] = ent_off[cw.t];
-    }
-    double pl[3], pm[3], pu[3], cl[3], cm[3];
-    parent_planes(L, i, extent, half, pl, pm, pu, cl, cm);
-    const float hf = (float)(pm[0] - pl[0]), hhf = 0.5f * hf;
-    int64_t pos = ent_off[cw.t] + (chunk_scan[w] - chunk_scan[cw.fw]);
-    for (int64_t base = cw.b; base < cw.e; base += 32) {
-        const int64_t q = base + lane;
-        int32_t out = 0;
-        bool keep = false;
-        if (q < cw.e) {
-            const int32_t x = L.ent[q];
-            if (x < 0) {
-                out = x;
-                keep = true;
-            } else {
-                const int c = entry_class(S, x, k, f, pl, pm, pu, cl, cm, hf, hhf);
-                keep = c != kDrop;
-                out = c == kPaint ? ~x : x;
-            }
-        }
-        const unsigned m = __ballot_sync(kFullMask, keep);
-        if (keep) nent[pos + __popc(m & ((1u << lane) - 1u))] = out;
-        pos += __popc(m);
     }
 }
 
@@ -838,71 +735,89 @@ __global__ void root_write(int64_t n, const int64_t* flag_scan, const int64_t* f
     if (s < n && flag[s]) ent[flag_scan[s]] = (int32_t)s;
 }
 
-// Merge of identical siblings, bottom-up: ckey = the common key of a cell's eight children, else kNotCollapsed.
-__global__ void collapse_level(int64_t n, const uint64_t* slot, const uint64_t* ckey_next, uint64_t* ckey, bool is_root) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint64_t k0 = 0;
-    bool same = !is_root;
-    for (int k = 0; k < 8 && same; ++k) {
-        const uint64_t v = slot[8 * i + k];
-        const uint64_t key = (v & kInternal) ? ckey_next[v & ~kInternal] : v;
-        if (key == kNotCollapsed) same = false;
-        else if (k == 0) k0 = key;
-        else if (key != k0) same = false;
+// Merge of identical siblings, bottom-up, an octet per cell (a lane per child): ckey = the common key of the eight
+// children, else kNotCollapsed. A cell that does not collapse survives as a record; place = its rank among its
+// block's surviving cells and the rank of its first leaf among the block's (kSurvives, bits 16.., bits 0..15), and
+// the block's sums of both.
+constexpr int kMergeCells = 32;  // cells per block (256 threads)
+constexpr uint32_t kSurvives = 1u << 31;
+__global__ void __launch_bounds__(8 * kMergeCells) collapse_level(int64_t n, const uint64_t* slot, const uint64_t* ckey_next,
+                                                                  uint64_t* ckey, bool is_root, uint32_t* place,
+                                                                  BlockSum* bs) {
+    __shared__ uint32_t s_sum[kMergeCells];  // leaves | survives << 16 per cell
+    const int64_t t = (int64_t)blockIdx.x * (8 * kMergeCells) + threadIdx.x, i = t >> 3;
+    const int o = threadIdx.x & 24, k = threadIdx.x & 7;
+    uint64_t key = 0;
+    if (i < n) {
+        const uint64_t v = slot[t];
+        key = (v & kInternal) ? ckey_next[v & ~kInternal] : v;
     }
-    ckey[i] = same ? k0 : kNotCollapsed;
-}
-
-// Surviving records and their stored-leaf counts.
-__global__ void survive_count(int64_t n, const uint64_t* slot, const uint64_t* ckey_next, const uint64_t* ckey,
-                              int64_t* surv, int64_t* nleaf) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const bool s = ckey[i] == kNotCollapsed;
-    int64_t c = 0;
-    if (s) {
-        for (int k = 0; k < 8; ++k) {
-            const uint64_t v = slot[8 * i + k];
-            const uint64_t key = (v & kInternal) ? ckey_next[v & ~kInternal] : v;
-            if (key != kNotCollapsed && key != 0) ++c;
+    const uint64_t k0 = __shfl_sync(kFullMask, key, o);
+    const unsigned eq = (__ballot_sync(kFullMask, key == k0 && key != kNotCollapsed) >> o) & 0xFFu;
+    const unsigned lf = (__ballot_sync(kFullMask, key != kNotCollapsed && key != 0) >> o) & 0xFFu;
+    const bool same = eq == 0xFFu && !is_root, surv = i < n && !same;
+    if (k == 0) {
+        if (i < n) ckey[i] = same ? k0 : kNotCollapsed;
+        s_sum[threadIdx.x >> 3] = surv ? (1u << 16) | __popc(lf) : 0u;
+    }
+    __syncthreads();
+    if (threadIdx.x < kMergeCells) {
+        const uint32_t own = s_sum[threadIdx.x];
+        uint32_t pre = own;
+#pragma unroll
+        for (int d = 1; d < kMergeCells; d <<= 1) {
+            const uint32_t u = __shfl_up_sync(kFullMask, pre, d);
+            if ((int)threadIdx.x >= d) pre += u;
         }
+        const int64_t c = (int64_t)blockIdx.x * kMergeCells + threadIdx.x;
+        if (c < n) place[c] = (pre - own) | (own ? kSurvives : 0u);
+        if (threadIdx.x == kMergeCells - 1) bs[blockIdx.x] = BlockSum{(int64_t)(pre & 0xFFFFu), (int64_t)(pre >> 16)};
     }
-    surv[i] = s ? 1 : 0;
-    nleaf[i] = c;
 }
 
-// Pool rows of the surviving records of one level.
+// Where a level's surviving cells go: place, the blocks' exclusive sums and the groups'.
+struct Ranks {
+    const uint32_t* place;
+    const BlockSum* bs;
+    const BlockSum* sup;
+};
+__device__ __forceinline__ int64_t record_rank(const Ranks& R, int64_t c) {
+    const int64_t b = c / kMergeCells;
+    return R.bs[b].cells + R.sup[b / kScanItems].cells + ((R.place[c] >> 16) & 0x7FFFu);
+}
+
+// Pool rows of the surviving records of one level, a lane per slot.
 // Leaf numbers (breadth-first slot order) are written modulo 2^31; the slot position 8 r + k of each leaf
 // whose number is a nonzero multiple m 2^31 goes to wraps[m - 1].
-__global__ void write_level(int64_t n, const uint64_t* slot, const uint64_t* ckey_next, const int64_t* rec_scan,
-                            const int64_t* leaf_scan, const int64_t* surv, int64_t rec_base, int64_t next_rec_base,
-                            int64_t leaf_base, const int64_t* next_rec_scan, int32_t* nodes, uint2* leaves,
-                            int64_t* wraps) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || !surv[i]) return;
-    const int64_t r = rec_base + rec_scan[i];
-    int64_t lf = leaf_base + leaf_scan[i];
-    for (int k = 0; k < 8; ++k) {
-        const uint64_t v = slot[8 * i + k];
-        int32_t out;
-        uint64_t key;
-        if ((v & kInternal) && ckey_next[v & ~kInternal] == kNotCollapsed) {
-            out = (int32_t)(next_rec_base + next_rec_scan[v & ~kInternal]);
-        } else {
-            key = (v & kInternal) ? ckey_next[v & ~kInternal] : v;
-            if (key == 0) {
-                out = 0;
-            } else {
-                leaves[lf] = make_uint2((uint32_t)key, (uint32_t)(key >> 32));
-                const int64_t low = lf & 0x7FFFFFFFll;
-                out = -(int32_t)low - 1;
-                if (low == 0 && lf > 0) wraps[(lf >> 31) - 1] = 8 * r + k;
-                ++lf;
-            }
-        }
-        nodes[8 * r + k] = out;
+__global__ void __launch_bounds__(8 * kMergeCells) write_level(int64_t n, const uint64_t* slot, const uint64_t* ckey_next,
+                                                               Ranks own, Ranks next, int64_t rec_base,
+                                                               int64_t next_rec_base, int64_t leaf_base, int32_t* nodes,
+                                                               uint2* leaves, int64_t* wraps) {
+    const int64_t t = (int64_t)blockIdx.x * (8 * kMergeCells) + threadIdx.x, i = t >> 3;
+    const int o = threadIdx.x & 24, k = threadIdx.x & 7;
+    uint32_t pl = 0;
+    uint64_t v = 0, key = 0;
+    if (i < n) {
+        pl = own.place[i];
+        v = slot[t];
+        key = (v & kInternal) ? ckey_next[v & ~kInternal] : v;
     }
+    const bool leaf = key != kNotCollapsed && key != 0;
+    const unsigned lf = (__ballot_sync(kFullMask, leaf) >> o) & 0xFFu;
+    if (!(pl & kSurvives)) return;
+    const BlockSum b = own.bs[blockIdx.x], g = own.sup[blockIdx.x / kScanItems];
+    const int64_t r = rec_base + b.cells + g.cells + ((pl >> 16) & 0x7FFFu);
+    int32_t out = 0;
+    if (leaf) {
+        const int64_t l = leaf_base + b.ent + g.ent + (pl & 0xFFFFu) + __popc(lf & ((1u << k) - 1u));
+        leaves[l] = make_uint2((uint32_t)key, (uint32_t)(key >> 32));
+        const int64_t low = l & 0x7FFFFFFFll;
+        out = -(int32_t)low - 1;
+        if (low == 0 && l > 0) wraps[(l >> 31) - 1] = 8 * r + k;
+    } else if (key == kNotCollapsed) {
+        out = (int32_t)(next_rec_base + record_rank(next, (int64_t)(v & ~kInternal)));
+    }
+    nodes[8 * r + k] = out;
 }
 
 // In-place exclusive scan of int64 (three phases; block sums scanned recursively).
@@ -929,6 +844,71 @@ __global__ void scan_add(int64_t* d, int64_t n, const int64_t* sums) {
 
 }  // namespace
 
+// ---------------------------------------------------------------------------
+// Device memory of the painter: a memory pool of its own. A paint makes about ten arrays per level; from the device
+// allocator each costs 30-50 us and a free 30 us (0.3 and 0.5 ms a GB), from the pool 1.5 us. Everything runs on the
+// legacy default stream, which orders frees and reuse. After a paint the pool gives back all but kPoolKeep bytes of
+// what it does not hold live, and canvox_release destroys it.
+// ---------------------------------------------------------------------------
+namespace {
+constexpr size_t kPoolKeep = (size_t)4 << 30;
+cudaMemPool_t g_pool = nullptr;
+
+cudaError_t pool_ready() {
+    if (g_pool) return cudaSuccess;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPoolProps props;
+    std::memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    e = cudaMemPoolCreate(&g_pool, &props);
+    if (e != cudaSuccess) {
+        g_pool = nullptr;
+        return e;
+    }
+    uint64_t keep = ~0ull;  // nothing is given back at the synchronisations of a paint
+    return cudaMemPoolSetAttribute(g_pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
+void pool_trim(size_t keep) {
+    if (g_pool && cudaDeviceSynchronize() == cudaSuccess) cudaMemPoolTrimTo(g_pool, keep);
+}
+
+// Retry an allocation that ran out of memory once the pool has given back what it does not hold live.
+template <typename F>
+cudaError_t with_retry(F alloc) {
+    cudaError_t e = alloc();
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        pool_trim(0);
+        e = alloc();
+    }
+    return e;
+}
+
+template <typename T>
+cudaError_t dalloc(T** p, int64_t n) {
+    *p = nullptr;
+    cudaError_t e = pool_ready();
+    if (e != cudaSuccess) return e;
+    const size_t bytes = sizeof(T) * (size_t)(n > 0 ? n : 1);
+    return with_retry([&] { return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, g_pool, 0); });
+}
+void dfree(void* p) {
+    if (p) cudaFreeAsync(p, 0);
+}
+}  // namespace
+
+void paint_pool_release() {
+    if (!g_pool) return;
+    cudaDeviceSynchronize();
+    cudaMemPoolDestroy(g_pool);
+    g_pool = nullptr;
+}
+
 // Exclusive scan of d[0..n) in place; returns the total through *total (synchronous).
 cudaError_t scan_i64(int64_t* d, int64_t n, int64_t* total) {
     if (n <= 0) {
@@ -937,7 +917,7 @@ cudaError_t scan_i64(int64_t* d, int64_t n, int64_t* total) {
     }
     const int64_t nb = (n + kScanBlock - 1) / kScanBlock;
     int64_t* sums = nullptr;
-    cudaError_t e = cudaMalloc(&sums, sizeof(int64_t) * (size_t)(nb + 1));
+    cudaError_t e = dalloc(&sums, nb + 1);
     if (e != cudaSuccess) return e;
     scan_block<<<(unsigned)nb, kScanBlock>>>(d, n, sums);
     e = cudaGetLastError();
@@ -953,7 +933,7 @@ cudaError_t scan_i64(int64_t* d, int64_t n, int64_t* total) {
             e = cudaMemcpy(&t, sums, sizeof(int64_t), cudaMemcpyDeviceToHost);
         }
     }
-    cudaFree(sums);
+    dfree(sums);
     *total = t;
     return e;
 }
@@ -963,25 +943,23 @@ namespace {
 struct DevBuf {
     std::vector<void*> ptrs;
     ~DevBuf() {
-        for (void* p : ptrs) cudaFree(p);
+        for (void* p : ptrs) dfree(p);
     }
     template <typename T>
     cudaError_t alloc(T** p, int64_t n) {
-        *p = nullptr;
-        cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * (size_t)(n > 0 ? n : 1));
+        const cudaError_t e = dalloc(p, n);
         if (e == cudaSuccess) ptrs.push_back(*p);
         return e;
-    }
-    void release(void* p) {
-        for (auto& q : ptrs)
-            if (q == p) {
-                cudaFree(q);
-                q = nullptr;
-            }
     }
 };
 
 unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
+
+void scan_sums(BlockSum* bs, int64_t n, BlockSum* sup, long long* tot) {
+    const int64_t ng = (n + kScanItems - 1) / kScanItems;
+    scan_groups<<<(unsigned)ng, kScanThreads>>>(bs, n, sup, tot);
+    if (ng > 1) scan_sup<<<1, kScanThreads>>>(sup, ng, tot);
+}
 
 // ---------------------------------------------------------------------------
 // Partitions for appends. The refined cells of one level P (the partition level)
@@ -991,14 +969,6 @@ unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 // appear among the new ones), so a partition whose stamp list at level P is
 // unchanged keeps its whole subtree, and only the others are painted again.
 // ---------------------------------------------------------------------------
-
-// pid_next[child index] = pid[parent] for every internal child (the partition a cell belongs to).
-__global__ void pid_propagate(int64_t n, const uint64_t* slot, const int32_t* pid, int32_t* pid_next) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 8 * n) return;
-    const uint64_t v = slot[t];
-    if (v & kInternal) pid_next[v & ~kInternal] = pid[t >> 3];
-}
 
 // off[p] = first index of partition p in the (nondecreasing) partition ids of one level, p = 0 .. nseg.
 __global__ void seg_offsets(int64_t n, const int32_t* pid, int64_t nseg, int64_t* off) {
@@ -1132,60 +1102,57 @@ cudaError_t finish_pools(const std::vector<uint64_t*>& slots, const std::vector<
                          uint2** d_leaves_out, int64_t* n_rec_out, int64_t* n_leaf_out,
                          std::vector<int64_t>* level_begin, int64_t* wrap_out, int32_t* n_wrap_out) {
     DevBuf buf;
-    // bottom-up merge of identical siblings
-    const int nl = (int)slots.size();
-    std::vector<uint64_t*> ckey((size_t)nl + 1, nullptr);
+    // bottom-up merge of identical siblings, with every level's ranks
+    const size_t nl = slots.size();
+    std::vector<uint64_t*> ckey(nl + 1, nullptr);
+    std::vector<Ranks> ranks(nl + 1);
     uint64_t* none;  // below the deepest level: no refined cells
-    PCK(buf.alloc(&none, 1));
-    ckey[(size_t)nl] = none;
-    for (int l = nl - 1; l >= 0; --l) {
-        PCK(buf.alloc(&ckey[(size_t)l], ncell[(size_t)l]));
-        collapse_level<<<blocks_for(ncell[(size_t)l], 256), 256>>>(ncell[(size_t)l], slots[(size_t)l], ckey[(size_t)l + 1],
-                                                                  ckey[(size_t)l], l == 0);
+    PCK(buf.alloc(&none, 2));
+    ckey[nl] = none;
+    ranks[nl] = Ranks{nullptr, nullptr, nullptr};
+    long long* d_tot;
+    PCK(buf.alloc(&d_tot, 2 * (int64_t)nl + 2));
+    for (size_t l = nl; l-- > 0;) {
+        const int64_t nc = ncell[l], nb = (nc + kMergeCells - 1) / kMergeCells, ng = (nb + kScanItems - 1) / kScanItems;
+        uint32_t* place;
+        BlockSum *bs, *sup;
+        PCK(buf.alloc(&ckey[l], nc));
+        PCK(buf.alloc(&place, nc));
+        PCK(buf.alloc(&bs, nb));
+        PCK(buf.alloc(&sup, ng));
+        collapse_level<<<(unsigned)nb, 8 * kMergeCells>>>(nc, slots[l], ckey[l + 1], ckey[l], l == 0, place, bs);
+        scan_sums(bs, nb, sup, d_tot + 2 * l);
         PCK(cudaGetLastError());
+        ranks[l] = Ranks{place, bs, sup};
     }
+    std::vector<long long> tot(2 * nl);
+    PCK(cudaMemcpy(tot.data(), d_tot, sizeof(long long) * tot.size(), cudaMemcpyDeviceToHost));
     // breadth-first numbering: records level by level, leaves in slot order
-    std::vector<int64_t*> rec_scan((size_t)nl + 1, nullptr), leaf_scan((size_t)nl, nullptr), surv((size_t)nl, nullptr);
-    std::vector<int64_t> rec_base((size_t)nl + 1, 0), leaf_base((size_t)nl + 1, 0);
-    for (int l = 0; l < nl; ++l) {
-        const int64_t nc = ncell[(size_t)l];
-        PCK(buf.alloc(&surv[(size_t)l], nc));
-        PCK(buf.alloc(&rec_scan[(size_t)l], nc));
-        PCK(buf.alloc(&leaf_scan[(size_t)l], nc));
-        survive_count<<<blocks_for(nc, 256), 256>>>(nc, slots[(size_t)l], ckey[(size_t)l + 1], ckey[(size_t)l],
-                                                     rec_scan[(size_t)l], leaf_scan[(size_t)l]);
-        PCK(cudaGetLastError());
-        PCK(cudaMemcpy(surv[(size_t)l], rec_scan[(size_t)l], sizeof(int64_t) * (size_t)nc, cudaMemcpyDeviceToDevice));
-        int64_t nr = 0, nlf = 0;
-        PCK(scan_i64(rec_scan[(size_t)l], nc, &nr));
-        PCK(scan_i64(leaf_scan[(size_t)l], nc, &nlf));
-        rec_base[(size_t)l + 1] = rec_base[(size_t)l] + nr;
-        leaf_base[(size_t)l + 1] = leaf_base[(size_t)l] + nlf;
+    std::vector<int64_t> rec_base(nl + 1, 0), leaf_base(nl + 1, 0);
+    for (size_t l = 0; l < nl; ++l) {
+        leaf_base[l + 1] = leaf_base[l] + tot[2 * l];
+        rec_base[l + 1] = rec_base[l] + tot[2 * l + 1];
     }
-    const int64_t n_rec = rec_base[(size_t)nl], n_leaf = leaf_base[(size_t)nl];
+    const int64_t n_rec = rec_base[nl], n_leaf = leaf_base[nl];
     if (n_rec > 0x7FFFFFFFll || n_leaf > kMaxLeaves) return cudaErrorMemoryAllocation;  // beyond the pool format
     const int32_t n_wrap = n_leaf > 0 ? (int32_t)((n_leaf - 1) >> 31) : 0;
     int64_t* d_wraps;
     PCK(buf.alloc(&d_wraps, kMaxWraps));
     int32_t* d_nodes = nullptr;
     uint2* d_leaves = nullptr;
-    PCK(cudaMalloc(&d_nodes, sizeof(int32_t) * 8 * (size_t)n_rec));
-    cudaError_t e = cudaMalloc(&d_leaves, sizeof(uint2) * (size_t)(n_leaf > 0 ? n_leaf : 1));
+    PCK(with_retry([&] { return cudaMalloc(&d_nodes, sizeof(int32_t) * 8 * (size_t)n_rec); }));
+    cudaError_t e = with_retry([&] { return cudaMalloc(&d_leaves, sizeof(uint2) * (size_t)(n_leaf > 0 ? n_leaf : 1)); });
     if (e != cudaSuccess) {
         cudaFree(d_nodes);
         return e;
     }
-    int64_t* zero_scan;
-    PCK(buf.alloc(&zero_scan, 1));
-    for (int l = 0; l < nl && e == cudaSuccess; ++l) {
-        const int64_t nc = ncell[(size_t)l];
-        write_level<<<blocks_for(nc, 256), 256>>>(nc, slots[(size_t)l], ckey[(size_t)l + 1], rec_scan[(size_t)l],
-                                                   leaf_scan[(size_t)l], surv[(size_t)l], rec_base[(size_t)l],
-                                                   rec_base[(size_t)l + 1], leaf_base[(size_t)l],
-                                                   l + 1 < nl ? rec_scan[(size_t)l + 1] : zero_scan, d_nodes, d_leaves,
-                                                   d_wraps);
-        e = cudaGetLastError();
+    for (size_t l = 0; l < nl; ++l) {
+        const int64_t nc = ncell[l];
+        write_level<<<blocks_for(nc, kMergeCells), 8 * kMergeCells>>>(nc, slots[l], ckey[l + 1], ranks[l], ranks[l + 1],
+                                                                       rec_base[l], rec_base[l + 1], leaf_base[l],
+                                                                       d_nodes, d_leaves, d_wraps);
     }
+    e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess && n_wrap > 0)
         e = cudaMemcpy(wrap_out, d_wraps, sizeof(int64_t) * (size_t)n_wrap, cudaMemcpyDeviceToHost);
@@ -1200,8 +1167,8 @@ cudaError_t finish_pools(const std::vector<uint64_t*>& slots, const std::vector<
     *n_rec_out = n_rec;
     *n_leaf_out = n_leaf;
     level_begin->clear();
-    for (int l = 0; l <= nl; ++l)
-        if (l == 0 || rec_base[(size_t)l] > rec_base[(size_t)l - 1]) level_begin->push_back(rec_base[(size_t)l]);
+    for (size_t l = 0; l <= nl; ++l)
+        if (l == 0 || rec_base[l] > rec_base[l - 1]) level_begin->push_back(rec_base[l]);
     return cudaSuccess;
 }
 
@@ -1212,15 +1179,20 @@ namespace {
 // Refined cells of one level with their ordered stamp lists (device arrays owned here).
 struct Level {
     int64_t n = 0;
+    int64_t n_ent = 0;    // entries of all lists
+    int64_t longest = 0;  // the longest list (0: none is longer than kLongList)
     int32_t level = 0;
     uint32_t* coord = nullptr;  // [n][3]
     int64_t* off = nullptr;     // [n + 1]
     int32_t* ent = nullptr;     // s: descends, ~s: paints the whole cell
-    LevelIn in() const { return LevelIn{n, level, coord, off, ent}; }
+    LevelIn in(double extent) const {
+        const double h = std::ldexp(extent, -(level + 1));
+        return LevelIn{n, level, coord, off, ent, h, (float)h};
+    }
     void free() {
-        cudaFree(coord);
-        cudaFree(off);
-        cudaFree(ent);
+        dfree(coord);
+        dfree(off);
+        dfree(ent);
         coord = nullptr;
         off = nullptr;
         ent = nullptr;
@@ -1228,126 +1200,82 @@ struct Level {
     }
 };
 
-template <typename T>
-cudaError_t dalloc(T** p, int64_t n) {
-    *p = nullptr;
-    return cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * (size_t)(n > 0 ? n : 1));
-}
-
-// The long cells of a level (lists longer than kChunkMinList) and the chunks of their children's lists (see
-// chunk_firstref); *skip marks them for the level's other passes. Nothing when the level has none.
-cudaError_t chunk_plan(const Level& L, DevBuf& buf, uint8_t** skip, std::vector<int64_t>* cells,
-                       std::vector<ChunkWork>* work) {
-    *skip = nullptr;
-    cells->clear();
-    work->clear();
-    int64_t total = 0;  // entries of the whole level: no cell is long if they are few
-    cudaError_t e = cudaMemcpy(&total, L.off + L.n, sizeof(int64_t), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess || total <= kChunkMinList) return e;
-    uint8_t* sk = nullptr;
-    int64_t *flag = nullptr, *out = nullptr;
-    if ((e = buf.alloc(&sk, L.n)) != cudaSuccess || (e = buf.alloc(&flag, L.n)) != cudaSuccess) return e;
-    flag_long<<<blocks_for(L.n, 256), 256>>>(L.in(), sk, flag);
-    int64_t n_long = 0;
-    if ((e = cudaGetLastError()) != cudaSuccess || (e = scan_i64(flag, L.n, &n_long)) != cudaSuccess) return e;
-    if (n_long == 0) return cudaSuccess;
-    if ((e = buf.alloc(&out, 3 * n_long)) != cudaSuccess) return e;
-    gather_long<<<blocks_for(L.n, 256), 256>>>(L.in(), sk, flag, out);
-    std::vector<int64_t> h((size_t)(3 * n_long));
-    if ((e = cudaGetLastError()) != cudaSuccess ||
-        (e = cudaMemcpy(h.data(), out, sizeof(int64_t) * h.size(), cudaMemcpyDeviceToHost)) != cudaSuccess)
-        return e;
-    for (int64_t j = 0; j < n_long; ++j) {
-        const int64_t i = h[(size_t)(3 * j)], b0 = h[(size_t)(3 * j + 1)], e0 = h[(size_t)(3 * j + 2)];
-        cells->push_back(i);
-        for (int k = 0; k < 8; ++k) {
-            const int64_t fw = (int64_t)work->size();
-            for (int64_t b = b0; b < e0; b += kChunk)
-                work->push_back(ChunkWork{8 * i + k, b, std::min(e0, b + kChunk), fw, b == b0 ? 1 : 0});
-        }
-    }
-    *skip = sk;
-    return cudaSuccess;
-}
-
 // Expand one level: the eight child slots of each cell (*slot_out, handed to the caller: a leaf key, or
-// kInternal | index in the next level) and the next level's refined cells with their lists.
-cudaError_t expand(const Level& L, const StampDev& S, int32_t depth, double extent, double half, uint64_t** slot_out,
-                   Level* next) {
+// kInternal | index in the next level) and the next level's refined cells with their lists; with pid (the cells'
+// partitions) also the next level's (*npid).
+cudaError_t expand(const Level& L, const StampDev& S, double extent, double half, uint64_t** slot_out, Level* next,
+                   const int32_t* pid, int32_t** npid) {
     DevBuf buf;
-    const int64_t nch = 8 * L.n;
-    int32_t* fr;
-    int64_t *cnt, *isint;
+    const int64_t nch = 8 * L.n, nb = (L.n + kCells - 1) / kCells, ng = (nb + kScanItems - 1) / kScanItems;
+    int32_t* cnt;
+    uint16_t* cls;
+    BlockSum *bs, *sup;
+    long long* tot;
     uint64_t* slot;
-    PCK(buf.alloc(&fr, nch));
     PCK(buf.alloc(&cnt, nch));
-    PCK(buf.alloc(&isint, nch));
+    PCK(buf.alloc(&cls, L.n_ent));
+    PCK(buf.alloc(&bs, nb));
+    PCK(buf.alloc(&sup, ng));
+    PCK(buf.alloc(&tot, 3));
     PCK(dalloc(&slot, nch));
     *slot_out = slot;
-    const LevelIn in = L.in();
-    const bool split = L.n < kSplitCells;  // few cells: a warp per child
-    // cells with long lists: a warp per chunk of a child's list (the passes below skip them)
-    uint8_t* skip = nullptr;
-    std::vector<int64_t> cells;
-    std::vector<ChunkWork> work;
-    PCK(chunk_plan(L, buf, &skip, &cells, &work));
-    const int64_t nw = (int64_t)work.size(), nj = 8 * (int64_t)cells.size();
-    ChunkWork* d_work = nullptr;
-    int64_t *d_cells = nullptr, *chunk_cnt = nullptr, *npaint = nullptr;
-    if (nw) {
-        PCK(buf.alloc(&d_work, nw));
-        PCK(buf.alloc(&d_cells, (int64_t)cells.size()));
-        PCK(buf.alloc(&chunk_cnt, nw));
-        PCK(buf.alloc(&npaint, nch));
-        PCK(cudaMemcpy(d_work, work.data(), sizeof(ChunkWork) * (size_t)nw, cudaMemcpyHostToDevice));
-        PCK(cudaMemcpy(d_cells, cells.data(), sizeof(int64_t) * cells.size(), cudaMemcpyHostToDevice));
-        chunk_init<<<blocks_for(nj, 256), 256>>>(d_cells, nj, fr, cnt, npaint);
-        chunk_firstref<<<blocks_for(nw, kWarpsPerBlock), 32 * kWarpsPerBlock>>>(in, S, depth, extent, half, d_work, nw, fr);
-        chunk_count<<<blocks_for(nw, kWarpsPerBlock), 32 * kWarpsPerBlock>>>(in, S, extent, half, d_work, nw, fr, chunk_cnt,
-                                                                             cnt, npaint);
-        chunk_child_finish<<<blocks_for(nj, kWarpsPerBlock), 32 * kWarpsPerBlock>>>(in, S, extent, half, d_cells, nj, fr,
-                                                                                   npaint, slot, cnt, isint);
+    const LevelIn in = L.in(extent);
+    PCK(cudaMemsetAsync(tot, 0, 3 * sizeof(long long), 0));
+    // cells with long lists: an octet per item of a list
+    unsigned long long h_long[2] = {0, 0};  // cells, items
+    Item* items = nullptr;
+    int32_t* icnt = nullptr;
+    if (L.longest > kLongList) {
+        LongCell* cells;
+        unsigned long long* ctr;
+        PCK(buf.alloc(&cells, L.n_ent / kLongList));
+        PCK(buf.alloc(&ctr, 2));
+        PCK(cudaMemsetAsync(ctr, 0, sizeof(h_long), 0));
+        find_long<<<blocks_for(L.n, 256), 256>>>(in, cells, ctr);
+        PCK(cudaGetLastError());
+        PCK(cudaMemcpy(h_long, ctr, sizeof(h_long), cudaMemcpyDeviceToHost));
+        const int64_t nlong = (int64_t)h_long[0], ni = (int64_t)h_long[1];
+        if (nlong) {
+            int32_t *fr, *npaint;
+            PCK(buf.alloc(&items, ni));
+            PCK(buf.alloc(&icnt, 8 * ni));
+            PCK(buf.alloc(&fr, 8 * nlong));
+            PCK(buf.alloc(&npaint, 8 * nlong));
+            long_items<<<(unsigned)nlong, 128>>>(cells, items, fr);
+            long_first<<<blocks_for(ni, 16), 128>>>(in, S, half, items, ni, fr);
+            long_count<<<blocks_for(ni, 16), 128>>>(in, S, half, items, ni, fr, cls, icnt);
+            long_sums<<<(unsigned)nlong, 8 * kSumRows>>>(cells, fr, icnt, slot, cnt, npaint);
+            long_blend<<<blocks_for(8 * nlong, 4), 128>>>(in, S, cells, nlong, npaint, cls, slot);
+            PCK(cudaGetLastError());
+        }
     }
-    if (split)
-        expand_child_count<<<blocks_for(nch, kWarpsPerBlock), 32 * kWarpsPerBlock>>>(in, S, depth, extent, half, fr, slot,
-                                                                                    cnt, isint, skip);
-    else
-        expand_parent_count<<<blocks_for(L.n, kWarpsPerBlock), 32 * kWarpsPerBlock>>>(in, S, depth, extent, half, fr,
-                                                                                     slot, cnt, isint, skip);
+    expand_count<<<(unsigned)nb, 8 * kCells>>>(in, S, half, slot, cnt, cls, bs, tot);
+    scan_sums(bs, nb, sup, tot);
     PCK(cudaGetLastError());
-    int64_t n_ent = 0, n_next = 0;
-    PCK(scan_i64(cnt, nch, &n_ent));
-    PCK(scan_i64(isint, nch, &n_next));
-    next->n = n_next;
+    long long h_tot[3];
+    PCK(cudaMemcpy(h_tot, tot, sizeof(h_tot), cudaMemcpyDeviceToHost));
+    next->n = h_tot[1];
+    next->n_ent = h_tot[0];
+    next->longest = h_tot[2];
     next->level = L.level + 1;
-    if (n_next == 0) return cudaSuccess;  // no internal child: the slots are all leaf keys
-    PCK(dalloc(&next->coord, 3 * n_next));
-    PCK(dalloc(&next->off, n_next + 1));
-    PCK(dalloc(&next->ent, n_ent));
-    PCK(cudaMemcpy(next->off + n_next, &n_ent, sizeof(int64_t), cudaMemcpyHostToDevice));
-    if (nw) {
-        int64_t n_chunked = 0;
-        PCK(scan_i64(chunk_cnt, nw, &n_chunked));  // per child: its list start plus the counts of earlier chunks
-        chunk_write<<<blocks_for(nw, kWarpsPerBlock), 32 * kWarpsPerBlock>>>(in, S, extent, half, d_work, nw, fr, slot, cnt,
-                                                                             isint, chunk_cnt, next->coord, next->off,
-                                                                             next->ent);
-    }
-    if (split)
-        expand_child_write<<<blocks_for(nch, kWarpsPerBlock), 32 * kWarpsPerBlock>>>(in, S, extent, half, fr, slot, cnt,
-                                                                                    isint, next->coord, next->off,
-                                                                                    next->ent, skip);
-    else
-        expand_parent_write<<<blocks_for(L.n, kWarpsPerBlock), 32 * kWarpsPerBlock>>>(in, S, extent, half, fr, slot,
-                                                                                     cnt, isint, next->coord, next->off,
-                                                                                     next->ent, skip);
-    PCK(cudaGetLastError());
-    return cudaDeviceSynchronize();
+    if (next->n == 0) return cudaSuccess;  // no internal child: the slots are all leaf keys
+    PCK(dalloc(&next->coord, 3 * next->n));
+    PCK(dalloc(&next->off, next->n + 1));
+    PCK(dalloc(&next->ent, next->n_ent));
+    if (pid) PCK(dalloc(npid, next->n));
+    PCK(cudaMemcpyAsync(next->off + next->n, tot, sizeof(int64_t), cudaMemcpyDeviceToDevice, 0));
+    expand_write<<<(unsigned)nb, 8 * kCells>>>(in, slot, cnt, cls, bs, sup, pid, next->coord, next->off, next->ent,
+                                               pid ? *npid : nullptr);
+    if (items)
+        long_write<<<blocks_for((int64_t)h_long[1], 16), 128>>>(in, items, (int64_t)h_long[1], slot, cls, icnt, next->off,
+                                                                next->ent);
+    return cudaGetLastError();
 }
 
 // Paint down from L (its arrays are freed on the way): slots and cell counts per level, until no refined cell is
 // left, or up to level `stop` (that level's cells are then left unexpanded in *rest). With track, the cells of L
 // are partitions 0 .. L.n - 1 and offs receives, per painted level, the first cell of each partition.
-cudaError_t paint_down(Level L, const StampDev& S, int32_t depth, double extent, double half, int stop, bool track,
+cudaError_t paint_down(Level L, const StampDev& S, double extent, double half, int stop, bool track,
                        std::vector<uint64_t*>* slots, std::vector<int64_t>* ncell, Level* rest,
                        std::vector<int64_t*>* offs) {
     const int64_t nseg = L.n;
@@ -1359,8 +1287,9 @@ cudaError_t paint_down(Level L, const StampDev& S, int32_t depth, double extent,
     }
     while (e == cudaSuccess && L.n > 0 && L.level != stop) {
         uint64_t* slot = nullptr;
+        int32_t* npid = nullptr;
         Level next;
-        e = expand(L, S, depth, extent, half, &slot, &next);
+        e = expand(L, S, extent, half, &slot, &next, pid, &npid);
         if (slot) {
             slots->push_back(slot);
             ncell->push_back(L.n);
@@ -1371,19 +1300,16 @@ cudaError_t paint_down(Level L, const StampDev& S, int32_t depth, double extent,
             if (e == cudaSuccess) {
                 offs->push_back(off);
                 seg_offsets<<<blocks_for(nseg + 1, 256), 256>>>(L.n, pid, nseg, off);
-                int32_t* pid_next = nullptr;
-                if (next.n > 0 && (e = dalloc(&pid_next, next.n)) == cudaSuccess)
-                    pid_propagate<<<blocks_for(8 * L.n, 256), 256>>>(L.n, slot, pid, pid_next);
-                if (e == cudaSuccess) e = cudaGetLastError();
-                cudaFree(pid);
-                pid = pid_next;
+                e = cudaGetLastError();
             }
         }
+        dfree(pid);
+        pid = npid;
         L.free();
         L = next;
         if (e != cudaSuccess) L.free();
     }
-    cudaFree(pid);
+    dfree(pid);
     if (e == cudaSuccess && L.n > 0 && L.level == stop) {
         *rest = L;
     } else {
@@ -1413,11 +1339,11 @@ struct PaintCache {
 
 void paint_cache_free(PaintCache* c) {
     if (!c) return;
-    cudaFree(c->code);
-    cudaFree(c->lst_off);
-    cudaFree(c->lst_ent);
-    for (auto* p : c->slots) cudaFree(p);
-    for (auto* p : c->off) cudaFree(p);
+    dfree(c->code);
+    dfree(c->lst_off);
+    dfree(c->lst_ent);
+    for (auto* p : c->slots) dfree(p);
+    for (auto* p : c->off) dfree(p);
     delete c;
 }
 
@@ -1426,11 +1352,11 @@ namespace {
 constexpr int kPartLevel = 5;  // partition level: up to 32,768 partitions
 
 void free_all(std::vector<uint64_t*>& v) {
-    for (auto* p : v) cudaFree(p);
+    for (auto* p : v) dfree(p);
     v.clear();
 }
 void free_all(std::vector<int64_t*>& v) {
-    for (auto* p : v) cudaFree(p);
+    for (auto* p : v) dfree(p);
     v.clear();
 }
 
@@ -1447,6 +1373,7 @@ cudaError_t root_level(const StampDev& S, int64_t n, double extent, double half,
         PCK(scan_i64(flag_scan, n, &n_root));
     }
     root->n = 1;
+    root->n_ent = root->longest = n_root;
     root->level = 0;
     PCK(dalloc(&root->coord, 3));
     PCK(dalloc(&root->off, 2));
@@ -1482,7 +1409,7 @@ cudaError_t assemble(int64_t n_part, const int32_t* reuse, const int32_t* rep, c
         PCK(scan_i64(off, n_part, &total));
         PCK(cudaMemcpy(off + n_part, &total, sizeof(int64_t), cudaMemcpyHostToDevice));
         if (total == 0) {
-            cudaFree(off);
+            dfree(off);
             offs->pop_back();
             break;
         }
@@ -1517,14 +1444,14 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     DevBuf buf;
     // squared radii and target depths (the host painter's integer loop, in the same FP64 operations)
     double* d_r2;
-    int32_t* d_kt;
+    StampRec* d_rec;
     cudaError_t e = buf.alloc(&d_r2, n);
-    if (e == cudaSuccess) e = buf.alloc(&d_kt, n);
+    if (e == cudaSuccess) e = buf.alloc(&d_rec, n);
     if (e == cudaSuccess && n > 0) {
-        stamp_prep<<<blocks_for(n, 256), 256>>>(d_r, n, depth, extent, d_r2, d_kt);
+        stamp_prep<<<blocks_for(n, 256), 256>>>(d_c, d_r, n, depth, extent, d_r2, d_rec);
         e = cudaGetLastError();
     }
-    const StampDev S{d_c, d_r2, d_kt, d_rgba};
+    const StampDev S{d_c, d_r2, d_rec, d_rgba};
     // levels 0 .. P - 1 from the root (always painted: every stamp reaches the root's list)
     std::vector<uint64_t*> slots_top, slots_bot, slots_r;
     std::vector<int64_t> ncell_top, ncell_bot, ncell_r;
@@ -1532,7 +1459,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     Level root, partP, rep_lvl, unused;
     PaintCache* nc = nullptr;
     if (e == cudaSuccess) e = root_level(S, n, extent, half, &root);
-    if (e == cudaSuccess) e = paint_down(root, S, depth, extent, half, kPartLevel, false, &slots_top, &ncell_top, &partP, nullptr);
+    if (e == cudaSuccess) e = paint_down(root, S, extent, half, kPartLevel, false, &slots_top, &ncell_top, &partP, nullptr);
     else root.free();
     if (e == cudaSuccess) {
         nc = new PaintCache();
@@ -1556,7 +1483,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
         if (e == cudaSuccess && partP.n > 0) {
             int64_t n_ent = 0;
             e = cudaMemcpy(&n_ent, partP.off + partP.n, sizeof(int64_t), cudaMemcpyDeviceToHost);
-            cudaFree(keep_ent);
+            dfree(keep_ent);
             keep_ent = nullptr;
             if (e == cudaSuccess) e = dalloc(&keep_ent, n_ent);
             if (e == cudaSuccess)
@@ -1567,7 +1494,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
         nc->lst_off = keep_off;
         nc->lst_ent = keep_ent;
         if (e == cudaSuccess)
-            e = paint_down(start, S, depth, extent, half, -1, true, &slots_bot, &ncell_bot, &unused, &offs_bot);
+            e = paint_down(start, S, extent, half, -1, true, &slots_bot, &ncell_bot, &unused, &offs_bot);
         else
             start.free();
         partP = Level();
@@ -1603,6 +1530,8 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
             list_lengths<<<blocks_for(m, 256), 256>>>(m, sel, partP.off, len);
             int64_t n_ent = 0;
             e = scan_i64(len, m, &n_ent);
+            rep_lvl.n_ent = n_ent;
+            rep_lvl.longest = partP.longest;
             if (e == cudaSuccess) e = cudaMemcpy(len + m, &n_ent, sizeof(int64_t), cudaMemcpyHostToDevice);
             if (e == cudaSuccess) e = dalloc(&rep_lvl.coord, 3 * m);
             if (e == cudaSuccess) e = dalloc(&rep_lvl.off, m + 1);
@@ -1616,7 +1545,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
                 e = cudaMemcpy(rep_lvl.off + m, &n_ent, sizeof(int64_t), cudaMemcpyHostToDevice);
         }
         if (e == cudaSuccess)
-            e = paint_down(rep_lvl, S, depth, extent, half, -1, true, &slots_r, &ncell_r, &unused, &offs_r);
+            e = paint_down(rep_lvl, S, extent, half, -1, true, &slots_r, &ncell_r, &unused, &offs_r);
         else
             rep_lvl.free();
         if (e == cudaSuccess) e = assemble(np, reuse, rep, *old, slots_r, offs_r, &slots_bot, &ncell_bot, &offs_bot);
@@ -1625,7 +1554,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
         // the new level-P lists are kept
         nc->lst_off = partP.off;
         nc->lst_ent = partP.ent;
-        cudaFree(partP.coord);
+        dfree(partP.coord);
         partP = Level();
     }
     paint_cache_free(old);
@@ -1638,6 +1567,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     }
     free_all(slots_top);
     partP.free();
+    pool_trim(kPoolKeep);
     if (e == cudaSuccess) {
         nc->slots = slots_bot;
         nc->ncell = ncell_bot;

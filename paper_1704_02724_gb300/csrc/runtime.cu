@@ -1009,6 +1009,7 @@ void canvox_release(void) {
     if (g.d_st_r) cudaFree(g.d_st_r);
     if (g.d_st_rgba) cudaFree(g.d_st_rgba);
     paint_cache_free(g.paint_cache);
+    paint_pool_release();
     if (g.done) cudaEventDestroy(g.done);
     g = Ctx();
 }
