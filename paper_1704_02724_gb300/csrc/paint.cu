@@ -61,7 +61,8 @@ constexpr int64_t kLongList = 512;      // longer lists are cut into items ...
 constexpr int64_t kItem = 128;          // ... of so many entries, one octet each
 constexpr int32_t kNoStamp = 0x7FFFFFFF;
 
-// What a child box test reads of a stamp: the centre as two FP32 words per axis, the squared radius, the target depth.
+// What a child box test reads of a stamp: the centre as two FP32 words per axis, the squared radius (both scaled by the
+// power of two that brings the canvas to a side in [1, 2), so that no FP32 square leaves its range), the target depth.
 struct StampRec {
     float ch[3], cl0;
     float cl1, cl2, r2;
@@ -119,7 +120,7 @@ struct LevelIn {
     const int64_t* off;     // [n + 1]
     const int32_t* ent;     // s: descends, ~s: paints the whole cell
     double h;               // side of the children
-    float hf;
+    float hf;               // the same scaled as the stamps' records are (NaN: a canvas for FP64 alone)
 };
 
 // How a stamp covers a box.
@@ -253,8 +254,8 @@ __device__ __forceinline__ int cover(const StampDev& S, int32_t v, const StampRe
 enum { kDrop = 0, kPaint = 1, kKeep = 2 };
 
 // Squared radius, target depth (the smallest k with extent 2^-k <= r/10, at most depth) and record of each stamp.
-__global__ void stamp_prep(const double* c, const double* r, int64_t n, int32_t depth, double extent, double* r2,
-                           StampRec* rec) {
+__global__ void stamp_prep(const double* c, const double* r, int64_t n, int32_t depth, double extent, double scale,
+                           double* r2, StampRec* rec) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const double rs = r[s];
@@ -269,8 +270,9 @@ __global__ void stamp_prep(const double* c, const double* r, int64_t n, int32_t 
     }
     float h[3], l[3];
     for (int a = 0; a < 3; ++a) {
-        h[a] = (float)c[3 * s + a];
-        l[a] = (float)(c[3 * s + a] - (double)h[a]);
+        const double x = c[3 * s + a] * scale;
+        h[a] = (float)x;
+        l[a] = (float)(x - (double)h[a]);
     }
     StampRec R;
     R.ch[0] = h[0];
@@ -279,7 +281,7 @@ __global__ void stamp_prep(const double* c, const double* r, int64_t n, int32_t 
     R.cl0 = l[0];
     R.cl1 = l[1];
     R.cl2 = l[2];
-    R.r2 = (float)rr;
+    R.r2 = (float)(rr * scale * scale);
     R.kt = k;
     rec[s] = R;
 }
@@ -1176,6 +1178,13 @@ cudaError_t finish_pools(const std::vector<uint64_t*>& slots, const std::vector<
 
 namespace {
 
+// The power of two that brings the canvas side to [1, 2). NaN past 2^+-400, where the FP64 squares themselves come near
+// the end of their range and the FP32 screen, which would not, is left out (every comparison with a NaN is open).
+double screen_scale(double extent) {
+    const int e = std::ilogb(extent);
+    return e < -400 || e > 400 ? std::nan("") : std::ldexp(1.0, -e);
+}
+
 // Refined cells of one level with their ordered stamp lists (device arrays owned here).
 struct Level {
     int64_t n = 0;
@@ -1187,7 +1196,7 @@ struct Level {
     int32_t* ent = nullptr;     // s: descends, ~s: paints the whole cell
     LevelIn in(double extent) const {
         const double h = std::ldexp(extent, -(level + 1));
-        return LevelIn{n, level, coord, off, ent, h, (float)h};
+        return LevelIn{n, level, coord, off, ent, h, (float)(h * screen_scale(extent))};
     }
     void free() {
         dfree(coord);
@@ -1448,7 +1457,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     cudaError_t e = buf.alloc(&d_r2, n);
     if (e == cudaSuccess) e = buf.alloc(&d_rec, n);
     if (e == cudaSuccess && n > 0) {
-        stamp_prep<<<blocks_for(n, 256), 256>>>(d_c, d_r, n, depth, extent, d_r2, d_rec);
+        stamp_prep<<<blocks_for(n, 256), 256>>>(d_c, d_r, n, depth, extent, screen_scale(extent), d_r2, d_rec);
         e = cudaGetLastError();
     }
     const StampDev S{d_c, d_r2, d_rec, d_rgba};
