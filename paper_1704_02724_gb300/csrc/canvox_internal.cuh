@@ -116,7 +116,7 @@ struct MixedParams {
     int32_t smem_records;
     int32_t use_ropes;   // 1: neighbour links (Tree::ropes), 0: stack of ancestors
     int32_t count_reads; // 1: count slot reads, leaf loads and record loads (canvox_stats)
-    // set by launch_mixed
+    // set by the launchers
     double inv_extent, unit;  // 1 / extent, extent 2^-31
     float side;               // extent
     float bound_t, bound_i;   // the colour bound of a boundary per local time and per ih (see ray_step)

@@ -1,25 +1,37 @@
 // FP64 twin of the mixed-precision traversal: the precision comparator.
 //
 // The same traversal as the mixed kernel (trace_mixed.cu): a persistent grid
-// whose warps pop tiles of rays from one global queue, exact integer cell
-// coordinates, the neighbour found as a sibling or through the parent's
-// neighbour link (the neighbour graph of Sec. 4.1.1, built at upload), a
-// descent while the cell is internal, front-to-back compositing to full
-// opacity or the canvas exit (Sec. 6.2). What differs is the arithmetic:
-// every crossing time is FP64 from the exact plane, t = P inv + nod in canvas
-// coordinates (no local frame, no FP32 screen, no error budget), every side
-// test is FP64, and colour and transmittance are FP64 sums. Timing this kernel
-// beside the mixed one isolates what the local frames of Sec. 6.1-6.3 buy on
-// this GPU, whose FP64 rate is a small fraction of its FP32 rate; the plain FP64
-// caster (trace_plain.cu) differs from the mixed kernel in its traversal too.
+// whose warps pop tiles of rays from one global queue, exact fixed-point cell
+// corners in the mirrored canvas, the neighbour found as a sibling or through
+// the parent's neighbour link (the neighbour graph of Sec. 4.1.1, built at
+// upload), a descent while the cell is internal, front-to-back compositing to
+// full opacity or the canvas exit (Sec. 6.2). What differs is the arithmetic:
+// every crossing time, position and sum is FP64 (no anchor, no FP32 screen, no
+// error budget). Timing this kernel beside the mixed one isolates what the
+// single-precision decisions buy on this GPU, whose FP64 rate is a small
+// fraction of its FP32 rate; the plain FP64 caster (trace_plain.cu) differs from
+// the mixed kernel in its traversal too.
 //
-// Decisions follow the FP64 oracle's conventions: a ray leaves a leaf by the
-// face with the smallest crossing time (ties to the lowest axis), and is on the
-// high side of a plane M just after t iff (M - o)/d <= t for d > 0, > t for
-// d < 0, and o >= M for d = 0 (here with the product form M inv + nod).
+// A plane's time is (X - eye) / |d|, the difference in units taken between
+// integers and the eye's rest below a unit (the ray's own 53 bits then count from
+// the eye, not from the canvas's centre); the sides below the old cell's level
+// are the bits of the position eye + t d. A ray leaves a leaf by the face with
+// the smallest crossing time (ties to the lowest axis); a position on a plane is
+// on the side the ray moves into, for d = 0 on the high side.
+//
+// What bounds it: the FP64 pipe, an instruction of which occupies an SM's unit
+// for 16 cycles however few lanes take part, so the step counts them: two per
+// axis for the exit times (an integer becomes a double by its bit pattern and
+// one addition), compares, half-to-double conversions and the termination test on
+// integer patterns, the opacity of thin leaves by its series, one position per
+// descent instead of a plane and a time per level and axis. 28 FP64 instructions
+// per warp and step (pipe 86 % busy): a depth-24 stereo pair of 540^2 with 205
+// leaves a ray takes 6.25 ms, 15.6 ms with a plane and a time per level and axis,
+// conversions and the library's opacity for every leaf.
 #include <cuda_fp16.h>
 
 #include "canvox_internal.cuh"
+#include "cells.cuh"
 
 namespace canvox {
 namespace {
@@ -27,72 +39,106 @@ namespace {
 constexpr unsigned kFull64 = 0xFFFFFFFFu;
 constexpr int kBlock64 = 256;
 
-__device__ __forceinline__ double p2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
-__device__ __forceinline__ double h2d(unsigned h) { return (double)__half2float(__ushort_as_half((unsigned short)h)); }
-
-// FP64 state of a lane that the step reads rarely: the output address and the colour sums.
-struct Cold64 {
-    double C[3];
-    uint32_t pix;
-    int32_t view;
+// Per-lane FP64 state that a step reads rarely, one 8-byte column per field and lane.
+enum Col64 {
+    kColC = 0,      // double: colour sums, three columns
+    kColDs = 3,     // double: |d_a| in units per length
+    kColRest = 6,   // double: the eye's rest below a unit (mirrored)
+    kColAt = 9,     // uint32: output pixel, view
+    kCols64 = 10
 };
 
 struct Ray64 {
-    Cold64* k;
-    double inv[3], nod[3];  // t(X) = X inv + nod; axis with d = 0: inv = 0, nod = o
+    char* base;             // the lane's shared columns
+    double iu[3], nr[3];    // t(X) = (X - U) iu + nr; axis with d = 0: 0 and a time past every other
     double t;               // parameter where the current leaf is entered
     double T;               // transmittance
-    uint32_t c[3];
+    uint32_t X[3], U[3];    // low corner of the current cell, the eye in whole units (mirrored)
     int32_t L;
-    uint32_t dpos, zmask;
+    uint32_t flip;
     uint2 val;
     int32_t pr;   // record holding the current leaf's slot
     uint32_t kc;  // child index of the current leaf in pr
     int32_t steps;
     uint32_t n_rays, n_steps, n_reads, n_leaf, n_rec;
+
+    template <typename V>
+    __device__ __forceinline__ V& col(int c) { return *reinterpret_cast<V*>(base + (size_t)c * (8 * kBlock64)); }
+    __device__ __forceinline__ double& C(int i) { return col<double>(kColC + i); }
+    __device__ __forceinline__ double& ds(int a) { return col<double>(kColDs + a); }
+    __device__ __forceinline__ double& rest(int a) { return col<double>(kColRest + a); }
+    __device__ __forceinline__ uint32_t& pix() { return col<uint32_t>(kColAt); }
+    __device__ __forceinline__ uint32_t& view() { return (&col<uint32_t>(kColAt))[1]; }
 };
 
-__device__ __forceinline__ bool zero_axis(const Ray64& r, int a) { return (r.zmask >> a) & 1u; }
-
-// Ray on the high side of the plane x_a = M just after t.
-__device__ __forceinline__ uint32_t high_side(const Ray64& r, int a, double M, double t) {
-    if (zero_axis(r, a)) return r.nod[a] >= M;
-    const double tm = fma(M, r.inv[a], r.nod[a]);
-    return r.inv[a] > 0.0 ? (tm <= t) : (tm > t);
+// A 32-bit integer as a double: 2^52 + x by its pattern, less 2^52 (exact).
+__device__ __forceinline__ double uint_to_double(uint32_t x) {
+    return __longlong_as_double(0x4330000000000000ll | (long long)x) - 4503599627370496.0;
+}
+// A binary16 value as a double, through its float (a normal one or zero) by exponent arithmetic.
+__device__ __forceinline__ double half_to_double(unsigned h) {
+    const uint32_t f = __float_as_uint(half_bits_to_float(h));
+    const uint32_t m = f & 0x7FFFFFFFu;
+    const long long d = ((long long)m << 29) + (m ? 0x3800000000000000ll : 0ll);
+    return __longlong_as_double(d | ((long long)(f >> 31) << 63));
+}
+__device__ __forceinline__ bool less_pos(double a, double b) {  // of numbers that are not both negative
+    return __double_as_longlong(a) < __double_as_longlong(b);
 }
 
-__device__ __forceinline__ double mid_plane(const Tree& T, uint32_t cc, int lev) {
-    return fma((double)(2u * cc + 1u), T.extent * p2d(-(lev + 1)), -T.half);
+// e^-x - 1. Below 1/8 (most leaves: thin paint, small cells) its series to x^10 / 10! (the next term is 2^-55 of the
+// value), 10 FP64 operations; else the library's.
+__device__ __forceinline__ double expm1_neg64(double x) {
+    const double y = -x;
+    if (less_pos(x, 0.125)) {
+        double p = fma(2.7557319223985893e-07, y, 2.7557319223985893e-06);
+        p = fma(p, y, 2.4801587301587302e-05);
+        p = fma(p, y, 1.9841269841269841e-04);
+        p = fma(p, y, 1.3888888888888889e-03);
+        p = fma(p, y, 8.3333333333333332e-03);
+        p = fma(p, y, 4.1666666666666664e-02);
+        p = fma(p, y, 0.16666666666666666);
+        p = fma(p, y, 0.5);
+        return fma(p * y, y, y);
+    }
+    return expm1(y);
 }
 
 // Composite the current leaf over [r.t, te].
 __device__ __forceinline__ void composite64(Ray64& r, double te) {
     if (r.val.y >> 16) {
-        const double s = h2d(r.val.y >> 16);
-        const double em = expm1(-s * (te - r.t));  // -(1 - e^{-sigma l})
+        const double em = expm1_neg64(half_to_double(r.val.y >> 16) * (te - r.t));  // -(1 - e^{-sigma l})
         const double w = -r.T * em;
-        r.k->C[0] += w * h2d(r.val.x & 0xFFFFu);
-        r.k->C[1] += w * h2d(r.val.x >> 16);
-        r.k->C[2] += w * h2d(r.val.y & 0xFFFFu);
-        r.T += r.T * em;
+        r.C(0) = fma(w, half_to_double(r.val.x & 0xFFFFu), r.C(0));
+        r.C(1) = fma(w, half_to_double(r.val.x >> 16), r.C(1));
+        r.C(2) = fma(w, half_to_double(r.val.y & 0xFFFFu), r.C(2));
+        r.T = fma(r.T, em, r.T);
     }
 }
 
 __device__ __forceinline__ void finish64(Ray64& r, const MixedParams& P) {
-    const View& V = P.views[r.k->view];
+    const View& V = P.views[r.view()];
     float4 o;
-    o.x = (float)(r.k->C[0] + r.T * (double)V.bg[0]);
-    o.y = (float)(r.k->C[1] + r.T * (double)V.bg[1]);
-    o.z = (float)(r.k->C[2] + r.T * (double)V.bg[2]);
+    o.x = (float)(r.C(0) + r.T * (double)V.bg[0]);
+    o.y = (float)(r.C(1) + r.T * (double)V.bg[1]);
+    o.z = (float)(r.C(2) + r.T * (double)V.bg[2]);
     o.w = (float)(1.0 - r.T);
-    const int64_t pix = V.out_offset + (int64_t)r.k->pix;
+    const int64_t pix = V.out_offset + (int64_t)r.pix();
     P.out[pix] = o;
     if (P.step_count) P.step_count[pix] = r.steps;
     r.n_rays += 1;
     r.n_steps += (uint32_t)r.steps;
 }
 
+// The ray's position on axis a at parameter t: the unit it lies in, kept within [X, X + s).
+__device__ __forceinline__ uint32_t locate64(Ray64& r, int a, double t, uint32_t X, uint32_t s) {
+    const int32_t n = __double2int_rd(fma(t, r.ds(a), r.rest(a)));
+    const int64_t rel = (int64_t)r.U[a] + n - (int64_t)X;
+    return X + (uint32_t)min(max(rel, (int64_t)0), (int64_t)s - 1);
+}
+
 // Start ray g of the launch. Returns true if it has a leaf to step from.
+template <bool kWrap>
 __device__ bool init64(Ray64& r, const MixedParams& P, unsigned long long g) {
     const Tree& T = P.tree;
     g += (unsigned long long)P.ray_base;
@@ -111,32 +157,39 @@ __device__ bool init64(Ray64& r, const MixedParams& P, unsigned long long g) {
     const int i = ((int)(tile - ty * (unsigned)V.tiles_x) << wl) + (lane & ((1 << wl) - 1));
     const int j = (int)ty * (32 >> wl) + (lane >> wl);
     if (i >= V.width || j >= V.height) return false;
-    r.k->view = lo;
-    r.k->pix = (uint32_t)j * (uint32_t)V.width + (uint32_t)i;
-    r.k->C[0] = r.k->C[1] = r.k->C[2] = 0.0;
+    r.view() = (uint32_t)lo;
+    r.pix() = (uint32_t)j * (uint32_t)V.width + (uint32_t)i;
+    r.C(0) = r.C(1) = r.C(2) = 0.0;
     r.T = 1.0;
     r.steps = 0;
     double d[3];
     pixel_ray(V, i, j, d);
-    r.dpos = 0;
-    r.zmask = 0;
+    r.flip = 0;
     double t0 = 0.0, t1 = __longlong_as_double(0x7FF0000000000000ll);
     bool miss = false;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const double da = d[a], o = V.eye[a];
+        const bool neg = d[a] < 0.0;
+        if (neg) r.flip |= 1u << a;
+        uint32_t u = (uint32_t)V.eye_unit[a];
+        double rest = V.eye_rest[a];
+        if (neg) {
+            rest = u ? -rest : 2147483648.0 - rest;
+            u = u ? 0x80000000u - u : 0u;
+        }
+        r.U[a] = u;
+        r.rest(a) = rest;
+        const double da = fabs(d[a]), o = neg ? -V.eye[a] : V.eye[a];
+        r.ds(a) = da * (P.inv_extent * 2147483648.0);
         if (da != 0.0) {
-            r.inv[a] = 1.0 / da;
-            r.nod[a] = -o * r.inv[a];
-            if (da > 0.0) r.dpos |= 1u << a;
-            const double ta = fma(-T.half, r.inv[a], r.nod[a]);
-            const double tb = fma(T.half, r.inv[a], r.nod[a]);
-            t0 = fmax(t0, da > 0.0 ? ta : tb);
-            t1 = fmin(t1, da > 0.0 ? tb : ta);
+            const double inv = 1.0 / da;
+            r.iu[a] = P.unit * inv;
+            r.nr[a] = -rest * r.iu[a];
+            t0 = fmax(t0, (-T.half - o) * inv);
+            t1 = fmin(t1, (T.half - o) * inv);
         } else {
-            r.inv[a] = 0.0;
-            r.nod[a] = o;
-            r.zmask |= 1u << a;
+            r.iu[a] = 0.0;
+            r.nr[a] = 1.0e300;
             if (!(o >= -T.half && o < T.half)) miss = true;
         }
     }
@@ -145,131 +198,111 @@ __device__ bool init64(Ray64& r, const MixedParams& P, unsigned long long g) {
         return false;
     }
     r.t = t0;
-    const EyePath& E = P.eye[r.k->view];
-    if (E.len > 0 && t0 == 0.0) {
+    r.steps = 1;
+    const EyePath& E = P.eye[lo];
+    if (E.len > 0) {  // (t0 is 0 for an eye inside the canvas)
         r.L = E.len;
         r.pr = E.rec[E.len - 1];
         r.kc = (E.c[0] & 1u) | ((E.c[1] & 1u) << 1) | ((E.c[2] & 1u) << 2);
-        r.c[0] = E.c[0];
-        r.c[1] = E.c[1];
-        r.c[2] = E.c[2];
+        const uint32_t last = (1u << E.len) - 1u;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) r.X[a] = (((r.flip >> a) & 1u) ? last - E.c[a] : E.c[a]) << (kFix - E.len);
         r.val = E.val;
         r.n_reads += r.L;
         r.n_leaf += (uint32_t)E.stored;
-        r.steps = 1;
         return true;
     }
     // locate the leaf that holds r(t0+) from the root
-    r.c[0] = r.c[1] = r.c[2] = 0u;
-    int lev = 0;
-    int32_t rec = 0, slot;
-    for (;;) {
-        int k = 0;
+    uint32_t q[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const uint32_t b = high_side(r, a, mid_plane(T, r.c[a], lev), t0);
-            r.c[a] = 2u * r.c[a] + b;
-            k |= (int)b << a;
-        }
-        slot = __ldg(T.nodes + (int64_t)rec * 8 + k);
+    for (int a = 0; a < 3; ++a) q[a] = locate64(r, a, t0, 0u, 0x80000000u);
+    int sh = kFix;
+    int32_t rec = 0, slot = 0;
+    do {
+        rec = slot;
+        --sh;
+        r.kc = (uint32_t)child_index_any(q, sh, r.flip);
+        slot = __ldg(T.nodes + (int64_t)rec * 8 + r.kc);
         r.n_rec += 1;
-        if (slot > 0) {
-            ++lev;
-            rec = slot;
-        } else {
-            r.pr = rec;
-            r.kc = (uint32_t)k;
-            break;
-        }
-    }
-    r.L = lev + 1;
+    } while (slot > 0);
+    r.pr = rec;
+    r.L = kFix - sh;
     r.n_reads += r.L;
+    r.val = make_uint2(0u, 0u);
     if (slot < 0) {
-        r.val = __ldg(T.leaves + leaf_index(T, rec, (int)r.kc, slot));
+        r.val = load_leaf<kWrap>(T, rec, (int)r.kc, slot);
         r.n_leaf += 1;
-    } else {
-        r.val = make_uint2(0u, 0u);
     }
-    r.steps = 1;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) r.X[a] = (q[a] >> sh) << sh;
     return true;
 }
 
 // One leaf step. Returns false once the ray is finished (its pixel written).
+template <bool kWrap>
 __device__ bool step64(Ray64& r, const MixedParams& P) {
     const Tree& T = P.tree;
     // 1. exit face: the smallest FP64 crossing time of the exact far planes (ties to the lowest axis)
-    const double w = T.extent * p2d(-r.L);
-    double te = __longlong_as_double(0x7FF0000000000000ll);
+    const uint32_t s = 1u << (kFix - r.L);
+    const double t0 = fma(uint_to_double(r.X[0] + s - r.U[0]), r.iu[0], r.nr[0]);
+    const double t1 = fma(uint_to_double(r.X[1] + s - r.U[1]), r.iu[1], r.nr[1]);
+    const double t2 = fma(uint_to_double(r.X[2] + s - r.U[2]), r.iu[2], r.nr[2]);
     int ax = 0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        if (zero_axis(r, a)) continue;
-        const double ta = fma(fma((double)(r.c[a] + ((r.dpos >> a) & 1u)), w, -T.half), r.inv[a], r.nod[a]);
-        if (ta < te) {
-            te = ta;
-            ax = a;
-        }
-    }
-    // 2. neighbour across the exit face
-    const uint32_t up = (r.dpos >> ax) & 1u;
-    const uint32_t cold = ax == 0 ? r.c[0] : (ax == 1 ? r.c[1] : r.c[2]);
-    const uint32_t cn = up ? cold + 1u : cold - 1u;
-    if ((cn >> r.L) != 0u) {  // leaving the canvas
+    double te = t0;
+    if (less_pos(t1, te)) { ax = 1; te = t1; }
+    if (less_pos(t2, te)) { ax = 2; te = t2; }
+    // 2. the neighbour across the exit face: its low corner is N on that axis
+    const uint32_t N = pick(ax, r.X[0], r.X[1], r.X[2]) + s;
+    if ((N >> kFix) != 0u) {  // leaving the canvas
         composite64(r, te);
         finish64(r, P);
         return false;
     }
-    const int lstar = r.L - (32 - __clz(cold ^ cn));
-    uint32_t cc[3] = {ax == 0 ? cn : r.c[0], ax == 1 ? cn : r.c[1], ax == 2 ? cn : r.c[2]};
-    int Lc = r.L;
-    int lv;
-    int32_t prec;
-    int kk;
-    if (lstar == r.L - 1) {
-        prec = r.pr;
-        kk = (int)(r.kc ^ (1u << ax));
-        lv = r.L;
-    } else {
-        const uint2 rp = __ldg(T.ropes + (int64_t)r.pr * 6 + 2 * ax + (int)up);
+    const int lstar = (kFix - 1) - (31 - __clz((N - s) ^ N));
+    uint32_t q[3] = {ax == 0 ? N : r.X[0], ax == 1 ? N : r.X[1], ax == 2 ? N : r.X[2]};
+    const int sh_old = kFix - r.L;
+    int32_t prec = r.pr;
+    int kk = (int)(r.kc ^ (1u << ax)), sh = sh_old;
+    if (!(N & s)) {  // not the high half of the same parent
+        const uint2 rp = __ldg(T.ropes + (int64_t)r.pr * 6 + 2 * ax + (int)(((r.flip >> ax) & 1u) ^ 1u));
         r.n_rec += 1;
         prec = (int32_t)rp.x;
         kk = (int)((rp.y >> 8) & 7u);
-        lv = (int)(rp.y & 255u);
+        sh = kFix - (int)(rp.y & 255u);
     }
     int32_t slot = __ldg(T.nodes + (int64_t)prec * 8 + kk);
     r.n_rec += 1;
-    // 3. descend while the cell is internal: integer bits down to the old level, then the ray's side at te
-    while (slot > 0) {
-        int k;
-        if (lv < Lc) {
-            const int sh = Lc - 1 - lv;
-            k = (int)((cc[0] >> sh) & 1u) | (int)(((cc[1] >> sh) & 1u) << 1) | (int)(((cc[2] >> sh) & 1u) << 2);
-        } else {
-            k = 0;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const uint32_t bit = a == ax ? (up ? 0u : 1u) : high_side(r, a, mid_plane(T, cc[a], lv), te);
-                cc[a] = 2u * cc[a] + bit;
-                k |= (int)bit << a;
-            }
-            ++Lc;
-        }
+    if (slot > 0 && sh != sh_old) {  // (a link names an internal cell only one level up)
         prec = slot;
-        kk = k;
-        ++lv;
+        sh = sh_old;
+        kk = child_index(q, sh, r.flip);
         slot = __ldg(T.nodes + (int64_t)prec * 8 + kk);
         r.n_rec += 1;
     }
-    const int Ln = lv;
-    r.n_reads += (uint32_t)(Ln - lstar);
+    // 3. finer than the old cell: near side on the exit axis, the ray's position at te on the others
+    if (slot > 0) {
+        const uint32_t q0 = locate64(r, 0, te, r.X[0], s), q1 = locate64(r, 1, te, r.X[1], s),
+                       q2 = locate64(r, 2, te, r.X[2], s);
+        q[0] = ax == 0 ? N : q0;
+        q[1] = ax == 1 ? N : q1;
+        q[2] = ax == 2 ? N : q2;
+        do {
+            --sh;
+            prec = slot;
+            kk = child_index(q, sh, r.flip);
+            slot = __ldg(T.nodes + (int64_t)prec * 8 + kk);
+            r.n_rec += 1;
+        } while (slot > 0);
+    }
+    r.n_reads += (uint32_t)(kFix - sh - lstar);
     uint2 nval = make_uint2(0u, 0u);
     if (slot < 0) {
-        nval = __ldg(T.leaves + leaf_index(T, prec, kk, slot));
+        nval = load_leaf<kWrap>(T, prec, kk, slot);
         r.n_leaf += 1;
     }
     // 4. composite the current leaf, then terminate or advance
     composite64(r, te);
-    if (r.T < (double)P.t_min) {
+    if (less_pos(r.T, (double)P.t_min)) {
         finish64(r, P);
         return false;
     }
@@ -279,11 +312,9 @@ __device__ bool step64(Ray64& r, const MixedParams& P) {
         finish64(r, P);
         return false;
     }
-    const int sh = Lc - Ln;
-    r.c[0] = cc[0] >> sh;
-    r.c[1] = cc[1] >> sh;
-    r.c[2] = cc[2] >> sh;
-    r.L = Ln;
+    r.L = kFix - sh;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) r.X[a] = (q[a] >> sh) << sh;
     r.val = nval;
     r.pr = prec;
     r.kc = (uint32_t)kk;
@@ -298,10 +329,11 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
     return v;
 }
 
+template <bool kWrap>
 __global__ void __launch_bounds__(kBlock64, 3) fp64links_kernel(MixedParams P) {
-    __shared__ Cold64 cold[kBlock64];
+    __shared__ double lanes[kCols64 * kBlock64];
     Ray64 r;
-    r.k = &cold[threadIdx.x];
+    r.base = reinterpret_cast<char*>(&lanes[threadIdx.x]);
     r.n_rays = r.n_steps = r.n_reads = r.n_leaf = r.n_rec = 0;
     const unsigned lane = threadIdx.x & 31u;
     bool alive = false;
@@ -316,7 +348,7 @@ __global__ void __launch_bounds__(kBlock64, 3) fp64links_kernel(MixedParams P) {
             if (base + __popc(idle) >= (unsigned long long)P.total_rays) drained = true;
             if (!alive) {
                 const unsigned long long g = base + __popc(idle & ((1u << lane) - 1u));
-                if (g < (unsigned long long)P.total_rays) alive = init64(r, P, g);
+                if (g < (unsigned long long)P.total_rays) alive = init64<kWrap>(r, P, g);
             }
             busy = __ballot_sync(kFull64, alive);
             if (!drained && __popc(busy) <= P.refill) continue;
@@ -326,7 +358,7 @@ __global__ void __launch_bounds__(kBlock64, 3) fp64links_kernel(MixedParams P) {
             continue;
         }
         do {
-            if (alive) alive = step64(r, P);
+            if (alive) alive = step64<kWrap>(r, P);
             busy = __ballot_sync(kFull64, alive);
         } while (busy != 0u && (drained || __popc(busy) > P.refill));
     }
@@ -340,14 +372,18 @@ __global__ void __launch_bounds__(kBlock64, 3) fp64links_kernel(MixedParams P) {
 
 }  // namespace
 
-cudaError_t launch_fp64links(const MixedParams& p, int grid, int block, cudaStream_t s) {
-    if (!p.tree.ropes) return cudaErrorInvalidValue;
-    fp64links_kernel<<<grid, block, 0, s>>>(p);
+cudaError_t launch_fp64links(const MixedParams& params, int grid, int block, cudaStream_t s) {
+    if (!params.tree.ropes) return cudaErrorInvalidValue;
+    MixedParams p = params;
+    p.inv_extent = 1.0 / p.tree.extent;
+    p.unit = p.tree.extent * 4.656612873077393e-10;  // 2^-31
+    if (p.tree.n_wrap > 0) fp64links_kernel<true><<<grid, block, 0, s>>>(p);
+    else fp64links_kernel<false><<<grid, block, 0, s>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t fp64links_max_blocks_per_sm(int block, int* out) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, fp64links_kernel, block, 0);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, fp64links_kernel<false>, block, 0);
 }
 
 }  // namespace canvox

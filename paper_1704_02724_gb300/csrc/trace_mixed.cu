@@ -59,12 +59,12 @@
 #include <cuda_fp16.h>
 
 #include "canvox_internal.cuh"
+#include "cells.cuh"
 
 namespace canvox {
 namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
-constexpr int kFix = 31;                            // the canvas is 2^31 fixed-point units wide
 constexpr float kEpsF = 3.5762786865234375e-07f;    // 6 * 2^-24: the exit-face screen's relative margin
 constexpr float kEpsG = 9.765625e-04f;              // 2^-10 = 2^31 * 2^-41: its absolute margin per ih
 constexpr float kEpsX = 7.152557373046875e-07f;     // 12 * 2^-24: the position's relative error bound, doubled
@@ -80,11 +80,6 @@ constexpr float kBigF = 1.0e28f;                    // time per unit of an axis 
 #define CANVOX_MIN_BLOCKS 4
 #endif
 
-// IEEE binary16 bits -> float (exact: every half is a float).
-__device__ __forceinline__ float half_bits_to_float(unsigned h) { return __half2float(__ushort_as_half((unsigned short)h)); }
-__device__ __forceinline__ float hsig(uint2 v) { return half_bits_to_float(v.y >> 16); }
-__device__ __forceinline__ float hlo(unsigned w) { return half_bits_to_float(w & 0xFFFFu); }
-__device__ __forceinline__ float hhi(unsigned w) { return half_bits_to_float(w >> 16); }
 // 1 / x to about an ulp (one instruction).
 __device__ __forceinline__ float rcp_approx(float x) {
     float r;
@@ -107,10 +102,6 @@ __device__ __forceinline__ float expm1_neg(float x) {
     return x < 1.0f ? -x * p : e - 1.0f;
 }
 
-// x[a] for a runtime axis without indexing an array (which would put it in local memory).
-template <typename V>
-__device__ __forceinline__ V pick(int a, V x0, V x1, V x2) { return a == 0 ? x0 : (a == 1 ? x1 : x2); }
-
 extern __shared__ int32_t s_nodes[];  // copy of the tree's first records (kernel instance with kSmem)
 
 // Child slot k of record rec: from the shared-memory copy of the tree's breadth-first prefix when the
@@ -120,13 +111,6 @@ __device__ __forceinline__ int32_t load_slot(const Tree& T, int32_t n_smem, int3
     if (kSmem && rec < n_smem) return s_nodes[rec * 8 + k];
     return __ldg(T.nodes + (int64_t)rec * 8 + k);
 }
-// Value of the leaf in slot k of record rec (slot value v < 0). kWrap: the canvas has more than 2^31 leaves (slots
-// hold leaf numbers modulo 2^31); an instance without it reads the number straight from the slot.
-template <bool kWrap>
-__device__ __forceinline__ uint2 load_leaf(const Tree& T, int32_t rec, int k, int32_t v) {
-    return __ldg(T.leaves + (kWrap ? leaf_index(T, rec, k, v) : (int64_t)(uint32_t)~v));
-}
-
 __device__ __forceinline__ void kahan_add(float& s, float& c, float x) {
     const float y = __fsub_rn(x, c);
     const float t = __fadd_rn(s, y);
@@ -315,19 +299,6 @@ __device__ __forceinline__ uint32_t locate(const Ray& r, int a, int32_t D, float
     const uint32_t h = s - (uint32_t)D + (uint32_t)__float2int_rd(__fadd_rn(x, e));
     open = l ^ h;  // an interval that reaches past the cell leaves every bit open
     return r.X[a] | (l & (s - 1u));
-}
-
-// Child index (not mirrored) at the bits `sh` <= 29 of the position q. (The shifts left lose bit 30 of q[2] only,
-// the child of the root.)
-__device__ __forceinline__ int child_index(const uint32_t q[3], int sh, uint32_t flip) {
-    uint32_t k = ((q[0] >> sh) & 1u) ^ flip;
-    k ^= ((q[1] << 1) >> sh) & 2u;
-    k ^= ((q[2] << 2) >> sh) & 4u;
-    return (int)k;
-}
-// The same for any bit (the root's children too).
-__device__ __forceinline__ int child_index_any(const uint32_t q[3], int sh, uint32_t flip) {
-    return (int)((((q[0] >> sh) & 1u) | (((q[1] >> sh) & 1u) << 1) | (((q[2] >> sh) & 1u) << 2)) ^ flip);
 }
 
 // Sides of the mid-planes of the cell that q's bits above `sh` name, on every axis but ax, just after FP64 time t:
