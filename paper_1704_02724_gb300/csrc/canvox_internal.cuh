@@ -143,6 +143,8 @@ cudaError_t fp64links_max_blocks_per_sm(int block, int* out);
 cudaError_t launch_plain(const PlainParams& p, int precision, long long n_pixels, cudaStream_t s);
 cudaError_t launch_local32(const PlainParams& p, int precision, long long n_pixels, cudaStream_t s);
 cudaError_t launch_hash(const Tree& t, unsigned long long* out, cudaStream_t s);
+// the terms of n leaves (numbers first, first + 1, ...) added to *out
+cudaError_t launch_hash_leaves(const uint2* leaves, int64_t first, int64_t n, unsigned long long* out, cudaStream_t s);
 cudaError_t launch_rope_level(const int32_t* nodes, uint2* ropes, int64_t lo, int64_t hi, int level, cudaStream_t s);
 cudaError_t launch_eye_paths(const Tree& t, const View* views, int n_views, EyePath* out, cudaStream_t s);
 cudaError_t probe_l2_gather(int64_t buffer_bytes, double* gbs);

@@ -6,11 +6,18 @@
 // grid (Sec. 6.1), launch of the traversal kernels, CUDA-graph replay,
 // counters, the schedule autotuner, the device painter's stamp table and the
 // measurement helpers' set-up.
+#include <algorithm>
+#include <atomic>
 #include <cmath>
+#include <condition_variable>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <exception>
+#include <functional>
+#include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "canvox_internal.cuh"
@@ -448,6 +455,225 @@ int check_stamps(const double* centers, const double* radii, const float* rgba, 
 }
 
 
+// The host's cores for the length of one call: run(n, fn) calls fn(i) for i in [0, n), the calling thread among them;
+// start() leaves it to the others until finish(). One thread for little work, and where no other can be started. The
+// pools of a canvas are validated and hashed element by element: one core takes about 2 ns an element, 10 ms for the
+// depth-8 canvas of 431,100 records, which bounded its upload.
+class HostTeam {
+  public:
+    explicit HostTeam(int64_t pieces) {
+        const int64_t cores = std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), 64);
+        try {
+            while ((int64_t)team_.size() + 1 < std::min(cores, pieces / 2)) team_.emplace_back([this] { serve(); });
+        } catch (...) {  // no more threads: the others and the caller do it
+        }
+    }
+    ~HostTeam() {
+        finish();
+        {
+            std::lock_guard<std::mutex> l(m_);
+            stop_ = true;
+        }
+        wake_.notify_all();
+        for (auto& t : team_) t.join();
+    }
+    HostTeam(const HostTeam&) = delete;
+    HostTeam& operator=(const HostTeam&) = delete;
+
+    void start(int64_t n, std::function<void(int64_t)> fn) {
+        finish();
+        {
+            std::lock_guard<std::mutex> l(m_);
+            fn_ = std::move(fn);
+            n_ = n;
+            next_.store(0);
+            busy_ = (int)team_.size();
+            ++job_;
+        }
+        wake_.notify_all();
+    }
+    void finish() {
+        work();
+        std::unique_lock<std::mutex> l(m_);
+        done_.wait(l, [this] { return busy_ == 0; });
+    }
+    void run(int64_t n, std::function<void(int64_t)> fn) {
+        start(n, std::move(fn));
+        finish();
+    }
+
+  private:
+    void work() {
+        for (int64_t i; (i = next_.fetch_add(1)) < n_;) fn_(i);
+    }
+    void serve() {
+        for (int64_t seen = 0;;) {
+            {
+                std::unique_lock<std::mutex> l(m_);
+                wake_.wait(l, [&] { return stop_ || job_ != seen; });
+                if (stop_) return;
+                seen = job_;
+            }
+            work();
+            std::lock_guard<std::mutex> l(m_);
+            if (--busy_ == 0) done_.notify_all();
+        }
+    }
+    std::mutex m_;
+    std::condition_variable wake_, done_;
+    std::function<void(int64_t)> fn_;
+    int64_t n_ = 0, job_ = 0;
+    int busy_ = 0;
+    bool stop_ = false;
+    std::atomic<int64_t> next_{0};
+    std::vector<std::thread> team_;
+};
+
+constexpr int64_t kHostChunk = 8192;  // records (256 KB) or leaves per piece of host work
+int64_t pieces_of(int64_t n) { return (n + kHostChunk - 1) / kHostChunk; }
+
+// First value of leaves [0, n) that is not allowed (-1: none): 0 non-finite, 1 negative extinction in *what.
+int64_t bad_leaf(const uint16_t* leaf_rgba, int64_t begin, int64_t end, int* what) {
+    for (int64_t i = begin; i < end; ++i) {
+        const uint16_t* q = leaf_rgba + 4 * i;
+        for (int c = 0; c < 4; ++c)
+            if (((q[c] >> 10) & 31) == 31) {
+                *what = 0;
+                return i;
+            }
+        if ((q[3] & 0x8000u) && (q[3] & 0x7FFFu)) {
+            *what = 1;
+            return i;
+        }
+    }
+    return -1;
+}
+
+// Checks the values of leaves [0, n), numbered from `first` in the message.
+int check_leaves(HostTeam& team, const uint16_t* leaf_rgba, int64_t n, int64_t first) {
+    const int64_t pieces = pieces_of(n);
+    std::vector<int64_t> bad((size_t)pieces, -1);
+    std::vector<int> what((size_t)pieces, 0);
+    team.run(pieces, [&](int64_t p) {
+        bad[(size_t)p] = bad_leaf(leaf_rgba, p * kHostChunk, std::min(n, (p + 1) * kHostChunk), &what[(size_t)p]);
+    });
+    for (int64_t p = 0; p < pieces; ++p)
+        if (bad[(size_t)p] >= 0)
+            return fail(CANVOX_ERR_BAD_TREE, what[(size_t)p] ? "leaf %lld: negative extinction" : "leaf %lld: non-finite FP16",
+                        (long long)(first + bad[(size_t)p]));
+    return CANVOX_OK;
+}
+
+// Hash terms of leaves [begin, end), numbered from `first`.
+unsigned long long hash_leaves(const uint16_t* leaf_rgba, int64_t begin, int64_t end, int64_t first) {
+    unsigned long long h = 0;
+    for (int64_t i = begin; i < end; ++i) {
+        unsigned long long v;
+        std::memcpy(&v, leaf_rgba + 4 * i, sizeof(v));  // R | G << 16 | B << 32 | sigma << 48
+        h += elem_hash(2ull, (unsigned long long)(first + i), v);
+    }
+    return h;
+}
+unsigned long long hash_slots(const int32_t* node_pool, int64_t begin, int64_t end) {  // records
+    unsigned long long h = 0;
+    for (int64_t i = 8 * begin; i < 8 * end; ++i)
+        h += elem_hash(1ull, (unsigned long long)i, (unsigned long long)(uint32_t)node_pool[i]);
+    return h;
+}
+
+// Validation of a node pool: breadth-first numbering of records and leaves, depth bound. Pieces of kHostChunk records
+// count their internal children and leaves, which gives every piece the numbers that it starts from (and, level by
+// level, where the levels of the breadth-first order begin); the pieces then check their slots. The error reported is
+// the first in pool order. Receives the levels' first records and the slots where leaf numbers pass multiples of 2^31.
+struct PoolError {
+    int kind = 0;
+    int64_t r = 0, a = 0, b = 0;
+    int k = 0;
+};
+int check_nodes(HostTeam& team, const int32_t* node_pool, int64_t n_records, int64_t n_leaves, int32_t depth,
+                std::vector<int64_t>* level_begin, int64_t* wraps, int32_t* n_wrap) {
+    const int64_t pieces = pieces_of(n_records);
+    std::vector<int64_t> rec((size_t)pieces + 1, 0), leaf((size_t)pieces + 1, 0);  // counts, then exclusive sums
+    auto internal_slots = [&](int64_t begin, int64_t end) {
+        int64_t c = 0;
+        for (int64_t i = 8 * begin; i < 8 * end; ++i) c += node_pool[i] > 0;
+        return c;
+    };
+    team.run(pieces, [&](int64_t p) {
+        const int64_t b = p * kHostChunk, e = std::min(n_records, b + kHostChunk);
+        int64_t neg = 0;
+        for (int64_t i = 8 * b; i < 8 * e; ++i) neg += node_pool[i] < 0;
+        rec[(size_t)p + 1] = internal_slots(b, e);
+        leaf[(size_t)p + 1] = neg;
+    });
+    for (int64_t p = 0; p < pieces; ++p) {
+        rec[(size_t)p + 1] += rec[(size_t)p];
+        leaf[(size_t)p + 1] += leaf[(size_t)p];
+    }
+    // records of level l: [begin[l], begin[l + 1]); the children of the records before begin[l] are numbered 1, 2, ...
+    std::vector<int64_t> begin{0, 1};
+    while (begin.back() < n_records) {
+        const int64_t b = begin.back(), p = b / kHostChunk;
+        const int64_t e = 1 + rec[(size_t)p] + internal_slots(p * kHostChunk, b);
+        if (e <= b) break;  // record b is not referenced before it appears
+        begin.push_back(std::min(e, n_records));
+    }
+    std::vector<PoolError> err((size_t)pieces);
+    std::atomic<int64_t> first_bad{pieces};
+    team.run(pieces, [&](int64_t p) {
+        if (p > first_bad.load()) return;
+        int64_t next_rec = 1 + rec[(size_t)p], next_leaf = leaf[(size_t)p];
+        const int64_t b = p * kHostChunk, e = std::min(n_records, b + kHostChunk);
+        int level = (int)(std::upper_bound(begin.begin(), begin.end(), b) - begin.begin()) - 1;
+        auto bad = [&](int kind, int64_t r, int k, int64_t x, int64_t y) {
+            err[(size_t)p] = PoolError{kind, r, x, y, k};
+            for (int64_t f = first_bad.load(); p < f && !first_bad.compare_exchange_weak(f, p);) {
+            }
+        };
+        for (int64_t r = b; r < e; ++r) {
+            if (r >= next_rec) return bad(1, r, 0, 0, 0);
+            while (level + 1 < (int)begin.size() && r >= begin[(size_t)level + 1]) ++level;
+            for (int k = 0; k < 8; ++k) {
+                const int32_t v = node_pool[8 * r + k];
+                if (v > 0) {
+                    if (v != next_rec) return bad(2, r, k, v, next_rec);
+                    if (v >= n_records) return bad(3, r, k, v, 0);
+                    if (level + 1 > depth - 1) return bad(4, r, k, v, level + 1);
+                    ++next_rec;
+                } else if (v < 0) {
+                    // leaves are numbered in breadth-first slot order; the slot holds the number modulo 2^31
+                    const int64_t li = -(int64_t)v - 1;
+                    if (li != (next_leaf & 0x7FFFFFFFll)) return bad(5, r, k, li, next_leaf & 0x7FFFFFFFll);
+                    if (next_leaf >= n_leaves) return bad(6, r, k, next_leaf, 0);
+                    if (next_leaf > 0 && li == 0) wraps[(next_leaf >> 31) - 1] = 8 * r + k;  // n_leaves <= 2^34: at most 7
+                    ++next_leaf;
+                }
+            }
+        }
+    });
+    if (first_bad.load() < pieces) {
+        const PoolError& x = err[(size_t)first_bad.load()];
+        switch (x.kind) {
+            case 1: return fail(CANVOX_ERR_BAD_TREE, "record %lld is not referenced before it appears", (long long)x.r);
+            case 2: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: child %d, expected %lld (breadth-first order)",
+                                (long long)x.r, x.k, (int)x.a, (long long)x.b);
+            case 3: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: child %d out of range", (long long)x.r, x.k, (int)x.a);
+            case 4: return fail(CANVOX_ERR_BAD_TREE, "record %d at level %d exceeds depth %d", (int)x.a, (int)x.b, depth);
+            case 5: return fail(CANVOX_ERR_BAD_TREE,
+                                "record %lld slot %d: leaf %lld, expected %lld (breadth-first order, modulo 2^31)",
+                                (long long)x.r, x.k, (long long)x.a, (long long)x.b);
+            default: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: leaf %lld out of range", (long long)x.r, x.k,
+                                 (long long)x.a);
+        }
+    }
+    const int64_t next_rec = 1 + rec[(size_t)pieces], next_leaf = leaf[(size_t)pieces];
+    if (next_rec != n_records) return fail(CANVOX_ERR_BAD_TREE, "%lld records unreachable", (long long)(n_records - next_rec));
+    if (next_leaf != n_leaves) return fail(CANVOX_ERR_BAD_TREE, "%lld leaves unreferenced", (long long)(n_leaves - next_leaf));
+    *n_wrap = n_leaves > 0 ? (int32_t)((n_leaves - 1) >> 31) : 0;
+    *level_begin = std::move(begin);
+    return CANVOX_OK;
+}
+
 // Neighbour links of the current pools, one launch per level (parents first).
 int build_links() {
     CK(cudaMalloc(&g.d_ropes, sizeof(uint2) * 6 * (size_t)g.n_rec), "cudaMalloc(ropes)");
@@ -490,6 +716,90 @@ int paint_table(int32_t depth, double extent, int64_t* n_records, int64_t* n_lea
     return CANVOX_OK;
 }
 
+// The work of canvox_upload_octree once its arguments are known to be good.
+int upload(const int32_t* node_pool, int64_t n_records, const uint16_t* leaf_rgba, int64_t n_leaves, int32_t depth,
+           double extent) {
+    // validation: breadth-first numbering of records and leaves, depth bound, finite FP16 values
+    const int64_t node_pieces = pieces_of(n_records), leaf_pieces = pieces_of(n_leaves);
+    HostTeam team(node_pieces + leaf_pieces);
+    std::vector<int64_t> level_begin;
+    int64_t wraps[kMaxWraps] = {};
+    int32_t n_wrap = 0;
+    int rc = check_nodes(team, node_pool, n_records, n_leaves, depth, &level_begin, wraps, &n_wrap);
+    if (rc) return rc;
+    if ((rc = check_leaves(team, leaf_rgba, n_leaves, 0))) return rc;
+    if ((rc = ensure_device())) return rc;
+    // the host pools' hash, beside the copies
+    std::atomic<unsigned long long> hash{0};
+    team.start(node_pieces + leaf_pieces, [&](int64_t p) {
+        if (p < node_pieces) {
+            hash += hash_slots(node_pool, p * kHostChunk, std::min(n_records, (p + 1) * kHostChunk));
+        } else {
+            const int64_t b = (p - node_pieces) * kHostChunk;
+            hash += hash_leaves(leaf_rgba, b, std::min(n_leaves, b + kHostChunk), 0);
+        }
+    });
+    struct Finish {  // (an early return waits for the team, whose work refers to the names above)
+        HostTeam& team;
+        ~Finish() { team.finish(); }
+    } finish{team};
+    // replace the device copy
+    if ((rc = drop_canvas())) return rc;
+    paint_cache_free(g.paint_cache);  // an uploaded canvas cannot be appended to
+    g.paint_cache = nullptr;
+    CK(cudaMalloc(&g.d_nodes, sizeof(int32_t) * 8 * (size_t)n_records), "cudaMalloc(nodes)");
+    CK(cudaMalloc(&g.d_leaves, sizeof(uint2) * (size_t)(n_leaves > 0 ? n_leaves : 1)), "cudaMalloc(leaves)");
+    CK(cudaMemcpy(g.d_nodes, node_pool, sizeof(int32_t) * 8 * (size_t)n_records, cudaMemcpyHostToDevice), "cudaMemcpy(nodes)");
+    if (n_leaves > 0)
+        CK(cudaMemcpy(g.d_leaves, leaf_rgba, sizeof(uint2) * (size_t)n_leaves, cudaMemcpyHostToDevice), "cudaMemcpy(leaves)");
+    g.n_rec = n_records;
+    g.n_leaf = n_leaves;
+    g.depth = depth;
+    g.extent = extent;
+    g.n_wrap = n_wrap;
+    for (int m = 0; m < kMaxWraps; ++m) g.wrap[m] = m < n_wrap ? wraps[m] : 0;
+    g.level_begin = std::move(level_begin);  // (breadth-first order keeps each level contiguous)
+    // bit-identity of the device copy
+    CK(cudaMemset(g.d_hash, 0, sizeof(unsigned long long)), "cudaMemset(hash)");
+    CK(launch_hash(device_tree(), g.d_hash, 0), "hash kernel launch");
+    team.finish();
+    g.host_hash = hash.load();
+    unsigned long long dh = 0;
+    CK(cudaMemcpy(&dh, g.d_hash, sizeof(dh), cudaMemcpyDeviceToHost), "cudaMemcpy(hash)");
+    if (dh != g.host_hash) return fail(CANVOX_ERR_CUDA, "device copy hash %016llx differs from host %016llx", dh, g.host_hash);
+    if ((rc = build_links())) return rc;
+    g.uploaded = true;
+    return CANVOX_OK;
+}
+
+// The work of canvox_update_leaves once its arguments are known to be good. The pool hash is a sum over elements: the
+// old values' terms, summed where they are, go out and the new ones', from the caller's values, come in.
+int update_range(int64_t first, int64_t count, const uint16_t* leaf_rgba) {
+    const int64_t pieces = pieces_of(count);
+    HostTeam team(pieces);
+    int rc = check_leaves(team, leaf_rgba, count, first);
+    if (rc) return rc;
+    if (count == 0) return CANVOX_OK;
+    std::atomic<unsigned long long> added{0};
+    team.start(pieces, [&](int64_t p) {
+        added += hash_leaves(leaf_rgba, p * kHostChunk, std::min(count, (p + 1) * kHostChunk), first);
+    });
+    struct Finish {
+        HostTeam& team;
+        ~Finish() { team.finish(); }
+    } finish{team};
+    if (g.any_render) CK(cudaEventSynchronize(g.done), "cudaEventSynchronize");
+    CK(cudaMemset(g.d_hash, 0, sizeof(unsigned long long)), "cudaMemset(hash)");
+    CK(launch_hash_leaves(g.d_leaves + first, first, count, g.d_hash, 0), "hash kernel launch");
+    unsigned long long gone = 0;
+    CK(cudaMemcpy(&gone, g.d_hash, sizeof(gone), cudaMemcpyDeviceToHost), "cudaMemcpy(hash)");
+    CK(cudaMemcpy(g.d_leaves + first, leaf_rgba, sizeof(uint2) * (size_t)count, cudaMemcpyHostToDevice), "cudaMemcpy(leaves)");
+    team.finish();
+    g.host_hash += added.load() - gone;
+    g.last_h2d = (int64_t)sizeof(uint2) * count;
+    return CANVOX_OK;
+}
+
 }  // namespace
 
 namespace canvox {
@@ -520,87 +830,11 @@ int canvox_upload_octree(const int32_t* node_pool, int64_t n_records, const uint
         return fail(CANVOX_ERR_INVALID_ARG, "pool beyond 2^31 - 1 records or 2^34 leaves");
     int rc = check_canvas_args(depth, extent);
     if (rc) return rc;
-    // validation: breadth-first numbering of records and leaves, depth bound, finite FP16 values
-    std::vector<uint8_t> level((size_t)n_records, 0);
-    int64_t next_rec = 1, next_leaf = 0;
-    unsigned long long hh = 0;
-    int64_t wraps[kMaxWraps] = {};
-    int32_t n_wrap = 0;
-    for (int64_t r = 0; r < n_records; ++r) {
-        if (r >= next_rec) return fail(CANVOX_ERR_BAD_TREE, "record %lld is not referenced before it appears", (long long)r);
-        for (int k = 0; k < 8; ++k) {
-            const int32_t v = node_pool[8 * r + k];
-            hh += elem_hash(1ull, (unsigned long long)(8 * r + k), (unsigned long long)(uint32_t)v);
-            if (v > 0) {
-                if (v != next_rec)
-                    return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: child %d, expected %lld (breadth-first order)",
-                                (long long)r, k, v, (long long)next_rec);
-                if (v >= n_records) return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: child %d out of range", (long long)r, k, v);
-                if (level[r] + 1 > depth - 1)
-                    return fail(CANVOX_ERR_BAD_TREE, "record %d at level %d exceeds depth %d", v, level[r] + 1, depth);
-                level[v] = (uint8_t)(level[r] + 1);
-                ++next_rec;
-            } else if (v < 0) {
-                // leaves are numbered in breadth-first slot order; the slot holds the number modulo 2^31
-                const int64_t li = -(int64_t)v - 1;
-                if (li != (next_leaf & 0x7FFFFFFFll))
-                    return fail(CANVOX_ERR_BAD_TREE,
-                                "record %lld slot %d: leaf %lld, expected %lld (breadth-first order, modulo 2^31)",
-                                (long long)r, k, (long long)li, (long long)(next_leaf & 0x7FFFFFFFll));
-                if (next_leaf >= n_leaves)
-                    return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: leaf %lld out of range", (long long)r, k,
-                                (long long)next_leaf);
-                if (next_leaf > 0 && li == 0) wraps[n_wrap++] = 8 * r + k;  // n_leaves <= 2^34: at most 7
-                ++next_leaf;
-            }
-        }
+    try {
+        return upload(node_pool, n_records, leaf_rgba, n_leaves, depth, extent);
+    } catch (const std::exception& e) {  // host memory
+        return fail(CANVOX_ERR_OOM, "upload: %s", e.what());
     }
-    if (next_rec != n_records) return fail(CANVOX_ERR_BAD_TREE, "%lld records unreachable", (long long)(n_records - next_rec));
-    if (next_leaf != n_leaves) return fail(CANVOX_ERR_BAD_TREE, "%lld leaves unreferenced", (long long)(n_leaves - next_leaf));
-    for (int64_t i = 0; i < n_leaves; ++i) {
-        const uint16_t* q = leaf_rgba + 4 * i;
-        for (int c = 0; c < 4; ++c)
-            if (((q[c] >> 10) & 31) == 31) return fail(CANVOX_ERR_BAD_TREE, "leaf %lld: non-finite FP16", (long long)i);
-        if ((q[3] & 0x8000u) && (q[3] & 0x7FFFu)) return fail(CANVOX_ERR_BAD_TREE, "leaf %lld: negative extinction", (long long)i);
-        unsigned long long val = (unsigned long long)q[0] | ((unsigned long long)q[1] << 16) |
-                                 ((unsigned long long)q[2] << 32) | ((unsigned long long)q[3] << 48);
-        hh += elem_hash(2ull, (unsigned long long)i, val);
-    }
-    rc = ensure_device();
-    if (rc) return rc;
-    // replace the device copy
-    if ((rc = drop_canvas())) return rc;
-    paint_cache_free(g.paint_cache);  // an uploaded canvas cannot be appended to
-    g.paint_cache = nullptr;
-    CK(cudaMalloc(&g.d_nodes, sizeof(int32_t) * 8 * (size_t)n_records), "cudaMalloc(nodes)");
-    CK(cudaMalloc(&g.d_leaves, sizeof(uint2) * (size_t)(n_leaves > 0 ? n_leaves : 1)), "cudaMalloc(leaves)");
-    CK(cudaMemcpy(g.d_nodes, node_pool, sizeof(int32_t) * 8 * (size_t)n_records, cudaMemcpyHostToDevice), "cudaMemcpy(nodes)");
-    if (n_leaves > 0)
-        CK(cudaMemcpy(g.d_leaves, leaf_rgba, sizeof(uint2) * (size_t)n_leaves, cudaMemcpyHostToDevice), "cudaMemcpy(leaves)");
-    g.n_rec = n_records;
-    g.n_leaf = n_leaves;
-    g.depth = depth;
-    g.extent = extent;
-    g.n_wrap = n_wrap;
-    for (int m = 0; m < kMaxWraps; ++m) g.wrap[m] = m < n_wrap ? wraps[m] : 0;
-    g.host_hash = hh;
-    // bit-identity of the device copy
-    CK(cudaMemset(g.d_hash, 0, sizeof(unsigned long long)), "cudaMemset(hash)");
-    CK(launch_hash(device_tree(), g.d_hash, 0), "hash kernel launch");
-    unsigned long long dh = 0;
-    CK(cudaMemcpy(&dh, g.d_hash, sizeof(dh), cudaMemcpyDeviceToHost), "cudaMemcpy(hash)");
-    if (dh != hh) return fail(CANVOX_ERR_CUDA, "device copy hash %016llx differs from host %016llx", dh, hh);
-    // records of each level (breadth-first order keeps each level contiguous)
-    g.level_begin.assign(1, 0);
-    for (int64_t lo = 0; lo < n_records;) {
-        int64_t hi = lo;
-        while (hi < n_records && level[(size_t)hi] == level[(size_t)lo]) ++hi;
-        g.level_begin.push_back(hi);
-        lo = hi;
-    }
-    if ((rc = build_links())) return rc;
-    g.uploaded = true;
-    return CANVOX_OK;
 }
 
 int canvox_paint_spheres(int32_t depth, double extent, const double* centers, const double* radii, const float* rgba,
@@ -671,31 +905,11 @@ int canvox_update_leaves(int64_t first, int64_t count, const uint16_t* leaf_rgba
     if (count < 0 || first < 0 || first > g.n_leaf || count > g.n_leaf - first || (count > 0 && !leaf_rgba))
         return fail(CANVOX_ERR_INVALID_ARG, "leaf range [%lld, %lld) outside the pool of %lld leaves",
                     (long long)first, (long long)(first + count), (long long)g.n_leaf);
-    for (int64_t i = 0; i < count; ++i) {
-        const uint16_t* q = leaf_rgba + 4 * i;
-        for (int c = 0; c < 4; ++c)
-            if (((q[c] >> 10) & 31) == 31) return fail(CANVOX_ERR_BAD_TREE, "leaf %lld: non-finite FP16", (long long)(first + i));
-        if ((q[3] & 0x8000u) && (q[3] & 0x7FFFu))
-            return fail(CANVOX_ERR_BAD_TREE, "leaf %lld: negative extinction", (long long)(first + i));
+    try {
+        return update_range(first, count, leaf_rgba);
+    } catch (const std::exception& e) {  // host memory
+        return fail(CANVOX_ERR_OOM, "leaf update: %s", e.what());
     }
-    if (count == 0) return CANVOX_OK;
-    if (g.any_render) CK(cudaEventSynchronize(g.done), "cudaEventSynchronize");
-    // the pool hash is a sum over elements: take the old values' terms out, put the new ones in
-    std::vector<uint2> old((size_t)count);
-    CK(cudaMemcpy(old.data(), g.d_leaves + first, sizeof(uint2) * (size_t)count, cudaMemcpyDeviceToHost), "cudaMemcpy(leaves)");
-    unsigned long long hh = g.host_hash;
-    for (int64_t i = 0; i < count; ++i) {
-        const uint16_t* q = leaf_rgba + 4 * i;
-        const unsigned long long nv = (unsigned long long)q[0] | ((unsigned long long)q[1] << 16) |
-                                      ((unsigned long long)q[2] << 32) | ((unsigned long long)q[3] << 48);
-        const unsigned long long ov = ((unsigned long long)old[(size_t)i].y << 32) | old[(size_t)i].x;
-        hh -= elem_hash(2ull, (unsigned long long)(first + i), ov);
-        hh += elem_hash(2ull, (unsigned long long)(first + i), nv);
-    }
-    CK(cudaMemcpy(g.d_leaves + first, leaf_rgba, sizeof(uint2) * (size_t)count, cudaMemcpyHostToDevice), "cudaMemcpy(leaves)");
-    g.host_hash = hh;
-    g.last_h2d = (int64_t)sizeof(uint2) * count;
-    return CANVOX_OK;
 }
 
 int canvox_octree_hash(uint64_t* host_hash, uint64_t* device_hash) {
