@@ -119,6 +119,7 @@ struct MixedParams {
     // set by the launchers
     double inv_extent, unit;  // 1 / extent, extent 2^-31
     float side;               // extent
+    int32_t steps;            // step_limit, at most 2^31 - 1
     float bound_t, bound_i;   // the colour bound of a boundary per local time and per ih (see ray_step)
 };
 
@@ -193,32 +194,58 @@ namespace canvox {
 //
 // The quotients take the reciprocal of their divisor, known for the width and height and formed once for the
 // norm: q = a r, then one correction by the exact remainder (Markstein 1990), 3 FP64 operations each instead of a
-// division's nine or so; the FP64 pipe (1/64 of the FP32 rate) bounds views of few leaves per ray. For the pixel
+// division's nine or so, and the norm's square root leaves its reciprocal; the FP64 pipe (1/64 of the FP32 rate) bounds views of few leaves per ray. For the pixel
 // coordinates the result is the rounded quotient always: 2i + 1 < 2^32 and W < 2^31, so a quotient lies at least
 // 2^-32 of an ulp from a rounding boundary, far more than the correction's error of 2^-51.
+// 1 / x: about 20 bits from the hardware, then one step of third order (1 + e + e^2) to 53.
 __device__ __forceinline__ double rcp64(double x) {
     double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));  // about 20 bits; two Newton steps to 53
-    r = fma(fma(-x, r, 1.0), r, r);
-    return fma(fma(-x, r, 1.0), r, r);
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+// sqrt(x), correctly rounded, and 1 / sqrt(x) to an ulp: two coupled Newton steps (Goldschmidt) from the hardware's
+// 20 bits, then the square root's own correction by its exact remainder (Markstein 1990).
+__device__ __forceinline__ double sqrt64(double x, double* rcp) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double g = x * y, h = 0.5 * y;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const double r = fma(-g, h, 0.5);
+        g = fma(g, r, g);
+        h = fma(h, r, h);
+    }
+    g = fma(fma(-g, g, x), h, g);
+    h += h;
+    *rcp = fma(h, fma(-g, h, 1.0), h);
+    return g;
+}
+// A 32-bit integer as a double: 2^52 + x by its pattern, less 2^52 (exact; one FP64 operation).
+__device__ __forceinline__ double uint_to_double(uint32_t x) {
+    return __longlong_as_double(0x4330000000000000ll | (long long)x) - 4503599627370496.0;
 }
 __device__ __forceinline__ double div64(double a, double b, double rcp_b) {
     const double q = __dmul_rn(a, rcp_b);
     return fma(fma(-b, q, a), rcp_b, q);
 }
 __device__ __forceinline__ void pixel_ray(const View& V, int i, int j, double d[3]) {
-    const double x = __dadd_rn(div64(2.0 * i + 1.0, (double)V.width, V.inv_w), -1.0);
-    const double y = __dsub_rn(1.0, div64(2.0 * j + 1.0, (double)V.height, V.inv_h));
+    const double x = __dadd_rn(div64(uint_to_double(2u * (uint32_t)i + 1u), uint_to_double((uint32_t)V.width), V.inv_w), -1.0);
+    const double y = __dsub_rn(1.0, div64(uint_to_double(2u * (uint32_t)j + 1u), uint_to_double((uint32_t)V.height), V.inv_h));
     const double u = __dmul_rn(__dmul_rn(x, V.sy), V.aspect);
     const double v = __dmul_rn(y, V.sy);
 #pragma unroll
     for (int a = 0; a < 3; ++a) d[a] = __dadd_rn(__dadd_rn(V.f[a], __dmul_rn(u, V.r[a])), __dmul_rn(v, V.u[a]));
-    const double n = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2])));
-    if (n < 1.0e100) {
-        const double r = rcp64(n);
+    const double n2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
+    // (the frame is orthonormal, so n2 is 1 or more but for rounding; a view wider than 10^75 takes the plain operations)
+    const int hi = (int)(__double_as_longlong(n2) >> 32);
+    if (hi > 0x3FE00000 && hi < 0x5F000000) {
+        double r;
+        const double n = sqrt64(n2, &r);
 #pragma unroll
         for (int a = 0; a < 3; ++a) d[a] = div64(d[a], n, r);
     } else {
+        const double n = __dsqrt_rn(n2);
 #pragma unroll
         for (int a = 0; a < 3; ++a) d[a] = __ddiv_rn(d[a], n);
     }

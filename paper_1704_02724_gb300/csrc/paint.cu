@@ -497,7 +497,7 @@ __device__ __forceinline__ int64_t warp_total(int64_t x) {
 
 // The children of every cell: slot (internal, or the leaf's key), list length, the entries' decisions; the block's
 // sums; tot[2] = the longest list. Cells with long lists only add their sums here.
-__global__ void __launch_bounds__(8 * kCells) expand_count(LevelIn L, StampDev S, double half, uint64_t* slot,
+__global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDev S, double half, uint64_t* slot,
                                                            int32_t* cnt, uint16_t* cls, BlockSum* bs, long long* tot) {
     __shared__ float4 s_rec[kCells * kStageRow];
     __shared__ int64_t s_ent[kCells / 4], s_int[kCells / 4];

@@ -71,10 +71,6 @@ struct Ray64 {
     __device__ __forceinline__ uint32_t& view() { return (&col<uint32_t>(kColAt))[1]; }
 };
 
-// A 32-bit integer as a double: 2^52 + x by its pattern, less 2^52 (exact).
-__device__ __forceinline__ double uint_to_double(uint32_t x) {
-    return __longlong_as_double(0x4330000000000000ll | (long long)x) - 4503599627370496.0;
-}
 // A binary16 value as a double, through its float (a normal one or zero) by exponent arithmetic.
 __device__ __forceinline__ double half_to_double(unsigned h) {
     const uint32_t f = __float_as_uint(half_bits_to_float(h));
@@ -138,7 +134,7 @@ __device__ __forceinline__ uint32_t locate64(Ray64& r, int a, double t, uint32_t
 }
 
 // Start ray g of the launch. Returns true if it has a leaf to step from.
-template <bool kWrap>
+template <int kPool>
 __device__ bool init64(Ray64& r, const MixedParams& P, unsigned long long g) {
     const Tree& T = P.tree;
     g += (unsigned long long)P.ray_base;
@@ -182,7 +178,7 @@ __device__ bool init64(Ray64& r, const MixedParams& P, unsigned long long g) {
         const double da = fabs(d[a]), o = neg ? -V.eye[a] : V.eye[a];
         r.ds(a) = da * (P.inv_extent * 2147483648.0);
         if (da != 0.0) {
-            const double inv = 1.0 / da;
+            const double inv = da > 1.0e-200 ? rcp64(da) : 1.0 / da;
             r.iu[a] = P.unit * inv;
             r.nr[a] = -rest * r.iu[a];
             t0 = fmax(t0, (-T.half - o) * inv);
@@ -230,7 +226,7 @@ __device__ bool init64(Ray64& r, const MixedParams& P, unsigned long long g) {
     r.n_reads += r.L;
     r.val = make_uint2(0u, 0u);
     if (slot < 0) {
-        r.val = load_leaf<kWrap>(T, rec, (int)r.kc, slot);
+        r.val = load_leaf<kPool>(T, rec, (int)r.kc, slot);
         r.n_leaf += 1;
     }
 #pragma unroll
@@ -239,7 +235,7 @@ __device__ bool init64(Ray64& r, const MixedParams& P, unsigned long long g) {
 }
 
 // One leaf step. Returns false once the ray is finished (its pixel written).
-template <bool kWrap>
+template <int kPool>
 __device__ bool step64(Ray64& r, const MixedParams& P) {
     const Tree& T = P.tree;
     // 1. exit face: the smallest FP64 crossing time of the exact far planes (ties to the lowest axis)
@@ -263,15 +259,19 @@ __device__ bool step64(Ray64& r, const MixedParams& P) {
     const int sh_old = kFix - r.L;
     int32_t prec = r.pr;
     int kk = (int)(r.kc ^ (1u << ax)), sh = sh_old;
+    int32_t slot = 0;
     if (!(N & s)) {  // not the high half of the same parent
         const uint2 rp = __ldg(T.ropes + (int64_t)r.pr * 6 + 2 * ax + (int)(((r.flip >> ax) & 1u) ^ 1u));
         r.n_rec += 1;
         prec = (int32_t)rp.x;
         kk = (int)((rp.y >> 8) & 7u);
         sh = kFix - (int)(rp.y & 255u);
+        if (rp.y & kLinkRecord) slot = prec;  // (a link to an internal cell names its record)
     }
-    int32_t slot = __ldg(T.nodes + (int64_t)prec * 8 + kk);
-    r.n_rec += 1;
+    if (slot == 0) {
+        slot = __ldg(T.nodes + (int64_t)prec * 8 + kk);
+        r.n_rec += 1;
+    }
     if (slot > 0 && sh != sh_old) {  // (a link names an internal cell only one level up)
         prec = slot;
         sh = sh_old;
@@ -297,7 +297,7 @@ __device__ bool step64(Ray64& r, const MixedParams& P) {
     r.n_reads += (uint32_t)(kFix - sh - lstar);
     uint2 nval = make_uint2(0u, 0u);
     if (slot < 0) {
-        nval = load_leaf<kWrap>(T, prec, kk, slot);
+        nval = load_leaf<kPool>(T, prec, kk, slot);
         r.n_leaf += 1;
     }
     // 4. composite the current leaf, then terminate or advance
@@ -329,7 +329,7 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
     return v;
 }
 
-template <bool kWrap>
+template <int kPool>
 __global__ void __launch_bounds__(kBlock64, 3) fp64links_kernel(MixedParams P) {
     __shared__ double lanes[kCols64 * kBlock64];
     Ray64 r;
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kBlock64, 3) fp64links_kernel(MixedParams P) {
             if (base + __popc(idle) >= (unsigned long long)P.total_rays) drained = true;
             if (!alive) {
                 const unsigned long long g = base + __popc(idle & ((1u << lane) - 1u));
-                if (g < (unsigned long long)P.total_rays) alive = init64<kWrap>(r, P, g);
+                if (g < (unsigned long long)P.total_rays) alive = init64<kPool>(r, P, g);
             }
             busy = __ballot_sync(kFull64, alive);
             if (!drained && __popc(busy) <= P.refill) continue;
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kBlock64, 3) fp64links_kernel(MixedParams P) {
             continue;
         }
         do {
-            if (alive) alive = step64<kWrap>(r, P);
+            if (alive) alive = step64<kPool>(r, P);
             busy = __ballot_sync(kFull64, alive);
         } while (busy != 0u && (drained || __popc(busy) > P.refill));
     }
@@ -377,13 +377,13 @@ cudaError_t launch_fp64links(const MixedParams& params, int grid, int block, cud
     MixedParams p = params;
     p.inv_extent = 1.0 / p.tree.extent;
     p.unit = p.tree.extent * 4.656612873077393e-10;  // 2^-31
-    if (p.tree.n_wrap > 0) fp64links_kernel<true><<<grid, block, 0, s>>>(p);
-    else fp64links_kernel<false><<<grid, block, 0, s>>>(p);
+    if (p.tree.n_wrap > 0) fp64links_kernel<kWrapPool><<<grid, block, 0, s>>>(p);
+    else fp64links_kernel<kPlainPool><<<grid, block, 0, s>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t fp64links_max_blocks_per_sm(int block, int* out) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, fp64links_kernel<false>, block, 0);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, fp64links_kernel<kPlainPool>, block, 0);
 }
 
 }  // namespace canvox

@@ -37,16 +37,24 @@
 // |dt|; each ray carries a budget for these bounds, and a boundary whose bound
 // would exceed it is recomputed in FP64.
 //
-// What bounds it: instruction issue (0.76 of the issue slots on a reduced
+// A step settles the boundary behind it, not the one ahead: the new leaf's value
+// is asked for last and first needed in the next step, for the colour bound of
+// the boundary it was entered by and then to composite the leaf before it, while
+// the next link is on its way. One dependent load of a step's five or six thus
+// leaves the chain that a single long ray waits for (a 256^2 view of the depth-8
+// cube, whose longest ray crosses 283 leaves, one after the other: 491 us before,
+// 444 us after; links that name an internal neighbour's own record take another).
+//
+// What bounds it: instruction issue (0.79 of the issue slots on a reduced
 // depth-24 stereo view, 28 of 32 warps resident), the loads being served by L1
-// and L2, and for views of few leaves per ray the FP64 pipe (0.84 busy on the
-// opaque depth-16 view, the per-ray set-up). So the step holds to integers and
-// few words: against frames of cells with planes as FP32 dyadics and two-word
-// reciprocals per axis, it issues 1.41 G instead of 2.09 G warp instructions on
-// that reduced view (1.64 ms instead of 2.44), spills nothing at 64 registers
-// (four blocks an SM), and the set-up takes 43 % fewer FP64 instructions (the
-// opaque view 0.40 ms instead of 0.69; the depth-24 stereo pair of 2160^2 in
-// 34.4 ms instead of 45.8).
+// and L2; for views of few leaves per ray the FP64 pipe (0.82 busy on the opaque
+// depth-16 view, the per-ray set-up); for small views the longest ray's chain.
+// So the step holds to integers and few words: against frames of cells with
+// planes as FP32 dyadics and two-word reciprocals per axis, it issues 1.40 G
+// instead of 2.09 G warp instructions on that reduced view (1.55 ms instead of
+// 2.44), with three spilled words at 64 registers (four blocks an SM), and the
+// set-up takes 57 % fewer FP64 instructions (the opaque view 0.31 ms instead of
+// 0.69; the depth-24 stereo pair of 2160^2 32.5 ms instead of 45.8).
 //
 // Compositing (emission-absorption reading of Sec. 6.2): per segment of signed
 // length l in a leaf (sigma, rgb): a = 1 - exp(-sigma l), C += T a rgb,
@@ -73,6 +81,7 @@ constexpr float kEpsT = 1.1368683772161603e-13f;    // 2^-43 = 2 * 2^-44: factor
 constexpr float kEpsI = 1.1920928955078125e-07f;    // 2^-23 = 2 * 2^-24: the same, per ih
 constexpr float kFar = 65536.0f;                    // a cell this many sides from the anchor asks for a new anchor
 constexpr int kBoxLevels = 16;                      // frames of fewer levels also end where the ray leaves their cell
+constexpr uint32_t kLeft = 4u;                      // (Ray::entry)
 constexpr float kBigF = 1.0e28f;                    // time per unit of an axis the ray never crosses (d_a = 0)
 
 // Resident 256-thread blocks per SM the register allocation must allow (occupancy knob).
@@ -106,34 +115,71 @@ extern __shared__ int32_t s_nodes[];  // copy of the tree's first records (kerne
 
 // Child slot k of record rec: from the shared-memory copy of the tree's breadth-first prefix when the
 // kernel keeps one and the record is in it (records [0, n_smem)), else through the read-only data cache.
-template <bool kSmem>
+template <bool kSmem, int kPool>
 __device__ __forceinline__ int32_t load_slot(const Tree& T, int32_t n_smem, int32_t rec, int k) {
     if (kSmem && rec < n_smem) return s_nodes[rec * 8 + k];
+    if (kPool == kSmallPool) return __ldg(byte_offset(T.nodes, (uint32_t)rec * 32u + (uint32_t)k * 4u));
     return __ldg(T.nodes + (int64_t)rec * 8 + k);
 }
-__device__ __forceinline__ void kahan_add(float& s, float& c, float x) {
-    const float y = __fsub_rn(x, c);
-    const float t = __fadd_rn(s, y);
-    c = __fsub_rn(__fsub_rn(t, s), y);
+// Link of record rec past its face 2 ax + s.
+template <int kPool>
+__device__ __forceinline__ uint2 load_link(const Tree& T, int32_t rec, int ax, uint32_t s) {
+    if (kPool == kSmallPool) return __ldg(byte_offset(T.ropes, (uint32_t)rec * 48u + (uint32_t)ax * 16u + s * 8u));
+    return __ldg(T.ropes + (int64_t)rec * 6 + 2 * ax + (int)s);
+}
+
+// Two FP32 operations in one instruction, on the words of a 64-bit register.
+typedef unsigned long long pair32;
+__device__ __forceinline__ pair32 pack2(float a, float b) {
+    pair32 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ pair32 add2(pair32 a, pair32 b) {
+    pair32 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ pair32 sub2(pair32 a, pair32 b) {
+    pair32 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ pair32 mul2(pair32 a, pair32 b) {
+    pair32 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// Kahan's compensated sum s (its compensation in c) of two channels.
+__device__ __forceinline__ void kahan_add2(pair32& s, pair32& c, pair32 x) {
+    const pair32 old = s, y = sub2(x, c), t = add2(old, y);
+    c = sub2(sub2(t, old), y);
     s = t;
+}
+__device__ __forceinline__ void kahan_add(float2& sc, float x) {
+    const float y = __fsub_rn(x, sc.y);
+    const float t = __fadd_rn(sc.x, y);
+    sc.y = __fsub_rn(__fsub_rn(t, sc.x), y);
+    sc.x = t;
 }
 
 constexpr int kBlock = 256;
 
 // Per-lane state in shared memory: the colour sums and the error budget of every step, and what only re-anchoring,
 // near-ties, start-up and the final write read. One 8-byte column per field and lane, so that every field of a
-// lane is its base address plus a constant, and 8-byte accesses of a warp meet no bank conflict. 120 bytes a
+// lane is its base address plus a constant, and 8-byte accesses of a warp meet no bank conflict. 128 bytes a
 // lane: four blocks stay within the 132 KB carve-out, which leaves 124 KB of the SM to L1.
 enum Col {
     kColInv = 0,    // double: 1 / |d_a| (0 for d_a = 0), three columns
     kColDir = 3,    // double: |d_a|, three columns
     kColTf = 6,     // double: FP64 ray parameter at the anchor
-    kColAcc = 7,    // float2: (sum, Kahan term) of the colour channels 0, 1, 2
+    kColAcc = 7,    // float2: sums of the colour channels 0, 1; their Kahan terms; (sum, Kahan term) of channel 2
     kColPix = 10,   // uint32: output pixel within the view; then the view
     kColCnt = 11,   // uint32: anchors, FP64 boundaries
     kColSum = 14,   // uint32: rays, leaf steps
+    kColG = 15,     // float: 2^-41 max_a 1 / |d_a| over the axes with d_a != 0, the exit screen's margin; uint32: slot reads
     kColIl = 12,    // float: low words of ih on axes 0, 1; then axis 2 and (uint32) the axes with d_a = 0
-    kCols = 15
+    kCols = 16
 };
 constexpr int kLaneShared = kCols * 8;
 static_assert(kLaneShared <= 128, "per-lane shared record: 128 bytes keep four blocks within the 132 KB carve-out");
@@ -144,25 +190,27 @@ struct Ray {
     float rr[3];                // - (the anchor position's part below a unit) * ih
     uint32_t X[3];              // low corner of the current cell: mirrored, in units
     int32_t A[3];               // the anchor: the ray's position at local time 0, rounded to a unit
-    float gscr;                 // 2^-41 max_a 1 / |d_a| over the axes with d_a != 0: the exit screen's margin term
     float cur_hi, cur_lo;       // local parameter of the current leaf's entry
+    float ell, dt;              // the leaf before: its segment's length, and the time bound of the boundary that ends it
     float T;
     float err;                  // colour-error bound spent so far (the budget of the FP32 boundaries)
     int32_t L, f;               // level of the current cell; level of the frame (anchor's neighbourhood)
     uint32_t flip;              // axes with d_a < 0: the canvas is mirrored there, so every ray runs upwards
-    uint2 val;
+    uint32_t entry;             // axis of the face the current leaf was entered by; kLeft: the ray has left the canvas
+    uint2 val, pval;            // values of the current leaf and of the one before
     int32_t pr;   // record holding the current leaf's slot (neighbour-link traversal)
     uint32_t kc;  // child index of the current leaf in pr (not mirrored)
     int32_t steps;
     // counters, summed over every ray the lane traces
-    uint32_t n_reads, n_leaf, n_rec;
+    uint32_t n_leaf, n_rec;
 
     template <typename V>
     __device__ __forceinline__ V& col(int c) { return *reinterpret_cast<V*>(base + (size_t)c * (8 * kBlock)); }
     __device__ __forceinline__ double& inv64(int a) { return col<double>(kColInv + a); }
     __device__ __forceinline__ double& dir64(int a) { return col<double>(kColDir + a); }
     __device__ __forceinline__ double& tf() { return col<double>(kColTf); }
-    __device__ __forceinline__ float2& acc(int i) { return col<float2>(kColAcc + i); }
+    __device__ __forceinline__ pair32& acc01(int i) { return col<pair32>(kColAcc + i); }
+    __device__ __forceinline__ float2& acc2() { return col<float2>(kColAcc + 2); }
     __device__ __forceinline__ uint32_t& pix() { return col<uint32_t>(kColPix); }
     __device__ __forceinline__ uint32_t& view() { return (&col<uint32_t>(kColPix))[1]; }
     __device__ __forceinline__ uint32_t& n_rebase() { return col<uint32_t>(kColCnt); }
@@ -170,6 +218,8 @@ struct Ray {
     __device__ __forceinline__ uint32_t& n_rays() { return col<uint32_t>(kColSum); }
     __device__ __forceinline__ uint32_t& n_steps() { return (&col<uint32_t>(kColSum))[1]; }
     __device__ __forceinline__ float& il(int a) { return (&col<float>(kColIl + (a >> 1)))[a & 1]; }
+    __device__ __forceinline__ float& gscr() { return col<float>(kColG); }
+    __device__ __forceinline__ uint32_t& n_reads() { return (&col<uint32_t>(kColG))[1]; }
     __device__ __forceinline__ uint32_t& zmask() { return (&col<uint32_t>(kColIl + 1))[1]; }
 };
 
@@ -250,25 +300,37 @@ __device__ __forceinline__ void set_anchor(Ray& r, const MixedParams& P, const V
     r.n_rebase() += 1;
 }
 
-// Composite the current leaf over [cursor, te]. The length is not clamped at
+// The anchor at the eye itself (of a view with the eye inside the canvas and eye_unit set): no FP64 arithmetic.
+__device__ __forceinline__ void set_anchor_eye(Ray& r, const View& V) {
+    r.tf() = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const bool m = (r.flip >> a) & 1u;
+        const float rest = m ? -(float)V.eye_rest[a] : (float)V.eye_rest[a];
+        r.A[a] = m ? (int32_t)(0x80000000u - (uint32_t)V.eye_unit[a]) : V.eye_unit[a];
+        r.rr[a] = r.ih[a] == kBigF ? 0.0f : -__fmaf_rn(rest, r.ih[a], rest * r.il(a));
+    }
+    r.cur_hi = 0.0f;
+    r.cur_lo = 0.0f;
+    r.n_rebase() += 1;
+}
+
+// Composite the leaf before the current one. The length is not clamped at
 // zero: a boundary can land slightly before the cursor (within its error
 // bound), and only the signed lengths of consecutive segments telescope, so a
 // boundary between two leaves of equal value then costs nothing.
-__device__ __forceinline__ void kahan_add2(float2& sc, float x) { kahan_add(sc.x, sc.y, x); }
-
-__device__ __forceinline__ void composite(Ray& r, float teh, float tel, float side) {
-    const float ell = ((teh - r.cur_hi) + (tel - r.cur_lo)) * side;
-    if (r.val.y >> 16) {
-        const float s = hsig(r.val);
-        const float em = expm1_neg(s * ell);  // -a
+__device__ __forceinline__ void composite(Ray& r) {
+    if (r.pval.y >> 16) {
+        const float s = hsig(r.pval);
+        const float em = expm1_neg(s * r.ell);  // -a
         const float w = -r.T * em;
-        float2 c0 = r.acc(0), c1 = r.acc(1), c2 = r.acc(2);
-        kahan_add2(c0, w * hlo(r.val.x));
-        kahan_add2(c1, w * hhi(r.val.x));
-        kahan_add2(c2, w * hlo(r.val.y));
-        r.acc(0) = c0;
-        r.acc(1) = c1;
-        r.acc(2) = c2;
+        pair32 s01 = r.acc01(0), c01 = r.acc01(1);
+        float2 s2 = r.acc2();
+        kahan_add2(s01, c01, mul2(pack2(w, w), pack2(hlo(r.pval.x), hhi(r.pval.x))));
+        kahan_add(s2, w * hlo(r.pval.y));
+        r.acc01(0) = s01;
+        r.acc01(1) = c01;
+        r.acc2() = s2;
         r.T = __fmaf_rn(r.T, em, r.T);  // T (1 - a)
     }
 }
@@ -276,9 +338,10 @@ __device__ __forceinline__ void composite(Ray& r, float teh, float tel, float si
 __device__ __forceinline__ void finish(Ray& r, const MixedParams& P) {
     const View& V = P.views[r.view()];
     float4 o;
-    o.x = r.acc(0).x + r.T * V.bg[0];
-    o.y = r.acc(1).x + r.T * V.bg[1];
-    o.z = r.acc(2).x + r.T * V.bg[2];
+    const float2 rg = r.col<float2>(kColAcc);
+    o.x = rg.x + r.T * V.bg[0];
+    o.y = rg.y + r.T * V.bg[1];
+    o.z = r.acc2().x + r.T * V.bg[2];
     o.w = 1.0f - r.T;
     const int64_t pix = V.out_offset + (int64_t)r.pix();
     P.out[pix] = o;
@@ -291,12 +354,12 @@ __device__ __forceinline__ void finish(Ray& r, const MixedParams& P) {
 // sides of every finer mid-plane at once. The way from the anchor, x = (th - rr) / ih, carries a relative error of
 // at most 6 * 2^-24 (th for th + tl, rr, ih, the reciprocal, the product) and, where th and rr cancel, 2^-24 units;
 // bits in which the ends of twice that interval differ, and all bits below them, are open (returned in `open`).
-__device__ __forceinline__ uint32_t locate(const Ray& r, int a, int32_t D, float th, uint32_t s, uint32_t& open) {
+__device__ __forceinline__ uint32_t locate(const Ray& r, int a, float th, uint32_t s, uint32_t& open) {
     const float x = __fsub_rn(th, r.rr[a]) * rcp_approx(r.ih[a]);
     const float e = __fmaf_rn(fabsf(x), kEpsX, kEpsU);
-    // from the cell's low corner: A + x - X = s - D + x
-    const uint32_t l = s - (uint32_t)D + (uint32_t)__float2int_rd(__fsub_rn(x, e));
-    const uint32_t h = s - (uint32_t)D + (uint32_t)__float2int_rd(__fadd_rn(x, e));
+    // from the cell's low corner
+    const uint32_t l = (uint32_t)r.A[a] - r.X[a] + (uint32_t)__float2int_rd(__fsub_rn(x, e));
+    const uint32_t h = (uint32_t)r.A[a] - r.X[a] + (uint32_t)__float2int_rd(__fadd_rn(x, e));
     open = l ^ h;  // an interval that reaches past the cell leaves every bit open
     return r.X[a] | (l & (s - 1u));
 }
@@ -331,7 +394,7 @@ __device__ __forceinline__ void split_inv(double inv, float& hi, float& lo) {
 __device__ __forceinline__ int deep_frame(int L, int depth, int K) { return max(L - K, min(max(0, depth - K), L)); }
 
 // Start ray g of the launch. Returns true if it has a leaf to step from.
-template <bool kSmem, bool kRopes, bool kCount, bool kWrap>
+template <bool kSmem, bool kRopes, bool kCount, int kPool>
 __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int32_t* stk) {
     const Tree& T = P.tree;
     g += (unsigned long long)P.ray_base;
@@ -352,7 +415,8 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
     if (i >= V.width || j >= V.height) return false;  // padding lane of a ragged tile
     r.view() = (uint32_t)lo;
     r.pix() = (uint32_t)j * (uint32_t)V.width + (uint32_t)i;
-    r.acc(0) = r.acc(1) = r.acc(2) = make_float2(0.0f, 0.0f);
+    r.acc01(0) = r.acc01(1) = 0;
+    r.acc2() = make_float2(0.0f, 0.0f);
     r.T = 1.0f;
     r.err = 0.0f;
     r.steps = 0;
@@ -384,7 +448,7 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
         }
     }
     r.zmask() = zmask;
-    r.gscr = kEpsG * g_inv;
+    r.gscr() = kEpsG * g_inv;
     const EyePath& E = P.eye[lo];
     double t0 = 0.0;
     if (E.len == 0) {
@@ -406,8 +470,11 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
             return false;
         }
     }
-    set_anchor(r, P, V, t0, -1);
-    r.steps = 1;
+    if (E.len > 0 && V.eye_unit[0] > 0 && V.eye_unit[1] > 0 && V.eye_unit[2] > 0) set_anchor_eye(r, V);
+    else set_anchor(r, P, V, t0, -1);
+    r.pval = make_uint2(0u, 0u);  // (nothing before the first leaf)
+    r.ell = r.dt = 0.0f;
+    r.entry = 0;
     if (E.len > 0) {
         // the eye's leaf, located once for the view
         r.L = E.len;
@@ -421,7 +488,7 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
 #pragma unroll
         for (int a = 0; a < 3; ++a) r.X[a] = (((r.flip >> a) & 1u) ? last - E.c[a] : E.c[a]) << (kFix - E.len);
         r.val = E.val;
-        if (kCount) r.n_reads += E.len;
+        if (kCount) atomicAdd(&r.n_reads(), (uint32_t)(E.len));
         if (kCount) r.n_leaf += (uint32_t)E.stored;
     } else {
         // locate the leaf that holds r(t0+) from the root
@@ -440,15 +507,15 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
             --sh;
             if (open >> sh) sides64(r, P, sh, -1, t0, q);
             r.kc = (uint32_t)child_index_any(q, sh, r.flip);
-            slot = load_slot<kSmem>(T, P.smem_records, rec, (int)r.kc);
+            slot = load_slot<kSmem, kPool>(T, P.smem_records, rec, (int)r.kc);
             if (kCount) r.n_rec += 1;
         } while (slot > 0);
         r.pr = rec;
         r.L = kFix - sh;
-        if (kCount) r.n_reads += r.L;
+        if (kCount) atomicAdd(&r.n_reads(), (uint32_t)(r.L));
         r.val = make_uint2(0u, 0u);
         if (slot < 0) {
-            r.val = load_leaf<kWrap>(T, rec, (int)r.kc, slot);
+            r.val = load_leaf<kPool>(T, rec, (int)r.kc, slot);
             if (kCount) r.n_leaf += 1;
         }
 #pragma unroll
@@ -461,7 +528,7 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
 }
 
 // One leaf step. Returns false once the ray is finished (its pixel written).
-template <bool kSmem, bool kRopes, bool kCount, bool kWrap>
+template <bool kSmem, bool kRopes, bool kCount, int kPool>
 __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
     const Tree& T = P.tree;
     // 1. exit of the current leaf: the far planes' distances from the anchor (exact integers) and their times.
@@ -484,7 +551,8 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
         if (F1 < Fb) { ax = 1; Fb = F1; }
         if (F2 < Fb) { ax = 2; Fb = F2; }
         const float Fs = fmaxf(fminf(F0, F1), fminf(fmaxf(F0, F1), F2));  // the median: runner-up
-        if (!(__fsub_rn(Fs, Fb) > __fmaf_rn(kEpsF, __fadd_rn(fabsf(Fs), fabsf(Fb)), r.gscr))) {
+        const bool clear = __fsub_rn(Fs, Fb) > __fmaf_rn(kEpsF, __fadd_rn(fabsf(Fs), fabsf(Fb)), r.gscr());
+        if (!clear && !(r.entry & kLeft)) {
             ax = exit_axis64(r.base, P.views, P.unit, T.half, r.flip, r.X[0] + s, r.X[1] + s, r.X[2] + s);
             rebase = fabsf(pick(ax, g0, g1, g2)) > kFar * (float)s;
         }
@@ -502,61 +570,96 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
         teh = __fadd_rn(p, lo);
         tel = __fsub_rn(lo, __fsub_rn(teh, p));
     }
-    // 2. the neighbour across the exit face: its low corner is N on that axis
+    // 2. the neighbour across the exit face: its low corner is N on that axis. Its link is asked for here, and the
+    //    boundary that ended the leaf before (whose other side, the current leaf's value, was still on its way when
+    //    that leaf was left) is settled while the link arrives
     const uint32_t N = pick(ax, r.X[0], r.X[1], r.X[2]) + s;
-    const bool leaves_canvas = (N >> kFix) != 0u;
-    uint32_t q[3] = {ax == 0 ? N : r.X[0], ax == 1 ? N : r.X[1], ax == 2 ? N : r.X[2]};
-    bool have64 = false;
-    double te64 = 0.0;
-    auto need64 = [&]() {
-        if (!have64) {
-            te64 = time64(r, P, ax, plane64(P.unit, T.half, N));
-            have64 = true;
-            const double tl = (te64 - r.tf()) * P.inv_extent;
-            teh = (float)tl;
-            tel = (float)(tl - (double)teh);
+    const bool linked = kRopes && !(N & s);  // not the high half of the same parent
+    uint2 rp = make_uint2(0u, 0u);
+    if (linked) rp = load_link<kPool>(T, r.pr, ax, ((r.flip >> ax) & 1u) ^ 1u);
+    {
+        const float bound = r.T * fmaxf(hsig(r.pval), hsig(r.val)) * r.dt;
+        const float spent = r.err + (((r.val.x ^ r.pval.x) | (r.val.y ^ r.pval.y)) ? bound : 0.0f);
+        if (spent > P.err_budget) {
+            // the boundary in FP64: the low plane, on the axis it was entered by, of the current cell (past the
+            // canvas, the canvas's far plane)
+            const int a = (int)(r.entry & 3u);
+            const double M = plane64(P.unit, T.half, pick(a, r.X[0], r.X[1], r.X[2]));
+            const double tl = (time64(r, P, a, M) - r.tf()) * P.inv_extent;
+            const float hi = (float)tl, lo = (float)(tl - (double)hi);
+            r.ell += ((hi - r.cur_hi) + (lo - r.cur_lo)) * P.side;
+            r.cur_hi = hi;
+            r.cur_lo = lo;
             r.n_f64() += 1;
-        }
-        return te64;
-    };
-    int sh = 0;
-    int32_t prec = 0;
-    int kk = 0;
-    uint2 nval = make_uint2(0u, 0u);  // the next leaf's value (empty past the canvas)
-    if (!leaves_canvas) {
-        // 3. the new leaf: start at the neighbouring cell (a sibling, the parent's neighbour link, or the common
-        //    ancestor on the stack), then descend while the cell is internal. The ray's way down to the old level
-        //    is in the cell's own coordinates; below it, in the bits of the ray's position.
-        const int sh_old = kFix - r.L;
-        int lstar = 0;  // level of the common ancestor (stack traversal and counters only)
-        if (!kRopes || kCount) lstar = (kFix - 1) - (31 - __clz((N - s) ^ N));
-        int32_t slot;
-        if (kRopes) {
-            prec = r.pr;
-            kk = (int)(r.kc ^ (1u << ax));
-            sh = sh_old;
-            if (!(N & s)) {  // not the high half of the same parent
-                const uint2 rp = __ldg(T.ropes + (int64_t)r.pr * 6 + 2 * ax + (int)(((r.flip >> ax) & 1u) ^ 1u));
-                if (kCount) r.n_rec += 1;
-                prec = (int32_t)rp.x;
-                kk = (int)((rp.y >> 8) & 7u);
-                sh = kFix - (int)(rp.y & 255u);
-            }
-            slot = load_slot<kSmem>(T, P.smem_records, prec, kk);
-            if (kCount) r.n_rec += 1;
-            if (slot > 0 && sh != sh_old) {  // (a link names an internal cell only one level up)
-                prec = slot;
-                sh = sh_old;
-                kk = child_index(q, sh, r.flip);
-                slot = load_slot<kSmem>(T, P.smem_records, prec, kk);
-                if (kCount) r.n_rec += 1;
-            }
         } else {
+            r.err = spent;
+        }
+    }
+    composite(r);
+    const bool done = (r.entry & kLeft) || (r.steps != 0 && r.T < P.t_min);
+    if (done || r.steps >= P.steps) {
+        if (!done) {
+            atomicOr(&P.scratch->status, 1ull);
+            atomicAdd(&P.scratch->stats[kStatStepLimited], 1ull);
+        }
+        finish(r, P);
+        return false;
+    }
+    r.steps += 1;
+    // 3. the current leaf's segment; where its end's time must be exact, in FP64 (formed anew where it is asked for
+    //    twice, so that it is not carried through the descent)
+    bool have64 = false;
+    auto exact_time = [&]() {
+        uint32_t x = N;
+        asm volatile("" : "+r"(x));  // (formed here: hoisted out of the descent, it cost every step 9 % more instructions)
+        const double t64 = time64(r, P, ax, plane64(P.unit, T.half, x));
+        const double tl = (t64 - r.tf()) * P.inv_extent;
+        teh = (float)tl;
+        tel = (float)(tl - (double)teh);
+        if (!have64) r.n_f64() += 1;
+        have64 = true;
+        return t64;
+    };
+    // 4. the new leaf: start at the neighbouring cell (a sibling, the parent's neighbour link, or the common ancestor on
+    //    the stack), then descend while the cell is internal. The ray's way down to the old level is in the cell's own
+    //    coordinates; below it, in the bits of the ray's position. Past the canvas the new leaf is an empty one, which
+    //    only settles the last boundary (its link reads as an empty slot).
+    uint32_t q[3] = {ax == 0 ? N : r.X[0], ax == 1 ? N : r.X[1], ax == 2 ? N : r.X[2]};
+    const uint32_t left = N >> kFix;
+    const int sh_old = kFix - r.L;
+    int lstar = 0;  // level of the common ancestor (stack traversal and counters only; -1 past the canvas)
+    if (!kRopes || kCount) lstar = (kFix - 1) - (31 - __clz((N - s) ^ N));
+    int32_t prec, slot;
+    int kk, sh = sh_old;
+    if (kRopes) {
+        prec = r.pr;
+        kk = (int)(r.kc ^ (1u << ax));
+        if (linked) {
+            if (kCount && !left) r.n_rec += 1;
+            prec = (int32_t)rp.x;
+            kk = (int)((rp.y >> 8) & 7u);
+            sh = kFix - (int)(rp.y & 255u);
+        }
+        slot = prec;  // (a link to an internal cell names its record)
+        if (!(rp.y & kLinkRecord)) {
+            slot = load_slot<kSmem, kPool>(T, P.smem_records, prec, kk);
+            if (kCount) r.n_rec += 1;
+        }
+        if (slot > 0 && sh != sh_old) {  // (a link names an internal cell only one level up)
+            prec = slot;
+            sh = sh_old;
+            kk = child_index(q, sh, r.flip);
+            slot = load_slot<kSmem, kPool>(T, P.smem_records, prec, kk);
+            if (kCount) r.n_rec += 1;
+        }
+    } else {
+        prec = kk = slot = 0;
+        if (!left) {
             prec = stk[lstar];
             sh = kFix - 1 - lstar;
             for (;;) {
                 kk = child_index_any(q, sh, r.flip);
-                slot = load_slot<kSmem>(T, P.smem_records, prec, kk);
+                slot = load_slot<kSmem, kPool>(T, P.smem_records, prec, kk);
                 if (kCount) r.n_rec += 1;
                 if (slot <= 0 || sh == sh_old) break;
                 stk[kFix - sh] = slot;
@@ -564,74 +667,59 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
                 --sh;
             }
         }
-        if (slot > 0) {
-            // finer than the old cell: near side on the exit axis, the ray's position on the others
-            uint32_t o0, o1, o2;
-            const uint32_t q0 = locate(r, 0, D0, teh, s, o0), q1 = locate(r, 1, D1, teh, s, o1),
-                           q2 = locate(r, 2, D2, teh, s, o2);
-            q[0] = ax == 0 ? N : q0;
-            q[1] = ax == 1 ? N : q1;
-            q[2] = ax == 2 ? N : q2;
-            const uint32_t open = (ax == 0 ? 0u : o0) | (ax == 1 ? 0u : o1) | (ax == 2 ? 0u : o2);
-            do {
-                if (!kRopes) stk[kFix - sh] = slot;
-                --sh;
-                if (open >> sh) {
-                    sides64(r, P, sh, ax, need64(), q);
-                    rebase = rebase || fabsf(teh) > kFar * ihx * (float)(1u << sh);
-                }
-                prec = slot;
-                kk = child_index(q, sh, r.flip);
-                slot = load_slot<kSmem>(T, P.smem_records, prec, kk);
-                if (kCount) r.n_rec += 1;
-            } while (slot > 0);
-        }
-        if (kCount) r.n_reads += (uint32_t)(kFix - sh - lstar);
-        if (slot < 0) {
-            nval = load_leaf<kWrap>(T, prec, kk, slot);
-            if (kCount) r.n_leaf += 1;
-        }
-        rebase = rebase || (uint32_t)(kFix - sh - r.f) > (uint32_t)P.frame_levels;
-        if (P.frame_levels < kBoxLevels && (((N - s) ^ N) >> (kFix - r.f)) != 0u) rebase = fexit = true;
     }
-    // 4. precision of this boundary (past the canvas: a boundary to sigma = 0)
-    {
-        const float dt = __fmaf_rn(P.bound_t, fabsf(teh), P.bound_i * ihx);
-        const float bound = r.T * fmaxf(hsig(r.val), hsig(nval)) * dt;
-        const float spent = r.err + (((nval.x ^ r.val.x) | (nval.y ^ r.val.y)) ? bound : 0.0f);
-        const bool exact = have64 || rebase || spent > P.err_budget;
-        if (exact) need64();
-        else r.err = spent;
+    if (slot > 0) {
+        // finer than the old cell: near side on the exit axis, the ray's position on the others
+        uint32_t o0, o1, o2;
+        const uint32_t q0 = locate(r, 0, teh, s, o0), q1 = locate(r, 1, teh, s, o1), q2 = locate(r, 2, teh, s, o2);
+        q[0] = ax == 0 ? N : q0;
+        q[1] = ax == 1 ? N : q1;
+        q[2] = ax == 2 ? N : q2;
+        const uint32_t open = (ax == 0 ? 0u : o0) | (ax == 1 ? 0u : o1) | (ax == 2 ? 0u : o2);
+        do {
+            if (!kRopes) stk[kFix - sh] = slot;
+            --sh;
+            if (open >> sh) {
+                sides64(r, P, sh, ax, exact_time(), q);
+                rebase = rebase || fabsf(teh) > kFar * ihx * (float)(1u << sh);
+            }
+            prec = slot;
+            kk = child_index(q, sh, r.flip);
+            slot = load_slot<kSmem, kPool>(T, P.smem_records, prec, kk);
+            if (kCount) r.n_rec += 1;
+        } while (slot > 0);
     }
-    // 5. composite the current leaf, then terminate or advance
-    composite(r, teh, tel, P.side);
-    bool end = leaves_canvas || r.T < P.t_min;
-    if (!end && r.steps >= P.step_limit) {
-        atomicOr(&P.scratch->status, 1ull);
-        atomicAdd(&P.scratch->stats[kStatStepLimited], 1ull);
-        end = true;
+    if (kCount && !left) atomicAdd(&r.n_reads(), (uint32_t)((uint32_t)(kFix - sh - lstar)));
+    r.pval = r.val;
+    r.val = make_uint2(0u, 0u);
+    if (slot < 0) {
+        r.val = load_leaf<kPool>(T, prec, kk, slot);
+        if (kCount) r.n_leaf += 1;
     }
-    if (end) {
-        finish(r, P);
-        return false;
-    }
-    r.val = nval;
+    rebase = rebase || (uint32_t)(kFix - sh - r.f) > (uint32_t)P.frame_levels;
+    if (P.frame_levels < kBoxLevels && (((N - s) ^ N) >> (kFix - r.f)) != 0u) rebase = fexit = true;
+    rebase = rebase && !left;
     if (kRopes) {
         r.pr = prec;
         r.kc = (uint32_t)kk;
     }
-    r.steps += 1;
+    r.entry = (uint32_t)ax | (left * kLeft);
     r.L = kFix - sh;
 #pragma unroll
     for (int a = 0; a < 3; ++a) r.X[a] = (q[a] >> sh) << sh;
-    r.cur_hi = teh;
-    r.cur_lo = tel;
     if (rebase) {
+        const double te64 = exact_time();
+        r.ell = ((teh - r.cur_hi) + (tel - r.cur_lo)) * P.side;
         // a leaf coarser than the frame takes the coarsest frame that holds it; a descent past the frame the deepest
         // one the canvas can need, so that deeper leaves do not anchor the ray again level by level
         r.f = fexit || r.L < r.f ? max(0, r.L - P.frame_levels) : deep_frame(r.L, T.depth, P.frame_levels);
         set_anchor(r, P, P.views[r.view()], te64, ax);
+    } else {
+        r.ell = ((teh - r.cur_hi) + (tel - r.cur_lo)) * P.side;
+        r.cur_hi = teh;
+        r.cur_lo = tel;
     }
+    r.dt = have64 ? 0.0f : __fmaf_rn(P.bound_t, fabsf(teh), P.bound_i * ihx);
     return true;
 }
 
@@ -641,7 +729,7 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
     return v;
 }
 
-template <bool kSmem, bool kRopes, bool kCount, bool kWrap>
+template <bool kSmem, bool kRopes, bool kCount, int kPool>
 __global__ void __launch_bounds__(kBlock, CANVOX_MIN_BLOCKS) mixed_kernel(MixedParams P) {
     __shared__ double lanes[kCols * kBlock];
     if (kSmem) {
@@ -652,7 +740,8 @@ __global__ void __launch_bounds__(kBlock, CANVOX_MIN_BLOCKS) mixed_kernel(MixedP
     Ray r;
     r.base = reinterpret_cast<char*>(&lanes[threadIdx.x]);
     r.n_f64() = r.n_rebase() = r.n_rays() = r.n_steps() = 0;
-    r.n_reads = r.n_leaf = r.n_rec = 0;
+    r.n_reads() = 0;
+    r.n_leaf = r.n_rec = 0;
     const unsigned lane = threadIdx.x & 31u;
     bool alive = false;
     bool drained = false;
@@ -666,7 +755,7 @@ __global__ void __launch_bounds__(kBlock, CANVOX_MIN_BLOCKS) mixed_kernel(MixedP
             if (base + __popc(idle) >= (unsigned long long)P.total_rays) drained = true;
             if (!alive) {
                 const unsigned long long g = base + __popc(idle & ((1u << lane) - 1u));
-                if (g < (unsigned long long)P.total_rays) alive = ray_init<kSmem, kRopes, kCount, kWrap>(r, P, g, stk);
+                if (g < (unsigned long long)P.total_rays) alive = ray_init<kSmem, kRopes, kCount, kPool>(r, P, g, stk);
             }
             busy = __ballot_sync(kFull, alive);
             if (!drained && __popc(busy) <= P.refill) continue;
@@ -676,12 +765,12 @@ __global__ void __launch_bounds__(kBlock, CANVOX_MIN_BLOCKS) mixed_kernel(MixedP
             continue;
         }
         do {
-            if (alive) alive = ray_step<kSmem, kRopes, kCount, kWrap>(r, P, stk);
+            if (alive) alive = ray_step<kSmem, kRopes, kCount, kPool>(r, P, stk);
             busy = __ballot_sync(kFull, alive);
             // (refill 0, the default: run until every lane is done; the uniform test skips the count)
         } while (busy != 0u && (drained || P.refill == 0 || __popc(busy) > P.refill));
     }
-    const unsigned long long v[7] = {r.n_rays(), r.n_steps(), kCount ? r.n_reads : 0u, kCount ? r.n_leaf : 0u,
+    const unsigned long long v[7] = {r.n_rays(), r.n_steps(), kCount ? r.n_reads() : 0u, kCount ? r.n_leaf : 0u,
                                      kCount ? r.n_rec : 0u, r.n_f64(), r.n_rebase()};
 #pragma unroll
     for (int i = 0; i < 7; ++i) {
@@ -692,25 +781,28 @@ __global__ void __launch_bounds__(kBlock, CANVOX_MIN_BLOCKS) mixed_kernel(MixedP
 
 }  // namespace
 
-template <bool kRopes, bool kCount, bool kWrap>
+template <bool kRopes, bool kCount, int kPool>
 cudaError_t launch_mixed_t(const MixedParams& p, int grid, int block, cudaStream_t s) {
     if (p.smem_records <= 0) {
-        mixed_kernel<false, kRopes, kCount, kWrap><<<grid, block, 0, s>>>(p);
+        mixed_kernel<false, kRopes, kCount, kPool><<<grid, block, 0, s>>>(p);
         return cudaGetLastError();
     }
     // static (per-lane records) plus dynamic shared memory passes the 48 KB default: always opt in
     const int smem = p.smem_records * 32;
     const cudaError_t e =
-        cudaFuncSetAttribute(mixed_kernel<true, kRopes, kCount, kWrap>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaFuncSetAttribute(mixed_kernel<true, kRopes, kCount, kPool>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    mixed_kernel<true, kRopes, kCount, kWrap><<<grid, block, smem, s>>>(p);
+    mixed_kernel<true, kRopes, kCount, kPool><<<grid, block, smem, s>>>(p);
     return cudaGetLastError();
 }
 
 template <bool kRopes, bool kCount>
 cudaError_t launch_mixed_w(const MixedParams& p, int grid, int block, cudaStream_t s) {
-    return p.tree.n_wrap > 0 ? launch_mixed_t<kRopes, kCount, true>(p, grid, block, s)
-                             : launch_mixed_t<kRopes, kCount, false>(p, grid, block, s);
+    switch (pool_kind(p.tree)) {
+        case kSmallPool: return launch_mixed_t<kRopes, kCount, kSmallPool>(p, grid, block, s);
+        case kPlainPool: return launch_mixed_t<kRopes, kCount, kPlainPool>(p, grid, block, s);
+        default: return launch_mixed_t<kRopes, kCount, kWrapPool>(p, grid, block, s);
+    }
 }
 
 cudaError_t launch_mixed(const MixedParams& params, int grid, int block, cudaStream_t s) {
@@ -720,6 +812,7 @@ cudaError_t launch_mixed(const MixedParams& params, int grid, int block, cudaStr
     p.side = (float)p.tree.extent;
     p.bound_t = kEpsT * p.side;
     p.bound_i = kEpsI * p.side;
+    p.steps = (int32_t)(p.step_limit < 0x7FFFFFFF ? p.step_limit : 0x7FFFFFFF);
     const bool ropes = p.use_ropes && p.tree.ropes;
     if (p.count_reads)
         return ropes ? launch_mixed_w<true, true>(p, grid, block, s) : launch_mixed_w<false, true>(p, grid, block, s);
@@ -729,11 +822,11 @@ cudaError_t launch_mixed(const MixedParams& params, int grid, int block, cudaStr
 cudaError_t mixed_max_blocks_per_sm(int block, int smem_bytes, int* out) {
     // all instances share the register and static shared-memory budget
     if (smem_bytes <= 0)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, mixed_kernel<false, true, true, false>, block, 0);
-    const cudaError_t e = cudaFuncSetAttribute(mixed_kernel<true, true, true, false>,
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, mixed_kernel<false, true, true, kPlainPool>, block, 0);
+    const cudaError_t e = cudaFuncSetAttribute(mixed_kernel<true, true, true, kPlainPool>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, mixed_kernel<true, true, true, false>, block, smem_bytes);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, mixed_kernel<true, true, true, kPlainPool>, block, smem_bytes);
 }
 
 }  // namespace canvox

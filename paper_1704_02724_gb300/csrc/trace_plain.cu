@@ -15,6 +15,7 @@
 #include <cuda_fp16.h>
 
 #include "canvox_internal.cuh"
+#include "cells.cuh"
 
 namespace canvox {
 namespace {
@@ -275,8 +276,10 @@ __global__ void eye_path_kernel(Tree t, const View* views, int n_views, EyePath*
 // Neighbour links (the paper's neighbour graph of Sec. 4.1.1, kept per record).
 // ropes[r][2a + s] names the cell across face (axis a, s = 1 high / 0 low) of
 // record r's cell: the same-level neighbour if it exists, else the coarser leaf
-// that covers it, as (record holding its slot, (child index << 8) | its level);
-// record -1 is outside the canvas. One launch per level, parents before
+// that covers it, as (record holding its slot, (child index << 8) | its level),
+// or, for an internal neighbour, as (its own record, kLinkRecord | the same),
+// which saves a ray the load of its slot; outside the canvas as (0, kLinkRecord),
+// which reads as an empty slot. One launch per level, parents before
 // children: a child's link is its sibling inside the parent, or the parent's
 // link, refined to the adjacent child when that neighbour is an internal cell.
 // Bound by memory (32 B of slots and 48 B of links read and 48 B written per
@@ -289,12 +292,12 @@ __global__ void __launch_bounds__(256) rope_level_kernel(const int32_t* nodes, u
     const long long r = lo + (t >> 3);
     const int k = (int)(t & 7);
     if (r >= hi) return;
-    if (level == 0 && k < 6) ropes[k] = make_uint2(0xFFFFFFFFu, 0u);
+    if (level == 0 && k < 6) ropes[k] = make_uint2(0u, kLinkRecord);
     const int32_t v = nodes[8 * r + k];
     if (v <= 0) return;
     uint2 R[6];
     if (level == 0) {
-        for (int f = 0; f < 6; ++f) R[f] = make_uint2(0xFFFFFFFFu, 0u);
+        for (int f = 0; f < 6; ++f) R[f] = make_uint2(0u, kLinkRecord);
     } else {
         const uint4* p = reinterpret_cast<const uint4*>(ropes + 6 * r);
 #pragma unroll
@@ -309,11 +312,14 @@ __global__ void __launch_bounds__(256) rope_level_kernel(const int32_t* nodes, u
     for (int a = 0; a < 3; ++a) {
         const uint32_t kk = (uint32_t)(k ^ (1 << a));
         const bool high = (k >> a) & 1;
-        const uint2 own = make_uint2((uint32_t)r, (kk << 8) | (uint32_t)(level + 1));  // the sibling inside r
-        uint2 far = high ? R[2 * a + 1] : R[2 * a];  // past r's face on the child's side
-        if ((int)far.x >= 0) {
-            const int32_t sv = nodes[(long long)(int)far.x * 8 + ((far.y >> 8) & 7u)];
-            if (sv > 0) far = make_uint2((uint32_t)sv, (kk << 8) | (uint32_t)(level + 1));
+        const uint32_t where = (kk << 8) | (uint32_t)(level + 1);
+        // the sibling inside r, and the cell past r's face on the child's side
+        const int32_t ov = nodes[8 * r + kk];
+        const uint2 own = ov > 0 ? make_uint2((uint32_t)ov, kLinkRecord | where) : make_uint2((uint32_t)r, where);
+        uint2 far = high ? R[2 * a + 1] : R[2 * a];
+        if ((far.y & kLinkRecord) && far.x != 0u) {
+            const int32_t cv = nodes[(long long)(int)far.x * 8 + kk];
+            far = cv > 0 ? make_uint2((uint32_t)cv, kLinkRecord | where) : make_uint2(far.x, where);
         }
         out[a] = high ? make_uint4(own.x, own.y, far.x, far.y) : make_uint4(far.x, far.y, own.x, own.y);
     }

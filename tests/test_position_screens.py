@@ -139,3 +139,25 @@ def test_pixel_quotients():
             q = rd(a * r)
             q = rd(rd(a - W * q) * r + q)
             assert q == Q((2 * i + 1) / W)
+
+
+def fma64(a, b, c):
+    return rd(a * b + c)
+
+
+def test_norm_square_root():
+    """sqrt by two coupled Newton steps from an approximation of 20 bits and the exact-remainder correction is the
+    rounded square root, and its reciprocal is within two ulps."""
+    rng = random.Random(4)
+    for k in range(1500):
+        x = Q(rng.choice((1.0, 4.0, 2.25, 1.0 + 2.0 ** -52)) if k < 8 else math.exp(rng.uniform(0.0, 12.0)))
+        y = Q(float(1.0 / math.sqrt(float(x))) * (1.0 + rng.uniform(-1, 1) * 2.0 ** -20))
+        g, h = rd(x * y), rd(y / 2)
+        for _ in range(2):
+            r = fma64(-g, h, Q(1, 2))
+            g, h = fma64(g, r, g), fma64(h, r, h)
+        g = fma64(fma64(-g, g, x), h, g)
+        assert float(g) == math.sqrt(float(x))
+        h = 2 * h
+        r = fma64(h, fma64(-g, h, Q(1)), h)
+        assert abs(r * g - 1) <= Q(1, 2 ** 51)
