@@ -456,15 +456,18 @@ int check_stamps(const double* centers, const double* radii, const float* rgba, 
 
 
 // The host's cores for the length of one call: run(n, fn) calls fn(i) for i in [0, n), the calling thread among them;
-// start() leaves it to the others until finish(). One thread for little work, and where no other can be started. The
-// pools of a canvas are validated and hashed element by element: one core takes about 2 ns an element, 10 ms for the
-// depth-8 canvas of 431,100 records, which bounded its upload.
+// start() leaves it to the others until finish(). The pools of a canvas are validated and hashed element by element:
+// one core takes about 1.5 ns an element, 10 ms for the depth-8 canvas of 431,100 records, which bounded its upload. A
+// thread takes 13 us to start, so there is one for every 80 us of work, kPieceUs a piece of kHostChunk leaves (and one
+// where no other can be started).
 class HostTeam {
   public:
-    explicit HostTeam(int64_t pieces) {
+    static constexpr int64_t kPieceUs = 13;
+    explicit HostTeam(int64_t leaf_pieces) {
         const int64_t cores = std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), 64);
+        const int64_t want = std::min(cores, 1 + leaf_pieces * kPieceUs / 80);
         try {
-            while ((int64_t)team_.size() + 1 < std::min(cores, pieces / 2)) team_.emplace_back([this] { serve(); });
+            while ((int64_t)team_.size() + 1 < want) team_.emplace_back([this] { serve(); });
         } catch (...) {  // no more threads: the others and the caller do it
         }
     }
@@ -532,46 +535,38 @@ class HostTeam {
 constexpr int64_t kHostChunk = 8192;  // records (256 KB) or leaves per piece of host work
 int64_t pieces_of(int64_t n) { return (n + kHostChunk - 1) / kHostChunk; }
 
-// First value of leaves [0, n) that is not allowed (-1: none): 0 non-finite, 1 negative extinction in *what.
-int64_t bad_leaf(const uint16_t* leaf_rgba, int64_t begin, int64_t end, int* what) {
-    for (int64_t i = begin; i < end; ++i) {
-        const uint16_t* q = leaf_rgba + 4 * i;
-        for (int c = 0; c < 4; ++c)
-            if (((q[c] >> 10) & 31) == 31) {
-                *what = 0;
-                return i;
-            }
-        if ((q[3] & 0x8000u) && (q[3] & 0x7FFFu)) {
-            *what = 1;
-            return i;
-        }
-    }
-    return -1;
+// The leaf's four binary16 words (R | G << 16 | B << 32 | sigma << 48), and whether they are allowed: all finite (an
+// exponent of 31 carries into bit 15 when 1 is added to it), the extinction not negative.
+unsigned long long leaf_word(const uint16_t* leaf_rgba, int64_t i) {
+    unsigned long long v;
+    std::memcpy(&v, leaf_rgba + 4 * i, sizeof(v));
+    return v;
 }
+bool leaf_finite(unsigned long long v) {
+    return (((v & 0x7C007C007C007C00ull) + 0x0400040004000400ull) & 0x8000800080008000ull) == 0;
+}
+bool leaf_allowed(unsigned long long v) { return leaf_finite(v) && (v >> 48) <= 0x8000u; }
 
-// Checks the values of leaves [0, n), numbered from `first` in the message.
-int check_leaves(HostTeam& team, const uint16_t* leaf_rgba, int64_t n, int64_t first) {
-    const int64_t pieces = pieces_of(n);
-    std::vector<int64_t> bad((size_t)pieces, -1);
-    std::vector<int> what((size_t)pieces, 0);
-    team.run(pieces, [&](int64_t p) {
-        bad[(size_t)p] = bad_leaf(leaf_rgba, p * kHostChunk, std::min(n, (p + 1) * kHostChunk), &what[(size_t)p]);
-    });
-    for (int64_t p = 0; p < pieces; ++p)
-        if (bad[(size_t)p] >= 0)
-            return fail(CANVOX_ERR_BAD_TREE, what[(size_t)p] ? "leaf %lld: negative extinction" : "leaf %lld: non-finite FP16",
-                        (long long)(first + bad[(size_t)p]));
+// The error of the first leaf that is not allowed in pieces' findings (-1: none), numbered from `first`.
+int leaf_error(const std::vector<int64_t>& bad, const uint16_t* leaf_rgba, int64_t first) {
+    for (int64_t i : bad)
+        if (i >= 0)
+            return fail(CANVOX_ERR_BAD_TREE,
+                        leaf_finite(leaf_word(leaf_rgba, i)) ? "leaf %lld: negative extinction" : "leaf %lld: non-finite FP16",
+                        (long long)(first + i));
     return CANVOX_OK;
+}
+int64_t first_bad_leaf(const uint16_t* leaf_rgba, int64_t begin, int64_t end) {
+    for (int64_t i = begin; i < end; ++i)
+        if (!leaf_allowed(leaf_word(leaf_rgba, i))) return i;
+    return -1;
 }
 
 // Hash terms of leaves [begin, end), numbered from `first`.
 unsigned long long hash_leaves(const uint16_t* leaf_rgba, int64_t begin, int64_t end, int64_t first) {
     unsigned long long h = 0;
-    for (int64_t i = begin; i < end; ++i) {
-        unsigned long long v;
-        std::memcpy(&v, leaf_rgba + 4 * i, sizeof(v));  // R | G << 16 | B << 32 | sigma << 48
-        h += elem_hash(2ull, (unsigned long long)(first + i), v);
-    }
+    for (int64_t i = begin; i < end; ++i)
+        h += elem_hash(2ull, (unsigned long long)(first + i), leaf_word(leaf_rgba, i));
     return h;
 }
 unsigned long long hash_slots(const int32_t* node_pool, int64_t begin, int64_t end) {  // records
@@ -721,13 +716,17 @@ int upload(const int32_t* node_pool, int64_t n_records, const uint16_t* leaf_rgb
            double extent) {
     // validation: breadth-first numbering of records and leaves, depth bound, finite FP16 values
     const int64_t node_pieces = pieces_of(n_records), leaf_pieces = pieces_of(n_leaves);
-    HostTeam team(node_pieces + leaf_pieces);
+    HostTeam team(9 * node_pieces + leaf_pieces);  // (eight slots a record)
     std::vector<int64_t> level_begin;
     int64_t wraps[kMaxWraps] = {};
     int32_t n_wrap = 0;
     int rc = check_nodes(team, node_pool, n_records, n_leaves, depth, &level_begin, wraps, &n_wrap);
     if (rc) return rc;
-    if ((rc = check_leaves(team, leaf_rgba, n_leaves, 0))) return rc;
+    std::vector<int64_t> bad((size_t)leaf_pieces, -1);
+    team.run(leaf_pieces, [&](int64_t p) {
+        bad[(size_t)p] = first_bad_leaf(leaf_rgba, p * kHostChunk, std::min(n_leaves, (p + 1) * kHostChunk));
+    });
+    if ((rc = leaf_error(bad, leaf_rgba, 0))) return rc;
     if ((rc = ensure_device())) return rc;
     // the host pools' hash, beside the copies
     std::atomic<unsigned long long> hash{0};
@@ -776,25 +775,29 @@ int upload(const int32_t* node_pool, int64_t n_records, const uint16_t* leaf_rgb
 // old values' terms, summed where they are, go out and the new ones', from the caller's values, come in.
 int update_range(int64_t first, int64_t count, const uint16_t* leaf_rgba) {
     const int64_t pieces = pieces_of(count);
-    HostTeam team(pieces);
-    int rc = check_leaves(team, leaf_rgba, count, first);
-    if (rc) return rc;
-    if (count == 0) return CANVOX_OK;
+    std::vector<int64_t> bad((size_t)pieces, -1);
     std::atomic<unsigned long long> added{0};
+    HostTeam team(pieces);
     team.start(pieces, [&](int64_t p) {
-        added += hash_leaves(leaf_rgba, p * kHostChunk, std::min(count, (p + 1) * kHostChunk), first);
+        const int64_t b = p * kHostChunk, e = std::min(count, b + kHostChunk);
+        bad[(size_t)p] = first_bad_leaf(leaf_rgba, b, e);
+        added += hash_leaves(leaf_rgba, b, e, first);
     });
-    struct Finish {
+    struct Finish {  // (an early return waits for the team, whose work refers to the names above)
         HostTeam& team;
         ~Finish() { team.finish(); }
     } finish{team};
-    if (g.any_render) CK(cudaEventSynchronize(g.done), "cudaEventSynchronize");
-    CK(cudaMemset(g.d_hash, 0, sizeof(unsigned long long)), "cudaMemset(hash)");
-    CK(launch_hash_leaves(g.d_leaves + first, first, count, g.d_hash, 0), "hash kernel launch");
-    unsigned long long gone = 0;
-    CK(cudaMemcpy(&gone, g.d_hash, sizeof(gone), cudaMemcpyDeviceToHost), "cudaMemcpy(hash)");
-    CK(cudaMemcpy(g.d_leaves + first, leaf_rgba, sizeof(uint2) * (size_t)count, cudaMemcpyHostToDevice), "cudaMemcpy(leaves)");
+    if (count > 0) {
+        if (g.any_render) CK(cudaStreamWaitEvent(0, g.done, 0), "cudaStreamWaitEvent");
+        CK(cudaMemsetAsync(g.d_hash, 0, sizeof(unsigned long long), 0), "cudaMemset(hash)");
+        CK(launch_hash_leaves(g.d_leaves + first, first, count, g.d_hash, 0), "hash kernel launch");
+    }
     team.finish();
+    const int rc = leaf_error(bad, leaf_rgba, first);
+    if (rc || count == 0) return rc;
+    unsigned long long gone = 0;
+    CK(cudaMemcpy(&gone, g.d_hash, sizeof(gone), cudaMemcpyDeviceToHost), "cudaMemcpy(hash)");  // (earlier renders done)
+    CK(cudaMemcpy(g.d_leaves + first, leaf_rgba, sizeof(uint2) * (size_t)count, cudaMemcpyHostToDevice), "cudaMemcpy(leaves)");
     g.host_hash += added.load() - gone;
     g.last_h2d = (int64_t)sizeof(uint2) * count;
     return CANVOX_OK;
