@@ -462,7 +462,7 @@ def main():
                        "schedule": "autotuned" if tuned else ("given" if opts else "built-in default")},
             "stereo_fps": (world / (ms_max * 1e-3)) if len(cams) == 2 else None,
             "wall_ms_per_step_incl_flush": wall * 1e3 / args.steps,
-            # per render: the eye-path kernel and the traversal kernel (one per view in per-view mode)
+            # per render: the set-up kernel and the traversal kernel (one per view in per-view mode)
             "gpu_launches": args.steps * (1 + (1 if not opts.get("per_view") else len(cams))),
             "roofline": roofline,
             "stats": {k: v for k, v in stats.items() if k != "status"},

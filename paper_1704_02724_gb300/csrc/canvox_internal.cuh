@@ -137,7 +137,9 @@ struct PlainParams {
 };
 
 // Launchers (trace_mixed.cu, trace_plain.cu, runtime.cu).
-cudaError_t launch_mixed(const MixedParams& p, int grid, int block, cudaStream_t s);  // smem from p.smem_records
+// smem from p.smem_records; after_setup: the launch right before it on the stream is launch_setup's, whose end the
+// kernel waits for itself (its blocks are resident by then)
+cudaError_t launch_mixed(const MixedParams& p, int grid, int block, cudaStream_t s, bool after_setup = false);
 cudaError_t mixed_max_blocks_per_sm(int block, int smem_bytes, int* out);
 cudaError_t launch_fp64links(const MixedParams& p, int grid, int block, cudaStream_t s);  // needs p.tree.ropes
 cudaError_t fp64links_max_blocks_per_sm(int block, int* out);
@@ -148,6 +150,11 @@ cudaError_t launch_hash(const Tree& t, unsigned long long* out, cudaStream_t s);
 cudaError_t launch_hash_leaves(const uint2* leaves, int64_t first, int64_t n, unsigned long long* out, cudaStream_t s);
 cudaError_t launch_rope_level(const int32_t* nodes, uint2* ropes, int64_t lo, int64_t hi, int level, cudaStream_t s);
 cudaError_t launch_eye_paths(const Tree& t, const View* views, int n_views, EyePath* out, cudaStream_t s);
+// One launch for what a render needs before its traversal: the view table (n <= kSetupViews, host memory, by value),
+// the eye paths, and `queues` ray-queue heads, the counters and the status word cleared.
+constexpr int kSetupViews = 64;
+cudaError_t launch_setup(const Tree& t, const View* host_views, int n, View* views, EyePath* eye, Scratch* scratch,
+                         int queues, cudaStream_t s);
 cudaError_t probe_l2_gather(int64_t buffer_bytes, double* gbs);
 cudaError_t probe_fp64(double* gflops);
 // The device painter. *cache: what it keeps of the last painted canvas for appends (null: none). When it holds

@@ -16,7 +16,7 @@
 namespace canvox {
 namespace {
 
-constexpr int kNoallocMaxViews = 64;
+constexpr int kNoallocMaxViews = kSetupViews;
 constexpr size_t kOffViews = 256;  // after the Scratch header (80 bytes), 256-byte aligned
 constexpr size_t kOffEye = kOffViews + ((sizeof(View) * kNoallocMaxViews + 255) / 256) * 256;
 constexpr size_t kNoallocBytes = kOffEye + ((sizeof(EyePath) * kNoallocMaxViews + 255) / 256) * 256;
@@ -27,25 +27,6 @@ static_assert(kNoallocBytes <= 24576, "the fixed scratch array is 24 KiB");
 // until the process exits. Host code must not use its name as a device address:
 // it takes the address from cudaGetSymbolAddress once per device (below).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[24576];
-
-// The view table of one call, passed by value as a kernel argument: the set-up kernel
-// copies it into the fixed array, so no host buffer has to outlive the call.
-struct ViewTable {
-    View v[kNoallocMaxViews];
-    int32_t n;
-};
-static_assert(sizeof(ViewTable) <= 32000, "kernel arguments are limited to 32764 bytes");
-
-// Clears the counters, status word and queue head, and stores the view table.
-__global__ void noalloc_setup_kernel(ViewTable t, Scratch* scratch, View* views) {
-    unsigned long long* z = reinterpret_cast<unsigned long long*>(scratch);
-    for (int i = threadIdx.x; i < (int)(sizeof(Scratch) / 8); i += blockDim.x) z[i] = 0ull;
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(t.v);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(views);
-    const int words = t.n * (int)(sizeof(View) / 4);
-    for (int i = threadIdx.x; i < words; i += blockDim.x) dst[i] = src[i];
-}
-static_assert(sizeof(Scratch) % 8 == 0 && sizeof(View) % 4 == 0, "word copies");
 
 constexpr int kMaxDevices = 64;
 // Device address of the array per device, looked up once (first call on that device). Atomic, so
@@ -94,12 +75,11 @@ extern "C" int canvox_render_noalloc(const int32_t* node_pool_dev, int64_t n_rec
         const double scaled = std::ldexp(std::frexp(extent, &ex), 23);
         if (scaled != std::floor(scaled)) return set_error(CANVOX_ERR_INVALID_ARG, "extent has more than 23 significant bits");
     }
-    ViewTable vt;  // host stack, no heap; travels as a kernel argument
-    vt.n = n_views;
+    View vt[kNoallocMaxViews];  // host stack, no heap; travels as a kernel argument
     int64_t total_rays = 0;
     canvox_render_opts o;
     builtin_render_opts(&o);
-    int rc = build_views(cams, n_views, o.tile_w, extent, vt.v, &total_rays);
+    int rc = build_views(cams, n_views, o.tile_w, extent, vt, &total_rays);
     if (rc) return rc;
     unsigned char* base = nullptr;
     rc = scratch_address(&base);
@@ -114,8 +94,6 @@ extern "C" int canvox_render_noalloc(const int32_t* node_pool_dev, int64_t n_rec
     View* views = reinterpret_cast<View*>(base + kOffViews);
     EyePath* eye = reinterpret_cast<EyePath*>(base + kOffEye);
     // the array keeps the previous call's contents: the counters and queue head start at zero
-    noalloc_setup_kernel<<<1, 256, 0, s>>>(vt, scratch, views);
-    e = cudaGetLastError();
     Tree t;
     t.nodes = node_pool_dev;
     t.ropes = nullptr;
@@ -126,7 +104,7 @@ extern "C" int canvox_render_noalloc(const int32_t* node_pool_dev, int64_t n_rec
     t.n_wrap = 0;  // n_leaves < 2^31: no leaf number passes 2^31
     t.extent = extent;
     t.half = 0.5 * extent;
-    if (e == cudaSuccess) e = launch_eye_paths(t, views, n_views, eye, s);
+    e = launch_setup(t, vt, n_views, views, eye, scratch, 1, s);
     if (e != cudaSuccess) return set_error(CANVOX_ERR_CUDA, cudaGetErrorString(e));
     MixedParams p;
     std::memset(&p, 0, sizeof(p));
@@ -149,7 +127,7 @@ extern "C" int canvox_render_noalloc(const int32_t* node_pool_dev, int64_t n_rec
     p.smem_records = 0;
     p.use_ropes = 0;  // no neighbour links without allocating them
     p.count_reads = 0;  // these calls report no counters
-    e = launch_mixed(p, sms * (bps > 0 ? bps : 1), o.block_threads, s);
+    e = launch_mixed(p, sms * (bps > 0 ? bps : 1), o.block_threads, s, true);
     if (e != cudaSuccess) return set_error(CANVOX_ERR_CUDA, cudaGetErrorString(e));
     return CANVOX_OK;
 }

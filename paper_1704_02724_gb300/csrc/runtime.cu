@@ -303,13 +303,20 @@ Tree device_tree() {
     return t;
 }
 
-// The launch sequence of one render: stage views, clear scratch, trace.
+// The launch sequence of one render: set up (views, cleared scratch, eye paths), trace. With hv (a pinned copy of the
+// views: renders replayed from a graph, which read the views of each replay there, and more views than a launch's
+// arguments hold) the set-up is a copy, a memset and a kernel, else one launch.
 int enqueue(const View* hv, const View* views_host, int n, int64_t total_rays, float* out,
             const canvox_render_opts& o, cudaStream_t s) {
     const int queues = o.per_view ? n : 1;
-    CK(cudaMemcpyAsync(g.d_views, hv, sizeof(View) * (size_t)n, cudaMemcpyHostToDevice, s), "cudaMemcpyAsync(views)");
-    CK(cudaMemsetAsync(g.d_scratch, 0, scratch_bytes(queues), s), "cudaMemsetAsync(scratch)");
     const Tree t = device_tree();
+    if (hv) {
+        CK(cudaMemcpyAsync(g.d_views, hv, sizeof(View) * (size_t)n, cudaMemcpyHostToDevice, s), "cudaMemcpyAsync(views)");
+        CK(cudaMemsetAsync(g.d_scratch, 0, scratch_bytes(queues), s), "cudaMemsetAsync(scratch)");
+        CK(launch_eye_paths(t, g.d_views, n, g.d_eye, s), "eye path kernel launch");
+    } else {
+        CK(launch_setup(t, views_host, n, g.d_views, g.d_eye, g.d_scratch, queues, s), "set-up kernel launch");
+    }
     if (o.precision == CANVOX_PREC_MIXED || o.precision == CANVOX_PREC_FP64_LINKS) {
         // the persistent traversal: mixed precision, or its FP64 twin (same traversal, FP64 arithmetic)
         const bool f64 = o.precision == CANVOX_PREC_FP64_LINKS;
@@ -320,9 +327,9 @@ int enqueue(const View* hv, const View* views_host, int n, int64_t total_rays, f
             bps = b > 0 ? (b < bps ? b : bps) : 1;
         }
         auto launch = [&](const MixedParams& p, int grid) {
-            return f64 ? launch_fp64links(p, grid, o.block_threads, s) : launch_mixed(p, grid, o.block_threads, s);
+            return f64 ? launch_fp64links(p, grid, o.block_threads, s)
+                       : launch_mixed(p, grid, o.block_threads, s, !hv && !o.per_view);
         };
-        CK(launch_eye_paths(t, g.d_views, n, g.d_eye, s), "eye path kernel launch");
         MixedParams p;
         std::memset(&p, 0, sizeof(p));
         p.tree = t;
@@ -947,11 +954,14 @@ int canvox_render_ex(const canvox_camera* cams, int32_t n_views, float* out_rgba
     if (rc) return rc;
     if ((rc = ensure_views(n_views)) || (rc = ensure_scratch(o.per_view ? n_views : 1))) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    const bool stage = o.use_graph || n_views > kSetupViews;
     const int b = g.next_buf;
-    g.next_buf ^= 1;
-    // the staging buffer b may still feed an earlier render's copy
-    CK(cudaEventSynchronize(g.staged[b]), "cudaEventSynchronize(staging)");
-    std::memcpy(g.h_views[b], views.data(), sizeof(View) * (size_t)n_views);
+    if (stage) {
+        g.next_buf ^= 1;
+        // the staging buffer b may still feed an earlier render's copy
+        CK(cudaEventSynchronize(g.staged[b]), "cudaEventSynchronize(staging)");
+        std::memcpy(g.h_views[b], views.data(), sizeof(View) * (size_t)n_views);
+    }
     // renders share the library's scratch: order this one after the previous one
     if (g.any_render) CK(cudaStreamWaitEvent(s, g.done, 0), "cudaStreamWaitEvent");
     if (o.use_graph) {
@@ -996,10 +1006,10 @@ int canvox_render_ex(const canvox_camera* cams, int32_t n_views, float* out_rgba
         }
         CK(cudaGraphLaunch(hit->exec, s), "cudaGraphLaunch");
     } else {
-        rc = enqueue(g.h_views[b], views.data(), n_views, total_rays, out_rgba_dev, o, s);
+        rc = enqueue(stage ? g.h_views[b] : nullptr, views.data(), n_views, total_rays, out_rgba_dev, o, s);
         if (rc) return rc;
     }
-    CK(cudaEventRecord(g.staged[b], s), "cudaEventRecord");
+    if (stage) CK(cudaEventRecord(g.staged[b], s), "cudaEventRecord");
     CK(cudaEventRecord(g.done, s), "cudaEventRecord");
     g.any_render = true;
     g.last_h2d = (int64_t)sizeof(View) * n_views;

@@ -732,6 +732,7 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 template <bool kSmem, bool kRopes, bool kCount, int kPool>
 __global__ void __launch_bounds__(kBlock, CANVOX_MIN_BLOCKS) mixed_kernel(MixedParams P) {
     __shared__ double lanes[kCols * kBlock];
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the set-up launch (views, eye paths, queue head)
     if (kSmem) {
         for (int i = threadIdx.x; i < P.smem_records * 8; i += blockDim.x) s_nodes[i] = __ldg(P.tree.nodes + i);
         __syncthreads();
@@ -782,30 +783,45 @@ __global__ void __launch_bounds__(kBlock, CANVOX_MIN_BLOCKS) mixed_kernel(MixedP
 }  // namespace
 
 template <bool kRopes, bool kCount, int kPool>
-cudaError_t launch_mixed_t(const MixedParams& p, int grid, int block, cudaStream_t s) {
-    if (p.smem_records <= 0) {
-        mixed_kernel<false, kRopes, kCount, kPool><<<grid, block, 0, s>>>(p);
+cudaError_t launch_mixed_t(const MixedParams& p, int grid, int block, cudaStream_t s, bool after_setup) {
+    void (*kernel)(MixedParams) = mixed_kernel<false, kRopes, kCount, kPool>;
+    int smem = 0;
+    if (p.smem_records > 0) {
+        // static (per-lane records) plus dynamic shared memory passes the 48 KB default: always opt in
+        kernel = mixed_kernel<true, kRopes, kCount, kPool>;
+        smem = p.smem_records * 32;
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    // a captured launch keeps its plain edge: graph queries of callers need not know programmatic ones
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (!after_setup || cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        kernel<<<grid, block, smem, s>>>(p);
         return cudaGetLastError();
     }
-    // static (per-lane records) plus dynamic shared memory passes the 48 KB default: always opt in
-    const int smem = p.smem_records * 32;
-    const cudaError_t e =
-        cudaFuncSetAttribute(mixed_kernel<true, kRopes, kCount, kPool>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    mixed_kernel<true, kRopes, kCount, kPool><<<grid, block, smem, s>>>(p);
-    return cudaGetLastError();
+    cudaLaunchAttribute overlap;
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cfg.attrs = &overlap;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
 template <bool kRopes, bool kCount>
-cudaError_t launch_mixed_w(const MixedParams& p, int grid, int block, cudaStream_t s) {
+cudaError_t launch_mixed_w(const MixedParams& p, int grid, int block, cudaStream_t s, bool after_setup) {
     switch (pool_kind(p.tree)) {
-        case kSmallPool: return launch_mixed_t<kRopes, kCount, kSmallPool>(p, grid, block, s);
-        case kPlainPool: return launch_mixed_t<kRopes, kCount, kPlainPool>(p, grid, block, s);
-        default: return launch_mixed_t<kRopes, kCount, kWrapPool>(p, grid, block, s);
+        case kSmallPool: return launch_mixed_t<kRopes, kCount, kSmallPool>(p, grid, block, s, after_setup);
+        case kPlainPool: return launch_mixed_t<kRopes, kCount, kPlainPool>(p, grid, block, s, after_setup);
+        default: return launch_mixed_t<kRopes, kCount, kWrapPool>(p, grid, block, s, after_setup);
     }
 }
 
-cudaError_t launch_mixed(const MixedParams& params, int grid, int block, cudaStream_t s) {
+cudaError_t launch_mixed(const MixedParams& params, int grid, int block, cudaStream_t s, bool after_setup) {
     MixedParams p = params;
     p.inv_extent = 1.0 / p.tree.extent;
     p.unit = p.tree.extent * 4.656612873077393e-10;  // 2^-31
@@ -815,8 +831,10 @@ cudaError_t launch_mixed(const MixedParams& params, int grid, int block, cudaStr
     p.steps = (int32_t)(p.step_limit < 0x7FFFFFFF ? p.step_limit : 0x7FFFFFFF);
     const bool ropes = p.use_ropes && p.tree.ropes;
     if (p.count_reads)
-        return ropes ? launch_mixed_w<true, true>(p, grid, block, s) : launch_mixed_w<false, true>(p, grid, block, s);
-    return ropes ? launch_mixed_w<true, false>(p, grid, block, s) : launch_mixed_w<false, false>(p, grid, block, s);
+        return ropes ? launch_mixed_w<true, true>(p, grid, block, s, after_setup)
+                     : launch_mixed_w<false, true>(p, grid, block, s, after_setup);
+    return ropes ? launch_mixed_w<true, false>(p, grid, block, s, after_setup)
+                 : launch_mixed_w<false, false>(p, grid, block, s, after_setup);
 }
 
 cudaError_t mixed_max_blocks_per_sm(int block, int smem_bytes, int* out) {
