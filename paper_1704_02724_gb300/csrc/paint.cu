@@ -27,8 +27,8 @@
 // knows whether an earlier stamp (or s itself) refines it, so one pass gives its
 // firstref, its blend and which stamps its own list keeps; that decision is left
 // as two bits per stamp and child, from which the next level's lists are written.
-// Lists of more than kLongList entries (near the root every stamp is on them;
-// around a room, its stamps) are cut into items of kItem entries that octets
+// Lists of more than 512 entries, 128 on levels of few cells (near the root every stamp is on them;
+// around a room, its stamps) are cut into items that octets
 // take in parallel: first the least refining stamp per child, then the decisions.
 // Geometry is FP32 with a proven margin, retaken in FP64 with the same operations
 // and order as the host painter inside the margin, so the pools are identical.
@@ -57,8 +57,13 @@ constexpr uint64_t kInternal = 1ull << 63;  // child slot: internal cell, low bi
 constexpr uint64_t kNotCollapsed = 1ull << 63;
 constexpr unsigned kFullMask = 0xFFFFFFFFu;
 constexpr int kCells = 16;              // cells per block of the octet kernels (128 threads)
-constexpr int64_t kLongList = 512;      // longer lists are cut into items ...
-constexpr int64_t kItem = 128;          // ... of so many entries, one octet each
+// Lists longer than this are cut into items, on levels of up to kFewCells cells and on those of more. A level of few cells
+// waits for the octet with the longest list (0.25 us an entry: 70-220 us for 300-500 entries on the levels where a room
+// begins), and the five launches for long lists cost some 30 us: 128 entries. With kLongFew 64, or kFewCells 4,096 or
+// 65,536, the painting session took the same within 1 %; with more cells the octets of other cells hide a list of 512.
+constexpr int64_t kFewCells = 16384;
+constexpr int64_t kLongFew = 128, kLongMany = 512;
+constexpr int kItemMin = 16, kItemMax = 128;  // ... of so many entries (item_size), one octet each
 constexpr int32_t kNoStamp = 0x7FFFFFFF;
 
 // What a child box test reads of a stamp: the centre as two FP32 words per axis, the squared radius (both scaled by the
@@ -119,6 +124,7 @@ struct LevelIn {
     const uint32_t* coord;  // [n][3]
     const int64_t* off;     // [n + 1]
     const int32_t* ent;     // s: descends, ~s: paints the whole cell
+    int64_t limit;          // longer lists are cut into items
     double h;               // side of the children
     float hf;               // the same scaled as the stamps' records are (NaN: a canvas for FP64 alone)
 };
@@ -131,26 +137,32 @@ enum { kOut = 0, kIn = 1, kPartCentreIn = 2, kPartCentreOut = 3 };
 // busy): j as two words too (the second 0 up to 2^24), the product's error from one fma. Within 2^-46 of the
 // corner's own size of the exact one.
 struct Child {
-    uint32_t cc[3];   // child coordinates
-    float lh[3], ll[3];
-    float hf, hh;     // side, half side
-    float g;          // the screen's margin: 2 sides per axis plus 2^-22 of the corner
+    uint32_t cc[3];      // child coordinates
+    float lh[3], ll[3];  // low corner
+    float uh[3], ul[3];  // high corner
+    float hh;            // half side
+    float a;             // the sum of the corners' sizes (the larger of the two per axis)
 };
+
+// j h as two FP32 words
+__device__ __forceinline__ void plane_words(int32_t j, float hf, float& hi, float& lo) {
+    const float jh = __int2float_rn(j), jl = __int2float_rn(j - __float2int_rn(jh));
+    const float p = __fmul_rn(jh, hf), t = __fmaf_rn(jl, hf, __fmaf_rn(jh, hf, -p));
+    hi = __fadd_rn(p, t);
+    lo = __fsub_rn(t, __fsub_rn(hi, p));
+}
 
 __device__ __forceinline__ Child child_box(const LevelIn& L, int64_t i, int k) {
     Child B;
-    B.hf = L.hf;
     B.hh = 0.5f * L.hf;
-    B.g = 6.0f * L.hf;
+    B.a = 0.0f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         B.cc[a] = 2u * L.coord[3 * i + a] + ((k >> a) & 1u);
         const int32_t j = (int32_t)B.cc[a] - (1 << L.level);
-        const float jh = __int2float_rn(j), jl = __int2float_rn(j - __float2int_rn(jh));
-        const float p = __fmul_rn(jh, L.hf), t = __fmaf_rn(jl, L.hf, __fmaf_rn(jh, L.hf, -p));
-        B.lh[a] = __fadd_rn(p, t);
-        B.ll[a] = __fsub_rn(t, __fsub_rn(B.lh[a], p));
-        B.g += 2.384185791015625e-07f * fabsf(B.lh[a]);
+        plane_words(j, L.hf, B.lh[a], B.ll[a]);
+        plane_words(j + 1, L.hf, B.uh[a], B.ul[a]);
+        B.a += fmaxf(fabsf(B.lh[a]), fabsf(B.uh[a]));
     }
     return B;
 }
@@ -173,21 +185,28 @@ __device__ __noinline__ int cover64(const double* c, double r2, uint32_t c0, uin
     return __dadd_rn(__dadd_rn(cen[0], cen[1]), cen[2]) < r2 ? kPartCentreIn : kPartCentreOut;
 }
 
-// The cover of a stamp, screened in FP32 (-1: open). With m >= M_a = |c_a - lo_a| + 2 h + 2^-22 |lo_a| on every axis,
-// the difference c_a - lo_a formed from two words each is within 2^-23 M_a of the exact one (the corner's words are
-// within 2^-46 of it, the centre's within 2^-48, and |c_a| <= |lo_a| + M_a), those to the far plane and the centre within 2^-22.4 M_a. The
-// squared distances to the far corner and the centre are then within 2^-20.9 m^2 (margin 2^-18 m^2), that to the box,
-// with n the sum of its terms' roots, within 2^-21.4 m n + 3 2^-44.8 m^2 + 2^-22 of itself (margin twice that and
-// more): a stamp far smaller than the box it lies in has n = 0 and is decided, where a margin in m^2 would leave
-// every room's stamps on every coarse level to FP64. Every comparison is false for a NaN or an infinite margin,
-// which leaves it open.
+// The cover of a stamp, screened in FP32 (-1: open). The difference x of the centre and a face's plane, formed from two
+// words each (the plane's within 2^-46 of it, the centre's within 2^-48), is within 2^-22.9 |x| + 2^-44.5 p of the exact
+// one, p the plane's size: next to a plane the words cancel exactly. So with A the sum of the planes' sizes and n that
+// of the distances outside the box per axis, the squared distance to the box is within 2^-21.1 of itself + 2^-43.5 A n +
+// 2^-88 A^2 (margin twice that and more). With m >= |x| + 2 h on every axis the squared distances to the far corner and
+// the centre are within 2^-20.9 (m + 2^-22 A)^2 (margin 2^-18). Without kExact the difference to the high face is formed
+// from the one to the low face, which is off by 2^-23 m: the squared distance to the box is then within 2^-21.4 m n +
+// 3 2^-44.8 m^2 + 2^-22 of itself. That leaves the stamps of a room that a plane of a far coarser cell crosses to FP64
+// (half of all tests on such a cell's list, 1 us an entry instead of 0.3), but next to cells of the stamps' own size
+// decides as many with fewer instructions and registers: expand_count
+// took 7.1 ms with kExact and 6.5 ms without over the levels of six paintings of 13,000 stamps.
+// Every comparison is false for a NaN or an infinite margin, which leaves it open.
+template <bool kExact>
 __device__ __forceinline__ int cover32(const Child& B, const StampRec& R, bool centre) {
     const float cl[3] = {R.cl0, R.cl1, R.cl2};
-    float dmin2 = 0.0f, dmax2 = 0.0f, cen2 = 0.0f, m = B.g, n = 0.0f;
+    float dmin2 = 0.0f, dmax2 = 0.0f, cen2 = 0.0f, m = 12.0f * B.hh + 2.384185791015625e-07f * B.a, n = 0.0f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float dl = __fadd_rn(__fsub_rn(R.ch[a], B.lh[a]), __fsub_rn(cl[a], B.ll[a]));
-        const float du = __fsub_rn(dl, B.hf), dc = __fsub_rn(dl, B.hh);
+        const float du = kExact ? __fadd_rn(__fsub_rn(R.ch[a], B.uh[a]), __fsub_rn(cl[a], B.ul[a]))
+                                : __fsub_rn(dl, 2.0f * B.hh);
+        const float dc = __fsub_rn(dl, B.hh);
         const float near = fmaxf(fmaxf(-dl, du), 0.0f), far = fmaxf(fabsf(dl), fabsf(du));
         dmin2 = fmaf(near, near, dmin2);
         dmax2 = fmaf(far, far, dmax2);
@@ -195,8 +214,11 @@ __device__ __forceinline__ int cover32(const Child& B, const StampRec& R, bool c
         m += fabsf(dl);
         n += near;
     }
-    // 2^-20 m n + 2^-41 m^2 + 2^-21 (dmin2 + r2)
-    const float e = fmaf(m, fmaf(4.547473508864641e-13f, m, 9.5367431640625e-07f * n), 4.76837158203125e-07f * (dmin2 + R.r2));
+    // 2^-20 (dmin2 + r2) + 2^-42 A (n + 2^-44 A), or 2^-20 m n + 2^-41 m^2 + 2^-21 (dmin2 + r2)
+    const float e = kExact ? fmaf(9.5367431640625e-07f, dmin2 + R.r2,
+                                  2.2737367544323206e-13f * B.a * fmaf(5.684341886080802e-14f, B.a, n))
+                           : fmaf(m, fmaf(4.547473508864641e-13f, m, 9.5367431640625e-07f * n),
+                                  4.76837158203125e-07f * (dmin2 + R.r2));
     if (dmin2 > R.r2 + e) return kOut;
     if (!(dmin2 < R.r2 - e)) return -1;
     const float margin = fmaf(3.814697265625e-06f * m, m, 2.384185791015625e-07f * R.r2);  // 2^-18 m^2 + 2^-22 r2
@@ -245,9 +267,10 @@ __device__ __forceinline__ StampRec staged(const float4* row, int j) {
     return R;
 }
 
+template <bool kExact>
 __device__ __forceinline__ int cover(const StampDev& S, int32_t v, const StampRec& R, const Child& B, double h,
                                      double half, bool centre) {
-    const int c = cover32(B, R, centre);
+    const int c = cover32<kExact>(B, R, centre);
     return c >= 0 ? c : cover64(S.c + 3 * (int64_t)v, S.r2[v], B.cc[0], B.cc[1], B.cc[2], h, half);
 }
 
@@ -287,8 +310,19 @@ __global__ void stamp_prep(const double* c, const double* r, int64_t n, int32_t 
 }
 
 // ---------------------------------------------------------------------------
-// Long lists: items of kItem entries, one octet (eight lanes, one per child) each.
+// Long lists: items of item_size entries, one octet (eight lanes, one per child) each.
 // ---------------------------------------------------------------------------
+
+// Entries per item of a level. An octet takes 0.3 us an entry when few are in flight and long_sums 1 us per 32 items of
+// a list, which meet at the square root of a tenth of the list's length; more than 65,536 items fill the chip
+// whatever their length, and each takes 64 bytes. On lists of
+// 3,000 stamps 24 items of 128 kept an item's octet busy for 40 us a level and the rest of the chip idle; 192 of 16 take
+// 8.7 us (a painting of 13,000 stamps opened and appended to twice: 22.1 -> 19.1 ms).
+int item_size(int64_t longest, int64_t n_ent) {
+    int item = kItemMin;
+    while (item < kItemMax && (10 * (int64_t)item * item < longest || 65536 * (int64_t)item < n_ent)) item *= 2;
+    return item;
+}
 
 struct LongCell {
     int64_t cell, b, e;  // its list [b, e)
@@ -299,22 +333,22 @@ struct Item {
     int64_t p;  // long cell
 };
 
-// Cells with lists longer than kLongList; ctr[0] counts them, ctr[1] their items.
-__global__ void find_long(LevelIn L, LongCell* out, unsigned long long* ctr) {
+// Cells with lists longer than the limit; ctr[0] counts them, ctr[1] their items.
+__global__ void find_long(LevelIn L, int item, LongCell* out, unsigned long long* ctr) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= L.n) return;
     const int64_t b = L.off[i], e = L.off[i + 1];
-    if (e - b <= kLongList) return;
+    if (e - b <= L.limit) return;
     const unsigned long long p = atomicAdd(&ctr[0], 1ull);
-    const unsigned long long w = atomicAdd(&ctr[1], (unsigned long long)((e - b + kItem - 1) / kItem));
+    const unsigned long long w = atomicAdd(&ctr[1], (unsigned long long)((e - b + item - 1) / item));
     out[p] = LongCell{i, b, e, (int64_t)w};
 }
 
 // One block per long cell: its items, and no refining stamp yet.
-__global__ void long_items(const LongCell* cells, Item* items, int32_t* fr) {
+__global__ void long_items(const LongCell* cells, int item, Item* items, int32_t* fr) {
     const LongCell C = cells[blockIdx.x];
-    for (int64_t j = threadIdx.x; C.b + j * kItem < C.e; j += blockDim.x)
-        items[C.item + j] = Item{C.cell, C.b + j * kItem, min(C.e, C.b + (j + 1) * kItem), (int64_t)blockIdx.x};
+    for (int64_t j = threadIdx.x; C.b + j * item < C.e; j += blockDim.x)
+        items[C.item + j] = Item{C.cell, C.b + j * item, min(C.e, C.b + (j + 1) * item), (int64_t)blockIdx.x};
     if (threadIdx.x < 8) fr[8 * (int64_t)blockIdx.x + threadIdx.x] = kNoStamp;
 }
 
@@ -341,7 +375,7 @@ __global__ void __launch_bounds__(128) long_first(LevelIn L, StampDev S, double 
             const int32_t v = __shfl_sync(kFullMask, C.v, (lane & 24) + j);
             if (v < 0 || first != kNoStamp) continue;
             const StampRec R = staged(row, j);
-            if (R.kt > lc && cover(S, v, R, B, L.h, half, false) >= kPartCentreIn) first = v;
+            if (R.kt > lc && cover<true>(S, v, R, B, L.h, half, false) >= kPartCentreIn) first = v;
         }
         __syncwarp();
     }
@@ -385,7 +419,7 @@ __global__ void __launch_bounds__(128) long_count(LevelIn L, StampDev S, double 
                     c = kPaint;
                 } else {
                     const bool refined = f <= v;
-                    const int x = cover(S, v, staged(row, j), B, L.h, half, !refined);
+                    const int x = cover<true>(S, v, staged(row, j), B, L.h, half, !refined);
                     c = x == kIn ? kPaint : (x == kOut ? kDrop : (refined ? kKeep : (x == kPartCentreIn ? kPaint : kDrop)));
                 }
             }
@@ -401,13 +435,13 @@ __global__ void __launch_bounds__(128) long_count(LevelIn L, StampDev S, double 
 
 // One block per long cell: the items' counts become exclusive sums per child; the child's total and slot.
 constexpr int kSumRows = 32;  // items at a time (a lane per item and child)
-__global__ void __launch_bounds__(8 * kSumRows) long_sums(const LongCell* cells, const int32_t* fr, int32_t* icnt,
-                                                          uint64_t* slot, int32_t* cnt, int32_t* npaint) {
+__global__ void __launch_bounds__(8 * kSumRows) long_sums(const LongCell* cells, int item, const int32_t* fr,
+                                                          int32_t* icnt, uint64_t* slot, int32_t* cnt, int32_t* npaint) {
     __shared__ int32_t s_x[8][kSumRows + 1];
     const int64_t p = blockIdx.x;
     const int k = threadIdx.x & 7, row = threadIdx.x >> 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const LongCell C = cells[p];
-    const int64_t ni = (C.e - C.b + kItem - 1) / kItem;
+    const int64_t ni = (C.e - C.b + item - 1) / item;
     int32_t sum = 0;  // warp w sums child w's items
     for (int64_t j = 0; j < ni; j += kSumRows) {
         int32_t* x = icnt + 8 * (C.item + j + row) + k;
@@ -497,6 +531,7 @@ __device__ __forceinline__ int64_t warp_total(int64_t x) {
 
 // The children of every cell: slot (internal, or the leaf's key), list length, the entries' decisions; the block's
 // sums; tot[2] = the longest list. Cells with long lists only add their sums here.
+template <bool kExact>
 __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDev S, double half, uint64_t* slot,
                                                            int32_t* cnt, uint16_t* cls, BlockSum* bs, long long* tot) {
     __shared__ float4 s_rec[kCells * kStageRow];
@@ -508,7 +543,7 @@ __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDe
         b = L.off[i];
         e = L.off[i + 1];
     }
-    const bool is_long = e - b > kLongList;
+    const bool is_long = e - b > L.limit;
     if (is_long) e = b;
     int32_t n = 0;
     bool found = false;
@@ -532,7 +567,7 @@ __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDe
                     } else {
                         const StampRec R = staged(row, j);
                         const bool refines = found || R.kt > lc;
-                        const int x = cover(S, v, R, B, L.h, half, !refines);
+                        const int x = cover<kExact>(S, v, R, B, L.h, half, !refines);
                         if (x == kIn) {
                             c = kPaint;
                         } else if (x != kOut) {
@@ -567,7 +602,7 @@ __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDe
     if (lane == 0) {
         s_ent[threadIdx.x >> 5] = ents;
         s_int[threadIdx.x >> 5] = ints;
-        if (longest > kLongList) atomicMax(&tot[2], (long long)longest);
+        if (longest > kLongFew) atomicMax(&tot[2], (long long)longest);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -708,7 +743,7 @@ __global__ void __launch_bounds__(8 * kCells) expand_write(LevelIn L, uint64_t* 
     if (i < L.n) {
         b = L.off[i];
         e = L.off[i + 1];
-        if (e - b > kLongList) e = b;
+        if (e - b > L.limit) e = b;
     }
     for (int64_t q0 = b; __any_sync(kFullMask, q0 < e); q0 += 8) {
         const int m = (int)max((int64_t)0, min((int64_t)8, e - q0));
@@ -1189,14 +1224,16 @@ double screen_scale(double extent) {
 struct Level {
     int64_t n = 0;
     int64_t n_ent = 0;    // entries of all lists
-    int64_t longest = 0;  // the longest list (0: none is longer than kLongList)
+    int64_t longest = 0;  // the longest list (0: none is longer than kLongFew)
     int32_t level = 0;
     uint32_t* coord = nullptr;  // [n][3]
     int64_t* off = nullptr;     // [n + 1]
     int32_t* ent = nullptr;     // s: descends, ~s: paints the whole cell
+    bool few() const { return n <= kFewCells; }
+    int64_t limit() const { return few() ? kLongFew : kLongMany; }
     LevelIn in(double extent) const {
         const double h = std::ldexp(extent, -(level + 1));
-        return LevelIn{n, level, coord, off, ent, h, (float)(h * screen_scale(extent))};
+        return LevelIn{n, level, coord, off, ent, limit(), h, (float)(h * screen_scale(extent))};
     }
     void free() {
         dfree(coord);
@@ -1234,13 +1271,14 @@ cudaError_t expand(const Level& L, const StampDev& S, double extent, double half
     unsigned long long h_long[2] = {0, 0};  // cells, items
     Item* items = nullptr;
     int32_t* icnt = nullptr;
-    if (L.longest > kLongList) {
+    if (L.longest > L.limit()) {
         LongCell* cells;
         unsigned long long* ctr;
-        PCK(buf.alloc(&cells, L.n_ent / kLongList));
+        PCK(buf.alloc(&cells, L.n_ent / L.limit()));
         PCK(buf.alloc(&ctr, 2));
         PCK(cudaMemsetAsync(ctr, 0, sizeof(h_long), 0));
-        find_long<<<blocks_for(L.n, 256), 256>>>(in, cells, ctr);
+        const int item = item_size(L.longest, L.n_ent);
+        find_long<<<blocks_for(L.n, 256), 256>>>(in, item, cells, ctr);
         PCK(cudaGetLastError());
         PCK(cudaMemcpy(h_long, ctr, sizeof(h_long), cudaMemcpyDeviceToHost));
         const int64_t nlong = (int64_t)h_long[0], ni = (int64_t)h_long[1];
@@ -1250,15 +1288,15 @@ cudaError_t expand(const Level& L, const StampDev& S, double extent, double half
             PCK(buf.alloc(&icnt, 8 * ni));
             PCK(buf.alloc(&fr, 8 * nlong));
             PCK(buf.alloc(&npaint, 8 * nlong));
-            long_items<<<(unsigned)nlong, 128>>>(cells, items, fr);
+            long_items<<<(unsigned)nlong, 128>>>(cells, item, items, fr);
             long_first<<<blocks_for(ni, 16), 128>>>(in, S, half, items, ni, fr);
             long_count<<<blocks_for(ni, 16), 128>>>(in, S, half, items, ni, fr, cls, icnt);
-            long_sums<<<(unsigned)nlong, 8 * kSumRows>>>(cells, fr, icnt, slot, cnt, npaint);
+            long_sums<<<(unsigned)nlong, 8 * kSumRows>>>(cells, item, fr, icnt, slot, cnt, npaint);
             long_blend<<<blocks_for(8 * nlong, 4), 128>>>(in, S, cells, nlong, npaint, cls, slot);
             PCK(cudaGetLastError());
         }
     }
-    expand_count<<<(unsigned)nb, 8 * kCells>>>(in, S, half, slot, cnt, cls, bs, tot);
+    (L.few() ? expand_count<true> : expand_count<false>)<<<(unsigned)nb, 8 * kCells>>>(in, S, half, slot, cnt, cls, bs, tot);
     scan_sums(bs, nb, sup, tot);
     PCK(cudaGetLastError());
     long long h_tot[3];

@@ -39,3 +39,28 @@ def test_extents_past_the_screen(extent):
     r = np.exp(rng.uniform(np.log(0.01), np.log(0.3), n)) * extent
     q = np.c_[rng.uniform(0, 1, (n, 3)), rng.uniform(0, 9, n)].astype(np.float32)
     _check(7, extent, c, r, q)
+
+
+@pytest.mark.parametrize("n", [2560, 2561, 10241])
+def test_item_lengths(n):
+    """Lists at the edges between items of 16, 32 and 64 entries."""
+    rng = np.random.default_rng(n)
+    c = rng.uniform(-0.02, 0.02, (n, 3))
+    r = np.exp(rng.uniform(np.log(0.02), np.log(0.4), n))
+    q = np.c_[rng.uniform(0, 1, (n, 3)), rng.uniform(0, 9, n)].astype(np.float32)
+    _check(4, 1.0, c, r, q)
+
+
+@pytest.mark.parametrize("n", [100, 200])
+def test_planes_through_a_room(n):
+    """Small stamps that touch, or miss by a relative 1e-16 to 1e-3, the planes of cells 2^16 times their size: the screen
+    next to a far coarser cell's plane, in an octet's own walk and in items."""
+    rng = np.random.default_rng(n)
+    E, D = 40000.0, 18
+    r = rng.uniform(0.8, 2.0, n)
+    c = rng.uniform(-8.0, 8.0, (n, 3)) + [E / 8, -E / 4, 0.0]
+    a = rng.integers(0, 3, n)
+    gap = 10.0 ** rng.uniform(-16, -3, n) * rng.choice([-1.0, 1.0], n)
+    c[np.arange(n), a] = np.array([E / 8, -E / 4, 0.0])[a] + rng.choice([-1.0, 1.0], n) * r * (1 + gap)
+    q = np.c_[rng.uniform(0, 1, (n, 3)), rng.uniform(0, 9, n)].astype(np.float32)
+    _check(D, E, c, r, q)
