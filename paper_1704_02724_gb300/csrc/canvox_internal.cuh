@@ -163,6 +163,7 @@ cudaError_t probe_fp64(double* gflops);
 struct PaintCache;
 void paint_cache_free(PaintCache* c);
 void paint_pool_release();  // after paint_cache_free: the painter's memory pool
+void paint_pool_trim();     // gives back what the pool does not hold live
 cudaError_t paint_pools(int32_t depth, double extent, const double* d_centers, const double* d_radii, const float4* d_rgba,
                         int64_t n, PaintCache** cache, int32_t** d_nodes, uint2** d_leaves, int64_t* n_rec,
                         int64_t* n_leaf, std::vector<int64_t>* level_begin, int64_t* wrap, int32_t* n_wrap);  // wrap: kMaxWraps

@@ -27,9 +27,9 @@
 // knows whether an earlier stamp (or s itself) refines it, so one pass gives its
 // firstref, its blend and which stamps its own list keeps; that decision is left
 // as two bits per stamp and child, from which the next level's lists are written.
-// Lists of more than 512 entries, 128 on levels of few cells (near the root every stamp is on them;
-// around a room, its stamps) are cut into items that octets
-// take in parallel: first the least refining stamp per child, then the decisions.
+// Lists of more than 512 entries, 128 on levels of few cells (near the root every
+// stamp is on them; around a room, its stamps) are cut into items that octets take
+// in parallel: first the least refining stamp per child, then the decisions.
 // Geometry is FP32 with a proven margin, retaken in FP64 with the same operations
 // and order as the host painter inside the margin, so the pools are identical.
 //
@@ -38,9 +38,9 @@
 // records. A lane per child suits the short lists most cells have: with a warp
 // per cell and a lane per stamp (32 stamps at a time, two passes), a list of five
 // left 27 lanes idle and its children were taken one after the other: the depth-24
-// table of 210,000 stamps took 251 ms then and 63 ms now (expand_count 32 ms of it,
+// table of 210,000 stamps took 251 ms then and 49 ms now (expand_count 30 ms of it,
 // its issue slots 52 % used at 26 of 48 possible warps), the 1,000 stamps of the
-// depth-8 cube with the read-back 7.5 and 2.4 ms.
+// depth-8 cube with the read-back 7.5 and 2.1 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -65,6 +65,10 @@ constexpr int64_t kFewCells = 16384;
 constexpr int64_t kLongFew = 128, kLongMany = 512;
 constexpr int kItemMin = 16, kItemMax = 128;  // ... of so many entries (item_size), one octet each
 constexpr int32_t kNoStamp = 0x7FFFFFFF;
+
+// Totals of a level on the device: the next level's entries and cells, its longest list, how many of its lists are
+// longer than kLongFew and than kLongMany and their entries, and find_long's two counters.
+enum { kTotEnt = 0, kTotCells = 1, kTotLongest = 2, kTotLong = 3, kLongCtr = 7, kTotWords = 9 };
 
 // What a child box test reads of a stamp: the centre as two FP32 words per axis, the squared radius (both scaled by the
 // power of two that brings the canvas to a side in [1, 2), so that no FP32 square leaves its range), the target depth.
@@ -333,33 +337,43 @@ struct Item {
     int64_t p;  // long cell
 };
 
-// Cells with lists longer than the limit; ctr[0] counts them, ctr[1] their items.
-__global__ void find_long(LevelIn L, int item, LongCell* out, unsigned long long* ctr) {
+// Cells with lists longer than the limit, their items, and no refining stamp yet; tot[kLongCtr] counts the cells, the
+// next word their items.
+__global__ void __launch_bounds__(256) find_long(LevelIn L, int item, LongCell* cells, Item* items, int32_t* fr,
+                                                 long long* tot) {
+    __shared__ LongCell s_cell[256];
+    __shared__ int64_t s_p[256];
+    __shared__ int s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L.n) return;
-    const int64_t b = L.off[i], e = L.off[i + 1];
-    if (e - b <= L.limit) return;
-    const unsigned long long p = atomicAdd(&ctr[0], 1ull);
-    const unsigned long long w = atomicAdd(&ctr[1], (unsigned long long)((e - b + item - 1) / item));
-    out[p] = LongCell{i, b, e, (int64_t)w};
-}
-
-// One block per long cell: its items, and no refining stamp yet.
-__global__ void long_items(const LongCell* cells, int item, Item* items, int32_t* fr) {
-    const LongCell C = cells[blockIdx.x];
-    for (int64_t j = threadIdx.x; C.b + j * item < C.e; j += blockDim.x)
-        items[C.item + j] = Item{C.cell, C.b + j * item, min(C.e, C.b + (j + 1) * item), (int64_t)blockIdx.x};
-    if (threadIdx.x < 8) fr[8 * (int64_t)blockIdx.x + threadIdx.x] = kNoStamp;
+    const int64_t b = i < L.n ? L.off[i] : 0, e = i < L.n ? L.off[i + 1] : 0;
+    if (e - b > L.limit) {
+        unsigned long long* ctr = reinterpret_cast<unsigned long long*>(tot + kLongCtr);
+        const int64_t p = (int64_t)atomicAdd(&ctr[0], 1ull);
+        const LongCell C{i, b, e, (int64_t)atomicAdd(&ctr[1], (unsigned long long)((e - b + item - 1) / item))};
+        const int j = atomicAdd(&s_n, 1);
+        cells[p] = s_cell[j] = C;
+        s_p[j] = p;
+    }
+    __syncthreads();
+    for (int j = 0; j < s_n; ++j) {
+        const LongCell C = s_cell[j];
+        const int64_t p = s_p[j];
+        for (int64_t q = threadIdx.x; C.b + q * item < C.e; q += blockDim.x)
+            items[C.item + q] = Item{C.cell, C.b + q * item, min(C.e, C.b + (q + 1) * item), p};
+        if (threadIdx.x < 8) fr[8 * p + threadIdx.x] = kNoStamp;
+    }
 }
 
 // The least stamp of each item that refines each child (entries are in stamp order, so the first that does).
 __global__ void __launch_bounds__(128) long_first(LevelIn L, StampDev S, double half, const Item* items,
-                                                  int64_t n_items, int32_t* fr) {
+                                                  const long long* tot, int32_t* fr) {
     __shared__ float4 s_rec[16 * kStageRow];
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
     const int lane = threadIdx.x & 31, k = threadIdx.x & 7, lc = L.level + 1;
     float4* row = s_rec + (threadIdx.x >> 3) * kStageRow;
-    const bool mine = w < n_items;
+    const bool mine = w < tot[kLongCtr + 1];
     const Item I = mine ? items[w] : Item{0, 0, 0, 0};
     const Child B = child_box(L, I.cell, k);
     int32_t first = kNoStamp;
@@ -391,12 +405,13 @@ __device__ __forceinline__ unsigned decision_bits(int c) {
 
 // Per item: the entries' decisions, and per child how many a refined child keeps or paint one that stays a leaf.
 __global__ void __launch_bounds__(128) long_count(LevelIn L, StampDev S, double half, const Item* items,
-                                                  int64_t n_items, const int32_t* fr, uint16_t* cls, int32_t* icnt) {
+                                                  const long long* tot, const int32_t* fr, uint16_t* cls,
+                                                  int32_t* icnt) {
     __shared__ float4 s_rec[16 * kStageRow];
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
     const int lane = threadIdx.x & 31, k = threadIdx.x & 7;
     float4* row = s_rec + (threadIdx.x >> 3) * kStageRow;
-    const bool mine = w < n_items;
+    const bool mine = w < tot[kLongCtr + 1];
     const Item I = mine ? items[w] : Item{0, 0, 0, 0};
     const Child B = child_box(L, I.cell, k);
     const int32_t f = mine ? fr[8 * I.p + k] : kNoStamp;
@@ -433,13 +448,16 @@ __global__ void __launch_bounds__(128) long_count(LevelIn L, StampDev S, double 
     if (mine) icnt[8 * w + k] = n;
 }
 
-// One block per long cell: the items' counts become exclusive sums per child; the child's total and slot.
+// One block per long cell: the items' counts become exclusive sums per child; the child's total and slot, and (a warp per
+// child) for a painted child that stays a leaf the blend, in order, of the stamps that paint it.
 constexpr int kSumRows = 32;  // items at a time (a lane per item and child)
-__global__ void __launch_bounds__(8 * kSumRows) long_sums(const LongCell* cells, int item, const int32_t* fr,
-                                                          int32_t* icnt, uint64_t* slot, int32_t* cnt, int32_t* npaint) {
+__global__ void __launch_bounds__(8 * kSumRows) long_sums(LevelIn L, StampDev S, const LongCell* cells, int item,
+                                                          const long long* tot, const int32_t* fr, const uint16_t* cls,
+                                                          int32_t* icnt, uint64_t* slot, int32_t* cnt) {
     __shared__ int32_t s_x[8][kSumRows + 1];
     const int64_t p = blockIdx.x;
     const int k = threadIdx.x & 7, row = threadIdx.x >> 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (p >= tot[kLongCtr]) return;
     const LongCell C = cells[p];
     const int64_t ni = (C.e - C.b + item - 1) / item;
     int32_t sum = 0;  // warp w sums child w's items
@@ -460,45 +478,39 @@ __global__ void __launch_bounds__(8 * kSumRows) long_sums(const LongCell* cells,
         if (j + row < ni) *x = s_x[k][row];
         __syncthreads();
     }
-    if (lane == 0) {
-        const int64_t t = 8 * C.cell + warp;
-        const bool internal = fr[8 * p + warp] != kNoStamp;
-        slot[t] = internal ? kInternal : 0ull;
-        cnt[t] = internal ? sum : 0;
-        npaint[8 * p + warp] = internal ? 0 : sum;
+    const int64_t t = 8 * C.cell + warp;
+    if (fr[8 * p + warp] != kNoStamp) {
+        if (lane == 0) {
+            slot[t] = kInternal;
+            cnt[t] = sum;
+        }
+        return;
     }
-}
-
-// One warp per child of a long cell that stays a leaf and is painted: the blend, in order, of the stamps that do.
-__global__ void __launch_bounds__(128) long_blend(LevelIn L, StampDev S, const LongCell* cells, int64_t n_long,
-                                                  const int32_t* npaint, const uint16_t* cls, uint64_t* slot) {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= 8 * n_long || npaint[w] == 0) return;  // warp-uniform
-    const LongCell C = cells[w >> 3];
-    const int k = (int)(w & 7);
     float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t base = C.b; base < C.e; base += 32) {
+    for (int64_t base = C.b; sum != 0 && base < C.e; base += 32) {
         const int64_t q = base + lane;
-        const bool p = q < C.e && ((cls[q] >> (8 + k)) & 1u);
-        const int32_t v = p ? L.ent[q] : 0;
-        unsigned m = __ballot_sync(kFullMask, p);
+        const bool paints = q < C.e && ((cls[q] >> (8 + warp)) & 1u);
+        const int32_t v = paints ? L.ent[q] : 0;
+        unsigned m = __ballot_sync(kFullMask, paints);
         while (m) {  // every lane folds the same sequence
             const int32_t x = __shfl_sync(kFullMask, v, __ffs(m) - 1);
             m &= m - 1;
             blend(val, S.rgba[x < 0 ? ~x : x]);
         }
     }
-    if (lane == 0) slot[8 * C.cell + k] = leaf_key(val);
+    if (lane == 0) {
+        slot[t] = leaf_key(val);
+        cnt[t] = 0;
+    }
 }
 
 // One octet per item: its kept entries at the child's list start plus the counts of the cell's earlier items.
-__global__ void __launch_bounds__(128) long_write(LevelIn L, const Item* items, int64_t n_items, const uint64_t* slot,
+__global__ void __launch_bounds__(128) long_write(LevelIn L, const Item* items, const long long* tot, const uint64_t* slot,
                                                   const uint16_t* cls, const int32_t* icnt, const int64_t* noff,
                                                   int32_t* nent) {
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
     const int k = threadIdx.x & 7;
-    if (w >= n_items) return;
+    if (w >= tot[kLongCtr + 1]) return;
     const Item I = items[w];
     const uint64_t s = slot[8 * I.cell + k];
     if (!(s & kInternal)) return;
@@ -530,7 +542,7 @@ __device__ __forceinline__ int64_t warp_total(int64_t x) {
 }
 
 // The children of every cell: slot (internal, or the leaf's key), list length, the entries' decisions; the block's
-// sums; tot[2] = the longest list. Cells with long lists only add their sums here.
+// sums; in tot the longest list and the long ones. Cells with long lists only add their sums here.
 template <bool kExact>
 __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDev S, double half, uint64_t* slot,
                                                            int32_t* cnt, uint16_t* cls, BlockSum* bs, long long* tot) {
@@ -596,13 +608,17 @@ __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDe
             cnt[t] = n;
         }
     }
+    if (n > kLongFew) {
+        unsigned long long* lists = reinterpret_cast<unsigned long long*>(tot + kTotLong);
+        for (int x = 0; x < (n > kLongMany ? 4 : 2); ++x) atomicAdd(&lists[x], (x & 1) ? (unsigned long long)n : 1ull);
+    }
     const int32_t longest = __reduce_max_sync(kFullMask, n);
     const int64_t ents = warp_total(n);
     const int ints = __popc(__ballot_sync(kFullMask, found));
     if (lane == 0) {
         s_ent[threadIdx.x >> 5] = ents;
         s_int[threadIdx.x >> 5] = ints;
-        if (longest > kLongFew) atomicMax(&tot[2], (long long)longest);
+        if (longest > kLongFew) atomicMax(&tot[kTotLongest], (long long)longest);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -676,8 +692,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_groups(BlockSum* bs, int64_
     if (threadIdx.x == 0) {
         sup[blockIdx.x] = gridDim.x == 1 ? BlockSum{0, 0} : total;
         if (gridDim.x == 1) {
-            tot[0] = total.ent;
-            tot[1] = total.cells;
+            tot[kTotEnt] = total.ent;
+            tot[kTotCells] = total.cells;
         }
     }
 }
@@ -695,16 +711,16 @@ __global__ void __launch_bounds__(kScanThreads) scan_sup(BlockSum* sup, int64_t 
         carry.cells += total.cells;
     }
     if (threadIdx.x == 0) {
-        tot[0] = carry.ent;
-        tot[1] = carry.cells;
+        tot[kTotEnt] = carry.ent;
+        tot[kTotCells] = carry.cells;
     }
 }
 
 // The next level: each refined child's index (into its slot), coordinates, list start and list, and with pid the
 // partition it belongs to. The lists of long cells are left to long_write.
 __global__ void __launch_bounds__(8 * kCells) expand_write(LevelIn L, uint64_t* slot, const int32_t* cnt, const uint16_t* cls,
-                                                           const BlockSum* bs, const BlockSum* sup, const int32_t* pid,
-                                                           uint32_t* ncoord, int64_t* noff, int32_t* nent, int32_t* npid) {
+                                                           const BlockSum* bs, const BlockSum* sup, const long long* tot,
+                                                           const int32_t* pid, uint32_t* ncoord, int64_t* noff, int32_t* nent, int32_t* npid) {
     __shared__ int64_t s_ent[kCells / 4];
     __shared__ int s_int[kCells / 4];
     const int64_t i = (int64_t)blockIdx.x * kCells + (threadIdx.x >> 3);
@@ -731,6 +747,7 @@ __global__ void __launch_bounds__(8 * kCells) expand_write(LevelIn L, uint64_t* 
         w += s_ent[q];
         j += s_int[q];
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) noff[tot[kTotCells]] = tot[kTotEnt];
     if (internal) {
         slot[t] = kInternal | (uint64_t)j;
         ncoord[3 * j] = 2u * L.coord[3 * i] + (k & 1u);
@@ -882,13 +899,15 @@ __global__ void scan_add(int64_t* d, int64_t n, const int64_t* sums) {
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// Device memory of the painter: a memory pool of its own. A paint makes about ten arrays per level; from the device
-// allocator each costs 30-50 us and a free 30 us (0.3 and 0.5 ms a GB), from the pool 1.5 us. Everything runs on the
-// legacy default stream, which orders frees and reuse. After a paint the pool gives back all but kPoolKeep bytes of
-// what it does not hold live, and canvox_release destroys it.
+// Device memory of the painter: a memory pool of its own. From the device allocator an array costs 30-50 us and a free
+// 30 us (0.3 and 0.5 ms a GB), from the pool 1.5 us each, so what a level needs only while it is painted is one
+// allocation. Everything runs on the legacy default stream, which orders frees and reuse. After a paint the pool gives
+// back all but kPoolKeep bytes (a 16th of the device's free memory, if that is less) of what it does not hold live, an
+// allocation of the library that finds no memory gets the rest (paint_pool_trim), and canvox_release destroys it. The depth-24 table of 210,000 stamps, whose arrays take 7 GB at once, took 57.4 ms with
+// 4 GiB kept and 48.6 ms with 8.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr size_t kPoolKeep = (size_t)4 << 30;
+constexpr size_t kPoolKeep = (size_t)8 << 30;
 cudaMemPool_t g_pool = nullptr;
 
 cudaError_t pool_ready() {
@@ -939,6 +958,8 @@ void dfree(void* p) {
 }
 }  // namespace
 
+void paint_pool_trim() { pool_trim(0); }
+
 void paint_pool_release() {
     if (!g_pool) return;
     cudaDeviceSynchronize();
@@ -987,6 +1008,22 @@ struct DevBuf {
         const cudaError_t e = dalloc(p, n);
         if (e == cudaSuccess) ptrs.push_back(*p);
         return e;
+    }
+};
+
+// Arrays in one allocation: sizes first, then alloc(), then the same calls of take().
+struct Arena {
+    size_t bytes = 0;
+    unsigned char* base = nullptr;
+    template <typename T>
+    void size(int64_t n) {
+        bytes += (sizeof(T) * (size_t)n + 255) / 256 * 256;
+    }
+    template <typename T>
+    T* take(int64_t n) {
+        T* p = reinterpret_cast<T*>(base);
+        base += (sizeof(T) * (size_t)n + 255) / 256 * 256;
+        return p;
     }
 };
 
@@ -1082,14 +1119,31 @@ __global__ void list_lengths(int64_t m, const int32_t* sel, const int64_t* off, 
     if (r < m) len[r] = off[sel[r] + 1] - off[sel[r]];
 }
 
-// Per new partition p, its cell count at one level: from the kept subtree (reuse[p] = q) or the repainted one
-// (rep[p] = r).
-__global__ void part_counts(int64_t n, const int32_t* reuse, const int32_t* rep, const int64_t* off_old,
-                            const int64_t* off_rep, int64_t* cnt) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int32_t q = reuse[p];
-    cnt[p] = q >= 0 ? (off_old ? off_old[q + 1] - off_old[q] : 0) : (off_rep ? off_rep[rep[p] + 1] - off_rep[rep[p]] : 0);
+// Per level (a block each) and new partition p, the first cell of p: the exclusive sums of the cell counts, from the
+// kept subtree (reuse[p] = q) or the repainted one (rep[p] = r); dst[n] = total[level] = the level's cells.
+struct PartLevels {
+    const int64_t *old[kMaxDepth], *rep[kMaxDepth];  // first cells per old and repainted partition (null: no such level)
+    int64_t* dst[kMaxDepth];
+};
+__global__ void __launch_bounds__(kScanThreads) part_offsets(int64_t n, const int32_t* reuse, const int32_t* rep,
+                                                             const __grid_constant__ PartLevels levels, int64_t* total) {
+    const int64_t *off_old = levels.old[blockIdx.x], *off_rep = levels.rep[blockIdx.x];
+    int64_t* dst = levels.dst[blockIdx.x];
+    int64_t carry = 0;
+    for (int64_t base = 0; base < n; base += kScanThreads) {
+        const int64_t p = base + threadIdx.x;
+        int64_t c = 0;
+        if (p < n) {
+            const int32_t q = reuse[p];
+            if (q >= 0) c = off_old ? off_old[q + 1] - off_old[q] : 0;
+            else if (off_rep) c = off_rep[rep[p] + 1] - off_rep[rep[p]];
+        }
+        BlockSum sum;
+        const BlockSum pre = block_scan(BlockSum{c, 0}, &sum);
+        if (p < n) dst[p] = carry + pre.ent;
+        carry += sum.ent;
+    }
+    if (threadIdx.x == 0) dst[n] = total[blockIdx.x] = carry;
 }
 
 // The assembled level: each cell's eight slots copied from its source, internal children renumbered to the
@@ -1143,20 +1197,28 @@ cudaError_t finish_pools(const std::vector<uint64_t*>& slots, const std::vector<
     const size_t nl = slots.size();
     std::vector<uint64_t*> ckey(nl + 1, nullptr);
     std::vector<Ranks> ranks(nl + 1);
-    uint64_t* none;  // below the deepest level: no refined cells
-    PCK(buf.alloc(&none, 2));
-    ckey[nl] = none;
+    const auto blocks = [](int64_t nc) { return (nc + kMergeCells - 1) / kMergeCells; };
+    const auto groups = [&](int64_t nc) { return (blocks(nc) + kScanItems - 1) / kScanItems; };
+    Arena A;
+    for (int64_t nc : ncell) {
+        A.size<uint64_t>(nc);
+        A.size<uint32_t>(nc);
+        A.size<BlockSum>(blocks(nc));
+        A.size<BlockSum>(groups(nc));
+    }
+    A.size<uint64_t>(2);
+    A.size<long long>(2 * (int64_t)nl + 2);
+    A.size<int64_t>(kMaxWraps);
+    PCK(buf.alloc(&A.base, (int64_t)A.bytes));
+    ckey[nl] = A.take<uint64_t>(2);  // below the deepest level: no refined cells
     ranks[nl] = Ranks{nullptr, nullptr, nullptr};
-    long long* d_tot;
-    PCK(buf.alloc(&d_tot, 2 * (int64_t)nl + 2));
+    long long* d_tot = A.take<long long>(2 * (int64_t)nl + 2);
+    int64_t* d_wraps = A.take<int64_t>(kMaxWraps);
     for (size_t l = nl; l-- > 0;) {
-        const int64_t nc = ncell[l], nb = (nc + kMergeCells - 1) / kMergeCells, ng = (nb + kScanItems - 1) / kScanItems;
-        uint32_t* place;
-        BlockSum *bs, *sup;
-        PCK(buf.alloc(&ckey[l], nc));
-        PCK(buf.alloc(&place, nc));
-        PCK(buf.alloc(&bs, nb));
-        PCK(buf.alloc(&sup, ng));
+        const int64_t nc = ncell[l], nb = blocks(nc), ng = groups(nc);
+        ckey[l] = A.take<uint64_t>(nc);
+        uint32_t* place = A.take<uint32_t>(nc);
+        BlockSum *bs = A.take<BlockSum>(nb), *sup = A.take<BlockSum>(ng);
         collapse_level<<<(unsigned)nb, 8 * kMergeCells>>>(nc, slots[l], ckey[l + 1], ckey[l], l == 0, place, bs);
         scan_sums(bs, nb, sup, d_tot + 2 * l);
         PCK(cudaGetLastError());
@@ -1173,8 +1235,6 @@ cudaError_t finish_pools(const std::vector<uint64_t*>& slots, const std::vector<
     const int64_t n_rec = rec_base[nl], n_leaf = leaf_base[nl];
     if (n_rec > 0x7FFFFFFFll || n_leaf > kMaxLeaves) return cudaErrorMemoryAllocation;  // beyond the pool format
     const int32_t n_wrap = n_leaf > 0 ? (int32_t)((n_leaf - 1) >> 31) : 0;
-    int64_t* d_wraps;
-    PCK(buf.alloc(&d_wraps, kMaxWraps));
     int32_t* d_nodes = nullptr;
     uint2* d_leaves = nullptr;
     PCK(with_retry([&] { return cudaMalloc(&d_nodes, sizeof(int32_t) * 8 * (size_t)n_rec); }));
@@ -1225,6 +1285,7 @@ struct Level {
     int64_t n = 0;
     int64_t n_ent = 0;    // entries of all lists
     int64_t longest = 0;  // the longest list (0: none is longer than kLongFew)
+    int64_t long_cells[2] = {0, 0}, long_ent[2] = {0, 0};  // at most: lists longer than kLongFew, kLongMany; their entries
     int32_t level = 0;
     uint32_t* coord = nullptr;  // [n][3]
     int64_t* off = nullptr;     // [n + 1]
@@ -1253,69 +1314,61 @@ cudaError_t expand(const Level& L, const StampDev& S, double extent, double half
                    const int32_t* pid, int32_t** npid) {
     DevBuf buf;
     const int64_t nch = 8 * L.n, nb = (L.n + kCells - 1) / kCells, ng = (nb + kScanItems - 1) / kScanItems;
-    int32_t* cnt;
-    uint16_t* cls;
-    BlockSum *bs, *sup;
-    long long* tot;
+    // cells with long lists: an octet per item of a list
+    const bool longs = L.longest > L.limit();
+    const int item = item_size(L.longest, L.n_ent), few = L.few() ? 0 : 1;
+    const int64_t nlong = longs ? L.long_cells[few] : 0, ni = longs ? L.long_ent[few] / item + nlong : 0;
+    Arena A;
+    A.size<int32_t>(nch);
+    A.size<uint16_t>(L.n_ent);
+    A.size<BlockSum>(nb);
+    A.size<BlockSum>(ng);
+    A.size<long long>(kTotWords);
+    A.size<LongCell>(nlong);
+    A.size<Item>(ni);
+    A.size<int32_t>(8 * ni);
+    A.size<int32_t>(8 * nlong);
+    PCK(buf.alloc(&A.base, (int64_t)A.bytes));
+    int32_t* cnt = A.take<int32_t>(nch);
+    uint16_t* cls = A.take<uint16_t>(L.n_ent);
+    BlockSum *bs = A.take<BlockSum>(nb), *sup = A.take<BlockSum>(ng);
+    long long* tot = A.take<long long>(kTotWords);
+    LongCell* cells = A.take<LongCell>(nlong);
+    Item* items = A.take<Item>(ni);
+    int32_t *icnt = A.take<int32_t>(8 * ni), *fr = A.take<int32_t>(8 * nlong);
     uint64_t* slot;
-    PCK(buf.alloc(&cnt, nch));
-    PCK(buf.alloc(&cls, L.n_ent));
-    PCK(buf.alloc(&bs, nb));
-    PCK(buf.alloc(&sup, ng));
-    PCK(buf.alloc(&tot, 3));
     PCK(dalloc(&slot, nch));
     *slot_out = slot;
     const LevelIn in = L.in(extent);
-    PCK(cudaMemsetAsync(tot, 0, 3 * sizeof(long long), 0));
-    // cells with long lists: an octet per item of a list
-    unsigned long long h_long[2] = {0, 0};  // cells, items
-    Item* items = nullptr;
-    int32_t* icnt = nullptr;
-    if (L.longest > L.limit()) {
-        LongCell* cells;
-        unsigned long long* ctr;
-        PCK(buf.alloc(&cells, L.n_ent / L.limit()));
-        PCK(buf.alloc(&ctr, 2));
-        PCK(cudaMemsetAsync(ctr, 0, sizeof(h_long), 0));
-        const int item = item_size(L.longest, L.n_ent);
-        find_long<<<blocks_for(L.n, 256), 256>>>(in, item, cells, ctr);
+    PCK(cudaMemsetAsync(tot, 0, kTotWords * sizeof(long long), 0));
+    if (longs) {
+        find_long<<<blocks_for(L.n, 256), 256>>>(in, item, cells, items, fr, tot);
+        long_first<<<blocks_for(ni, 16), 128>>>(in, S, half, items, tot, fr);
+        long_count<<<blocks_for(ni, 16), 128>>>(in, S, half, items, tot, fr, cls, icnt);
+        long_sums<<<(unsigned)nlong, 8 * kSumRows>>>(in, S, cells, item, tot, fr, cls, icnt, slot, cnt);
         PCK(cudaGetLastError());
-        PCK(cudaMemcpy(h_long, ctr, sizeof(h_long), cudaMemcpyDeviceToHost));
-        const int64_t nlong = (int64_t)h_long[0], ni = (int64_t)h_long[1];
-        if (nlong) {
-            int32_t *fr, *npaint;
-            PCK(buf.alloc(&items, ni));
-            PCK(buf.alloc(&icnt, 8 * ni));
-            PCK(buf.alloc(&fr, 8 * nlong));
-            PCK(buf.alloc(&npaint, 8 * nlong));
-            long_items<<<(unsigned)nlong, 128>>>(cells, item, items, fr);
-            long_first<<<blocks_for(ni, 16), 128>>>(in, S, half, items, ni, fr);
-            long_count<<<blocks_for(ni, 16), 128>>>(in, S, half, items, ni, fr, cls, icnt);
-            long_sums<<<(unsigned)nlong, 8 * kSumRows>>>(cells, item, fr, icnt, slot, cnt, npaint);
-            long_blend<<<blocks_for(8 * nlong, 4), 128>>>(in, S, cells, nlong, npaint, cls, slot);
-            PCK(cudaGetLastError());
-        }
     }
     (L.few() ? expand_count<true> : expand_count<false>)<<<(unsigned)nb, 8 * kCells>>>(in, S, half, slot, cnt, cls, bs, tot);
     scan_sums(bs, nb, sup, tot);
     PCK(cudaGetLastError());
-    long long h_tot[3];
+    long long h_tot[kTotWords];
     PCK(cudaMemcpy(h_tot, tot, sizeof(h_tot), cudaMemcpyDeviceToHost));
-    next->n = h_tot[1];
-    next->n_ent = h_tot[0];
-    next->longest = h_tot[2];
+    next->n = h_tot[kTotCells];
+    next->n_ent = h_tot[kTotEnt];
+    next->longest = h_tot[kTotLongest];
+    for (int x = 0; x < 2; ++x) {
+        next->long_cells[x] = h_tot[kTotLong + 2 * x];
+        next->long_ent[x] = h_tot[kTotLong + 2 * x + 1];
+    }
     next->level = L.level + 1;
     if (next->n == 0) return cudaSuccess;  // no internal child: the slots are all leaf keys
     PCK(dalloc(&next->coord, 3 * next->n));
     PCK(dalloc(&next->off, next->n + 1));
     PCK(dalloc(&next->ent, next->n_ent));
     if (pid) PCK(dalloc(npid, next->n));
-    PCK(cudaMemcpyAsync(next->off + next->n, tot, sizeof(int64_t), cudaMemcpyDeviceToDevice, 0));
-    expand_write<<<(unsigned)nb, 8 * kCells>>>(in, slot, cnt, cls, bs, sup, pid, next->coord, next->off, next->ent,
+    expand_write<<<(unsigned)nb, 8 * kCells>>>(in, slot, cnt, cls, bs, sup, tot, pid, next->coord, next->off, next->ent,
                                                pid ? *npid : nullptr);
-    if (items)
-        long_write<<<blocks_for((int64_t)h_long[1], 16), 128>>>(in, items, (int64_t)h_long[1], slot, cls, icnt, next->off,
-                                                                next->ent);
+    if (longs) long_write<<<blocks_for(ni, 16), 128>>>(in, items, tot, slot, cls, icnt, next->off, next->ent);
     return cudaGetLastError();
 }
 
@@ -1421,6 +1474,10 @@ cudaError_t root_level(const StampDev& S, int64_t n, double extent, double half,
     }
     root->n = 1;
     root->n_ent = root->longest = n_root;
+    for (int x = 0; x < 2; ++x) {
+        root->long_cells[x] = 1;
+        root->long_ent[x] = n_root;
+    }
     root->level = 0;
     PCK(dalloc(&root->coord, 3));
     PCK(dalloc(&root->off, 2));
@@ -1441,27 +1498,26 @@ cudaError_t assemble(int64_t n_part, const int32_t* reuse, const int32_t* rep, c
                      const std::vector<uint64_t*>& slots_r, const std::vector<int64_t*>& offs_r,
                      std::vector<uint64_t*>* slots, std::vector<int64_t>* ncell, std::vector<int64_t*>* offs) {
     DevBuf buf;
-    int64_t* cnt;
-    PCK(buf.alloc(&cnt, n_part));
     const size_t depth_max = std::max(old.slots.size(), slots_r.size());
+    if (n_part == 0 || depth_max == 0) return cudaDeviceSynchronize();
+    int64_t* d_total;
+    PCK(buf.alloc(&d_total, (int64_t)depth_max));
+    PartLevels levels = {};
     for (size_t d = 0; d < depth_max; ++d) {
-        part_counts<<<blocks_for(n_part, 256), 256>>>(n_part, reuse, rep, d < old.off.size() ? old.off[d] : nullptr,
-                                                      d < offs_r.size() ? offs_r[d] : nullptr, cnt);
-        PCK(cudaGetLastError());
         int64_t* off;
         PCK(dalloc(&off, n_part + 1));
         offs->push_back(off);
-        PCK(cudaMemcpy(off, cnt, sizeof(int64_t) * (size_t)n_part, cudaMemcpyDeviceToDevice));
-        int64_t total = 0;
-        PCK(scan_i64(off, n_part, &total));
-        PCK(cudaMemcpy(off + n_part, &total, sizeof(int64_t), cudaMemcpyHostToDevice));
-        if (total == 0) {
-            dfree(off);
-            offs->pop_back();
-            break;
-        }
-        ncell->push_back(total);
+        levels.old[d] = d < old.off.size() ? old.off[d] : nullptr;
+        levels.rep[d] = d < offs_r.size() ? offs_r[d] : nullptr;
+        levels.dst[d] = off;
     }
+    part_offsets<<<(unsigned)depth_max, kScanThreads>>>(n_part, reuse, rep, levels, d_total);
+    PCK(cudaGetLastError());
+    std::vector<int64_t> total(depth_max);
+    PCK(cudaMemcpy(total.data(), d_total, sizeof(int64_t) * depth_max, cudaMemcpyDeviceToHost));
+    for (size_t d = 0; d < depth_max && total[d] > 0; ++d) ncell->push_back(total[d]);
+    for (size_t d = ncell->size(); d < depth_max; ++d) dfree((*offs)[d]);
+    offs->resize(ncell->size());
     for (size_t d = 0; d < ncell->size(); ++d) {
         uint64_t* slot;
         PCK(dalloc(&slot, 8 * (*ncell)[d]));
@@ -1579,6 +1635,10 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
             e = scan_i64(len, m, &n_ent);
             rep_lvl.n_ent = n_ent;
             rep_lvl.longest = partP.longest;
+            for (int x = 0; x < 2; ++x) {
+                rep_lvl.long_cells[x] = partP.long_cells[x];
+                rep_lvl.long_ent[x] = partP.long_ent[x];
+            }
             if (e == cudaSuccess) e = cudaMemcpy(len + m, &n_ent, sizeof(int64_t), cudaMemcpyHostToDevice);
             if (e == cudaSuccess) e = dalloc(&rep_lvl.coord, 3 * m);
             if (e == cudaSuccess) e = dalloc(&rep_lvl.off, m + 1);
@@ -1614,7 +1674,9 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     }
     free_all(slots_top);
     partP.free();
-    pool_trim(kPoolKeep);
+    size_t spare = 0, total = 0;
+    if (cudaMemGetInfo(&spare, &total) != cudaSuccess) spare = 0;
+    pool_trim(std::min(kPoolKeep, spare / 16));
     if (e == cudaSuccess) {
         nc->slots = slots_bot;
         nc->ncell = ncell_bot;

@@ -131,6 +131,18 @@ void builtin_defaults(canvox_render_opts* o) {
     o->count_reads = 1;
 }
 
+// cudaMalloc; where there is no memory left, once more with what the painter's pool keeps for the next paint.
+template <typename T>
+cudaError_t device_malloc(T** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        paint_pool_trim();
+        e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    }
+    return e;
+}
+
 int ensure_device() {
     int dev;
     CK(cudaGetDevice(&dev), "cudaGetDevice");
@@ -425,9 +437,9 @@ int reserve_stamps(int64_t n, int64_t keep) {
     while (cap < n) cap *= 2;
     double *c = nullptr, *r = nullptr;
     float4* q = nullptr;
-    cudaError_t e = cudaMalloc(&c, sizeof(double) * 3 * (size_t)cap);
-    if (e == cudaSuccess) e = cudaMalloc(&r, sizeof(double) * (size_t)cap);
-    if (e == cudaSuccess) e = cudaMalloc(&q, sizeof(float4) * (size_t)cap);
+    cudaError_t e = device_malloc(&c, sizeof(double) * 3 * (size_t)cap);
+    if (e == cudaSuccess) e = device_malloc(&r, sizeof(double) * (size_t)cap);
+    if (e == cudaSuccess) e = device_malloc(&q, sizeof(float4) * (size_t)cap);
     if (e == cudaSuccess && keep > 0) e = cudaMemcpy(c, g.d_st_c, sizeof(double) * 3 * (size_t)keep, cudaMemcpyDeviceToDevice);
     if (e == cudaSuccess && keep > 0) e = cudaMemcpy(r, g.d_st_r, sizeof(double) * (size_t)keep, cudaMemcpyDeviceToDevice);
     if (e == cudaSuccess && keep > 0) e = cudaMemcpy(q, g.d_st_rgba, sizeof(float4) * (size_t)keep, cudaMemcpyDeviceToDevice);
@@ -678,7 +690,7 @@ int check_nodes(HostTeam& team, const int32_t* node_pool, int64_t n_records, int
 
 // Neighbour links of the current pools, one launch per level (parents first).
 int build_links() {
-    CK(cudaMalloc(&g.d_ropes, sizeof(uint2) * 6 * (size_t)g.n_rec), "cudaMalloc(ropes)");
+    CK(device_malloc(&g.d_ropes, sizeof(uint2) * 6 * (size_t)g.n_rec), "cudaMalloc(ropes)");
     for (size_t l = 0; l + 1 < g.level_begin.size(); ++l)
         CK(launch_rope_level(g.d_nodes, g.d_ropes, g.level_begin[l], g.level_begin[l + 1], (int)l, 0), "rope kernel launch");
     CK(cudaDeviceSynchronize(), "rope build");
@@ -753,8 +765,8 @@ int upload(const int32_t* node_pool, int64_t n_records, const uint16_t* leaf_rgb
     if ((rc = drop_canvas())) return rc;
     paint_cache_free(g.paint_cache);  // an uploaded canvas cannot be appended to
     g.paint_cache = nullptr;
-    CK(cudaMalloc(&g.d_nodes, sizeof(int32_t) * 8 * (size_t)n_records), "cudaMalloc(nodes)");
-    CK(cudaMalloc(&g.d_leaves, sizeof(uint2) * (size_t)(n_leaves > 0 ? n_leaves : 1)), "cudaMalloc(leaves)");
+    CK(device_malloc(&g.d_nodes, sizeof(int32_t) * 8 * (size_t)n_records), "cudaMalloc(nodes)");
+    CK(device_malloc(&g.d_leaves, sizeof(uint2) * (size_t)(n_leaves > 0 ? n_leaves : 1)), "cudaMalloc(leaves)");
     CK(cudaMemcpy(g.d_nodes, node_pool, sizeof(int32_t) * 8 * (size_t)n_records, cudaMemcpyHostToDevice), "cudaMemcpy(nodes)");
     if (n_leaves > 0)
         CK(cudaMemcpy(g.d_leaves, leaf_rgba, sizeof(uint2) * (size_t)n_leaves, cudaMemcpyHostToDevice), "cudaMemcpy(leaves)");
@@ -1061,7 +1073,7 @@ int canvox_render_host(const canvox_camera* cams, int32_t n_views, float* out_rg
         if (g.d_host_out) cudaFree(g.d_host_out);
         g.d_host_out = nullptr;
         g.host_out_cap = 0;
-        CK(cudaMalloc(&g.d_host_out, sizeof(float4) * (size_t)npx), "cudaMalloc(host render target)");
+        CK(device_malloc(&g.d_host_out, sizeof(float4) * (size_t)npx), "cudaMalloc(host render target)");
         g.host_out_cap = npx;
     }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -1087,7 +1099,7 @@ int canvox_autotune(const canvox_camera* cams, int32_t n_views, void* stream, ca
         if (e > npx) npx = e;
     }
     float4* out = nullptr;
-    CK(cudaMalloc(&out, sizeof(float4) * (size_t)(npx > 0 ? npx : 1)), "cudaMalloc(autotune target)");
+    CK(device_malloc(&out, sizeof(float4) * (size_t)(npx > 0 ? npx : 1)), "cudaMalloc(autotune target)");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
@@ -1165,7 +1177,7 @@ int canvox_footprint(const canvox_camera* cams, int32_t n_views, void* stream, i
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int64_t rec_words = (g.n_rec + 31) / 32, leaf_words = (g.n_leaf + 31) / 32;
     uint32_t* bits = nullptr;
-    CK(cudaMalloc(&bits, sizeof(uint32_t) * (size_t)(rec_words + leaf_words + 4)), "cudaMalloc(footprint)");
+    CK(device_malloc(&bits, sizeof(uint32_t) * (size_t)(rec_words + leaf_words + 4)), "cudaMalloc(footprint)");
     struct Free {
         uint32_t* p;
         ~Free() { cudaFree(p); }
