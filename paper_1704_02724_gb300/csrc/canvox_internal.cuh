@@ -121,6 +121,7 @@ struct MixedParams {
     float side;               // extent
     int32_t steps;            // step_limit, at most 2^31 - 1
     float bound_t, bound_i;   // the colour bound of a boundary per local time and per ih (see ray_step)
+    int32_t take, per_block;  // a launch of one wave: rays a warp takes, warps a block uses (0: rays from the queue)
 };
 
 struct PlainParams {

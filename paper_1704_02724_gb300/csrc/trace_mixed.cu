@@ -749,15 +749,21 @@ __global__ void __launch_bounds__(kBlock, CANVOX_MIN_BLOCKS) mixed_kernel(MixedP
     for (;;) {
         unsigned busy = __ballot_sync(kFull, alive);
         if (!drained && __popc(busy) <= P.refill) {
-            const unsigned idle = ~busy;
-            unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(P.queue, (unsigned long long)__popc(idle));
-            base = __shfl_sync(kFull, base, 0);
-            if (base + __popc(idle) >= (unsigned long long)P.total_rays) drained = true;
-            if (!alive) {
-                const unsigned long long g = base + __popc(idle & ((1u << lane) - 1u));
-                if (g < (unsigned long long)P.total_rays) alive = ray_init<kSmem, kRopes, kCount, kPool>(r, P, g, stk);
+            unsigned long long g = (unsigned long long)P.total_rays;
+            if (P.per_block) {
+                const unsigned w = threadIdx.x >> 5;
+                if (w < (unsigned)P.per_block && lane < (unsigned)P.take)
+                    g = (blockIdx.x * (unsigned)P.per_block + w) * (unsigned)P.take + lane;
+                drained = true;
+            } else {
+                const unsigned idle = ~busy;
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(P.queue, (unsigned long long)__popc(idle));
+                base = __shfl_sync(kFull, base, 0);
+                if (base + __popc(idle) >= (unsigned long long)P.total_rays) drained = true;
+                if (!alive) g = base + __popc(idle & ((1u << lane) - 1u));
             }
+            if (g < (unsigned long long)P.total_rays) alive = ray_init<kSmem, kRopes, kCount, kPool>(r, P, g, stk);
             busy = __ballot_sync(kFull, alive);
             if (!drained && __popc(busy) <= P.refill) continue;
         }
@@ -829,6 +835,19 @@ cudaError_t launch_mixed(const MixedParams& params, int grid, int block, cudaStr
     p.bound_t = kEpsT * p.side;
     p.bound_i = kEpsI * p.side;
     p.steps = (int32_t)(p.step_limit < 0x7FFFFFFF ? p.step_limit : 0x7FFFFFFF);
+    // Rays that fit the resident lanes are dealt out evenly, neighbouring ones to the warps of a block, instead of to
+    // whichever warp asks first (the first blocks: some SMs then work for others). While half of the resident warps
+    // would do, a warp takes half as many rays, down to one: a warp's steps follow every path that one of its lanes
+    // takes, and a small launch waits for the longest ray's chain of steps. Beyond half, the FP64 set-up of a warp, the
+    // same for one lane as for 32, and the shared issue slots cost more than that (256 x 256 pixels of the depth-24
+    // canvas with 16 rays a warp: 532 us). From the queue by 32, dealt out by 32 and by this rule, in us: depth-8 cube 64
+    // x 64 374, 369, 249, 128 x 128 409, 410, 339; depth-27 canvas 128 x 128 1278, 1265, 892; depth-24 canvas 128 x 128
+    // 452, 438, 390, 256 x 256 489, 421, 421; opaque paint 64 x 64 35, 34, 37, 128 x 128 38, 34, 38, 392 x 392 52, 48, 48.
+    const int64_t room = (int64_t)grid * (block / 32);  // warps
+    p.take = 32;
+    while (p.refill == 0 && p.take > 1 && p.total_rays <= room / 2 * (p.take / 2)) p.take /= 2;
+    const int64_t warps = (p.total_rays + p.take - 1) / p.take;
+    p.per_block = warps <= room ? (int32_t)((warps + grid - 1) / grid) : 0;
     const bool ropes = p.use_ropes && p.tree.ropes;
     if (p.count_reads)
         return ropes ? launch_mixed_w<true, true>(p, grid, block, s, after_setup)
