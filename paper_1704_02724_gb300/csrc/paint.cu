@@ -244,6 +244,7 @@ struct Entries {
     float4 x, y;    // its record
 };
 constexpr int kStageRow = 17;  // float4 per octet: eight records and a pad
+constexpr int kColourRow = 25; // the same with the eight stamps' colours
 __device__ __forceinline__ void load_entries(Entries& E, const LevelIn& L, const StampDev& S, int k) {
     E.m = (int)max((int64_t)0, min((int64_t)8, E.e - E.q0));
     E.v = k < E.m ? L.ent[E.q0 + k] : -1;
@@ -546,7 +547,7 @@ __device__ __forceinline__ int64_t warp_total(int64_t x) {
 template <bool kExact>
 __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDev S, double half, uint64_t* slot,
                                                            int32_t* cnt, uint16_t* cls, BlockSum* bs, long long* tot) {
-    __shared__ float4 s_rec[kCells * kStageRow];
+    __shared__ float4 s_rec[kCells * kColourRow];
     __shared__ int64_t s_ent[kCells / 4], s_int[kCells / 4];
     const int64_t i = (int64_t)blockIdx.x * kCells + (threadIdx.x >> 3);
     const int lane = threadIdx.x & 31, k = threadIdx.x & 7, lc = L.level + 1;
@@ -562,10 +563,12 @@ __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDe
     float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
     if (__any_sync(kFullMask, b < e)) {
         const Child B = child_box(L, i < L.n ? i : 0, k);
-        float4* row = s_rec + (threadIdx.x >> 3) * kStageRow;
+        float4* row = s_rec + (threadIdx.x >> 3) * kColourRow;
         Entries C{b, e, -1, 0, {}, {}};
         for (; __any_sync(kFullMask, C.q0 < C.e); C.q0 += 8) {
             load_entries(C, L, S, k);  // (most lists are short: no loads ahead, which cost registers)
+            // (the colours too: asked for by the child that an entry paints, each was a wait; 1 % of a depth-24 paint)
+            if (k < C.m) row[16 + k] = __ldg(S.rgba + (C.v < 0 ? ~C.v : C.v));
             stage_entries(C, row, k);
             __syncwarp();
             const int mm = __reduce_max_sync(kFullMask, C.m);
@@ -591,7 +594,7 @@ __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDe
                 const unsigned bits = decision_bits(c);
                 if (k == j) own = bits;
                 n += c != kDrop;
-                if (c == kPaint && !found) blend(val, S.rgba[v < 0 ? ~v : v]);
+                if (c == kPaint && !found) blend(val, row[16 + j]);
             }
             if (k < C.m) cls[C.q0 + k] = (uint16_t)own;
             __syncwarp();
@@ -613,7 +616,7 @@ __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDe
         for (int x = 0; x < (n > kLongMany ? 4 : 2); ++x) atomicAdd(&lists[x], (x & 1) ? (unsigned long long)n : 1ull);
     }
     const int32_t longest = __reduce_max_sync(kFullMask, n);
-    const int64_t ents = warp_total(n);
+    const int64_t ents = longest < (1 << 26) ? (int64_t)__reduce_add_sync(kFullMask, n) : warp_total(n);
     const int ints = __popc(__ballot_sync(kFullMask, found));
     if (lane == 0) {
         s_ent[threadIdx.x >> 5] = ents;
