@@ -164,6 +164,11 @@ cudaError_t probe_fp64(double* gflops);
 struct PaintCache;
 void paint_cache_free(PaintCache* c);
 void paint_pool_release();  // after paint_cache_free: the painter's memory pool
+// Memory of the current canvas's three pools. A call that replaces the canvas lays the new pools into the old ones'
+// memory where they fit (spares; canvas_malloc), and gives back the rest when it ends.
+enum { kPoolNodes = 0, kPoolLeaves = 1, kPoolLinks = 2, kCanvasPools = 3 };
+cudaError_t canvas_malloc(int pool, void** p, size_t bytes);
+void canvas_spares_free();
 void paint_pool_trim();     // gives back what the pool does not hold live
 cudaError_t paint_pools(int32_t depth, double extent, const double* d_centers, const double* d_radii, const float4* d_rgba,
                         int64_t n, PaintCache** cache, int32_t** d_nodes, uint2** d_leaves, int64_t* n_rec,

@@ -936,25 +936,20 @@ void pool_trim(size_t keep) {
     if (g_pool && cudaDeviceSynchronize() == cudaSuccess) cudaMemPoolTrimTo(g_pool, keep);
 }
 
-// Retry an allocation that ran out of memory once the pool has given back what it does not hold live.
-template <typename F>
-cudaError_t with_retry(F alloc) {
-    cudaError_t e = alloc();
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        pool_trim(0);
-        e = alloc();
-    }
-    return e;
-}
-
 template <typename T>
 cudaError_t dalloc(T** p, int64_t n) {
     *p = nullptr;
     cudaError_t e = pool_ready();
     if (e != cudaSuccess) return e;
     const size_t bytes = sizeof(T) * (size_t)(n > 0 ? n : 1);
-    return with_retry([&] { return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, g_pool, 0); });
+    e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, g_pool, 0);
+    if (e == cudaErrorMemoryAllocation) {  // once more, with what the pool does not hold live and the canvas before
+        cudaGetLastError();
+        canvas_spares_free();
+        pool_trim(0);
+        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, g_pool, 0);
+    }
+    return e;
 }
 void dfree(void* p) {
     if (p) cudaFreeAsync(p, 0);
@@ -1240,8 +1235,8 @@ cudaError_t finish_pools(const std::vector<uint64_t*>& slots, const std::vector<
     const int32_t n_wrap = n_leaf > 0 ? (int32_t)((n_leaf - 1) >> 31) : 0;
     int32_t* d_nodes = nullptr;
     uint2* d_leaves = nullptr;
-    PCK(with_retry([&] { return cudaMalloc(&d_nodes, sizeof(int32_t) * 8 * (size_t)n_rec); }));
-    cudaError_t e = with_retry([&] { return cudaMalloc(&d_leaves, sizeof(uint2) * (size_t)(n_leaf > 0 ? n_leaf : 1)); });
+    PCK(canvas_malloc(kPoolNodes, reinterpret_cast<void**>(&d_nodes), sizeof(int32_t) * 8 * (size_t)n_rec));
+    cudaError_t e = canvas_malloc(kPoolLeaves, reinterpret_cast<void**>(&d_leaves), sizeof(uint2) * (size_t)(n_leaf > 0 ? n_leaf : 1));
     if (e != cudaSuccess) {
         cudaFree(d_nodes);
         return e;
