@@ -38,9 +38,9 @@
 // records. A lane per child suits the short lists most cells have: with a warp
 // per cell and a lane per stamp (32 stamps at a time, two passes), a list of five
 // left 27 lanes idle and its children were taken one after the other: the depth-24
-// table of 210,000 stamps took 251 ms then and 49 ms now (expand_count 30 ms of it,
-// its issue slots 52 % used at 26 of 48 possible warps), the 1,000 stamps of the
-// depth-8 cube with the read-back 7.5 and 2.1 ms.
+// table of 210,000 stamps took 251 ms then and 35 ms now (expand_last 11.2 ms of it,
+// expand_count 8, their issue slots 66-69 % used at 33 of 36 resident warps), the
+// 1,000 stamps of the depth-8 cube with the read-back 7.5 and 1.6 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -632,6 +632,68 @@ __global__ void __launch_bounds__(8 * kCells, 9) expand_count(LevelIn L, StampDe
         }
         bs[blockIdx.x] = x;
     }
+}
+
+// The children of the cells of the level above the deepest: leaves all, each the blend of the stamps that hold its centre
+// (one that holds the whole leaf holds its centre too, and one that does not touch it does not: also in FP64, whose
+// rounding is monotone), in order. A distance instead of three, and neither decisions nor lists: 28.8 million cells of
+// the depth-24 table take 11.2 ms instead of 18.9 (expand_count), bound by the waits for records (69 % of the issue slots).
+__global__ void __launch_bounds__(8 * kCells, 9) expand_last(LevelIn L, StampDev S, double half, uint64_t* slot) {
+    __shared__ float4 s_rec[kCells * kColourRow];
+    const int64_t i = (int64_t)blockIdx.x * kCells + (threadIdx.x >> 3);
+    const int lane = threadIdx.x & 31, k = threadIdx.x & 7;
+    int64_t b = 0, e = 0;
+    if (i < L.n) {
+        b = L.off[i];
+        e = L.off[i + 1];
+    }
+    const bool is_long = e - b > L.limit;
+    if (is_long) e = b;
+    float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (__any_sync(kFullMask, b < e)) {
+        // the leaf's centre, (2 j + 1) h / 2, as two words per axis, and the margin's terms (cover32)
+        const uint32_t* coord = L.coord + 3 * (i < L.n ? i : 0);
+        float mh[3], ml[3], A = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const uint32_t cc = 2u * coord[a] + ((k >> a) & 1u);
+            plane_words(2 * ((int32_t)cc - (1 << L.level)) + 1, 0.5f * L.hf, mh[a], ml[a]);
+            A += fabsf(mh[a]);
+        }
+        const float g1 = 2.2737367544323206e-13f * A, g2 = 5.684341886080802e-14f * A;  // 2^-42, 2^-44
+        float4* row = s_rec + (threadIdx.x >> 3) * kColourRow;
+        Entries C{b, e, -1, 0, {}, {}};
+        for (; __any_sync(kFullMask, C.q0 < C.e); C.q0 += 8) {
+            load_entries(C, L, S, k);
+            if (k < C.m) row[16 + k] = __ldg(S.rgba + (C.v < 0 ? ~C.v : C.v));
+            stage_entries(C, row, k);
+            __syncwarp();
+            const int mm = __reduce_max_sync(kFullMask, C.m);
+            for (int j = 0; j < mm; ++j) {
+                const int32_t v = __shfl_sync(kFullMask, C.v, (lane & 24) + j);
+                if (j >= C.m) continue;
+                bool paints = v < 0;
+                if (!paints) {
+                    const StampRec R = staged(row, j);
+                    const float x0 = __fadd_rn(__fsub_rn(R.ch[0], mh[0]), __fsub_rn(R.cl0, ml[0]));
+                    const float x1 = __fadd_rn(__fsub_rn(R.ch[1], mh[1]), __fsub_rn(R.cl1, ml[1]));
+                    const float x2 = __fadd_rn(__fsub_rn(R.ch[2], mh[2]), __fsub_rn(R.cl2, ml[2]));
+                    const float cen2 = fmaf(x2, x2, fmaf(x1, x1, x0 * x0)), d = cen2 - R.r2;
+                    const float n = fabsf(x0) + fabsf(x1) + fabsf(x2);
+                    const float margin = fmaf(9.5367431640625e-07f, cen2 + R.r2, g1 * (n + g2));  // 2^-20 (cen2 + r2) + ...
+                    paints = d < 0.0f;
+                    if (!(fabsf(d) > margin)) {
+                        const int x = cover64(S.c + 3 * (int64_t)v, S.r2[v], 2u * coord[0] + (k & 1u),
+                                              2u * coord[1] + ((k >> 1) & 1u), 2u * coord[2] + ((k >> 2) & 1u), L.h, half);
+                        paints = x == kIn || x == kPartCentreIn;
+                    }
+                }
+                if (paints) blend(val, row[16 + j]);
+            }
+            __syncwarp();
+        }
+    }
+    if (i < L.n && !is_long) slot[8 * i + k] = leaf_key(val);
 }
 
 // Exclusive sums over the blocks, two levels: within kScanItems of them in place, and over those groups (sup).
@@ -1308,17 +1370,19 @@ struct Level {
 // Expand one level: the eight child slots of each cell (*slot_out, handed to the caller: a leaf key, or
 // kInternal | index in the next level) and the next level's refined cells with their lists; with pid (the cells'
 // partitions) also the next level's (*npid).
-cudaError_t expand(const Level& L, const StampDev& S, double extent, double half, uint64_t** slot_out, Level* next,
-                   const int32_t* pid, int32_t** npid) {
+cudaError_t expand(const Level& L, const StampDev& S, double extent, double half, int depth, uint64_t** slot_out,
+                   Level* next, const int32_t* pid, int32_t** npid) {
     DevBuf buf;
     const int64_t nch = 8 * L.n, nb = (L.n + kCells - 1) / kCells, ng = (nb + kScanItems - 1) / kScanItems;
     // cells with long lists: an octet per item of a list
     const bool longs = L.longest > L.limit();
     const int item = item_size(L.longest, L.n_ent), few = L.few() ? 0 : 1;
     const int64_t nlong = longs ? L.long_cells[few] : 0, ni = longs ? L.long_ent[few] / item + nlong : 0;
+    const bool last = L.level + 1 == depth;  // (the children are leaves all)
+    const int64_t n_cnt = last && !longs ? 0 : nch, n_cls = last && !longs ? 0 : L.n_ent;
     Arena A;
-    A.size<int32_t>(nch);
-    A.size<uint16_t>(L.n_ent);
+    A.size<int32_t>(n_cnt);
+    A.size<uint16_t>(n_cls);
     A.size<BlockSum>(nb);
     A.size<BlockSum>(ng);
     A.size<long long>(kTotWords);
@@ -1327,8 +1391,8 @@ cudaError_t expand(const Level& L, const StampDev& S, double extent, double half
     A.size<int32_t>(8 * ni);
     A.size<int32_t>(8 * nlong);
     PCK(buf.alloc(&A.base, (int64_t)A.bytes));
-    int32_t* cnt = A.take<int32_t>(nch);
-    uint16_t* cls = A.take<uint16_t>(L.n_ent);
+    int32_t* cnt = A.take<int32_t>(n_cnt);
+    uint16_t* cls = A.take<uint16_t>(n_cls);
     BlockSum *bs = A.take<BlockSum>(nb), *sup = A.take<BlockSum>(ng);
     long long* tot = A.take<long long>(kTotWords);
     LongCell* cells = A.take<LongCell>(nlong);
@@ -1345,6 +1409,12 @@ cudaError_t expand(const Level& L, const StampDev& S, double extent, double half
         long_count<<<blocks_for(ni, 16), 128>>>(in, S, half, items, tot, fr, cls, icnt);
         long_sums<<<(unsigned)nlong, 8 * kSumRows>>>(in, S, cells, item, tot, fr, cls, icnt, slot, cnt);
         PCK(cudaGetLastError());
+    }
+    if (last) {
+        expand_last<<<(unsigned)nb, 8 * kCells>>>(in, S, half, slot);
+        next->n = 0;
+        next->level = depth;
+        return cudaGetLastError();
     }
     (L.few() ? expand_count<true> : expand_count<false>)<<<(unsigned)nb, 8 * kCells>>>(in, S, half, slot, cnt, cls, bs, tot);
     scan_sums(bs, nb, sup, tot);
@@ -1373,7 +1443,7 @@ cudaError_t expand(const Level& L, const StampDev& S, double extent, double half
 // Paint down from L (its arrays are freed on the way): slots and cell counts per level, until no refined cell is
 // left, or up to level `stop` (that level's cells are then left unexpanded in *rest). With track, the cells of L
 // are partitions 0 .. L.n - 1 and offs receives, per painted level, the first cell of each partition.
-cudaError_t paint_down(Level L, const StampDev& S, double extent, double half, int stop, bool track,
+cudaError_t paint_down(Level L, const StampDev& S, double extent, double half, int depth, int stop, bool track,
                        std::vector<uint64_t*>* slots, std::vector<int64_t>* ncell, Level* rest,
                        std::vector<int64_t*>* offs) {
     const int64_t nseg = L.n;
@@ -1387,7 +1457,7 @@ cudaError_t paint_down(Level L, const StampDev& S, double extent, double half, i
         uint64_t* slot = nullptr;
         int32_t* npid = nullptr;
         Level next;
-        e = expand(L, S, extent, half, &slot, &next, pid, &npid);
+        e = expand(L, S, extent, half, depth, &slot, &next, pid, &npid);
         if (slot) {
             slots->push_back(slot);
             ncell->push_back(L.n);
@@ -1560,7 +1630,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     Level root, partP, rep_lvl, unused;
     PaintCache* nc = nullptr;
     if (e == cudaSuccess) e = root_level(S, n, extent, half, &root);
-    if (e == cudaSuccess) e = paint_down(root, S, extent, half, kPartLevel, false, &slots_top, &ncell_top, &partP, nullptr);
+    if (e == cudaSuccess) e = paint_down(root, S, extent, half, depth, kPartLevel, false, &slots_top, &ncell_top, &partP, nullptr);
     else root.free();
     if (e == cudaSuccess) {
         nc = new PaintCache();
@@ -1595,7 +1665,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
         nc->lst_off = keep_off;
         nc->lst_ent = keep_ent;
         if (e == cudaSuccess)
-            e = paint_down(start, S, extent, half, -1, true, &slots_bot, &ncell_bot, &unused, &offs_bot);
+            e = paint_down(start, S, extent, half, depth, -1, true, &slots_bot, &ncell_bot, &unused, &offs_bot);
         else
             start.free();
         partP = Level();
@@ -1650,7 +1720,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
                 e = cudaMemcpy(rep_lvl.off + m, &n_ent, sizeof(int64_t), cudaMemcpyHostToDevice);
         }
         if (e == cudaSuccess)
-            e = paint_down(rep_lvl, S, extent, half, -1, true, &slots_r, &ncell_r, &unused, &offs_r);
+            e = paint_down(rep_lvl, S, extent, half, depth, -1, true, &slots_r, &ncell_r, &unused, &offs_r);
         else
             rep_lvl.free();
         if (e == cudaSuccess) e = assemble(np, reuse, rep, *old, slots_r, offs_r, &slots_bot, &ncell_bot, &offs_bot);

@@ -64,3 +64,16 @@ def test_planes_through_a_room(n):
     c[np.arange(n), a] = np.array([E / 8, -E / 4, 0.0])[a] + rng.choice([-1.0, 1.0], n) * r * (1 + gap)
     q = np.c_[rng.uniform(0, 1, (n, 3)), rng.uniform(0, 9, n)].astype(np.float32)
     _check(D, E, c, r, q)
+
+
+@pytest.mark.parametrize("depth", [1, 2, 5, 7])
+def test_centres_at_the_radius(depth):
+    """Stamps whose surface passes exactly, or an ulp inside or outside, through centres of the deepest leaves."""
+    rng = np.random.default_rng(depth)
+    n, h = 150, 2.0 ** -depth
+    c = (rng.integers(0, 2 ** depth, (n, 3)) + 0.5) * h - 0.5             # leaf centres
+    r = rng.integers(1, max(2, 2 ** depth // 8), n) * h
+    r[::5] = h * np.sqrt(rng.integers(1, 12, len(r[::5])))
+    r = r * (1.0 + rng.integers(-1, 2, n) * 2.0 ** -52)
+    q = np.c_[rng.uniform(0, 1, (n, 3)), rng.uniform(0, 9, n)].astype(np.float32)
+    _check(depth, 1.0, c, r, q)
