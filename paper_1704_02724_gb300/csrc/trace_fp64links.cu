@@ -259,26 +259,18 @@ __device__ bool step64(Ray64& r, const MixedParams& P) {
     const int sh_old = kFix - r.L;
     int32_t prec = r.pr;
     int kk = (int)(r.kc ^ (1u << ax)), sh = sh_old;
-    int32_t slot = 0;
     if (!(N & s)) {  // not the high half of the same parent
         const uint2 rp = __ldg(T.ropes + (int64_t)r.pr * 6 + 2 * ax + (int)(((r.flip >> ax) & 1u) ^ 1u));
         r.n_rec += 1;
         prec = (int32_t)rp.x;
-        kk = (int)((rp.y >> 8) & 7u);
-        sh = kFix - (int)(rp.y & 255u);
-        if (rp.y & kLinkRecord) slot = prec;  // (a link to an internal cell names its record)
+        // (an internal neighbour is named by its own record: its child next to the old cell has a sibling's index)
+        if (!(rp.y & kLinkRecord)) {
+            kk = (int)((rp.y >> 8) & 7u);
+            sh = kFix - (int)(rp.y & 255u);
+        }
     }
-    if (slot == 0) {
-        slot = __ldg(T.nodes + (int64_t)prec * 8 + kk);
-        r.n_rec += 1;
-    }
-    if (slot > 0 && sh != sh_old) {  // (a link names an internal cell only one level up)
-        prec = slot;
-        sh = sh_old;
-        kk = child_index(q, sh, r.flip);
-        slot = __ldg(T.nodes + (int64_t)prec * 8 + kk);
-        r.n_rec += 1;
-    }
+    int32_t slot = __ldg(T.nodes + (int64_t)prec * 8 + kk);
+    r.n_rec += 1;
     // 3. finer than the old cell: near side on the exit axis, the ray's position at te on the others
     if (slot > 0) {
         const uint32_t q0 = locate64(r, 0, te, r.X[0], s), q1 = locate64(r, 1, te, r.X[1], s),

@@ -194,7 +194,7 @@ struct Ray {
     float ell, dt;              // the leaf before: its segment's length, and the time bound of the boundary that ends it
     float T;
     float err;                  // colour-error bound spent so far (the budget of the FP32 boundaries)
-    int32_t L, f;               // level of the current cell; level of the frame (anchor's neighbourhood)
+    int32_t sh, fs;             // the current cell's side is 2^sh units; that of the frame (anchor's neighbourhood) 2^fs
     uint32_t flip;              // axes with d_a < 0: the canvas is mirrored there, so every ray runs upwards
     uint32_t entry;             // axis of the face the current leaf was entered by; kLeft: the ray has left the canvas
     uint2 val, pval;            // values of the current leaf and of the one before
@@ -477,7 +477,7 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
     r.entry = 0;
     if (E.len > 0) {
         // the eye's leaf, located once for the view
-        r.L = E.len;
+        r.sh = kFix - E.len;
         if (kRopes) {
             r.pr = E.rec[E.len - 1];
             r.kc = (E.c[0] & 1u) | ((E.c[1] & 1u) << 1) | ((E.c[2] & 1u) << 2);
@@ -511,8 +511,8 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
             if (kCount) r.n_rec += 1;
         } while (slot > 0);
         r.pr = rec;
-        r.L = kFix - sh;
-        if (kCount) atomicAdd(&r.n_reads(), (uint32_t)(r.L));
+        r.sh = sh;
+        if (kCount) atomicAdd(&r.n_reads(), (uint32_t)(kFix - sh));
         r.val = make_uint2(0u, 0u);
         if (slot < 0) {
             r.val = load_leaf<kPool>(T, rec, (int)r.kc, slot);
@@ -523,7 +523,7 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
     }
     // the frame a descent would settle in (depth - K, within [L - K, L]): rays that start in a deep subtree are not
     // anchored again on their first descent past the first leaf's frame
-    r.f = deep_frame(r.L, T.depth, P.frame_levels);
+    r.fs = kFix - deep_frame(kFix - r.sh, T.depth, P.frame_levels);
     return true;
 }
 
@@ -536,7 +536,7 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
     // the runner-up F_s exceeds the smallest F_b by more than 6 * 2^-24 (|F_s| + |F_b|) + gscr, F_b's face is the
     // exit face and only its double-float time is formed. Otherwise (a ray that passes within about 2^-22 of its way
     // from the anchor of an edge of the leaf) the face is chosen in FP64 from the exact planes.
-    const uint32_t s = 1u << (kFix - r.L);
+    const uint32_t s = 1u << r.sh;
     const int32_t D0 = (int32_t)(r.X[0] + s - (uint32_t)r.A[0]);
     const int32_t D1 = (int32_t)(r.X[1] + s - (uint32_t)r.A[1]);
     const int32_t D2 = (int32_t)(r.X[2] + s - (uint32_t)r.A[2]);
@@ -626,32 +626,25 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
     //    only settles the last boundary (its link reads as an empty slot).
     uint32_t q[3] = {ax == 0 ? N : r.X[0], ax == 1 ? N : r.X[1], ax == 2 ? N : r.X[2]};
     const uint32_t left = N >> kFix;
-    const int sh_old = kFix - r.L;
+    const int sh_old = r.sh;
     int lstar = 0;  // level of the common ancestor (stack traversal and counters only; -1 past the canvas)
     if (!kRopes || kCount) lstar = (kFix - 1) - (31 - __clz((N - s) ^ N));
     int32_t prec, slot;
     int kk, sh = sh_old;
     if (kRopes) {
+        // one load for every lane: a sibling's slot, the slot a link names, or, where the parent's neighbour is an internal
+        // cell (named by its own record), that of its child next to the old cell, which has a sibling's index; past the
+        // canvas the root's, unused
         prec = r.pr;
         kk = (int)(r.kc ^ (1u << ax));
-        if (linked) {
-            if (kCount && !left) r.n_rec += 1;
-            prec = (int32_t)rp.x;
-            kk = (int)((rp.y >> 8) & 7u);
-            sh = kFix - (int)(rp.y & 255u);
-        }
-        slot = prec;  // (a link to an internal cell names its record)
-        if (!(rp.y & kLinkRecord)) {
-            slot = load_slot<kSmem, kPool>(T, P.smem_records, prec, kk);
-            if (kCount) r.n_rec += 1;
-        }
-        if (slot > 0 && sh != sh_old) {  // (a link names an internal cell only one level up)
-            prec = slot;
-            sh = sh_old;
-            kk = child_index(q, sh, r.flip);
-            slot = load_slot<kSmem, kPool>(T, P.smem_records, prec, kk);
-            if (kCount) r.n_rec += 1;
-        }
+        if (kCount && linked && !left) r.n_rec += 1;
+        const bool named = linked && !(rp.y & kLinkRecord);
+        prec = linked ? (int32_t)rp.x : prec;
+        kk = named ? (int)((rp.y >> 8) & 7u) : kk;
+        sh = named ? kFix - (int)(rp.y & 255u) : sh;
+        slot = load_slot<kSmem, kPool>(T, P.smem_records, prec, kk);
+        if (left) slot = 0;
+        if (kCount && !left) r.n_rec += 1;
     } else {
         prec = kk = slot = 0;
         if (!left) {
@@ -696,15 +689,15 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
         r.val = load_leaf<kPool>(T, prec, kk, slot);
         if (kCount) r.n_leaf += 1;
     }
-    rebase = rebase || (uint32_t)(kFix - sh - r.f) > (uint32_t)P.frame_levels;
-    if (P.frame_levels < kBoxLevels && (((N - s) ^ N) >> (kFix - r.f)) != 0u) rebase = fexit = true;
+    rebase = rebase || (uint32_t)(r.fs - sh) > (uint32_t)P.frame_levels;
+    if (P.frame_levels < kBoxLevels && (((N - s) ^ N) >> r.fs) != 0u) rebase = fexit = true;
     rebase = rebase && !left;
     if (kRopes) {
         r.pr = prec;
         r.kc = (uint32_t)kk;
     }
     r.entry = (uint32_t)ax | (left * kLeft);
-    r.L = kFix - sh;
+    r.sh = sh;
 #pragma unroll
     for (int a = 0; a < 3; ++a) r.X[a] = (q[a] >> sh) << sh;
     if (rebase) {
@@ -712,7 +705,8 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
         r.ell = ((teh - r.cur_hi) + (tel - r.cur_lo)) * P.side;
         // a leaf coarser than the frame takes the coarsest frame that holds it; a descent past the frame the deepest
         // one the canvas can need, so that deeper leaves do not anchor the ray again level by level
-        r.f = fexit || r.L < r.f ? max(0, r.L - P.frame_levels) : deep_frame(r.L, T.depth, P.frame_levels);
+        const int L = kFix - sh;
+        r.fs = kFix - (fexit || sh > r.fs ? max(0, L - P.frame_levels) : deep_frame(L, T.depth, P.frame_levels));
         set_anchor(r, P, P.views[r.view()], te64, ax);
     } else {
         r.ell = ((teh - r.cur_hi) + (tel - r.cur_lo)) * P.side;
