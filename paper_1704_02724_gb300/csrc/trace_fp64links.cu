@@ -265,8 +265,8 @@ __device__ bool step64(Ray64& r, const MixedParams& P) {
         prec = (int32_t)rp.x;
         // (an internal neighbour is named by its own record: its child next to the old cell has a sibling's index)
         if (!(rp.y & kLinkRecord)) {
-            kk = (int)((rp.y >> 8) & 7u);
-            sh = kFix - (int)(rp.y & 255u);
+            kk = (int)(rp.y >> 8);
+            sh = (int)(rp.y & 255u);
         }
     }
     int32_t slot = __ldg(T.nodes + (int64_t)prec * 8 + kk);

@@ -562,7 +562,8 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
     {
         // te = D ih + rr as hi + lo: D as two FP32 words, the product's error from one fma (Dekker). Within
         // 2^-45 |te| + 2^-25 ih.
-        const float dh = pick(ax, g0, g1, g2), dl = __int2float_rn(pick(ax, D0, D1, D2) - __float2int_rn(dh));
+        const int32_t D = pick(ax, D0, D1, D2);
+        const float dh = __int2float_rn(D), dl = __int2float_rn(D - __float2int_rn(dh));
         const float p = __fmul_rn(dh, ihx);
         const float lo = __fadd_rn(__fmaf_rn(dh, r.il(ax),
                                              __fmaf_rn(dl, ihx, __fmaf_rn(dh, ihx, -p))),
@@ -640,8 +641,8 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
         if (kCount && linked && !left) r.n_rec += 1;
         const bool named = linked && !(rp.y & kLinkRecord);
         prec = linked ? (int32_t)rp.x : prec;
-        kk = named ? (int)((rp.y >> 8) & 7u) : kk;
-        sh = named ? kFix - (int)(rp.y & 255u) : sh;
+        kk = named ? (int)(rp.y >> 8) : kk;
+        sh = named ? (int)(rp.y & 255u) : sh;
         slot = load_slot<kSmem, kPool>(T, P.smem_records, prec, kk);
         if (left) slot = 0;
         if (kCount && !left) r.n_rec += 1;

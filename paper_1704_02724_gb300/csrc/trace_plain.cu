@@ -310,7 +310,7 @@ cudaError_t setup_launch(const Tree& t, const View* host_views, int n, View* vie
 // Neighbour links (the paper's neighbour graph of Sec. 4.1.1, kept per record).
 // ropes[r][2a + s] names the cell across face (axis a, s = 1 high / 0 low) of
 // record r's cell: the same-level neighbour if it exists, else the coarser leaf
-// that covers it, as (record holding its slot, (child index << 8) | its level),
+// that covers it, as (record holding its slot, (child index << 8) | the shift of its side, 31 - level),
 // or, for an internal neighbour, as (its own record, kLinkRecord | the same),
 // which saves a ray the load of its slot; outside the canvas as (0, kLinkRecord),
 // which reads as an empty slot. One launch per level, parents before
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(256) rope_level_kernel(const int32_t* nodes, u
     for (int a = 0; a < 3; ++a) {
         const uint32_t kk = (uint32_t)(k ^ (1 << a));
         const bool high = (k >> a) & 1;
-        const uint32_t where = (kk << 8) | (uint32_t)(level + 1);
+        const uint32_t where = (kk << 8) | (uint32_t)(kFix - (level + 1));
         // the sibling inside r, and the cell past r's face on the child's side
         const int32_t ov = nodes[8 * r + kk];
         const uint2 own = ov > 0 ? make_uint2((uint32_t)ov, kLinkRecord | where) : make_uint2((uint32_t)r, where);
