@@ -65,7 +65,7 @@ struct View {
     int32_t tile_wl;  // log2 of the tile width
 };
 
-// Leaf holding the eye of a view, located once per render by eye_path_kernel.
+// Leaf holding the eye of a view, located once per render (eye_path).
 // Valid (len > 0) when the eye is inside the canvas and on no cell plane of its
 // path: every ray of the view then starts in this leaf at t = 0 (the ray is on
 // the high side of a plane just after t = 0 iff the eye is above it).

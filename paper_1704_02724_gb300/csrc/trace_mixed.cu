@@ -42,19 +42,21 @@
 // the boundary it was entered by and then to composite the leaf before it, while
 // the next link is on its way. One dependent load of a step's five or six thus
 // leaves the chain that a single long ray waits for (a 256^2 view of the depth-8
-// cube, whose longest ray crosses 283 leaves, one after the other: 491 us before,
-// 444 us after; links that name an internal neighbour's own record take another).
+// cube, whose longest ray crosses 283 leaves, one after the other: 491 -> 444 us).
+// The new slot then takes one load after the link, whichever way it is found
+// (398 -> 359 us; three, one after the other, before).
 //
-// What bounds it: instruction issue (0.79 of the issue slots on a reduced
+// What bounds it: instruction issue (0.84 of the issue slots on a reduced
 // depth-24 stereo view, 28 of 32 warps resident), the loads being served by L1
 // and L2; for views of few leaves per ray the FP64 pipe (0.82 busy on the opaque
-// depth-16 view, the per-ray set-up); for small views the longest ray's chain.
-// So the step holds to integers and few words: against frames of cells with
-// planes as FP32 dyadics and two-word reciprocals per axis, it issues 1.40 G
-// instead of 2.09 G warp instructions on that reduced view (1.55 ms instead of
-// 2.44), with three spilled words at 64 registers (four blocks an SM), and the
-// set-up takes 57 % fewer FP64 instructions (the opaque view 0.31 ms instead of
-// 0.69; the depth-24 stereo pair of 2160^2 32.5 ms instead of 45.8).
+// depth-16 view, the per-ray set-up); for small views the longest ray's chain
+// (0.10 of the issue slots on the cube). So the step holds to integers and few
+// words: against frames of cells with planes as FP32 dyadics and two-word
+// reciprocals per axis, it issues 1.30 G instead of 2.09 G warp instructions on
+// that reduced view (1.35 ms instead of 2.44), without spills at 64 registers
+// (four blocks an SM), and the set-up takes 57 % fewer FP64 instructions (the
+// opaque view 0.30 ms instead of 0.69; the depth-24 stereo pair of 2160^2 29.3 ms
+// instead of 45.8).
 //
 // Compositing (emission-absorption reading of Sec. 6.2): per segment of signed
 // length l in a leaf (sigma, rgb): a = 1 - exp(-sigma l), C += T a rgb,
@@ -440,6 +442,10 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
             r.inv64(a) = inv;
             split_inv(inv, r.ih[a], r.il(a));
             g_inv = fmaxf(g_inv, r.ih[a]);
+            if (!(r.ih[a] < kBigF)) {  // never crossed either, within FP32's range (no screen decides: g_inv)
+                r.ih[a] = kBigF;
+                r.il(a) = 0.0f;
+            }
         } else {
             r.inv64(a) = 0.0;
             r.ih[a] = kBigF;
