@@ -36,7 +36,7 @@ extern "C" {
 #define CANVOX_ERR_OOM (-5)          /* device or pinned host allocation failed */
 #define CANVOX_ERR_STEP_LIMIT (-6)   /* some ray hit the per-ray step limit (partial pixel written) */
 
-#define CANVOX_PREC_MIXED 0 /* FP32 cell-local frames, FP64 rebase and error-budgeted FP64 boundaries */
+#define CANVOX_PREC_MIXED 0 /* FP32 around FP64 anchors on the ray, error-budgeted FP64 boundaries */
 #define CANVOX_PREC_FP64 1  /* plain FP64: canvas coordinates, leaf located from the root each step */
 #define CANVOX_PREC_FP32 2  /* plain FP32 in canvas coordinates (the failing baseline of Sec. 6.3) */
 #define CANVOX_PREC_CELL32 3  /* the paper's FP32 cell-local walk, p' s + c per step (Sec. 6.2-6.3) */
@@ -91,7 +91,7 @@ typedef struct canvox_camera {
  *   refill        : a warp refetches rays when at most this many lanes are still busy (0..31).
  *   smem_records  : records of the breadth-first tree prefix (the top of the tree) copied to shared
  *                   memory at kernel start (0 = none, at most 6144; blocks per SM shrink to fit).
- *   frame_levels  : K, the most levels a local frame may sit above its cell (1..22).
+ *   frame_levels  : K, the levels a ray may descend below its last anchor's before it is anchored again (1..22).
  *   tile_w        : pixel tile a warp starts with: tile_w x (32 / tile_w), tile_w in {4, 8, 16, 32}.
  *   traversal     : 0 = neighbour links (the paper's neighbour graph, Sec. 4.1.1, built at upload),
  *                   1 = stack of ancestor records with re-descent from the common ancestor.
@@ -134,7 +134,7 @@ typedef struct canvox_stats {
     int64_t leaf_loads;      /* non-empty leaf values read (8 B each) */
     int64_t record_loads;    /* child-slot loads actually issued (stack restarts included) */
     int64_t fp64_boundaries; /* leaf boundaries whose crossing time was taken in FP64 */
-    int64_t rebases;         /* local frames entered (FP64 rebase of the ray) */
+    int64_t rebases;         /* anchors set (the ray's FP64 position and parameter) */
     int64_t step_limited;    /* rays stopped by the step limit */
     int64_t h2d_bytes;       /* host-to-device bytes the call copied (view table) */
     int64_t d2h_bytes;       /* device-to-host bytes the call copied (image, canvox_render_host only) */
@@ -185,8 +185,10 @@ int canvox_upload_octree(const int32_t* node_pool, int64_t n_records, const uint
  * eight identical siblings merge bottom-up (the root stays), and the pools are written
  * in the breadth-first layout of canvox_upload_octree. The result is bit-identical to
  * painting the stamps one by one in that order. Synchronous; the previous canvas is
- * freed first (also on failure). Temporary device memory: per tree level, the ordered
- * stamp lists of the refined cells. n_records, n_leaves (optional) receive the pool
+ * dropped first (also on failure), its memory given to the new one where that fits, else
+ * back. Temporary device memory: per tree level, the ordered stamp lists of the refined
+ * cells, of which the library keeps at most 8 GiB (a 16th of the free memory) for the next
+ * paint. n_records, n_leaves (optional) receive the pool
  * sizes. Errors: INVALID_ARG (non-finite input, negative radius or extinction, bad
  * depth/extent), OOM (device memory, or pools beyond 2^31 - 1 records or 2^34 leaves), CUDA.
  */
