@@ -841,9 +841,10 @@ cudaError_t launch_mixed(const MixedParams& params, int grid, int block, cudaStr
     // would do, a warp takes half as many rays, down to one: a warp's steps follow every path that one of its lanes
     // takes, and a small launch waits for the longest ray's chain of steps. Beyond half, the FP64 set-up of a warp, the
     // same for one lane as for 32, and the shared issue slots cost more than that (256 x 256 pixels of the depth-24
-    // canvas with 16 rays a warp: 532 us). From the queue by 32, dealt out by 32 and by this rule, in us: depth-8 cube 64
-    // x 64 374, 369, 249, 128 x 128 409, 410, 339; depth-27 canvas 128 x 128 1278, 1265, 892; depth-24 canvas 128 x 128
-    // 452, 438, 390, 256 x 256 489, 421, 421; opaque paint 64 x 64 35, 34, 37, 128 x 128 38, 34, 38, 392 x 392 52, 48, 48.
+    // canvas: 443 us with 16 rays a warp, 383 with 32). From the queue by 32, dealt out by 32 and by this rule, in us:
+    // depth-8 cube 64 x 64 329, 323, 227, 128 x 128 363, 364, 307; depth-27 canvas 64 x 64 927, 867, 437, 128 x 128 1157,
+    // 1136, 808; depth-24 canvas 128 x 128 409, 391, 350, 256 x 256 457, 383, 383; opaque paint 32 x 32 32, 31, 27, 64 x
+    // 64 34, 30, 32, 128 x 128 36, 30, 34, 256 x 256 43, 35, 35.
     const int64_t room = (int64_t)grid * (block / 32);  // warps
     p.take = 32;
     while (p.refill == 0 && p.take > 1 && p.total_rays <= room / 2 * (p.take / 2)) p.take /= 2;
