@@ -639,9 +639,10 @@ int check_nodes(HostTeam& team, const int32_t* node_pool, int64_t n_records, int
         rec[(size_t)p + 1] += rec[(size_t)p];
         leaf[(size_t)p + 1] += leaf[(size_t)p];
     }
-    // records of level l: [begin[l], begin[l + 1]); the children of the records before begin[l] are numbered 1, 2, ...
+    // records of level l: [begin[l], begin[l + 1]); the children of the records before begin[l] are numbered 1, 2, ... (Not
+    // past level `depth`, whose records the check reports: a chain of records has as many levels, each a piece to walk.)
     std::vector<int64_t> begin{0, 1};
-    while (begin.back() < n_records) {
+    while (begin.back() < n_records && (int)begin.size() <= depth) {
         const int64_t b = begin.back(), p = b / kHostChunk;
         const int64_t e = 1 + rec[(size_t)p] + internal_slots(p * kHostChunk, b);
         if (e <= b) break;  // record b is not referenced before it appears
