@@ -20,6 +20,8 @@
 #include <thread>
 #include <vector>
 
+#include <sched.h>
+
 #include "canvox_internal.cuh"
 
 using namespace canvox;
@@ -489,6 +491,13 @@ int check_stamps(const double* centers, const double* radii, const float* rgba, 
 }
 
 
+// Cores this thread may run on (a process is often held to a few of the host's).
+int64_t cores_allowed() {
+    cpu_set_t set;
+    if (sched_getaffinity(0, sizeof(set), &set) == 0) return std::max(1, CPU_COUNT(&set));
+    return std::max(1u, std::thread::hardware_concurrency());
+}
+
 // The host's cores for the length of one call: run(n, fn) calls fn(i) for i in [0, n), the calling thread among them;
 // start() leaves it to the others until finish(). The pools of a canvas are validated and hashed element by element:
 // one core takes about 1.5 ns an element, 10 ms for the depth-8 canvas of 431,100 records, which bounded its upload. A
@@ -498,7 +507,7 @@ class HostTeam {
   public:
     static constexpr int64_t kPieceUs = 13;
     explicit HostTeam(int64_t leaf_pieces) {
-        const int64_t cores = std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), 64);
+        const int64_t cores = std::min<int64_t>(cores_allowed(), 64);
         const int64_t want = std::min(cores, 1 + leaf_pieces * kPieceUs / 80);
         try {
             while ((int64_t)team_.size() + 1 < want) team_.emplace_back([this] { serve(); });
@@ -517,6 +526,7 @@ class HostTeam {
     HostTeam(const HostTeam&) = delete;
     HostTeam& operator=(const HostTeam&) = delete;
 
+    bool alone() const { return team_.empty(); }  // no thread but the caller's
     void start(int64_t n, std::function<void(int64_t)> fn) {
         finish();
         {
@@ -614,89 +624,124 @@ unsigned long long hash_slots(const int32_t* node_pool, int64_t begin, int64_t e
 // count their internal children and leaves, which gives every piece the numbers that it starts from (and, level by
 // level, where the levels of the breadth-first order begin); the pieces then check their slots. The error reported is
 // the first in pool order. Receives the levels' first records and the slots where leaf numbers pass multiples of 2^31.
+// Without helpers the caller's thread takes the pieces in order, which brings the numbers along, and adds the slots' hash
+// terms to *hash on the same walk (the multiplications hide behind the checks; counted, checked and hashed apart, a pool of
+// 408,085 records and 1.85 million leaves took one core 36 ms instead of 24).
 struct PoolError {
     int kind = 0;
     int64_t r = 0, a = 0, b = 0;
     int k = 0;
 };
+struct PoolWalk {  // where a piece begins, then where it ended
+    int64_t next_rec, next_leaf;
+    unsigned long long hash;
+    PoolError err;
+};
+// Checks records [b, e). `begin`: the levels' first records; with kAlone they are found on the way.
+template <bool kAlone>
+void check_piece(const int32_t* node_pool, int64_t n_records, int64_t n_leaves, int32_t depth, int64_t b, int64_t e,
+                 std::vector<int64_t>& begin, int64_t* wraps, PoolWalk& w) {
+    int64_t next_rec = w.next_rec, next_leaf = w.next_leaf;
+    unsigned long long h = 0;
+    int level = (int)(std::upper_bound(begin.begin(), begin.end(), b) - begin.begin()) - 1;
+    auto bad = [&](int kind, int64_t r, int k, int64_t x, int64_t y) { w.err = PoolError{kind, r, x, y, k}; };
+    for (int64_t r = b; r < e; ++r) {
+        if (r >= next_rec) return bad(1, r, 0, 0, 0);
+        while (level + 1 < (int)begin.size() && r >= begin[(size_t)level + 1]) {
+            ++level;
+            if (kAlone && level + 1 == (int)begin.size()) begin.push_back(next_rec);  // (the records before r name those)
+        }
+        for (int k = 0; k < 8; ++k) {
+            const int32_t v = node_pool[8 * r + k];
+            if (kAlone) h += elem_hash(1ull, (unsigned long long)(8 * r + k), (unsigned long long)(uint32_t)v);
+            if (v > 0) {
+                if (v != next_rec) return bad(2, r, k, v, next_rec);
+                if (v >= n_records) return bad(3, r, k, v, 0);
+                if (level + 1 > depth - 1) return bad(4, r, k, v, level + 1);
+                ++next_rec;
+            } else if (v < 0) {
+                // leaves are numbered in breadth-first slot order; the slot holds the number modulo 2^31
+                const int64_t li = -(int64_t)v - 1;
+                if (li != (next_leaf & 0x7FFFFFFFll)) return bad(5, r, k, li, next_leaf & 0x7FFFFFFFll);
+                if (next_leaf >= n_leaves) return bad(6, r, k, next_leaf, 0);
+                if (next_leaf > 0 && li == 0) wraps[(next_leaf >> 31) - 1] = 8 * r + k;  // n_leaves <= 2^34: at most 7
+                ++next_leaf;
+            }
+        }
+    }
+    w.next_rec = next_rec;
+    w.next_leaf = next_leaf;
+    w.hash += h;
+}
+
+int pool_error(const PoolError& x, int32_t depth) {
+    switch (x.kind) {
+        case 1: return fail(CANVOX_ERR_BAD_TREE, "record %lld is not referenced before it appears", (long long)x.r);
+        case 2: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: child %d, expected %lld (breadth-first order)",
+                            (long long)x.r, x.k, (int)x.a, (long long)x.b);
+        case 3: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: child %d out of range", (long long)x.r, x.k, (int)x.a);
+        case 4: return fail(CANVOX_ERR_BAD_TREE, "record %d at level %d exceeds depth %d", (int)x.a, (int)x.b, depth);
+        case 5: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: leaf %lld, expected %lld (breadth-first order, modulo 2^31)",
+                            (long long)x.r, x.k, (long long)x.a, (long long)x.b);
+        default: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: leaf %lld out of range", (long long)x.r, x.k,
+                             (long long)x.a);
+    }
+}
+
 int check_nodes(HostTeam& team, const int32_t* node_pool, int64_t n_records, int64_t n_leaves, int32_t depth,
-                std::vector<int64_t>* level_begin, int64_t* wraps, int32_t* n_wrap) {
+                std::vector<int64_t>* level_begin, int64_t* wraps, int32_t* n_wrap, unsigned long long* hash) {
     const int64_t pieces = pieces_of(n_records);
-    std::vector<int64_t> rec((size_t)pieces + 1, 0), leaf((size_t)pieces + 1, 0);  // counts, then exclusive sums
-    auto internal_slots = [&](int64_t begin, int64_t end) {
-        int64_t c = 0;
-        for (int64_t i = 8 * begin; i < 8 * end; ++i) c += node_pool[i] > 0;
-        return c;
-    };
-    team.run(pieces, [&](int64_t p) {
-        const int64_t b = p * kHostChunk, e = std::min(n_records, b + kHostChunk);
-        int64_t neg = 0;
-        for (int64_t i = 8 * b; i < 8 * e; ++i) neg += node_pool[i] < 0;
-        rec[(size_t)p + 1] = internal_slots(b, e);
-        leaf[(size_t)p + 1] = neg;
-    });
-    for (int64_t p = 0; p < pieces; ++p) {
-        rec[(size_t)p + 1] += rec[(size_t)p];
-        leaf[(size_t)p + 1] += leaf[(size_t)p];
-    }
-    // records of level l: [begin[l], begin[l + 1]); the children of the records before begin[l] are numbered 1, 2, ... (Not
-    // past level `depth`, whose records the check reports: a chain of records has as many levels, each a piece to walk.)
-    std::vector<int64_t> begin{0, 1};
-    while (begin.back() < n_records && (int)begin.size() <= depth) {
-        const int64_t b = begin.back(), p = b / kHostChunk;
-        const int64_t e = 1 + rec[(size_t)p] + internal_slots(p * kHostChunk, b);
-        if (e <= b) break;  // record b is not referenced before it appears
-        begin.push_back(std::min(e, n_records));
-    }
-    std::vector<PoolError> err((size_t)pieces);
-    std::atomic<int64_t> first_bad{pieces};
-    team.run(pieces, [&](int64_t p) {
-        if (p > first_bad.load()) return;
-        int64_t next_rec = 1 + rec[(size_t)p], next_leaf = leaf[(size_t)p];
-        const int64_t b = p * kHostChunk, e = std::min(n_records, b + kHostChunk);
-        int level = (int)(std::upper_bound(begin.begin(), begin.end(), b) - begin.begin()) - 1;
-        auto bad = [&](int kind, int64_t r, int k, int64_t x, int64_t y) {
-            err[(size_t)p] = PoolError{kind, r, x, y, k};
+    std::vector<int64_t> begin{0, 1};  // records of level l: [begin[l], begin[l + 1])
+    int64_t next_rec, next_leaf;
+    if (team.alone()) {
+        PoolWalk w{1, 0, 0, {}};
+        check_piece<true>(node_pool, n_records, n_leaves, depth, 0, n_records, begin, wraps, w);
+        if (w.err.kind) return pool_error(w.err, depth);
+        next_rec = w.next_rec;
+        next_leaf = w.next_leaf;
+        *hash += w.hash;
+    } else {
+        std::vector<int64_t> rec((size_t)pieces + 1, 0), leaf((size_t)pieces + 1, 0);  // counts, then exclusive sums
+        auto internal_slots = [&](int64_t from, int64_t to) {
+            int64_t c = 0;
+            for (int64_t i = 8 * from; i < 8 * to; ++i) c += node_pool[i] > 0;
+            return c;
+        };
+        team.run(pieces, [&](int64_t p) {
+            const int64_t b = p * kHostChunk, e = std::min(n_records, b + kHostChunk);
+            int64_t neg = 0;
+            for (int64_t i = 8 * b; i < 8 * e; ++i) neg += node_pool[i] < 0;
+            rec[(size_t)p + 1] = internal_slots(b, e);
+            leaf[(size_t)p + 1] = neg;
+        });
+        for (int64_t p = 0; p < pieces; ++p) {
+            rec[(size_t)p + 1] += rec[(size_t)p];
+            leaf[(size_t)p + 1] += leaf[(size_t)p];
+        }
+        // the children of the records before begin[l] are numbered 1, 2, ... (Not past level `depth`, whose records the
+        // check reports: a chain of records has as many levels, each a piece to walk.)
+        while (begin.back() < n_records && (int)begin.size() <= depth) {
+            const int64_t b = begin.back(), p = b / kHostChunk;
+            const int64_t e = 1 + rec[(size_t)p] + internal_slots(p * kHostChunk, b);
+            if (e <= b) break;  // record b is not referenced before it appears
+            begin.push_back(std::min(e, n_records));
+        }
+        std::vector<PoolError> err((size_t)pieces);
+        std::atomic<int64_t> first_bad{pieces};
+        team.run(pieces, [&](int64_t p) {
+            if (p > first_bad.load()) return;
+            PoolWalk w{1 + rec[(size_t)p], leaf[(size_t)p], 0, {}};
+            const int64_t b = p * kHostChunk;
+            check_piece<false>(node_pool, n_records, n_leaves, depth, b, std::min(n_records, b + kHostChunk), begin, wraps, w);
+            if (!w.err.kind) return;
+            err[(size_t)p] = w.err;
             for (int64_t f = first_bad.load(); p < f && !first_bad.compare_exchange_weak(f, p);) {
             }
-        };
-        for (int64_t r = b; r < e; ++r) {
-            if (r >= next_rec) return bad(1, r, 0, 0, 0);
-            while (level + 1 < (int)begin.size() && r >= begin[(size_t)level + 1]) ++level;
-            for (int k = 0; k < 8; ++k) {
-                const int32_t v = node_pool[8 * r + k];
-                if (v > 0) {
-                    if (v != next_rec) return bad(2, r, k, v, next_rec);
-                    if (v >= n_records) return bad(3, r, k, v, 0);
-                    if (level + 1 > depth - 1) return bad(4, r, k, v, level + 1);
-                    ++next_rec;
-                } else if (v < 0) {
-                    // leaves are numbered in breadth-first slot order; the slot holds the number modulo 2^31
-                    const int64_t li = -(int64_t)v - 1;
-                    if (li != (next_leaf & 0x7FFFFFFFll)) return bad(5, r, k, li, next_leaf & 0x7FFFFFFFll);
-                    if (next_leaf >= n_leaves) return bad(6, r, k, next_leaf, 0);
-                    if (next_leaf > 0 && li == 0) wraps[(next_leaf >> 31) - 1] = 8 * r + k;  // n_leaves <= 2^34: at most 7
-                    ++next_leaf;
-                }
-            }
-        }
-    });
-    if (first_bad.load() < pieces) {
-        const PoolError& x = err[(size_t)first_bad.load()];
-        switch (x.kind) {
-            case 1: return fail(CANVOX_ERR_BAD_TREE, "record %lld is not referenced before it appears", (long long)x.r);
-            case 2: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: child %d, expected %lld (breadth-first order)",
-                                (long long)x.r, x.k, (int)x.a, (long long)x.b);
-            case 3: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: child %d out of range", (long long)x.r, x.k, (int)x.a);
-            case 4: return fail(CANVOX_ERR_BAD_TREE, "record %d at level %d exceeds depth %d", (int)x.a, (int)x.b, depth);
-            case 5: return fail(CANVOX_ERR_BAD_TREE,
-                                "record %lld slot %d: leaf %lld, expected %lld (breadth-first order, modulo 2^31)",
-                                (long long)x.r, x.k, (long long)x.a, (long long)x.b);
-            default: return fail(CANVOX_ERR_BAD_TREE, "record %lld slot %d: leaf %lld out of range", (long long)x.r, x.k,
-                                 (long long)x.a);
-        }
+        });
+        if (first_bad.load() < pieces) return pool_error(err[(size_t)first_bad.load()], depth);
+        next_rec = 1 + rec[(size_t)pieces];
+        next_leaf = leaf[(size_t)pieces];
     }
-    const int64_t next_rec = 1 + rec[(size_t)pieces], next_leaf = leaf[(size_t)pieces];
     if (next_rec != n_records) return fail(CANVOX_ERR_BAD_TREE, "%lld records unreachable", (long long)(n_records - next_rec));
     if (next_leaf != n_leaves) return fail(CANVOX_ERR_BAD_TREE, "%lld leaves unreferenced", (long long)(n_leaves - next_leaf));
     *n_wrap = n_leaves > 0 ? (int32_t)((n_leaves - 1) >> 31) : 0;
@@ -755,17 +800,29 @@ int upload(const int32_t* node_pool, int64_t n_records, const uint16_t* leaf_rgb
     std::vector<int64_t> level_begin;
     int64_t wraps[kMaxWraps] = {};
     int32_t n_wrap = 0;
-    int rc = check_nodes(team, node_pool, n_records, n_leaves, depth, &level_begin, wraps, &n_wrap);
+    std::atomic<unsigned long long> hash{0};
+    unsigned long long walked = 0;
+    int rc = check_nodes(team, node_pool, n_records, n_leaves, depth, &level_begin, wraps, &n_wrap, &walked);
     if (rc) return rc;
     std::vector<int64_t> bad((size_t)leaf_pieces, -1);
+    const bool alone = team.alone();
     team.run(leaf_pieces, [&](int64_t p) {
-        bad[(size_t)p] = first_bad_leaf(leaf_rgba, p * kHostChunk, std::min(n_leaves, (p + 1) * kHostChunk));
+        const int64_t b = p * kHostChunk, e = std::min(n_leaves, b + kHostChunk);
+        if (!alone) {
+            bad[(size_t)p] = first_bad_leaf(leaf_rgba, b, e);
+            return;
+        }
+        for (int64_t i = e; i-- > b;) {  // (one walk, as over the records; backwards, so that the first bad leaf stays)
+            const unsigned long long v = leaf_word(leaf_rgba, i);
+            if (!leaf_allowed(v)) bad[(size_t)p] = i;
+            walked += elem_hash(2ull, (unsigned long long)i, v);
+        }
     });
     if ((rc = leaf_error(bad, leaf_rgba, 0))) return rc;
     if ((rc = ensure_device())) return rc;
     // the host pools' hash, beside the copies
-    std::atomic<unsigned long long> hash{0};
-    team.start(node_pieces + leaf_pieces, [&](int64_t p) {
+    hash = walked;
+    team.start(alone ? 0 : node_pieces + leaf_pieces, [&](int64_t p) {
         if (p < node_pieces) {
             hash += hash_slots(node_pool, p * kHostChunk, std::min(n_records, (p + 1) * kHostChunk));
         } else {
