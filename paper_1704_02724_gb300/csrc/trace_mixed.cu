@@ -84,6 +84,7 @@ constexpr float kEpsI = 1.1920928955078125e-07f;    // 2^-23 = 2 * 2^-24: the sa
 constexpr float kFar = 65536.0f;                    // a cell this many sides from the anchor asks for a new anchor
 constexpr int kBoxLevels = 16;                      // frames of fewer levels also end where the ray leaves their cell
 constexpr uint32_t kLeft = 4u;                      // (Ray::entry)
+constexpr float kMaxWay = 2147483520.0f;            // the largest float below 2^31
 constexpr float kBigF = 1.0e28f;                    // time per unit of an axis the ray never crosses (d_a = 0)
 
 // Resident 256-thread blocks per SM the register allocation must allow (occupancy knob).
@@ -585,9 +586,10 @@ __device__ bool ray_step(Ray& r, const MixedParams& P, int32_t* stk) {
     float teh, tel;
     {
         // te = D ih + rr as hi + lo: D as two FP32 words, the product's error from one fma (Dekker). Within
-        // 2^-45 |te| + 2^-25 ih.
+        // 2^-45 |te| + 2^-25 ih. (dh at most the float below 2^31: rounded up to 2^31 itself, as for the canvas's far face
+        // seen from its near one, it is past the largest integer, and the conversion back would leave dl a unit short.)
         const int32_t D = pick(ax, D0, D1, D2);
-        const float dh = __int2float_rn(D), dl = __int2float_rn(D - __float2int_rn(dh));
+        const float dh = fminf(__int2float_rn(D), kMaxWay), dl = __int2float_rn(D - __float2int_rn(dh));
         const float p = __fmul_rn(dh, ihx);
         const float lo = __fadd_rn(__fmaf_rn(dh, r.il(ax),
                                              __fmaf_rn(dl, ihx, __fmaf_rn(dh, ihx, -p))),
