@@ -178,7 +178,8 @@ __device__ bool init64(Ray64& r, const MixedParams& P, unsigned long long g) {
         const double da = fabs(d[a]), o = neg ? -V.eye[a] : V.eye[a];
         r.ds(a) = da * (P.inv_extent * 2147483648.0);
         if (da != 0.0) {
-            const double inv = da > 1.0e-200 ? rcp64(da) : 1.0 / da;
+            // (smaller components are never crossed: a time of 1e200 per length keeps the products below finite)
+            const double inv = da > 1.0e-200 ? rcp64(da) : 1.0e200;
             r.iu[a] = P.unit * inv;
             r.nr[a] = -rest * r.iu[a];
             t0 = fmax(t0, (-T.half - o) * inv);

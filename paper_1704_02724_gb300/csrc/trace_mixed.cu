@@ -457,7 +457,8 @@ __device__ bool ray_init(Ray& r, const MixedParams& P, unsigned long long g, int
         r.dir64(a) = da;
         if (mag != 0) {
             if (bits < 0) r.flip |= 1u << a;
-            const double inv = mag > 0x0100000000000000ll ? rcp64(da) : 1.0 / da;
+            // (below 2^-1007 the reciprocal nears infinity, which is no time: 0 for a plane the eye is on, else past all)
+            const double inv = mag > 0x0100000000000000ll ? rcp64(da) : 1.0e300;
             r.inv64(a) = inv;
             split_inv(inv, r.ih[a], r.il(a));
             g_inv = fmaxf(g_inv, r.ih[a]);
