@@ -211,7 +211,9 @@ namespace canvox {
 // division's nine or so, and the norm's square root leaves its reciprocal; the FP64 pipe (1/64 of the FP32 rate) bounds views of few leaves per ray. For the pixel
 // coordinates the result is the rounded quotient always: 2i + 1 < 2^32 and W < 2^31, so a quotient lies at least
 // 2^-32 of an ulp from a rounding boundary, far more than the correction's error of 2^-51.
-// 1 / x: about 20 bits from the hardware, then one step of third order (1 + e + e^2) to 53.
+// 1 / x: about 20 bits from the hardware, r0 = (1 - e) / x, then one third-order Newton step (the geometric series
+// (1 + e + e^2) r0, Householder 1970), which leaves e^3 = 2^-60 and one rounding: within 0.51 ulp, the correctly rounded
+// quotient but for near-ties.
 __device__ __forceinline__ double rcp64(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));

@@ -32,6 +32,7 @@
 
 #include "canvox_internal.cuh"
 #include "cells.cuh"
+#include "opacity.cuh"
 
 namespace canvox {
 namespace {
@@ -77,27 +78,6 @@ __device__ __forceinline__ double half_to_double(unsigned h) {
     const uint32_t m = f & 0x7FFFFFFFu;
     const long long d = ((long long)m << 29) + (m ? 0x3800000000000000ll : 0ll);
     return __longlong_as_double(d | ((long long)(f >> 31) << 63));
-}
-__device__ __forceinline__ bool less_pos(double a, double b) {  // of numbers that are not both negative
-    return __double_as_longlong(a) < __double_as_longlong(b);
-}
-
-// e^-x - 1. Below 1/8 (most leaves: thin paint, small cells) its series to x^10 / 10! (the next term is 2^-55 of the
-// value), 10 FP64 operations; else the library's.
-__device__ __forceinline__ double expm1_neg64(double x) {
-    const double y = -x;
-    if (less_pos(x, 0.125)) {
-        double p = fma(2.7557319223985893e-07, y, 2.7557319223985893e-06);
-        p = fma(p, y, 2.4801587301587302e-05);
-        p = fma(p, y, 1.9841269841269841e-04);
-        p = fma(p, y, 1.3888888888888889e-03);
-        p = fma(p, y, 8.3333333333333332e-03);
-        p = fma(p, y, 4.1666666666666664e-02);
-        p = fma(p, y, 0.16666666666666666);
-        p = fma(p, y, 0.5);
-        return fma(p * y, y, y);
-    }
-    return expm1(y);
 }
 
 // Composite the current leaf over [r.t, te].

@@ -70,6 +70,7 @@
 
 #include "canvox_internal.cuh"
 #include "cells.cuh"
+#include "opacity.cuh"
 
 namespace canvox {
 namespace {
@@ -97,21 +98,6 @@ __device__ __forceinline__ float rcp_approx(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
-}
-
-// e^-x - 1 for x >= 0 (and just below 0): on [0, 1] - x (1 + x r(x)) with r the degree-5 minimax polynomial (Remez,
-// relative error 2^-28.5), beyond it by the hardware exponential, where the 1 dominates. Within 1.1 ulp; 12
-// instructions without a branch, against about 20 of expm1f.
-__device__ __forceinline__ float expm1_neg(float x) {
-    float p = __fmaf_rn(0.000129130945f, x, -0.00130112655f);
-    p = __fmaf_rn(p, x, 0.0082762083f);
-    p = __fmaf_rn(p, x, -0.0416474678f);
-    p = __fmaf_rn(p, x, 0.166663662f);
-    p = __fmaf_rn(p, x, -0.499999851f);
-    p = __fmaf_rn(p, x, 1.0f);
-    float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * -1.44269504f));
-    return x < 1.0f ? -x * p : e - 1.0f;
 }
 
 extern __shared__ int32_t s_nodes[];  // copy of the tree's first records (kernel instance with kSmem)
