@@ -187,8 +187,13 @@ int canvox_upload_octree(const int32_t* node_pool, int64_t n_records, const uint
  * painting the stamps one by one in that order. Synchronous; the previous canvas is
  * dropped first (also on failure), its memory given to the new one where that fits, else
  * back. Temporary device memory: per tree level, the ordered stamp lists of the refined
- * cells, of which the library keeps at most 8 GiB (a 16th of the free memory) for the next
- * paint. n_records, n_leaves (optional) receive the pool
+ * cells. The library keeps for the next paint at most twice what this one had in use at
+ * once, and no more than a 16th of the device's free memory; its own allocations that find no
+ * memory get that back, other allocators in the process only by canvox_release. Canvas pools (of
+ * painted and uploaded canvases alike) are allocated an eighth larger than needed, at most
+ * 256 MiB, so that a canvas that grows keeps its memory; a smaller canvas stays in the
+ * memory of the one before while that leaves no more than 512 MiB, nor more than its
+ * own size and a MiB, unused per pool. n_records, n_leaves (optional) receive the pool
  * sizes. Errors: INVALID_ARG (non-finite input, negative radius or extinction, bad
  * depth/extent), OOM (device memory, or pools beyond 2^31 - 1 records or 2^34 leaves), CUDA.
  */

@@ -966,13 +966,16 @@ __global__ void scan_add(int64_t* d, int64_t n, const int64_t* sums) {
 // ---------------------------------------------------------------------------
 // Device memory of the painter: a memory pool of its own. From the device allocator an array costs 30-50 us and a free
 // 30 us (0.3 and 0.5 ms a GB), from the pool 1.5 us each, so what a level needs only while it is painted is one
-// allocation. Everything runs on the legacy default stream, which orders frees and reuse. After a paint the pool gives
-// back all but kPoolKeep bytes (a 16th of the device's free memory, if that is less) of what it does not hold live, an
-// allocation of the library that finds no memory gets the rest (paint_pool_trim), and canvox_release destroys it. The depth-24 table of 210,000 stamps, whose arrays take 7 GB at once, took 57.4 ms with
-// 4 GiB kept and 48.6 ms with 8.
+// allocation. Everything runs on the legacy default stream, which orders frees and reuse. After a paint the pool keeps
+// at most twice what the last painting (its appends among it) had live at once, as arrays of other sizes leave gaps: the
+// same painting changed and painted again then allocates nothing (with an eighth instead of as much again the depth-24 table
+// of 210,000 stamps took 36.5 ms for 35.2, a session of appends 13.2 for 12.7); and no more than a kPoolShare-th of the
+// device's free memory. The rest is given back. An allocation of the library that finds no memory gets what is not live
+// (paint_pool_trim), and canvox_release destroys the pool. (The depth-24 table of 210,000 stamps, whose arrays take 7 GB at
+// once, took 57.4 ms with 4 GiB kept and 48.6 ms with 8; a small painting after it holds a few MB again.)
 // ---------------------------------------------------------------------------
 namespace {
-constexpr size_t kPoolKeep = (size_t)8 << 30;
+constexpr size_t kPoolShare = 16;
 cudaMemPool_t g_pool = nullptr;
 
 cudaError_t pool_ready() {
@@ -996,6 +999,17 @@ cudaError_t pool_ready() {
 
 void pool_trim(size_t keep) {
     if (g_pool && cudaDeviceSynchronize() == cudaSuccess) cudaMemPoolTrimTo(g_pool, keep);
+}
+
+// The most bytes live at once since the mark was last set back (to what is live then).
+uint64_t pool_high_water() {
+    uint64_t high = 0;
+    if (!g_pool || cudaMemPoolGetAttribute(g_pool, cudaMemPoolAttrUsedMemHigh, &high) != cudaSuccess) return 0;
+    return high;
+}
+void pool_reset_high_water() {
+    uint64_t zero = 0;
+    if (g_pool) cudaMemPoolSetAttribute(g_pool, cudaMemPoolAttrUsedMemHigh, &zero);
 }
 
 template <typename T>
@@ -1612,6 +1626,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     *cache = nullptr;
     // an append: the same canvas, and the stamps the cache was painted with come first in the table
     const bool append = old && old->depth == depth && old->extent == extent && old->n_stamps <= n;
+    if (!append) pool_reset_high_water();
     DevBuf buf;
     // squared radii and target depths (the host painter's integer loop, in the same FP64 operations)
     double* d_r2;
@@ -1744,7 +1759,8 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     partP.free();
     size_t spare = 0, total = 0;
     if (cudaMemGetInfo(&spare, &total) != cudaSuccess) spare = 0;
-    pool_trim(std::min(kPoolKeep, spare / 16));
+    const size_t high = (size_t)pool_high_water();
+    pool_trim(std::min(2 * high, spare / kPoolShare));
     if (e == cudaSuccess) {
         nc->slots = slots_bot;
         nc->ncell = ncell_bot;
