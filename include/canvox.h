@@ -187,9 +187,10 @@ int canvox_upload_octree(const int32_t* node_pool, int64_t n_records, const uint
  * painting the stamps one by one in that order. Synchronous; the previous canvas is
  * dropped first (also on failure), its memory given to the new one where that fits, else
  * back. Temporary device memory: per tree level, the ordered stamp lists of the refined
- * cells. The library keeps for the next paint at most twice what this one had in use at
- * once, and no more than a 16th of the device's free memory; its own allocations that find no
- * memory get that back, other allocators in the process only by canvox_release. Canvas pools (of
+ * cells. The library keeps for the next paint what the last two (and their appends) had in
+ * use at once, the more of them, with a quarter and 64 MiB for gaps, and no more than a 16th
+ * of the device's free memory; its own allocations that find no memory get that back, other
+ * allocators in the process only by canvox_release. Canvas pools (of
  * painted and uploaded canvases alike) are allocated an eighth larger than needed, at most
  * 256 MiB, so that a canvas that grows keeps its memory; a smaller canvas stays in the
  * memory of the one before while that leaves no more than 512 MiB, nor more than its

@@ -967,15 +967,18 @@ __global__ void scan_add(int64_t* d, int64_t n, const int64_t* sums) {
 // Device memory of the painter: a memory pool of its own. From the device allocator an array costs 30-50 us and a free
 // 30 us (0.3 and 0.5 ms a GB), from the pool 1.5 us each, so what a level needs only while it is painted is one
 // allocation. Everything runs on the legacy default stream, which orders frees and reuse. After a paint the pool keeps
-// at most twice what the last painting (its appends among it) had live at once, as arrays of other sizes leave gaps: the
-// same painting changed and painted again then allocates nothing (with an eighth instead of as much again the depth-24 table
-// of 210,000 stamps took 36.5 ms for 35.2, a session of appends 13.2 for 12.7); and no more than a kPoolShare-th of the
-// device's free memory. The rest is given back. An allocation of the library that finds no memory gets what is not live
-// (paint_pool_trim), and canvox_release destroys the pool. (The depth-24 table of 210,000 stamps, whose arrays take 7 GB at
-// once, took 57.4 ms with 4 GiB kept and 48.6 ms with 8; a small painting after it holds a few MB again.)
+// what the last two paintings (their appends among them) had live at once, whichever is more, and room for the gaps
+// between arrays (with_gaps), but no more than a kPoolShare-th of the device's free memory; the rest is given back. The
+// same paintings, changed and painted again, then allocate nothing: the depth-24 table of 210,000 stamps, 6 GB live at once,
+// takes 35.3 ms, with an eighth of that for the gaps 36.5, and a session of appends 12.8 and 13.2. An allocation of the
+// library that finds no memory gets what is not live (paint_pool_trim), and canvox_release destroys the pool.
 // ---------------------------------------------------------------------------
 namespace {
 constexpr size_t kPoolShare = 16;
+// 1.16 to 1.21 of the bytes live were reserved for paintings of 0.6 and 6 GB, and 72 MB more than the 62 MB of a small one
+// (the pool takes the device's memory 32 MiB at a time).
+size_t with_gaps(size_t live) { return live + live / 4 + ((size_t)64 << 20); }
+size_t g_live_before = 0;  // the painting's before the last
 cudaMemPool_t g_pool = nullptr;
 
 cudaError_t pool_ready() {
@@ -1007,7 +1010,8 @@ uint64_t pool_high_water() {
     if (!g_pool || cudaMemPoolGetAttribute(g_pool, cudaMemPoolAttrUsedMemHigh, &high) != cudaSuccess) return 0;
     return high;
 }
-void pool_reset_high_water() {
+void new_painting() {
+    g_live_before = (size_t)pool_high_water();
     uint64_t zero = 0;
     if (g_pool) cudaMemPoolSetAttribute(g_pool, cudaMemPoolAttrUsedMemHigh, &zero);
 }
@@ -1039,6 +1043,7 @@ void paint_pool_release() {
     cudaDeviceSynchronize();
     cudaMemPoolDestroy(g_pool);
     g_pool = nullptr;
+    g_live_before = 0;
 }
 
 // Exclusive scan of d[0..n) in place; returns the total through *total (synchronous).
@@ -1626,7 +1631,7 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     *cache = nullptr;
     // an append: the same canvas, and the stamps the cache was painted with come first in the table
     const bool append = old && old->depth == depth && old->extent == extent && old->n_stamps <= n;
-    if (!append) pool_reset_high_water();
+    if (!append) new_painting();
     DevBuf buf;
     // squared radii and target depths (the host painter's integer loop, in the same FP64 operations)
     double* d_r2;
@@ -1759,8 +1764,8 @@ cudaError_t paint_pools(int32_t depth, double extent, const double* d_c, const d
     partP.free();
     size_t spare = 0, total = 0;
     if (cudaMemGetInfo(&spare, &total) != cudaSuccess) spare = 0;
-    const size_t high = (size_t)pool_high_water();
-    pool_trim(std::min(2 * high, spare / kPoolShare));
+    const size_t live = std::max((size_t)pool_high_water(), g_live_before);
+    pool_trim(std::min(with_gaps(live), spare / kPoolShare));
     if (e == cudaSuccess) {
         nc->slots = slots_bot;
         nc->ncell = ncell_bot;
