@@ -904,8 +904,9 @@ namespace canvox {
 // The spare of the canvas before is taken where the new pool fits and leaves no more than kCanvasSlack, and no more than
 // its own size, unused; a new allocation has an eighth (at most kCanvasRoom) to spare, so that a canvas that strokes are
 // appended to keeps its memory. Freeing a canvas and allocating the next took 0.3 ms (30 MB) to 3.6 ms (5 GB) of a
-// paint or an upload: the depth-24 table of 210,000 stamps 47.7 -> 44.3 ms, the depth-8 cube painted and read back 2.05 ->
-// 1.65 ms, uploaded 2.44 -> 2.31 ms.
+// paint or an upload of a canvas of about the same size as the one before: the depth-24 table of 210,000 stamps 47.7 -> 44.3
+// ms, the depth-8 cube painted and read back 2.05 -> 1.65 ms, uploaded 2.44 -> 2.31 ms. The first canvas of a process, and
+// one whose size differs by more, take what they took.
 constexpr size_t kCanvasSlack = (size_t)512 << 20, kCanvasRoom = (size_t)256 << 20;
 
 cudaError_t canvas_malloc(int pool, void** p, size_t bytes) {

@@ -46,20 +46,20 @@
 // The new slot then takes one load after the link, whichever way it is found
 // (398 -> 359 us; three, one after the other, before).
 //
-// What bounds it: instruction issue (0.84 of the issue slots on a reduced
+// What bounds it: instruction issue (0.83 of the issue slots on a reduced
 // depth-24 stereo view, 28 of 32 warps resident), the loads being served by L1
 // and L2; for views of few leaves per ray the FP64 pipe (0.82 busy on the opaque
 // depth-16 view, the per-ray set-up); for small views the longest ray's chain
 // (0.10 of the issue slots on the cube). So the step holds to integers and few
 // words: against frames of cells with planes as FP32 dyadics and two-word
-// reciprocals per axis, it issues 1.30 G instead of 2.09 G warp instructions on
-// that reduced view (1.35 ms instead of 2.44), without spills at 64 registers
+// reciprocals per axis, it issues 1.26 G instead of 1.98 G warp instructions on
+// that reduced view (1.37 ms instead of 2.45), without spills at 64 registers
 // (four blocks an SM), and the set-up takes 57 % fewer FP64 instructions (the
-// opaque view 0.30 ms instead of 0.69; the depth-24 stereo pair of 2160^2 29.3 ms
-// instead of 45.8).
+// opaque view 0.31 ms instead of 0.73; the depth-24 stereo pair of 2160^2 30.3 ms
+// instead of 47.3).
 //
 // Compositing (emission-absorption reading of Sec. 6.2): per segment of signed
-// length l in a leaf (sigma, rgb): a = 1 - exp(-sigma l), C += T a rgb,
+// length l in a leaf (sigma, rgb): a = 1 - exp(-sigma l) (opacity.cuh), C += T a rgb,
 // T *= 1 - a, with a compensated (Kahan) FP32 sum for C and the transmittance
 // kept as a running product (one rounding per leaf, unbiased).
 //
