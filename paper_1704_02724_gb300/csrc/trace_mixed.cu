@@ -367,7 +367,10 @@ __device__ __forceinline__ uint32_t locate(const Ray& r, int a, float th, uint32
     // from the cell's low corner
     const uint32_t l = (uint32_t)r.A[a] - r.X[a] + (uint32_t)__float2int_rd(__fsub_rn(x, e));
     const uint32_t h = (uint32_t)r.A[a] - r.X[a] + (uint32_t)__float2int_rd(__fadd_rn(x, e));
-    open = l ^ h;  // an interval that reaches past the cell leaves every bit open
+    // An interval that reaches past the cell, or lies past it, leaves every bit open: at a corner the next plane can come out
+    // a little before the last one (an FP64 time from a far eye, around an anchor next to it), and the bits of a position
+    // below the cell are those of its far end.
+    open = (l ^ h) | ((l | h) & ~(s - 1u));
     return r.X[a] | (l & (s - 1u));
 }
 
