@@ -52,8 +52,8 @@ struct View {
     double sy;                // tan
     double aspect;            // width / height
     double inv_w, inv_h;      // 1 / width, 1 / height (rounded to nearest)
-    // the eye from the canvas's low corner, in units of 2^-31 canvas sides: eye_unit[a] + eye_rest[a], the rest at
-    // most half a unit (a far eye: 0 and the whole distance)
+    // the eye from the canvas's low corner, in units of 2^-31 canvas sides, per axis: within the canvas eye_unit[a] (1 ..
+    // 2^31 - 1) + eye_rest[a], the rest at most half a unit, or a unit next to a face; else 0 and the whole distance
     double eye_rest[3];
     int32_t eye_unit[3];
     int32_t pad;

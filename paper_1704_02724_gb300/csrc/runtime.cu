@@ -252,8 +252,8 @@ int setup_views(const canvox_camera* cams, int n, int tile_w, double extent, Vie
             // eye + half exactly as s + e (Knuth's two-sum); the rest of s over a unit count is exact (one fma)
             const double half = 0.5 * extent, unit = std::ldexp(extent, -31);
             const double s = c.eye[a] + half, b = s - c.eye[a], e = (c.eye[a] - (s - b)) + (half - b);
-            const double k = std::nearbyint(s / unit);
-            if (k >= 1.0 && k <= 2147483647.0) {
+            if (c.eye[a] > -half && c.eye[a] < half) {
+                const double k = std::min(std::max(std::nearbyint(s / unit), 1.0), 2147483647.0);
                 V.eye_unit[a] = (int32_t)k;
                 V.eye_rest[a] = (std::fma(-k, unit, s) + e) / unit;
             } else {

@@ -150,7 +150,8 @@ __device__ bool init64(Ray64& r, const MixedParams& P, unsigned long long g) {
         uint32_t u = (uint32_t)V.eye_unit[a];
         double rest = V.eye_rest[a];
         if (neg) {
-            rest = u ? -rest : 2147483648.0 - rest;
+            // (an eye outside: from the face it looks at, whose distance keeps its own precision)
+            rest = u ? -rest : (T.half - V.eye[a]) * (P.inv_extent * 2147483648.0);
             u = u ? 0x80000000u - u : 0u;
         }
         r.U[a] = u;

@@ -275,7 +275,7 @@ __device__ __forceinline__ void anchor_zero_axes(Ray& r, const View& V) {
 }
 
 // Anchor the ray at FP64 parameter t: local time 0, at the ray's position there, which is formed from the eye's
-// (a whole number of units and a rest of half a unit at most, so that it keeps its precision near the eye). On axis
+// (a whole number of units and a rest of a unit at most, so that it keeps its precision near the eye). On axis
 // ax (the face just crossed; -1: none) it is the current cell's low plane exactly.
 __device__ __forceinline__ void set_anchor(Ray& r, const MixedParams& P, const View& V, double t, int ax) {
     r.tf() = t;

@@ -241,52 +241,23 @@ __device__ __forceinline__ void eye_path(const Tree& t, const View& V, EyePath& 
         if (!(V.eye[a] > -t.half && V.eye[a] < t.half)) return;  // (on the low face the direction decides)
     int32_t rec = 0;
     const int32_t* unit = V.eye_unit;
-    if (unit[0] > 0 && unit[1] > 0 && unit[2] > 0) {
-        // The eye in whole units and an exactly signed rest: the bits of the unit it is in are its path, and the path's
-        // first mid-plane that it lies on is the lowest bit of a whole number of units. So the chain has no FP64
-        // (fma and three comparisons a level), only the loads: 3 us less of
-        // a render at depth 16 (a view of 32 x 32 pixels 29.5 -> 26.3 us), 9 us at depths 24 and 27.
-        uint32_t v[3];
-        int on = kMaxDepth + 1;
-        for (int a = 0; a < 3; ++a) {
-            const long long rest = __double_as_longlong(V.eye_rest[a]);
-            const bool zero = (rest << 1) == 0;
-            v[a] = (uint32_t)unit[a] - (rest < 0 && !zero ? 1u : 0u);
-            if (zero) on = min(on, kFix - __ffs(unit[a]));
-        }
-        for (int lev = 0; lev < kMaxDepth; ++lev) {
-            E.rec[lev] = rec;
-            if (lev == on) return;
-            const int sh = kFix - 1 - lev;
-            const int k = (int)(((v[0] >> sh) & 1u) | (((v[1] >> sh) & 1u) << 1) | (((v[2] >> sh) & 1u) << 2));
-            const int32_t slot = __ldg(t.nodes + (long long)rec * 8 + k);
-            if (slot > 0) {
-                rec = slot;
-                continue;
-            }
-            if (slot < 0) {
-                E.val = t.leaves[leaf_index(t, rec, k, slot)];
-                E.stored = 1;
-            }
-            for (int a = 0; a < 3; ++a) E.c[a] = v[a] >> sh;
-            E.len = lev + 1;
-            return;
-        }
-        return;
+    // The eye in whole units (set for an eye inside the canvas) and an exactly signed rest: the bits of the unit it is in are
+    // its path, and the path's first mid-plane that it lies on is the lowest bit of a whole number of units. So the chain
+    // has no FP64 (fma and three comparisons a level), only the loads: 3 us less of a render at depth 16 (a view of
+    // 32 x 32 pixels 29.5 -> 26.3 us), 9 us at depths 24 and 27.
+    uint32_t v[3];
+    int on = kMaxDepth + 1;
+    for (int a = 0; a < 3; ++a) {
+        const long long rest = __double_as_longlong(V.eye_rest[a]);
+        const bool zero = (rest << 1) == 0;
+        v[a] = (uint32_t)unit[a] - (rest < 0 && !zero ? 1u : 0u);
+        if (zero) on = min(on, kFix - __ffs(unit[a]));
     }
-    // within half a unit of a face of the canvas
-    unsigned c[3] = {0u, 0u, 0u};
     for (int lev = 0; lev < kMaxDepth; ++lev) {
         E.rec[lev] = rec;
-        const double w = t.extent * __longlong_as_double((long long)(1023 - (lev + 1)) << 52);
-        int k = 0;
-        for (int a = 0; a < 3; ++a) {
-            const double M = fma((double)(2u * c[a] + 1u), w, -t.half);
-            if (V.eye[a] == M) return;  // on the plane: the direction decides
-            const unsigned b = V.eye[a] > M;
-            c[a] = 2u * c[a] + b;
-            k |= (int)b << a;
-        }
+        if (lev == on) return;
+        const int sh = kFix - 1 - lev;
+        const int k = (int)(((v[0] >> sh) & 1u) | (((v[1] >> sh) & 1u) << 1) | (((v[2] >> sh) & 1u) << 2));
         const int32_t slot = __ldg(t.nodes + (long long)rec * 8 + k);
         if (slot > 0) {
             rec = slot;
@@ -296,9 +267,7 @@ __device__ __forceinline__ void eye_path(const Tree& t, const View& V, EyePath& 
             E.val = t.leaves[leaf_index(t, rec, k, slot)];
             E.stored = 1;
         }
-        E.c[0] = c[0];
-        E.c[1] = c[1];
-        E.c[2] = c[2];
+        for (int a = 0; a < 3; ++a) E.c[a] = v[a] >> sh;
         E.len = lev + 1;
         return;
     }
