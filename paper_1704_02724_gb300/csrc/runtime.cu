@@ -167,6 +167,24 @@ int ensure_device() {
     return CANVOX_OK;
 }
 
+// The canvas's device for the length of a call that launches kernels on its pools (a leaf edit, an append, a hash),
+// whatever device the caller has current: on another one they would read addresses that it does not have.
+class OnCanvasDevice {
+  public:
+    OnCanvasDevice() {
+        if (cudaGetDevice(&before_) != cudaSuccess || before_ == g.device) before_ = -1;
+        else cudaSetDevice(g.device);
+    }
+    ~OnCanvasDevice() {
+        if (before_ >= 0) cudaSetDevice(before_);
+    }
+    OnCanvasDevice(const OnCanvasDevice&) = delete;
+    OnCanvasDevice& operator=(const OnCanvasDevice&) = delete;
+
+  private:
+    int before_ = -1;
+};
+
 void drop_graphs() {
     for (auto& e : g.graphs) {
         if (e.exec) cudaGraphExecDestroy(e.exec);
@@ -1000,6 +1018,7 @@ int canvox_paint_append(const double* centers, const double* radii, const float*
     if (g.st_n + n >= 0x7FFFFFFFll) return fail(CANVOX_ERR_INVALID_ARG, "stamp table beyond 2^31 - 1 stamps");
     const int32_t depth = g.depth;
     const double extent = g.extent;
+    const OnCanvasDevice device;
     if ((rc = reserve_stamps(g.st_n + n, g.st_n))) return rc;
     if (n > 0) {
         CK(cudaMemcpy(g.d_st_c + 3 * g.st_n, centers, sizeof(double) * 3 * (size_t)n, cudaMemcpyHostToDevice),
@@ -1040,6 +1059,7 @@ int canvox_update_leaves(int64_t first, int64_t count, const uint16_t* leaf_rgba
     if (count < 0 || first < 0 || first > g.n_leaf || count > g.n_leaf - first || (count > 0 && !leaf_rgba))
         return fail(CANVOX_ERR_INVALID_ARG, "leaf range [%lld, %lld) outside the pool of %lld leaves",
                     (long long)first, (long long)(first + count), (long long)g.n_leaf);
+    const OnCanvasDevice device;
     try {
         return update_range(first, count, leaf_rgba);
     } catch (const std::exception& e) {  // host memory
@@ -1052,6 +1072,7 @@ int canvox_octree_hash(uint64_t* host_hash, uint64_t* device_hash) {
     if (!g.uploaded) return fail(CANVOX_ERR_NOT_UPLOADED, "no canvas uploaded");
     if (host_hash) *host_hash = g.host_hash;
     if (device_hash) {
+        const OnCanvasDevice device;
         if (g.any_render) CK(cudaEventSynchronize(g.done), "cudaEventSynchronize");
         CK(cudaMemset(g.d_hash, 0, sizeof(unsigned long long)), "cudaMemset(hash)");
         CK(launch_hash(device_tree(), g.d_hash, 0), "hash kernel launch");

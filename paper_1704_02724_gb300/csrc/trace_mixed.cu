@@ -270,6 +270,7 @@ __device__ __forceinline__ void anchor_zero_axes(Ray& r, const View& V) {
     for (int a = 0; a < 3; ++a) {
         if (!((zm >> a) & 1u)) continue;
         const long long rest = __double_as_longlong(V.eye_rest[a]);  // (below 0: the sign bit set, and not -0)
+        // (eye_unit is 0 only for an eye on the low face: a ray that meets the canvas has its eye within it on such an axis)
         r.A[a] = V.eye_unit[a] ? V.eye_unit[a] - (rest < 0 && (rest << 1) != 0 ? 1 : 0) : __double2int_rd(V.eye_rest[a]);
     }
 }
