@@ -8,21 +8,22 @@ namespace {
 
 // e^-x - 1 for x >= 0, and just below 0 (a segment can come out that much too short). The argument is reduced by a whole
 // number n of ln 2 (Cody and Waite 1980; one word of ln 2 does, as the part it leaves out is scaled by 2^n too):
-// -x = n ln 2 + f, |f| <= 0.347, e^f - 1 = f + f^2 q(f) with q the degree-4 minimax polynomial (relative error 2^-26.1),
-// e^-x - 1 = 2^n (e^f - 1) + (2^n - 1). Within 0.98 ulp of every argument (all binary32 values from 2^-40 on compared;
+// -x = n ln 2 + f, |f| <= 0.347, e^f - 1 = f + f^2 q(f) with q the degree-4 minimax polynomial (relative error 2^-26),
+// e^-x - 1 = 2^n (e^f - 1) + (2^n - 1). Within 0.96 ulp for every argument (all binary32 values from 2^-40 on compared;
 // the library's has 1), in 13 instructions without a branch, against about 20 of expm1f. x (1 + x r(x)) on [0, 1) with
-// the hardware exponential beyond took 12, but reached 1.58 ulp and, by that instruction's documented error, 1.9; the
-// difference is 0.3 to 0.7 % of the depth-24 and -27 views (32.12 ms for 31.9 of a stereo pair of 2160^2).
+// the hardware exponential beyond took 12, but reached 1.58 ulp and, by that instruction's documented error, 1.9. The
+// difference is 0 to 0.8 % of the views (a depth-24 stereo pair of 2160^2 30.3 -> 30.4 ms, two depth-27 pairs 7.33 -> 7.40,
+// a 256^2 view of the depth-8 cube 0.3413 -> 0.3422); with the polynomial as one chain of products, two operations longer,
+// it was 0.3 to 0.7 % more of the same.
 __device__ __forceinline__ float expm1_neg(float x) {
     constexpr float kRound = 12583039.0f;  // 1.5 2^23 + 127: adding it rounds to a whole number, n + 127 in the low bits
     const float y = fminf(x, 88.0f);       // (beyond, e^-x is below half an ulp of 1 either way)
     const float t = __fmaf_rn(y, -1.44269504f, kRound);
     const float f = __fmaf_rn(__fsub_rn(t, kRound), -0.693147181f, -y);
-    float q = __fmaf_rn(0.0013882489f, f, 0.0083666919f);
-    q = __fmaf_rn(q, f, 0.0416672044f);
-    q = __fmaf_rn(q, f, 0.16666542f);
-    q = __fmaf_rn(q, f, 0.49999997f);
-    const float p = __fmaf_rn(__fmul_rn(q, f), f, f);
+    const float f2 = __fmul_rn(f, f);      // (even and odd terms apart: two operations less on the chain)
+    const float q = __fmaf_rn(__fmaf_rn(0.00138824887f, f2, __fmaf_rn(0.00836669188f, f, 0.0416672826f)), f2,
+                              __fmaf_rn(0.16666536f, f, 0.49999997f));
+    const float p = __fmaf_rn(q, f2, f);
     const float s = __int_as_float(__float_as_int(t) << 23);  // 2^n
     return __fmaf_rn(p, s, __fsub_rn(s, 1.0f));
 }
