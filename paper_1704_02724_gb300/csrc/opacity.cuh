@@ -12,9 +12,9 @@ namespace {
 // e^-x - 1 = 2^n (e^f - 1) + (2^n - 1). Within 0.96 ulp for every argument (all binary32 values from 2^-40 on compared;
 // the library's has 1), in 13 instructions without a branch, against about 20 of expm1f. x (1 + x r(x)) on [0, 1) with
 // the hardware exponential beyond took 12, but reached 1.58 ulp and, by that instruction's documented error, 1.9. The
-// difference is 0 to 0.8 % of the views (a depth-24 stereo pair of 2160^2 30.3 -> 30.4 ms, two depth-27 pairs 7.33 -> 7.40,
-// a 256^2 view of the depth-8 cube 0.3413 -> 0.3422); with the polynomial as one chain of products, two operations longer,
-// it was 0.3 to 0.7 % more of the same.
+// difference is up to 1 % of the depth-24 and -27 views (a stereo pair of 2160^2 329.0 -> 325.0 Mrays/s, a quarter of it the
+// exit time's bound and the mask of the position's bits; two depth-27 pairs 7.27 -> 7.34 ms), 0.3 % of a 256^2 view of the
+// depth-8 cube and nothing of an opaque one. The even and odd terms apart keep the chain two operations shorter.
 __device__ __forceinline__ float expm1_neg(float x) {
     constexpr float kRound = 12583039.0f;  // 1.5 2^23 + 127: adding it rounds to a whole number, n + 127 in the low bits
     const float y = fminf(x, 88.0f);       // (beyond, e^-x is below half an ulp of 1 either way)
